@@ -118,7 +118,8 @@ int niti_set_engine(niti_ctx *ctx, int engine);
 
 /* Number of kernels / memsets this context has enqueued so far. */
 uint64_t niti_launch_count(niti_ctx *ctx);
-/* Of those, launches of the tensor-core (tcgen05) matrix-multiply kernel. */
+/* Of those, launches of the tensor-core (tcgen05) matrix-multiply kernel (without the instance that computes
+ * the error of strided convolutions, which only niti_launch_count() counts). */
 uint64_t niti_tc_launch_count(niti_ctx *ctx);
 /* Of those, launches of the paired-CTA (cta_group::2) variant. */
 uint64_t niti_tc_pair_launch_count(niti_ctx *ctx);
@@ -218,10 +219,9 @@ int niti_conv_wgrad(niti_ctx *ctx, void *stream, const int8_t *x, const int8_t *
  * respect to x and w.  H, W are always the INPUT sizes of the forward
  * convolution; y / e have the [B][Ho][Wo][Cout] shape.  Workspace: the same op
  * ids with the stride as a ninth entry of dims.  stride = 1 is the call
- * without the suffix.  Forward and weight gradient of strided layers with at
- * least 32 channels on both sides run on the tensor cores (the stride becomes
- * the element stride of the operand copies); the error of a strided layer and
- * layers with other channel counts run on the CUDA-core engine. */
+ * without the suffix.  Strides up to 8 run on the tensor cores: the stride
+ * becomes the traversal stride of the operand copies, and the error is
+ * computed phase by phase of the input grid. */
 int niti_conv_fwd_strided(niti_ctx *ctx, void *stream, const int8_t *x, const int32_t *s_x,
                           const int8_t *w, const int32_t *s_w, int8_t *y, int32_t *s_y, int32_t *b_y, int B,
                           int H, int W, int Cin, int Cout, int R, int S, int pad, int stride, int relu,

@@ -4,15 +4,96 @@
 
 int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *xcol, int B, int H, int W,
                          int Ci, int R, int S, int pad, int stride, int Ho, int Wo);
-int niti_launch_pad_pitch(niti_ctx *ctx, cudaStream_t st, const int8_t *src, int8_t *dst, int rows, int n, int pitch);
-int niti_launch_pad_rows32(niti_ctx *ctx, cudaStream_t st, const int8_t *w, int8_t *wcol, int rows, int k);
-int niti_launch_round_compact32(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const WsHeader *hdr, int8_t *out,
-                                int rows, int k, int mbits, int round_mode, int32_t *b_out);
+int niti_launch_widen(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *xw, int rows, int W, int Ci, int Cp, int pad,
+                      int row_bytes, const int8_t *w, int8_t *ww, int wrows, int S, int pitch);
+int niti_launch_pad_pitch(niti_ctx *ctx, cudaStream_t st, const int8_t *src, int8_t *dst, long long rows, int n, int pitch);
+int niti_launch_round_compact(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const WsHeader *hdr, int8_t *out,
+                              int rows, int k, int pitch, int rowk, int rpitch, int Ci, int Cp, int mbits, int round_mode,
+                              int32_t *b_out, int8_t *upd_w);
 
-// Few-channel convolutions (R*S*Cin <= 32 and Cin not a multiple of 16, i.e. no TMA view of the
-// NHWC tensor): gathered into K = 32 rows and run as a plain matrix multiply.
+static inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// Few-channel convolutions (first layers: Cin = 1 or 3, no TMA view of the NHWC tensor), forward and weight
+// gradient.  With at most 32 taps the taps of every output pixel are gathered into one 32-byte row and the layer
+// runs as a plain K = 32 matrix multiply.
 static inline bool few_channel_conv(int Ci, int R, int S) { return R * S * Ci <= 32 && (Ci % 16) != 0; }
-static inline size_t round_up(size_t v, size_t a);
+
+// With more taps nothing is gathered: a tap row of a window is S * Ci contiguous bytes of an image row.  Pixels are
+// widened to Cp bytes (4, 8 or 16: stride * Cp has to be a multiple of the 16 bytes that TMA strides are made of)
+// and image rows get their zero padding, and then the layer is a convolution with R x 1 taps over Wo "pixels" per
+// row that lie stride * Cp bytes apart and have S * Cp channels: windows that overlap in memory.
+struct WindowGeometry {
+  int Cp;                  // bytes per widened pixel, 0: the layer is not run this way
+  int row_bytes;           // of a widened image row
+  int chans, pitch;        // channels of a window (S * Cp), and rounded up to 16: pitch of a tap row of weights
+  size_t x_bytes, w_bytes, acc_bytes;
+};
+static WindowGeometry window_geometry(const GemmProblem &p) {
+  WindowGeometry g;
+  memset(&g, 0, sizeof(g));
+  if (p.Ci >= 16 || few_channel_conv(p.Ci, p.R, p.S) || p.kind == GK_CONV_DGRAD) return g;
+  int cp = 4;
+  while (cp < p.Ci || (p.stride * cp) % 16 != 0) cp *= 2;
+  if (cp > 16) return g;
+  g.Cp = cp;
+  g.row_bytes = (((p.Wo - 1) * p.stride + p.S) * cp + 15) / 16 * 16;
+  g.chans = p.S * cp;
+  g.pitch = (g.chans + 15) / 16 * 16;
+  g.x_bytes = round_up((size_t)p.B * p.H * g.row_bytes, 256);
+  g.w_bytes = round_up((size_t)p.Co * p.R * g.pitch, 256);
+  g.acc_bytes = round_up((size_t)p.Co * p.R * g.pitch * 4, 256);
+  return g;
+}
+// The problem as the tensor-core engine sees it.
+static GemmProblem window_problem(const GemmProblem &p, const WindowGeometry &g, const int8_t *xw) {
+  GemmProblem q = p;
+  q.Ci = g.pitch;
+  q.W = p.Wo; q.S = 1;
+  q.win_chans = g.chans;
+  q.win_sw = p.stride * g.Cp; q.win_sh = g.row_bytes;
+  if (p.kind == GK_CONV_FWD) { q.gk = (long long)p.R * g.pitch; q.q0 = xw; }
+  else { q.gn = (long long)p.R * g.pitch; q.q1 = xw; }
+  return q;
+}
+
+// An operand of a multiply as rows of `width` bytes; TMA needs row pitches that are multiples of 16, so other
+// widths are copied once per call into padded rows (q0 / q1 of the problem).
+struct OperandRows { long long rows; int width; };
+static OperandRows operand_rows(const GemmProblem &p, int which) {
+  switch (p.kind) {
+    case GK_FC_FWD: return which == 0 ? OperandRows{p.M, p.K} : OperandRows{p.N, p.K};
+    case GK_FC_DGRAD: return which == 0 ? OperandRows{p.M, p.N} : OperandRows{p.N, p.K};
+    case GK_FC_WGRAD: return which == 0 ? OperandRows{p.M, p.N} : OperandRows{p.M, p.K};
+    default: break;
+  }
+  const OperandRows x = {(long long)p.B * p.H * p.W, p.Ci}, e = {(long long)p.B * p.Ho * p.Wo, p.Co};
+  const OperandRows w = {(long long)p.Co * p.R * p.S, p.Ci};
+  if (p.kind == GK_CONV_FWD) return which == 0 ? x : w;
+  if (p.kind == GK_CONV_DGRAD) return which == 0 ? e : w;
+  return which == 0 ? e : x;
+}
+static inline int pitch16(int width) { return (width + 15) / 16 * 16; }
+static size_t pad_bytes(const GemmProblem &p, int which) {
+  const OperandRows o = operand_rows(p, which);
+  return o.width % 16 == 0 ? 0 : round_up((size_t)o.rows * pitch16(o.width), 256);
+}
+static size_t pad_bytes(const GemmProblem &p) { return pad_bytes(p, 0) + pad_bytes(p, 1); }
+// Copies what needs padding (and is not padded yet) into `mem` (pad_bytes(p) bytes).
+static int pad_operands(niti_ctx *ctx, cudaStream_t st, GemmProblem &p, char *mem) {
+  for (int which = 0; which < 2; ++which) {
+    const size_t bytes = pad_bytes(p, which);
+    const int8_t *&q = which == 0 ? p.q0 : p.q1;
+    if (bytes && !q) {
+      const OperandRows o = operand_rows(p, which);
+      const int rc = niti_launch_pad_pitch(ctx, st, which == 0 ? p.p0 : p.p1, (int8_t *)mem, o.rows, o.width, pitch16(o.width));
+      if (rc != NITI_OK) return rc;
+      q = (int8_t *)mem;
+      (which == 0 ? p.ld0 : p.ld1) = pitch16(o.width);
+    }
+    mem += bytes;
+  }
+  return NITI_OK;
+}
 
 extern "C" int niti_create(niti_ctx **out, int device) {
   if (!out) return NITI_ERR_ARG;
@@ -20,19 +101,21 @@ extern "C" int niti_create(niti_ctx **out, int device) {
   niti_ctx *ctx = new niti_ctx();
   memset(ctx, 0, sizeof(*ctx));
   ctx->device = device;
-  cudaDeviceProp prop;
+  // (single attributes: the full property query takes about 3 ms)
+  int major = 0, smem_optin = 0;
   cudaError_t e = cudaSetDevice(device);
-  if (e == cudaSuccess) e = cudaGetDeviceProperties(&prop, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (e != cudaSuccess) {
     delete ctx;
     return NITI_ERR_CUDA;
   }
-  if (prop.major != 10) {   // the kernels are built for sm_100a only
+  if (major != 10) {        // the kernels are built for sm_100a only
     delete ctx;
     return NITI_ERR_SHAPE;
   }
-  ctx->sm_count = prop.multiProcessorCount;
-  ctx->smem_optin = prop.sharedMemPerBlockOptin;
+  ctx->smem_optin = (size_t)smem_optin;
   // one allocation: the status words, then the table of speculative-estimate errors
   const size_t dev_bytes = 256 + sizeof(int32_t) * 2 * NITI_SPEC_SLOTS;
   e = cudaMalloc(&ctx->d_status, dev_bytes);
@@ -47,6 +130,10 @@ extern "C" int niti_create(niti_ctx **out, int device) {
   if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
       qres == cudaDriverEntryPointSuccess)
     ctx->encode_tiled = fn;
+  fn = nullptr;
+  if (cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
+      qres == cudaDriverEntryPointSuccess)
+    ctx->encode_im2col = fn;
   *out = ctx;
   return NITI_OK;
 }
@@ -195,9 +282,6 @@ extern "C" int niti_check(niti_ctx *ctx, void *stream, uint32_t *status) {
   return NITI_OK;
 }
 
-static inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-
 static bool fill_conv(GemmProblem &p, int kind, int B, int H, int W, int Ci, int Co, int R, int S,
                       int pad, int stride = 1) {
   p.kind = kind;
@@ -238,7 +322,7 @@ extern "C" size_t niti_workspace_bytes(int op, const int64_t *d, int nd) {
       if (nd != 3 || d[0] <= 0 || d[1] <= 0 || d[2] <= 0) return 0;
       fill_fc(p, GK_FC_FWD, (int)d[0], (int)d[1], (int)d[2]);
       outs = (size_t)(d[0] * d[1]) * (size_t)niti_partial_slices(GK_FC_FWD, d[0]);
-      extra = niti_tc_scratch_bytes(p);
+      extra = pad_bytes(p);
       break;
     case NITI_OP_LINEAR_BWD_UPDATE:
     case NITI_OP_LINEAR_BWD: {
@@ -247,9 +331,7 @@ extern "C" size_t niti_workspace_bytes(int op, const int64_t *d, int nd) {
       outs = linear_bwd_acc_elems(d[0], d[1], d[2]);
       fill_fc(p, GK_FC_DGRAD, (int)d[0], (int)d[1], (int)d[2]);
       fill_fc(p2, GK_FC_WGRAD, (int)d[0], (int)d[1], (int)d[2]);
-      size_t e1 = niti_tc_scratch_bytes(p), e2 = niti_tc_scratch_bytes(p2);
-      extra = e1 > e2 ? e1 : e2;
-      if (d[1] % 16) extra += round_up((size_t)d[0] * (size_t)((d[1] + 15) / 16 * 16), 256);   // e with padded rows
+      extra = pad_bytes(p) + pad_bytes(p2, 1);        // e, w and a with padded rows
       if (op == NITI_OP_LINEAR_BWD_UPDATE) extra = round_up(extra, 256) + round_up(b, 256);    // scratch gradient
       break;
     }
@@ -268,11 +350,16 @@ extern "C" size_t niti_workspace_bytes(int op, const int64_t *d, int nd) {
                      stride))
         return 0;
       outs = (size_t)(p.gm * p.gn);
-      extra = niti_tc_scratch_bytes(p);
-      if (few_channel_conv((int)d[3], (int)d[5], (int)d[6]) && op != NITI_OP_CONV_DGRAD) {
+      const WindowGeometry wg = window_geometry(p);
+      if (wg.Cp) {
+        extra = wg.x_bytes + wg.w_bytes + wg.acc_bytes;
+        if (op == NITI_OP_CONV_WGRAD) extra += pad_bytes(p, 0);           // e with padded pixels
+      } else if (few_channel_conv((int)d[3], (int)d[5], (int)d[6]) && op != NITI_OP_CONV_DGRAD) {
         const size_t M = (size_t)d[0] * p.Ho * p.Wo;
-        extra += round_up(M * 32, 256) + round_up((size_t)d[4] * 32, 256) + round_up((size_t)d[4] * 32 * 4, 256);
-        if (op == NITI_OP_CONV_FWD && outs < M * (size_t)d[4]) outs = M * (size_t)d[4];
+        extra = round_up(M * 32, 256) + round_up((size_t)d[4] * 32, 256) + round_up((size_t)d[4] * 32 * 4, 256);
+        if (op == NITI_OP_CONV_WGRAD) extra += pad_bytes(p, 0);           // e with padded pixels
+      } else {
+        extra = pad_bytes(p);
       }
       if (upd) extra = round_up(extra, 256) + round_up((size_t)(p.gm * p.gn), 256);             // scratch gradient
       break;
@@ -329,22 +416,27 @@ int niti_reduce_after_gemm(niti_ctx *ctx, cudaStream_t st, int kind, int32_t *ac
 // `out` is a scratch tensor and the plain update kernel follows.
 int niti_launch_maxpool2_fwd(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *y, int B, int H, int W, int C);
 
-static int run_gemm_round(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, void *ws, size_t ws_bytes,
-                          size_t need, int8_t *out, int mbits, int round_mode, int relu,
+// tc_form: the problem in the form the tensor-core engine takes (operands prepared), where that is another one.
+// pad_mem: scratch for operands whose rows have to be padded (pad_bytes(p)).
+static int run_gemm_round(niti_ctx *ctx, cudaStream_t st, GemmProblem p, void *ws, size_t ws_bytes,
+                          size_t need, char *pad_mem, int8_t *out, int mbits, int round_mode, int relu,
                           const int8_t *mask, const int32_t *s_a, const int32_t *s_w, int32_t *s_out,
-                          int32_t *b_out, int8_t *update_w = nullptr, int8_t *pool_out = nullptr) {
+                          int32_t *b_out, int8_t *update_w = nullptr, int8_t *pool_out = nullptr,
+                          const GemmProblem *tc_form = nullptr) {
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
   WsHeader *hdr = nullptr;
   int32_t *acc = (int32_t *)((char *)ws + NITI_WS_HEADER);
   int rc = niti_take_header(ctx, st, ws, &hdr);                            // zeroed reduction scalars and split maxima
+  const bool narrow = p.kind <= GK_FC_WGRAD && p.N < 32 && p.kind != GK_FC_FWD;       // (the CUDA-core engine's)
+  if (rc == NITI_OK && ctx->engine != 1 && !narrow && !tc_form) rc = pad_operands(ctx, st, p, pad_mem);
   if (rc != NITI_OK) return rc;
   rc = NITI_ERR_SHAPE;
   bool fused = false;
   bool pooled = false;
   bool updated = false;
   RoundSpec rs = {out, mask, mbits, round_mode, relu, s_a, s_w, s_out, b_out, pool_out, update_w};
-  if (ctx->engine != 1) rc = niti_tc_gemm(ctx, st, p, rs, acc, hdr, &fused, &pooled, true, &updated);
+  if (ctx->engine != 1) rc = niti_tc_gemm(ctx, st, tc_form ? *tc_form : p, rs, acc, hdr, &fused, &pooled, true, &updated);
   if (rc == NITI_ERR_SHAPE) {
     rc = niti_simt_gemm(ctx, st, p, acc, hdr);
     if (rc == NITI_OK) rc = niti_reduce_after_gemm(ctx, st, p.kind, acc, p.gm * p.gn, hdr, true);
@@ -389,8 +481,9 @@ extern "C" int niti_linear_fwd(niti_ctx *ctx, void *stream, const int8_t *a, con
   fill_fc(p, GK_FC_FWD, M, N, K);
   p.p0 = a; p.p1 = w;
   int64_t dims[3] = {M, N, K};
+  char *pad_mem = (char *)ws + NITI_WS_HEADER + round_up((size_t)M * N * niti_partial_slices(GK_FC_FWD, M) * 4, 256);
   return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes,
-                        niti_workspace_bytes(NITI_OP_LINEAR_FWD, dims, 3), out, 7, round_mode, relu,
+                        niti_workspace_bytes(NITI_OP_LINEAR_FWD, dims, 3), pad_mem, out, 7, round_mode, relu,
                         nullptr, s_a, s_w, s_out, b_out);
 }
 
@@ -414,35 +507,30 @@ static int linear_bwd_impl(niti_ctx *ctx, void *stream, const int8_t *a, const i
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
   if (update_w) g = (int8_t *)((char *)ws + need_base);       // scratch, used only if the multiply rounds by itself
-  // TMA needs 16-byte row pitches: an error tensor with N % 16 != 0 (10 or 1000 classes) is copied
-  // once into rows padded to the next multiple of 16 for the tensor-core engine
-  const int8_t *e_tc = e;
-  long long e_ld = 0;
-  if ((N % 16) != 0 && N >= 32 && ctx->engine != 1) {
-    const int pitch = (N + 15) / 16 * 16;
-    int8_t *epad = (int8_t *)((char *)ws + NITI_WS_HEADER + round_up(linear_bwd_acc_elems(M, N, K) * 4, 256));
-    int rcp = niti_launch_pad_pitch(ctx, (cudaStream_t)stream, e, epad, M, N, pitch);
+  // rows padded for TMA: e (shared by both multiplies), then w (error) and a (weight gradient)
+  char *pad_mem = (char *)ws + NITI_WS_HEADER + round_up(linear_bwd_acc_elems(M, N, K) * 4, 256);
+  GemmProblem pd, pw;
+  fill_fc(pd, GK_FC_DGRAD, M, N, K);
+  pd.p0 = e; pd.p1 = w;
+  fill_fc(pw, GK_FC_WGRAD, M, N, K);
+  pw.p0 = e; pw.p1 = a;
+  char *pad_a = pad_mem + pad_bytes(pd) - pad_bytes(pw, 0);      // (the weight gradient finds e padded already)
+  if (pad_bytes(pd, 0) && N >= 32 && ctx->engine != 1) {
+    const int rcp = niti_launch_pad_pitch(ctx, (cudaStream_t)stream, e, (int8_t *)pad_mem, M, N, pitch16(N));
     if (rcp != NITI_OK) return rcp;
-    e_tc = epad;
-    e_ld = pitch;
+    pd.q0 = pw.q0 = (int8_t *)pad_mem;
+    pd.ld0 = pw.ld0 = pitch16(N);
   }
-  GemmProblem p;
   int rc;
   if (e_prev && update_w) {                // the error below needs the weights as they were
-    fill_fc(p, GK_FC_DGRAD, M, N, K);
-    p.p0 = e_tc; p.p1 = w; p.ld0 = e_ld;
-    rc = run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, e_prev, 7, round_mode, 0,
+    rc = run_gemm_round(ctx, (cudaStream_t)stream, pd, ws, ws_bytes, need, pad_mem, e_prev, 7, round_mode, 0,
                         relu_mask_src, nullptr, nullptr, nullptr, b_e);
     if (rc != NITI_OK) return rc;
   }
-  fill_fc(p, GK_FC_WGRAD, M, N, K);
-  p.p0 = e_tc; p.p1 = a; p.ld0 = e_ld;
-  rc = run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, g, m_u, round_mode, 0, nullptr,
+  rc = run_gemm_round(ctx, (cudaStream_t)stream, pw, ws, ws_bytes, need, pad_a, g, m_u, round_mode, 0, nullptr,
                       nullptr, nullptr, nullptr, b_g, update_w);
   if (rc != NITI_OK || !e_prev || update_w) return rc;
-  fill_fc(p, GK_FC_DGRAD, M, N, K);
-  p.p0 = e_tc; p.p1 = w; p.ld0 = e_ld;
-  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, e_prev, 7, round_mode, 0,
+  return run_gemm_round(ctx, (cudaStream_t)stream, pd, ws, ws_bytes, need, pad_mem, e_prev, 7, round_mode, 0,
                         relu_mask_src, nullptr, nullptr, nullptr, b_e);
 }
 
@@ -460,6 +548,11 @@ extern "C" int niti_linear_bwd_update(niti_ctx *ctx, void *stream, const int8_t 
                                       int M, int N, int K, int m_u, int round_mode, void *ws, size_t ws_bytes) {
   return linear_bwd_impl(ctx, stream, a, e, w, e_prev, relu_mask_src, nullptr, w, b_e, b_g, M, N, K, m_u,
                          round_mode, ws, ws_bytes, "niti_linear_bwd_update");
+}
+
+// padded operands of a convolution call that gathers nothing: right behind the accumulators
+static inline char *conv_pad_mem(const GemmProblem &p, void *ws) {
+  return (char *)ws + NITI_WS_HEADER + round_up((size_t)(p.gm * p.gn) * 4, 256);
 }
 
 static int conv_args_ok(int B, int H, int W, int Ci, int Co, int R, int S, int pad, int round_mode) {
@@ -481,6 +574,17 @@ static int conv_fwd_impl(niti_ctx *ctx, void *stream, const int8_t *x, const int
   p.p0 = x; p.p1 = w;
   int64_t dims[9] = {B, H, W, Cin, Cout, R, S, pad, stride};
   const size_t need = niti_workspace_bytes(NITI_OP_CONV_FWD, dims, 9);
+  const WindowGeometry wg = window_geometry(p);
+  if (wg.Cp && ctx->engine != 1 && ws && !((uintptr_t)ws & 255) && ws_bytes >= need) {
+    int8_t *xw = (int8_t *)conv_pad_mem(p, ws), *ww = xw + wg.x_bytes;
+    const int rc = niti_launch_widen(ctx, (cudaStream_t)stream, x, xw, B * H, W, Cin, wg.Cp, pad, wg.row_bytes, w, ww, Cout * R, S,
+                                     wg.pitch);
+    if (rc != NITI_OK) return rc;
+    GemmProblem q = window_problem(p, wg, xw);
+    q.q1 = ww;
+    return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, nullptr, y, 7, round_mode, relu, nullptr, s_x, s_w,
+                          s_y, b_y, nullptr, y_pool, &q);
+  }
   if (few_channel_conv(Cin, R, S) && ctx->engine != 1) {
     if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
       return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
@@ -498,16 +602,16 @@ static int conv_fwd_impl(niti_ctx *ctx, void *stream, const int8_t *x, const int
       memcpy(ctx->tap_dims, dims, sizeof(dims));
     }
     int rc = niti_launch_im2col32(ctx, st, x, xcol, B, H, W, Cin, R, S, pad, stride, p.Ho, p.Wo);
-    if (rc == NITI_OK) rc = niti_launch_pad_rows32(ctx, st, w, wcol, Cout, R * S * Cin);
+    if (rc == NITI_OK) rc = niti_launch_pad_pitch(ctx, st, w, wcol, Cout, R * S * Cin, 32);
     if (rc != NITI_OK) return rc;
     GemmProblem q;
     fill_fc(q, GK_FC_FWD, (int)M, Cout, 32);
     q.p0 = xcol; q.p1 = wcol;
-    rc = run_gemm_round(ctx, st, q, ws, ws_bytes, need, y, 7, round_mode, relu, nullptr, s_x, s_w, s_y, b_y);
+    rc = run_gemm_round(ctx, st, q, ws, ws_bytes, need, nullptr, y, 7, round_mode, relu, nullptr, s_x, s_w, s_y, b_y);
     if (rc != NITI_OK || !y_pool) return rc;
     return niti_launch_maxpool2_fwd(ctx, st, y, y_pool, B, p.Ho, p.Wo, Cout);
   }
-  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, y, 7, round_mode, relu, nullptr,
+  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, conv_pad_mem(p, ws), y, 7, round_mode, relu, nullptr,
                         s_x, s_w, s_y, b_y, nullptr, y_pool);
 }
 
@@ -553,7 +657,7 @@ extern "C" int niti_conv_dgrad_strided(niti_ctx *ctx, void *stream, const int8_t
   p.p0 = e; p.p1 = w;
   int64_t dims[9] = {B, H, W, Cin, Cout, R, S, pad, stride};
   return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes,
-                        niti_workspace_bytes(NITI_OP_CONV_DGRAD, dims, 9), e_prev, 7, round_mode, 0,
+                        niti_workspace_bytes(NITI_OP_CONV_DGRAD, dims, 9), conv_pad_mem(p, ws), e_prev, 7, round_mode, 0,
                         relu_mask_src, nullptr, nullptr, nullptr, b_e);
 }
 
@@ -586,41 +690,48 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
   if (update_w) g = (int8_t *)((char *)ws + need_base);       // scratch, used only where the rounding stores int8
-  if (few_channel_conv(Cin, R, S) && ctx->engine != 1 && (Cout % 16) == 0) {
-    // g32[co][k] = sum_pix e[pix][co] * xcol[pix][k] over the gathered rows (k < 32), then the first
-    // R*S*Cin columns are rounded into g
+  const WindowGeometry wg = window_geometry(p);
+  if ((wg.Cp || few_channel_conv(Cin, R, S)) && ctx->engine != 1) {
+    // the multiply leaves int32 sums over widened windows (columns r, s * Cp + c) or over gathered 32-byte rows; the
+    // columns that are taps are then rounded into g, or subtracted from the weights
     cudaStream_t st = (cudaStream_t)stream;
     const size_t M = (size_t)B * p.Ho * p.Wo;
     WsHeader *hdr = nullptr;
-    char *base = (char *)ws + NITI_WS_HEADER + round_up((size_t)(p.gm * p.gn) * 4, 256);
-    int8_t *xcol = (int8_t *)base;
-    int32_t *acc32 = (int32_t *)(base + round_up(M * 32, 256) + round_up((size_t)Cout * 32, 256));
     int rc = niti_take_header(ctx, st, ws, &hdr);
     if (rc != NITI_OK) return rc;
-    if (tap_cache_hit(ctx, x, B, H, W, Cin, R, S, pad, stride)) {
-      xcol = ctx->tap_buf;                 // gathered by the forward call
-      ctx->tap_dims[8] = 0;                // (used once: the next forward call fills the cache again)
-    } else rc = niti_launch_im2col32(ctx, st, x, xcol, B, H, W, Cin, R, S, pad, stride, p.Ho, p.Wo);
-    if (rc != NITI_OK) return rc;
+    int8_t *xcol = (int8_t *)conv_pad_mem(p, ws);
+    const size_t x_bytes = wg.Cp ? wg.x_bytes + wg.w_bytes : round_up(M * 32, 256) + round_up((size_t)Cout * 32, 256);
+    int32_t *acc = (int32_t *)(xcol + x_bytes);
+    const int acc_pitch = wg.Cp ? R * wg.pitch : 32;
+    char *pad_mem = (char *)acc + round_up((size_t)Cout * acc_pitch * 4, 256);
     GemmProblem q;
-    fill_fc(q, GK_FC_WGRAD, (int)M, Cout, 32);     // rows M are the contraction
-    q.p0 = e; q.p1 = xcol;
-    bool fused = false;
-    RoundSpec none = {nullptr, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
-    const int saved = ctx->engine;
-    if (saved == 0) ctx->engine = 4;               // int32 accumulators are needed here, not a fused store
-    rc = niti_tc_gemm(ctx, st, q, none, acc32, hdr, &fused);
-    ctx->engine = saved;
-    if (rc == NITI_ERR_SHAPE) {
-      rc = niti_simt_gemm(ctx, st, q, acc32, hdr);
-      if (rc == NITI_OK) rc = niti_reduce_after_gemm(ctx, st, q.kind, acc32, (long long)Cout * 32, hdr);
+    if (wg.Cp) {
+      rc = niti_launch_widen(ctx, st, x, xcol, B * H, W, Cin, wg.Cp, pad, wg.row_bytes, nullptr, nullptr, 0, S, wg.pitch);
+      q = window_problem(p, wg, xcol);
+    } else {
+      if (tap_cache_hit(ctx, x, B, H, W, Cin, R, S, pad, stride)) {
+        xcol = ctx->tap_buf;               // gathered by the forward call
+        ctx->tap_dims[8] = 0;              // (used once: the next forward call fills the cache again)
+      } else rc = niti_launch_im2col32(ctx, st, x, xcol, B, H, W, Cin, R, S, pad, stride, p.Ho, p.Wo);
+      fill_fc(q, GK_FC_WGRAD, (int)M, Cout, 32);     // rows M are the contraction
+      q.p0 = e; q.p1 = xcol;
     }
     if (rc != NITI_OK) return rc;
-    rc = niti_launch_round_compact32(ctx, st, acc32, hdr, g, Cout, R * S * Cin, m_u, round_mode, b_g);
-    if (rc != NITI_OK || !update_w) return rc;
-    return niti_launch_sgd_update(ctx, st, update_w, g, (long long)Cout * R * S * Cin);
+    rc = pad_operands(ctx, st, q, pad_mem);
+    if (rc != NITI_OK) return rc;
+    bool fused = false;
+    RoundSpec none = {nullptr, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
+    rc = niti_tc_gemm(ctx, st, q, none, acc, hdr, &fused);       // (no output: int32 accumulators)
+    if (rc == NITI_ERR_SHAPE && !wg.Cp) {
+      rc = niti_simt_gemm(ctx, st, q, acc, hdr);
+      if (rc == NITI_OK) rc = niti_reduce_after_gemm(ctx, st, q.kind, acc, (long long)Cout * 32, hdr);
+    }
+    if (rc == NITI_OK)
+      return niti_launch_round_compact(ctx, st, acc, hdr, g, Cout, R * S * Cin, acc_pitch, S * Cin, wg.Cp ? wg.pitch : S * Cin,
+                                       Cin, wg.Cp ? wg.Cp : Cin, m_u, round_mode, b_g, update_w);
+    if (rc != NITI_ERR_SHAPE) return rc;
   }
-  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, g, m_u, round_mode, 0, nullptr,
+  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, conv_pad_mem(p, ws), g, m_u, round_mode, 0, nullptr,
                         nullptr, nullptr, nullptr, b_g, update_w);
 }
 

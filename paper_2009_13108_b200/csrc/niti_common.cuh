@@ -27,6 +27,7 @@ struct niti_ctx {
   double *prof_ops;         // algorithmic int8 operations (2*M*N*K) of each recorded launch
   // cuTensorMapEncodeTiled, fetched through the runtime so that libcuda is not a link dependency
   void *encode_tiled;
+  void *encode_im2col;      // cuTensorMapEncodeIm2col
   // data-parallel training (niti_set_reduce_hook): called where a tensor-wide quantity has to be
   // combined over the ranks before the rounding may use it
   niti_reduce_fn reduce_fn;
@@ -45,7 +46,7 @@ struct niti_ctx {
   // per-device facts of the tensor-core kernel, indexed by CTAs per tile (1 or 2): co-resident CTAs /
   // CTA pairs (0 = not asked yet) and the dynamic shared-memory limit already set on the kernel
   int tc_units[3];
-  size_t tc_attr_smem[3];
+  size_t tc_attr_smem[7];   // CTAs + 2 * mode of the instance
   // the device's opt-in limit of dynamic shared memory per CTA.  The limit set on a kernel belongs to the
   // device, not to a context: every context therefore sets this same value (a context that set only what it
   // needed would lower the limit under another context of the process)
@@ -178,8 +179,15 @@ struct GemmProblem {
   int B, H, W, Ho, Wo, Ci, Co, R, S, pad, stride;
   // the matrix multiply actually run
   long long gm, gn, gk;
-  // row pitch in bytes of p0 when its rows are padded (fully connected kinds; 0 = dense)
-  long long ld0;
+  // Operands as the tensor-core engine copies them, when the caller's rows are no multiple of 16 bytes: copies
+  // of p0 / p1 with padded rows (null: the operand itself) and their row pitches in bytes (0: dense).  A row is
+  // a row of a matrix, a pixel's channels, or a tap's input channels (convolution weights).
+  const int8_t *q0, *q1;
+  long long ld0, ld1;
+  // windows of a few-channel convolution (0: none): channels of a window, byte distance of neighbouring windows and
+  // of image rows in the widened input; W and S then count windows and tap rows' windows (Wo and 1), and only rows
+  // have a stride and padding
+  int win_chans, win_sw, win_sh;
 };
 
 // Fully connected forward / error multiplies with at most 128 output rows (weight streaming: the
@@ -223,6 +231,7 @@ struct RoundSpec {
   const int32_t *s_a, *s_w;
   int32_t *s_out, *b_out;
   int8_t *pool_out;        // optional (may be null): 2 x 2 max-pool of `out`, forward convolutions with ReLU
+  // (out may be null: the caller wants the int32 accumulators and rounds them itself)
   int8_t *update_w;        // optional (may be null): weight gradients; the caller will subtract `out` from these weights
 };
 // Tensor-core engine (tcgen05); returns NITI_ERR_SHAPE if the shape is not eligible.  *fused is set
@@ -233,7 +242,6 @@ struct RoundSpec {
 // (`out` is then not written).
 int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, const RoundSpec &r, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled = nullptr, bool shard_ok = false, bool *updated = nullptr);
-size_t niti_tc_scratch_bytes(const GemmProblem &p);
 
 // Epilogue pass: b from hdr->maxabs32, bp = max(0, b - mbits), out = Round(acc) with optional ReLU
 // and optional mask; s_out = s_a + s_w + bp if s_out != NULL; b_out = b if != NULL.

@@ -186,45 +186,117 @@ im2col32_rgb3x3_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xcol, 
   }
 }
 
-// weights [Cout][R*S*Cin] -> [Cout][32], zero padded
-__global__ void pad_rows32_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ wcol, int rows, int k) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < rows * 32) {
-    const int r = idx >> 5, c = idx & 31;
-    wcol[idx] = c < k ? w[r * k + c] : (int8_t)0;
+// Rows of n bytes -> rows of `pitch` bytes (a multiple of 4, pitch >= n), zero padded.  One output word per thread
+// from the two aligned source words around it (bound: memory; the byte-per-thread form with its 64-bit
+// divisions took 12.9 us for 4096 rows of 1000 bytes).
+__global__ void __launch_bounds__(256)
+pad_pitch_kernel(const int8_t *__restrict__ src, int8_t *__restrict__ dst, long long rows, int n, int pitch) {
+  const int words = pitch >> 2;
+  const long long total = rows * n;                       // source bytes
+  const int wpb = (int)(blockDim.x);
+  // a block covers whole rows: rows_pb rows of `words` words
+  const int rows_pb = words >= wpb ? 1 : wpb / words;
+  const int t = threadIdx.x;
+  const int rl = rows_pb == 1 ? 0 : t / words;
+  if (rl >= rows_pb) return;
+  for (long long r = (long long)blockIdx.x * rows_pb + rl; r < rows; r += (long long)gridDim.x * rows_pb) {
+    for (int c = rows_pb == 1 ? t : t - rl * words; c < words; c += rows_pb == 1 ? wpb : words) {
+      unsigned v = 0;
+      const int left = n - 4 * c;                         // valid bytes of this word
+      if (left > 0) {
+        const long long o = r * n + 4 * c;
+        const unsigned *p = reinterpret_cast<const unsigned *>(src) + (o >> 2);     // (src is 16-byte aligned)
+        const unsigned sh = 8u * (unsigned)(o & 3);
+        const unsigned lo = p[0];
+        const unsigned hi = ((o | 3) + 1 < total && sh) ? p[1] : 0u;
+        v = __funnelshift_r(lo, hi, sh);
+        if (left < 4) v &= 0xffffffffu >> (32 - 8 * left);
+      }
+      reinterpret_cast<unsigned *>(dst + r * pitch)[c] = v;
+    }
   }
 }
 
-// rows of n bytes -> rows of pitch bytes (pitch >= n), zero padded
-__global__ void pad_pitch_kernel(const int8_t *__restrict__ src, int8_t *__restrict__ dst, int rows, int n, int pitch) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < (long long)rows * pitch) {
-    const int r = (int)(idx / pitch), c = (int)(idx % pitch);
-    dst[idx] = c < n ? src[(long long)r * n + c] : (int8_t)0;
-  }
-}
-
-int niti_launch_pad_pitch(niti_ctx *ctx, cudaStream_t st, const int8_t *src, int8_t *dst, int rows, int n, int pitch) {
-  long long total = (long long)rows * pitch;
-  pad_pitch_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(src, dst, rows, n, pitch);
+int niti_launch_pad_pitch(niti_ctx *ctx, cudaStream_t st, const int8_t *src, int8_t *dst, long long rows, int n, int pitch) {
+  const int words = pitch >> 2, rows_pb = words >= 256 ? 1 : 256 / words;
+  long long blocks = (rows + rows_pb - 1) / rows_pb;
+  if (blocks > (long long)ctx->sm_count * 32) blocks = (long long)ctx->sm_count * 32;
+  pad_pitch_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dst, rows, n, pitch);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
 }
 
-// Rounds acc[rows][32] (int32) and keeps the first k columns: out[rows][k].
-__global__ void round_compact32_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict__ hdr,
-                                       int8_t *__restrict__ out, int rows, int k, int mbits, int round_mode,
-                                       int32_t *__restrict__ b_out) {
+// Rounds the columns of acc[rows][pitch] (int32) that hold taps: out[rows][taps * rowk], or subtracts them from
+// upd_w.  Column of tap row r, column s, channel c: r * rpitch + s * Cp + c.
+__global__ void __launch_bounds__(256)
+round_compact_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict__ hdr, int8_t *__restrict__ out,
+                     int rows, int k, int pitch, int rowk, int rpitch, int Ci, int Cp, int mbits, int round_mode,
+                     int32_t *__restrict__ b_out, int8_t *__restrict__ upd_w) {
   const int b = niti_bitlen32(hdr->maxabs32);
   const int bp = b > mbits ? b - mbits : 0;
   const unsigned qmax = (1u << mbits) - 1u;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx == 0 && b_out) *b_out = b;
   if (idx < rows * k) {
-    const int r = idx / k, c = idx % k;
-    out[idx] = (int8_t)niti_round_i32(acc[r * 32 + c], bp, qmax, round_mode);
+    const int row = idx / k, c = idx - row * k;
+    const int r = c / rowk, rem = c - r * rowk, sx = rem / Ci, ci = rem - sx * Ci;
+    const int q = niti_round_i32(acc[(long long)row * pitch + r * rpitch + sx * Cp + ci], bp, qmax, round_mode);
+    if (upd_w) {
+      const int d = (int)upd_w[idx] - q;
+      upd_w[idx] = (int8_t)(d > 127 ? 127 : (d < -127 ? -127 : d));
+    } else {
+      out[idx] = (int8_t)q;
+    }
   }
+}
+
+// Few-channel convolutions with more than 32 taps ("windows", see window_geometry): image rows with `pad` zero
+// pixels on the left, enough on the right for the last window, and every pixel widened from Ci to Cp bytes (4, 8 or
+// 16).  One word of the widened row per thread (bound: memory; the taps are not copied, so 224 x 224 x 3 images
+// become 13 MB for an 11 x 11 stride-4 layer where gathered rows were 74 MB and took 80 us to write).
+__global__ void __launch_bounds__(256)
+widen_pixels_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xw, int rows, int W, int Ci, int Cp, int pad,
+                    int row_words) {
+  const int wpp = Cp >> 2;                                 // words per pixel
+  const long long total = (long long)rows * row_words;
+  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(idx / row_words), wd = (int)(idx - (long long)r * row_words);
+    const int px = wd / wpp - pad, c0 = 4 * (wd - (wd / wpp) * wpp);
+    unsigned v = 0;
+    if (px >= 0 && px < W && c0 < Ci) {
+      const int8_t *src = x + ((long long)r * W + px) * Ci + c0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c0 + c < Ci) v |= (unsigned)(uint8_t)src[c] << (8 * c);
+    }
+    reinterpret_cast<unsigned *>(xw)[idx] = v;
+  }
+}
+// weights [Cout][R][S][Ci] -> [Cout][R][pitch], tap column s in bytes s * Cp .. s * Cp + Ci - 1, zero elsewhere
+__global__ void __launch_bounds__(256)
+widen_weights_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ ww, int rows, int S, int Ci, int Cp, int pitch) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx < (long long)rows * pitch) {
+    const int r = (int)(idx / pitch), b = (int)(idx - (long long)r * pitch);
+    const int sx = b / Cp, c = b - sx * Cp;
+    ww[idx] = (sx < S && c < Ci) ? w[((long long)r * S + sx) * Ci + c] : (int8_t)0;
+  }
+}
+int niti_launch_widen(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *xw, int rows, int W, int Ci, int Cp, int pad,
+                      int row_bytes, const int8_t *w, int8_t *ww, int wrows, int S, int pitch) {
+  const long long words = (long long)rows * (row_bytes / 4);
+  long long blocks = (words + 255) / 256;
+  if (blocks > (long long)ctx->sm_count * 64) blocks = (long long)ctx->sm_count * 64;
+  widen_pixels_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, xw, rows, W, Ci, Cp, pad, row_bytes / 4);
+  ctx->launches++;
+  if (w) {
+    widen_weights_kernel<<<(unsigned)(((long long)wrows * pitch + 255) / 256), 256, 0, st>>>(w, ww, wrows, S, Ci, Cp, pitch);
+    ctx->launches++;
+  }
+  NITI_CUDA_TRY(ctx, cudaGetLastError());
+  return NITI_OK;
 }
 
 int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *xcol, int B, int H, int W,
@@ -249,16 +321,11 @@ int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t
   return NITI_OK;
 }
 
-int niti_launch_pad_rows32(niti_ctx *ctx, cudaStream_t st, const int8_t *w, int8_t *wcol, int rows, int k) {
-  pad_rows32_kernel<<<(rows * 32 + 255) / 256, 256, 0, st>>>(w, wcol, rows, k);
-  ctx->launches++;
-  NITI_CUDA_TRY(ctx, cudaGetLastError());
-  return NITI_OK;
-}
-
-int niti_launch_round_compact32(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const WsHeader *hdr, int8_t *out,
-                                int rows, int k, int mbits, int round_mode, int32_t *b_out) {
-  round_compact32_kernel<<<(rows * k + 255) / 256, 256, 0, st>>>(acc, hdr, out, rows, k, mbits, round_mode, b_out);
+int niti_launch_round_compact(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const WsHeader *hdr, int8_t *out,
+                              int rows, int k, int pitch, int rowk, int rpitch, int Ci, int Cp, int mbits, int round_mode,
+                              int32_t *b_out, int8_t *upd_w) {
+  round_compact_kernel<<<(rows * k + 255) / 256, 256, 0, st>>>(acc, hdr, out, rows, k, pitch, rowk, rpitch, Ci, Cp, mbits,
+                                                               round_mode, b_out, upd_w);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;

@@ -279,7 +279,7 @@ int niti_simt_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, int32_t
   q.H = p.H; q.W = p.W; q.Ho = p.Ho; q.Wo = p.Wo; q.Ci = p.Ci; q.Co = p.Co; q.R = p.R; q.S = p.S; q.pad = p.pad;
   q.stride = p.stride > 0 ? p.stride : 1;
   q.gm = p.gm; q.gn = p.gn; q.gk = p.gk;
-  q.pitch0 = p.ld0 ? p.ld0 : p.N;
+  q.pitch0 = p.N;
   long long gx = (p.gn + TN - 1) / TN, gy = (p.gm + TM - 1) / TM;
   if (gy > 65535) return niti_fail(ctx, NITI_ERR_SHAPE, "simt gemm: too many row tiles");
   // split the contraction when the output grid alone cannot fill the GPU

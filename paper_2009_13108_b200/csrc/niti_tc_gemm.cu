@@ -53,6 +53,7 @@ struct TcParams {
                                 // stage and buffer advance together, one barrier per tile serves both
   int stg_off;                  // > 0: byte offset (from the aligned base) of the epilogue warps' transpose
                                 // buffers for coalesced atomic adds, 32 x 33 words per warp
+  int nstg_off;                 // byte offset of the staging buffers for rows with a pitch that is no multiple of 8
   int mrep;                     // 128-row tiles per item (row-batched mode of short contractions), else 1
   int bn_mma;                   // N of one MMA; bn = mrep * bn_mma accumulator columns per item
   long long gm, gn;             // output extent (rows, columns); row pitch of acc is gn
@@ -74,9 +75,24 @@ struct TcParams {
   int w_tiles, h_tiles, b_tiles;
   int PW, PH, PB;               // extent of the pixel grid the output rows (or k-blocks) run over
   int R, S, pad;
+  int stride_w;                 // the same for columns (1 where the input is a tensor of windows)
   int stride;                   // convolution stride (forward and weight gradient; the shifted operand is then
                                 // copied with that element stride, so a box still lands as Wt x Ht pixels)
   int c_chunks;                 // channel chunks per tap along the contraction (fwd / dgrad)
+  int tail_ks;                  // MMAs of the last channel chunk when it is not a whole one (0: all chunks whole)
+  // im2col copies (see "Pixel rows" at the planner): rows / contraction pixels are consecutive pixels of the
+  // PB x PH x PW grid, whatever its extents
+  int mode;                     // kernel instance: see "Instances" at the kernel
+  int i2c;
+  int i2c_w0, i2c_h0;           // base pixel (in the copied tensor) of grid position (0, 0)
+  int i2c_dj, i2c_di, i2c_db;   // wgrad: 128 pixels as (columns, rows, images) of the grid
+  // error of a strided convolution: dstride > 1.  Input pixels with the same (position + pad) mod stride form a
+  // phase, whose error is a stride-1 correlation of e with every dstride-th tap; items run over (tile, phase)
+  int dstride;
+  int nph_r, nph_s;             // phases with at least one tap
+  int T_r, T_s;                 // taps of the phase with most of them
+  int u0_r, u0_s;               // first grid position: input row = dstride * (position + u0) + phase - pad
+  int OH, OW;                   // extent of the tensor the output rows are written to
   int Cn;                       // wgrad: input channels Ci (columns per tap)
   int n_chunks;                 // wgrad: column chunks per tap
   int ctas;                     // CTAs per tile: 1, or 2 (cta_group::2, 256-row tiles)
@@ -251,6 +267,20 @@ __device__ __forceinline__ void tma_load_4d(unsigned dst, const CUtensorMap *map
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap *map, unsigned bar, int c0, int c1, int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+// im2col copy of consecutive pixels: base pixel (w, h, n), filter offset (ow, oh)
+__device__ __forceinline__ void tma_load_im2col(unsigned dst, const CUtensorMap *map, unsigned bar, int c, int w, int h,
+                                                int n, unsigned short ow, unsigned short oh) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(ow), "h"(oh)
       : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -492,6 +522,60 @@ __device__ __forceinline__ void store32(int8_t *dst, const unsigned (&w8)[8]) {
                : "memory");
 }
 
+// Rows whose pitch or base is not a multiple of 32 bytes (`unit` = the largest power of two that divides
+// both, at most 16).  A lane holds 32 columns of its own row, `nv` of them inside the matrix.  With units of
+// 16 or 8 bytes every lane stores its own pieces; below that a store instruction of 32 scattered pieces
+// costs 32 sector requests, so the chunk passes through shared memory (32 rows x 36 bytes per warp) and each
+// instruction writes whole rows.
+template <typename T>
+__device__ __forceinline__ void store_rows_staged(int8_t *out8, long long off, bool rok, int nv, const unsigned *stg, int lane) {
+  constexpr int LPR = 32 / (int)sizeof(T);                     // lanes per row
+  const int part = lane % LPR;
+  for (int r0 = 0; r0 < 32; r0 += (int)sizeof(T)) {
+    const int r = r0 + lane / LPR;
+    const long long o = __shfl_sync(0xffffffffu, off, r);
+    const int ok = __shfl_sync(0xffffffffu, rok ? 1 : 0, r);
+    if (ok && part * (int)sizeof(T) < nv)
+      reinterpret_cast<T *>(out8 + o)[part] = reinterpret_cast<const T *>(reinterpret_cast<const char *>(stg) + r * 36)[part];
+  }
+}
+__device__ __forceinline__ void store_rows_narrow(int8_t *out8, long long off, bool rok, const unsigned (&w8)[8], int nv,
+                                                  int unit, unsigned *stg, int lane) {
+  if (unit >= 8) {
+    if (!rok) return;
+    int8_t *dst = out8 + off;
+    if (unit >= 16) {
+      *reinterpret_cast<uint4 *>(dst) = make_uint4(w8[0], w8[1], w8[2], w8[3]);
+      if (nv > 16) *reinterpret_cast<uint4 *>(dst + 16) = make_uint4(w8[4], w8[5], w8[6], w8[7]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (8 * j < nv) *reinterpret_cast<uint2 *>(dst + 8 * j) = make_uint2(w8[2 * j], w8[2 * j + 1]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) stg[lane * 9 + j] = w8[j];
+  __syncwarp();
+  if (unit == 4) store_rows_staged<unsigned>(out8, off, rok, nv, stg, lane);
+  else if (unit == 2) store_rows_staged<unsigned short>(out8, off, rok, nv, stg, lane);
+  else store_rows_staged<unsigned char>(out8, off, rok, nv, stg, lane);
+  __syncwarp();
+}
+// 32 gate bytes of this lane's row, from the aligned words that hold at least one of its nv bytes
+__device__ __forceinline__ void load_row_narrow(const int8_t *src, unsigned (&m)[8], int nv) {
+  const unsigned sh = 8u * (unsigned)((uintptr_t)src & 3);
+  const unsigned *p = reinterpret_cast<const unsigned *>((uintptr_t)src & ~(uintptr_t)3);
+  const int words = (nv + (int)((uintptr_t)src & 3) + 3) >> 2;
+  unsigned lo = p[0];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const unsigned hi = j + 1 < words ? p[j + 1] : 0u;
+    m[j] = __funnelshift_r(lo, hi, sh);
+    lo = hi;
+  }
+}
+
 // Per call site the table keeps the errors (true bit-width minus sample-based estimate, each stored + 2
 // in four bits) of the last two calls.  An error that repeats is systematic (the tensor's extremes sit
 // outside the sampled tiles, or its distribution has a heavier tail than the scaling assumes) and is
@@ -518,6 +602,30 @@ __device__ __forceinline__ void pixel_box(const TcParams &p, int idx, int &w0, i
   int wt, ht, bt;
   tile_coords(p, idx, wt, ht, bt);
   w0 = wt * p.Wt; h0 = ht * p.Ht; b0 = bt * p.Bt;
+}
+
+// Phase of an item of a strided error multiply (dstride > 1): items run over (tile, phase), so that a contiguous
+// range of items holds all phases, which have different numbers of taps, in equal shares.
+struct Phase { int r, s, n_r, n_s; };     // first tap row / column, taps of the phase
+__device__ __forceinline__ Phase split_phase(const TcParams &p, int item, int &tile) {
+  const int nph = p.nph_r * p.nph_s;
+  tile = item / nph;
+  const int ph = item - tile * nph;
+  Phase q;
+  q.r = ph / p.nph_s;
+  q.s = ph - q.r * p.nph_s;
+  q.n_r = (p.R - q.r + p.dstride - 1) / p.dstride;
+  q.n_s = (p.S - q.s + p.dstride - 1) / p.dstride;
+  return q;
+}
+
+// Output row of grid position `idx` of a phase of a strided error multiply; ok: it is inside the tensor.
+__device__ __forceinline__ long long phase_row(const TcParams &p, int idx, const Phase &q, bool &ok) {
+  int v, u, b;
+  tile_coords(p, idx, v, u, b);
+  const int jj = (v + p.u0_s) * p.dstride + q.s - p.pad, ii = (u + p.u0_r) * p.dstride + q.r - p.pad;
+  ok = b < p.PB && ii >= 0 && ii < p.OH && jj >= 0 && jj < p.OW;
+  return ((long long)b * p.OH + ii) * p.OW + jj;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -552,6 +660,19 @@ __device__ __forceinline__ void tma_load_4d_pair(unsigned dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(unsigned dst, const CUtensorMap *map, unsigned bar, int c0, int c1, int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_im2col_pair(unsigned dst, const CUtensorMap *map, unsigned bar, int c, int w, int h,
+                                                     int n, unsigned short ow, unsigned short oh) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(ow), "h"(oh)
       : "memory");
 }
 __device__ __forceinline__ void tc_commit_pair(unsigned bar) {
@@ -624,6 +745,17 @@ __device__ __forceinline__ void load2(unsigned dst, const CUtensorMap *m, unsign
 template <int CTAS>
 __device__ __forceinline__ void load4(unsigned dst, const CUtensorMap *m, unsigned bar, int c0, int c1, int c2, int c3) {
   if (CTAS == 2) tma_load_4d_pair(dst, m, bar, c0, c1, c2, c3); else tma_load_4d(dst, m, bar, c0, c1, c2, c3);
+}
+
+template <int CTAS>
+__device__ __forceinline__ void load3(unsigned dst, const CUtensorMap *m, unsigned bar, int c0, int c1, int c2) {
+  if (CTAS == 2) tma_load_3d_pair(dst, m, bar, c0, c1, c2); else tma_load_3d(dst, m, bar, c0, c1, c2);
+}
+template <int CTAS>
+__device__ __forceinline__ void load_im2col(unsigned dst, const CUtensorMap *m, unsigned bar, int c, int w, int h, int n,
+                                            int ow, int oh) {
+  if (CTAS == 2) tma_load_im2col_pair(dst, m, bar, c, w, h, n, (unsigned short)ow, (unsigned short)oh);
+  else tma_load_im2col(dst, m, bar, c, w, h, n, (unsigned short)ow, (unsigned short)oh);
 }
 
 // item -> (row unit, column tile, split).  Row units (one CTA's 128 rows, or a pair's 256) are
@@ -716,12 +848,19 @@ __device__ __forceinline__ void halo_mma_loop(const TcParams &p, int issuer, int
     }
   }
 }
-template <int CTAS>
+// Instances.  MODE 0: pixel boxes and plain matrices whose operands are whole chunks and whose output rows are
+// 32-byte aligned (the layers of the benchmark networks).  MODE 1: everything else that has no phases: im2col
+// copies, short channel chunks, output rows of any pitch.  MODE 2: MODE 1 for the error of a strided
+// convolution (items run over the phases of the input grid).  With one kernel for all of them the index
+// arithmetic and the registers of the general forms cost the aligned layers 1 - 4 % (13 spilled registers more;
+// 14 x 14 weight gradients 28.8 -> 30.4 us, 56 x 56 ones 86.2 -> 89.7 us).
+template <int CTAS, int MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const TcParams p, int32_t *__restrict__ acc, WsHeader *hdr, uint32_t *status,
                int8_t *__restrict__ out8, const int8_t *__restrict__ mask8, const int32_t *s_a,
                const int32_t *s_w, int32_t *s_out, int32_t *b_out, int32_t *spec_slot, int8_t *__restrict__ pool8) {
+  constexpr bool I2C = MODE >= 1, STRIDED = MODE == 2, GENERAL = MODE >= 1;
   if (p.epi_mode == EPI_SPECULATE && !p.single_wave) {
     // the follow-up launch may be scheduled now (it is launched as a programmatic dependent): its CTAs
     // take the SMs as this grid's CTAs retire and wait there for the whole grid to finish
@@ -916,34 +1055,45 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       // next tile no copy is issued and the ring runs dry; measured: ~1500 cycles of integer divisions
       // per tile cost a third of a 256-channel convolution).  Consecutive items of the convolutions
       // are consecutive tiles, so tile and pixel-box coordinates are stepped, not divided.
-      const bool stepped = p.blocked && p.splits == 1 && p.raster_g <= 0;
+      const bool stepped = p.blocked && p.splits == 1 && p.raster_g <= 0 && !STRIDED;
       int c_mu = 0, c_nt = 0, c_wt = 0, c_ht = 0, c_bt = 0;
       for (int item = first_item; ok && item < item_end; item += item_step) {
         int mu, nt, split;
         int w0 = 0, h0 = 0, b0 = 0, tap_n = 0, ci0 = 0;
+        Phase phq = {0, 0, p.R, p.S};
         if (stepped) {
           if (item == first_item) {
             decode_item(p, item, c_mu, c_nt, split);
             const int mt0 = c_mu * CTAS + (int)rank;
-            tile_coords(p, mt0, c_wt, c_ht, c_bt);
+            tile_coords(p, (I2C && p.i2c) ? mt0 * BM : mt0, c_wt, c_ht, c_bt);
           } else if (++c_nt == p.n_tiles_n) {
             c_nt = 0;
             ++c_mu;
-            c_wt += CTAS;
-            while (c_wt >= p.w_tiles) { c_wt -= p.w_tiles; if (++c_ht == p.h_tiles) { c_ht = 0; ++c_bt; } }
+            if (I2C && p.i2c) {
+              tile_coords(p, (c_mu * CTAS + (int)rank) * BM, c_wt, c_ht, c_bt);
+            } else {
+              c_wt += CTAS;
+              while (c_wt >= p.w_tiles) { c_wt -= p.w_tiles; if (++c_ht == p.h_tiles) { c_ht = 0; ++c_bt; } }
+            }
           }
           mu = c_mu; nt = c_nt; split = 0;
           w0 = c_wt * p.Wt; h0 = c_ht * p.Ht; b0 = c_bt * p.Bt;
         } else {
-          decode_item(p, item, mu, nt, split);
-          if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) pixel_box(p, mu * CTAS + (int)rank, w0, h0, b0);
+          int tile = item;
+          if (STRIDED) phq = split_phase(p, item, tile);
+          decode_item(p, tile, mu, nt, split);
+          if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD)
+            pixel_box(p, (mu * CTAS + (int)rank) * ((I2C && p.i2c) ? BM : 1), w0, h0, b0);
         }
-        if (p.kind == GK_CONV_FWD) { w0 *= p.stride; h0 *= p.stride; }     // output pixel -> window origin in x
+        if (p.kind == GK_CONV_FWD) { w0 *= p.stride_w; h0 *= p.stride; }     // output pixel -> window origin in x
+        if (I2C && p.i2c) { w0 += p.i2c_w0; h0 += p.i2c_h0; }
+        const int n_ts = phq.n_s;
         const int mt = mu * CTAS + (int)rank;     // this CTA's 128-row tile
         const int nb = nt * p.bn + (int)rank * bn_cta;
         const int kb0 = split * p.kb_per_split;
         int kb1 = kb0 + p.kb_per_split;
         if (kb1 > p.kb_total) kb1 = p.kb_total;
+        if (STRIDED) kb1 = phq.n_r * phq.n_s * p.c_chunks;
         if (p.kind == GK_CONV_WGRAD) {
           tap_n = nt / p.n_chunks;
           ci0 = (nt % p.n_chunks) * p.bn + (int)rank * bn_cta;
@@ -958,9 +1108,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             const int tap = kb0 / p.c_chunks;
             cc = kb0 % p.c_chunks; tr = tap / p.S; ts = tap % p.S;
           } else if (p.kind == GK_CONV_WGRAD) {
-            kwt = kb0 % p.w_tiles;
-            const int t = kb0 / p.w_tiles;
-            kht = t % p.h_tiles; kbt = t / p.h_tiles;
+            tile_coords(p, (I2C && p.i2c) ? kb0 * BM : kb0, kwt, kht, kbt);
           }
         }
         int wg_r = 0, wg_s = 0;
@@ -991,19 +1139,35 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               for (int j = 0; j < p.b_boxes; ++j)
                 load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
               break;
-            case GK_CONV_FWD:     // k-block = (tap, channel chunk)
-              load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 + ts - p.pad, h0 + tr - p.pad, b0);
-              load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+            case GK_CONV_FWD:     // k-block = (tap, channel chunk); B = w[co][tap][ci]
+              if (I2C && p.i2c) load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, ts, tr);
+              else load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 + ts - p.pad, h0 + tr - p.pad, b0);
+              if (GENERAL) load3<CTAS>(sb, &map_b, full, cc * p.kdepth, tr * p.S + ts, nb);
+              else load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
               break;
             case GK_CONV_DGRAD: { // A = e shifted the other way; B(ci, (tap, co)) = w[co][tap][ci]
-              load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 - ts + p.pad, h0 - tr + p.pad, b0);
-              const int col = (tr * p.S + ts) * p.Cn + nb;
+              int tap = tr * p.S + ts;
+              if (I2C && p.i2c) {
+                load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, p.T_s - 1 - ts, p.T_r - 1 - tr);
+                if (STRIDED) tap = (phq.r + p.dstride * tr) * p.S + phq.s + p.dstride * ts;
+              } else {
+                load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 - ts + p.pad, h0 - tr + p.pad, b0);
+              }
               for (int j = 0; j < p.b_boxes; ++j)
-                load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, col + j * p.b_box_step, cc * p.kdepth);
+                if (GENERAL) load3<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, tap, cc * p.kdepth);
+                else load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, tap * p.Cn + nb + j * p.b_box_step, cc * p.kdepth);
               break;
             }
             default: {            // GK_CONV_WGRAD: k-block = pixel box; A = e, B = x shifted by the tap
               const int kw0 = kwt * p.Wt, kh0 = kht * p.Ht, kbb0 = kbt * p.Bt;
+              if (I2C && p.i2c) {        // consecutive pixels: e as a plain matrix, x as im2col rows of the same pixels
+                for (int j = 0; j < p.a_boxes; ++j)
+                  load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * BM);
+                for (int j = 0; j < p.b_boxes; ++j)
+                  load_im2col<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + j * p.b_box_step,
+                                    kwt * p.stride_w + p.i2c_w0, kht * p.stride + p.i2c_h0, kbt, wg_s, wg_r);
+                break;
+              }
               for (int j = 0; j < p.a_boxes; ++j)
                 load4<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kw0, kh0, kbb0);
               for (int j = 0; j < p.b_boxes; ++j)
@@ -1015,9 +1179,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
          }
           if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) {
-            if (++cc == p.c_chunks) { cc = 0; if (++ts == p.S) { ts = 0; ++tr; } }
+            if (++cc == p.c_chunks) { cc = 0; if (++ts == n_ts) { ts = 0; ++tr; } }
           } else if (p.kind == GK_CONV_WGRAD) {
-            if (++kwt == p.w_tiles) { kwt = 0; if (++kht == p.h_tiles) { kht = 0; ++kbt; } }
+            if (I2C && p.i2c) {          // 128 pixels further in the grid
+              kwt += p.i2c_dj;
+              if (kwt >= p.w_tiles) { kwt -= p.w_tiles; ++kht; }
+              kht += p.i2c_di;
+              if (kht >= p.h_tiles) { kht -= p.h_tiles; ++kbt; }
+              kbt += p.i2c_db;
+            } else if (++kwt == p.w_tiles) { kwt = 0; if (++kht == p.h_tiles) { kht = 0; ++kbt; } }
           }
           if (++owner == nprod) owner = 0;
           if (++stage == p.stages) { stage = 0; phase ^= 1; }
@@ -1084,7 +1254,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const unsigned g_a_lo0 = (unsigned)p.a_desc, g_b_lo0 = (unsigned)p.b_desc;
       const unsigned g_a_hi = (unsigned)(p.a_desc >> 32), g_b_hi = (unsigned)(p.b_desc >> 32);
       const unsigned g_ak = p.a_kstep16, g_bk = p.b_kstep16, g_idesc = p.idesc, g_a_bytes = (unsigned)p.a_bytes;
-      const int g_ksteps = p.ksteps, g_mrep = p.mrep;
+      const int g_ksteps = p.ksteps, g_mrep = p.mrep, g_tail = GENERAL ? p.tail_ks : 0;
       const unsigned g_bn_mma = (unsigned)p.bn_mma, g_slice16 = (unsigned)p.a_box_bytes >> 4;
       unsigned gbuf = 0, gpar = 0;            // use % nbuf, (use / nbuf) & 1, counted
       for (int item = first_item; ok && item < item_end; item += item_step, ++use) {
@@ -1092,6 +1262,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int kb0 = split * p.kb_per_split;
         int kb1 = kb0 + p.kb_per_split;
         if (kb1 > p.kb_total) kb1 = p.kb_total;
+        if (STRIDED) {
+          int tile;
+          const Phase q = split_phase(p, item, tile);
+          kb1 = q.n_r * q.n_s * p.c_chunks;
+        }
+        int cc_left = g_tail ? p.c_chunks - kb0 % p.c_chunks : 0;     // chunks up to the short one (counted)
         const unsigned buf = gbuf;
         // wait until the epilogue has drained this accumulator buffer (the first nbuf uses pass at once)
         if (!mbar_wait_warp(tempty0 + 8 * buf, gpar ^ 1u, &abort_flag, status)) { ok = false; break; }
@@ -1104,6 +1280,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           const unsigned sa = smem_base + stage * stage_bytes;
           const unsigned a_lo = g_a_lo0 + ((sa >> 4) & 0x3fff), b_lo = g_b_lo0 + (((sa + g_a_bytes) >> 4) & 0x3fff);
           const unsigned first_acc = kb > kb0 ? 1u : 0u;
+          int ks = g_ksteps;
+          if (g_tail && --cc_left == 0) { ks = g_tail; cc_left = p.c_chunks; }
           if (leader) {
             if (g_mrep > 1) {
               for (int j = 0; j < g_mrep; ++j) {
@@ -1114,9 +1292,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 else issue_kblock<CTAS, 3>(td, aj, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
               }
             }
-            else if (g_ksteps == 4) issue_kblock<CTAS, 4>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
-            else if (g_ksteps == 2) issue_kblock<CTAS, 2>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
-            else if (g_ksteps == 1) issue_kblock<CTAS, 1>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
+            else if (ks == 4) issue_kblock<CTAS, 4>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
+            else if (ks == 2) issue_kblock<CTAS, 2>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
+            else if (ks == 1) issue_kblock<CTAS, 1>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
             else issue_kblock<CTAS, 3>(tmem_d, a_lo, g_a_hi, b_lo, g_b_hi, g_ak, g_bk, g_idesc, first_acc);
             // frees the stage (in every CTA of the pair) once these MMAs have read it
             if (CTAS == 2) tc_commit_pair(empty0 + 8 * stage); else tc_commit(empty0 + 8 * stage);
@@ -1137,7 +1315,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int row_in_tile = quarter * 32 + lane;
     unsigned use = 0;
     unsigned mx = 0;
-    unsigned spec_max = 0;
     int bp = 0;
     int h_wt = 0, h_ht = 0, h_bt = 0;
     if (p.epi_mode == EPI_KNOWN_B) {
@@ -1188,9 +1365,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             (mask8 == nullptr || ((uintptr_t)mask8 & 31) == 0);
     // the lean loop takes over after a warp's first item (which may be the CTA's speculative first
     // tile) when every chunk of every tile is whole and aligned
-    const bool lean_ok = (p.epi_mode == EPI_KNOWN_B || p.epi_mode == EPI_SPECULATE) && io_aligned && p.splits == 1 &&
+    const bool lean_ok = (p.epi_mode == EPI_KNOWN_B || p.epi_mode == EPI_SPECULATE) && p.splits == 1 &&
                          (p.bn & 31) == 0 && p.halo != 2 && p.kind != GK_CONV_WGRAD &&
-                         (p.mrep == 1 || (p.gn == p.bn_mma && mask8 == nullptr));
+                         (p.mrep == 1 || (io_aligned && p.gn == p.bn_mma && mask8 == nullptr));
+    // (otherwise: the largest store unit of the output rows, and this warp's staging buffer)
+    const unsigned io_bits = (unsigned)p.gn | (unsigned)(uintptr_t)out8 | 16u | (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
+    const int io_unit = (int)(io_bits & (0u - io_bits));
+    unsigned *nstg = reinterpret_cast<unsigned *>(smem_raw + (smem_base - smem_u32(smem_raw)) + p.nstg_off) +
+                     (warp - EPI_WARP0) * (32 * 9);
     int lean_item = -1;
     Extremes ex_all = {0, 0, 0u};
     // this thread's pixel inside a pixel box (generic convolutions): the box sides are powers of two
@@ -1200,7 +1382,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     for (int item = first_item + egroup * item_step; ok && item < item_end;
          item += item_step * egroups, use += (unsigned)egroups) {
       int mu = 0, nt = 0, split = 0;
-      if (!p.halo) decode_item(p, item, mu, nt, split);
+      Phase phq = {0, 0, 1, 1};
+      if (!p.halo) {
+        int tile = item;
+        if (STRIDED) phq = split_phase(p, item, tile);
+        decode_item(p, tile, mu, nt, split);
+      }
       const int mt = mu * CTAS + (int)rank;
       const unsigned buf = ebuf;
       const unsigned tpar = epar;
@@ -1223,7 +1410,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ncols_valid = (int)p.gn;
         for (int st = 0; st < egroups; ++st)
           if (++h_wt == p.w_tiles) { h_wt = 0; if (++h_ht == p.h_tiles) { h_ht = 0; ++h_bt; } }
-      } else if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) {
+      } else if (STRIDED) {
+        out_row = phase_row(p, mt * BM + row_in_tile, phq, row_ok);
+        col0 = (long long)nt * p.bn;
+        long long rem = p.gn - col0;
+        ncols_valid = rem < p.bn ? (int)rem : p.bn;
+      } else if ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) {
         int w0, h0, b0;
         pixel_box(p, mt, w0, h0, b0);
         const int ww = r_ww, hh = r_hh, bb = r_bb;
@@ -1447,8 +1639,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           bp = spec_bp_ready - 1;
           rk = make_round_const(bp, p.mbits, p.round_mode);
         }
-        const bool vec_ok = ((p.gn & 15) == 0) && ((col0 & 15) == 0);
-        const bool vec32_ok = ((p.gn & 31) == 0) && ((col0 & 31) == 0) && (((uintptr_t)out8 & 31) == 0);
         // Whole 32-column chunks with 32-byte aligned rows (every layer of the networks): the chunk
         // loop below does nothing per chunk but load, round and store; pointers are stepped.  (The
         // epilogue warps share their schedulers' integer pipe, which is the bound of layers with few
@@ -1506,7 +1696,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             cc += cstep;
             while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (mrow) mrow += sub_stride; }
           }
-        } else
+        } else if (GENERAL)
         for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
           int v[32];
           // chunk geometry: in row-batched mode chunk c holds columns cc of the item's tile c / bn_mma
@@ -1519,56 +1709,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             orow = out_row + (long long)jt * BM;
             rok = orow < p.gm;
           }
-          int8_t *dst8 = out8 + orow * p.gn + col0;
-          const int8_t *msk = mask8 ? mask8 + orow * p.gn + col0 : nullptr;
-          // the ReLU mask bytes are fetched first so that their latency overlaps the TMEM load and
-          // the rounding arithmetic
-          int4 m0v = make_int4(0x01010101, 0x01010101, 0x01010101, 0x01010101), m1v = m0v;
-          if (msk && vec_ok && rok && cc + 32 <= ncols_valid) {
-            if (vec32_ok && (((uintptr_t)mask8 & 31) == 0)) {
-              asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                           : "=r"(m0v.x), "=r"(m0v.y), "=r"(m0v.z), "=r"(m0v.w), "=r"(m1v.x), "=r"(m1v.y), "=r"(m1v.z),
-                             "=r"(m1v.w)
-                           : "l"(msk + cc));
-            } else {
-              m0v = *reinterpret_cast<const int4 *>(msk + cc);
-              m1v = *reinterpret_cast<const int4 *>(msk + cc + 16);
-            }
-          }
+          const int nv = ncols_valid - cc;                       // (uniform across the warp)
+          if (nv <= 0) continue;
+          const long long off = orow * p.gn + col0 + cc;
+          // (the ReLU mask bytes are fetched first: their latency overlaps the TMEM load and the rounding)
+          unsigned m[8], w8[8];
+          if (mask8 && rok) load_row_narrow(mask8 + off, m, nv < 32 ? nv : 32);
           tc_ld32(tm_row + (unsigned)c, v);
-          if (rok && cc < ncols_valid) {
-            unsigned w8[8];
-            Extremes ex = {0, 0, 0u};
+          if (rok) {
+            Extremes ex = {0, 0, 0u};                            // (columns beyond the matrix accumulate zeros)
             round_chunk32(v, w8, rk, p.relu != 0, ex);
-            if (vec_ok && cc + 32 <= ncols_valid) {
-              mx |= ex.magnitude_bits();
-              if (msk) {
-                w8[0] &= bytes_gt0(m0v.x); w8[1] &= bytes_gt0(m0v.y);
-                w8[2] &= bytes_gt0(m0v.z); w8[3] &= bytes_gt0(m0v.w);
-                w8[4] &= bytes_gt0(m1v.x); w8[5] &= bytes_gt0(m1v.y);
-                w8[6] &= bytes_gt0(m1v.z); w8[7] &= bytes_gt0(m1v.w);
-              }
-              if (vec32_ok) {
-                // one 32-byte sector per lane in a single request (half as many store requests)
-                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                             ::"l"(dst8 + cc), "r"(w8[0]), "r"(w8[1]), "r"(w8[2]), "r"(w8[3]), "r"(w8[4]), "r"(w8[5]),
-                               "r"(w8[6]), "r"(w8[7])
-                             : "memory");
-              } else {
-                *reinterpret_cast<int4 *>(dst8 + cc) = make_int4(w8[0], w8[1], w8[2], w8[3]);
-                *reinterpret_cast<int4 *>(dst8 + cc + 16) = make_int4(w8[4], w8[5], w8[6], w8[7]);
-              }
-            } else {
+            mx |= ex.magnitude_bits();
+            if (mask8) {
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (cc + j < ncols_valid) {
-                  mx |= (unsigned)abs(v[j]);
-                  int8_t q = (int8_t)((w8[j >> 2] >> (8 * (j & 3))) & 0xff);
-                  if (msk && msk[cc + j] <= 0) q = 0;
-                  dst8[cc + j] = q;
-                }
+              for (int j = 0; j < 8; ++j) w8[j] &= bytes_gt0(m[j]);
             }
           }
+          store_rows_narrow(out8, off, rok, w8, nv, io_unit, nstg, lane);
         }
       }
       tc_fence_before();
@@ -1589,21 +1746,27 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // executes only what changes (measured on the first layer: the general loop above spends a third
     // of its integer instructions on tests whose outcome is the same for every tile).
     if (ok && lean_item >= 0) {
-      auto lean = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c) {
+      auto lean = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c, auto narrow_c) {
+        constexpr bool NARROW = decltype(narrow_c)::value;   // output rows that are not 32-byte aligned, short last chunks
         constexpr bool RELU = decltype(relu_c)::value, MASK = decltype(mask_c)::value, BATCHED = decltype(batched_c)::value;
         constexpr bool POOL = decltype(pool_c)::value;       // fused 2 x 2 max-pool of the ReLU'd tile
         constexpr bool UPD = decltype(upd_c)::value;         // the output rows are weights: subtract the rounded gradient
         const int pool_xh = p.pool_xh;
         const bool pool_lane = (lane & (1 | pool_xh)) == 0;  // the window's top-left pixel stores the maximum
-        const int kind = p.halo ? 0 : ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) ? 1 : 2);
+        const int kind = STRIDED ? 3 : (p.halo ? 0 : (((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) ? 1 : 2));
         const int istep = item_step * egroups, nbuf = p.nbuf, bn = p.bn, n_tiles_n = p.n_tiles_n;
         const int cstep = 32 * wpq, c_first = 32 * chunk_phase;
         const long long gn = p.gn, gm = p.gm;
         const int bn_mma = BATCHED ? p.bn_mma : p.bn;
         const long long sub_stride = (long long)BM * gn;
-        const bool counted = p.blocked && p.raster_g <= 0;     // consecutive items: (mu, nt) are stepped
+        const bool counted = p.blocked && p.raster_g <= 0 && kind != 3;     // consecutive items: (mu, nt) are stepped
         int mu = 0, nt = 0, split = 0;
-        if (kind != 0) decode_item(p, lean_item, mu, nt, split);
+        Phase phq = {0, 0, 1, 1};
+        if (kind == 3) {
+          int tile;
+          phq = split_phase(p, lean_item, tile);
+          decode_item(p, tile, mu, nt, split);
+        } else if (kind != 0) decode_item(p, lean_item, mu, nt, split);
         for (int item = lean_item; item < item_end; item += istep) {
           const unsigned buf = ebuf, tpar = epar;
           ebuf += (unsigned)egroups;
@@ -1625,16 +1788,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             row_ok = w < p.PW && h < p.PH && b < p.PB;
             out_row = ((long long)b * p.PH + h) * p.PW + w;
             if (POOL) pool_row = ((long long)b * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
+          } else if (kind == 3) {
+            out_row = phase_row(p, (mu * CTAS + (int)rank) * BM + row_in_tile, phq, row_ok);
           } else {
             out_row = (long long)(mu * CTAS + (int)rank) * (BM * p.mrep) + row_in_tile;
             row_ok = out_row < gm;
           }
           const int col0 = nt * bn;
-          int cend = BATCHED ? bn : (int)(gn - col0);          // (whole chunks: gn is a multiple of 32)
+          int cend = BATCHED ? bn : (int)(gn - col0);          // (whole chunks unless NARROW)
           if (cend > bn) cend = bn;
           if (kind != 0) {                                      // next item of this warp
             if (counted) { nt += egroups; while (nt >= n_tiles_n) { nt -= n_tiles_n; ++mu; } }
-            else if (item + istep < item_end) decode_item(p, item + istep, mu, nt, split);
+            else if (item + istep < item_end) {
+              int tile = item + istep;
+              if (kind == 3) phq = split_phase(p, item + istep, tile);
+              decode_item(p, tile, mu, nt, split);
+            }
           }
           if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
           tc_fence_after();
@@ -1650,7 +1819,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             int v[32];
             const bool rok = BATCHED ? (row_ok && orow < gm) : row_ok;
             unsigned m[8];
-            if ((MASK || UPD) && rok)
+            if (NARROW) {
+              if (MASK && rok) load_row_narrow(mrow + cc, m, cend - c < 32 ? cend - c : 32);
+            } else if ((MASK || UPD) && rok)
               asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                            : "=r"(m[0]), "=r"(m[1]), "=r"(m[2]), "=r"(m[3]), "=r"(m[4]), "=r"(m[5]), "=r"(m[6]), "=r"(m[7])
                            : "l"((UPD ? (const int8_t *)drow : mrow) + cc));
@@ -1667,8 +1838,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (MASK) w8[j] &= bytes_gt0(m[j]);
                 if (UPD) w8[j] = bytes_sub_clamp127(m[j], w8[j]);
               }
-              store32(drow + cc, w8);
+              if (!NARROW) store32(drow + cc, w8);
             }
+            if (NARROW) store_rows_narrow(out8, row_off + cc, rok, w8, cend - c, io_unit, nstg, lane);
             if (POOL) {                                        // (warp-uniform: all lanes exchange)
               pool_chunk32(w8, pool_xh);
               if (rok && pool_lane) store32(prow + cc, w8);
@@ -1687,11 +1859,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       using T = std::true_type;
       using F = std::false_type;
       const bool relu = p.relu != 0, masked = mask8 != nullptr, batched = p.mrep > 1;
-      if (batched) { if (relu) lean(T{}, F{}, T{}, F{}, F{}); else lean(F{}, F{}, T{}, F{}, F{}); }   // (row-batched: forward only)
-      else if (p.update) lean(F{}, F{}, F{}, F{}, T{});                                              // (weight gradients: signed, no mask)
-      else if (p.pool) lean(T{}, F{}, F{}, T{}, F{});                                                // (pooling: ReLU, no mask)
-      else if (relu) { if (masked) lean(T{}, T{}, F{}, F{}, F{}); else lean(T{}, F{}, F{}, F{}, F{}); }
-      else { if (masked) lean(F{}, T{}, F{}, F{}, F{}); else lean(F{}, F{}, F{}, F{}, F{}); }
+      if (batched) { if (relu) lean(T{}, F{}, T{}, F{}, F{}, F{}); else lean(F{}, F{}, T{}, F{}, F{}, F{}); }   // (row-batched: forward only)
+      else if (GENERAL && !io_aligned) {
+        if (relu) lean(T{}, F{}, F{}, F{}, F{}, T{});                                                      // (ReLU: forward, no mask)
+        else if (masked) lean(F{}, T{}, F{}, F{}, F{}, T{});
+        else lean(F{}, F{}, F{}, F{}, F{}, T{});
+      }
+      else if (p.update) lean(F{}, F{}, F{}, F{}, T{}, F{});                                              // (weight gradients: signed, no mask)
+      else if (p.pool) lean(T{}, F{}, F{}, T{}, F{}, F{});                                                // (pooling: ReLU, no mask)
+      else if (relu) lean(T{}, F{}, F{}, F{}, F{}, F{});
+      else { if (masked) lean(F{}, T{}, F{}, F{}, F{}, F{}); else lean(F{}, F{}, F{}, F{}, F{}, F{}); }
       mx |= ex_all.magnitude_bits();
     }
     if (p.epi_mode == EPI_SPILL || p.epi_mode == EPI_SPECULATE) {
@@ -1759,6 +1936,10 @@ __global__ void timeout_probe_kernel(uint32_t *status) {
 // ------------------------------------------------------------------------------------------
 // Host side: tensor maps, descriptors, eligibility
 // ------------------------------------------------------------------------------------------
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                   const cuuint64_t *, const int *, const int *, cuuint32_t, cuuint32_t,
+                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
@@ -1788,7 +1969,16 @@ static unsigned long long desc_mnmajor(int sw, int kdepth) {
   d |= (unsigned long long)1 << 46;
   return d | layout_bits(sw);
 }
-static int pick_swizzle(long long extent) { return extent >= 128 ? 128 : (extent >= 64 ? 64 : (extent >= 32 ? 32 : 0)); }
+// Swizzle width (= bytes of a copied row) of an operand with `extent` elements along its rows.  Copies past the
+// extent are filled with zeros, so a short last chunk costs no memory traffic, and the MMAs that would only
+// see zeros are left out.
+static int pick_swizzle(long long extent) { return extent > 64 ? 128 : (extent > 32 ? 64 : 32); }
+// Swizzle width of an MN-major operand of which a CTA stages `n` columns: the width that copies the fewest
+// columns, the wider one of two equals.
+static int pick_swizzle_mn(int n) {
+  if (n <= 32) return 32;
+  return (n + 127) / 128 * 128 <= (n + 63) / 64 * 64 ? 128 : 64;
+}
 
 struct MapSpec {
   int nd;
@@ -1798,6 +1988,8 @@ struct MapSpec {
   int swizzle;
   const void *base;
   cuuint32_t estr[4];      // element (traversal) stride per dimension; 0 = 1
+  int im2col;              // 1: im2col map; box[0] = channels per pixel, box[1] = pixels per copy
+  int lo[2], hi[2];        // its bounding box: first base pixel (W, H), last base pixel relative to the last pixel
 };
 
 static bool encode(niti_ctx *ctx, CUtensorMap *m, const MapSpec &s) {
@@ -1805,6 +1997,18 @@ static bool encode(niti_ctx *ctx, CUtensorMap *m, const MapSpec &s) {
   if (((uintptr_t)s.base & 15) != 0) return false;
   for (int i = 0; i + 1 < s.nd; ++i)
     if (s.strides[i] % 16 != 0) return false;
+  if (s.im2col) {
+    if (!ctx->encode_im2col || s.box[1] > 256) return false;
+    for (int i = 0; i < 2; ++i)
+      if (s.lo[i] < -128 || s.lo[i] > 127 || s.hi[i] < -128 || s.hi[i] > 127) return false;
+    const cuuint32_t es[4] = {1, s.estr[1] > 1 ? s.estr[1] : 1, s.estr[2] > 1 ? s.estr[2] : 1, 1};
+    if (es[1] > 8 || es[2] > 8) return false;
+    return ((EncodeIm2colFn)ctx->encode_im2col)(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(s.base), s.dims,
+                                                s.strides, s.lo, s.hi, s.box[0], s.box[1], es,
+                                                CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_enum(s.swizzle),
+                                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  }
   for (int i = 0; i < s.nd; ++i)
     if (s.box[i] == 0 || s.box[i] > 256) return false;
   cuuint32_t es[4] = {1, 1, 1, 1};
@@ -1829,10 +2033,28 @@ static bool pick_pixel_box(int W, int H, int B, int &Wt, int &Ht, int &Bt) {
   return Wt <= W && Ht <= H && Bt <= B;
 }
 
+// Extents and strides of a tensor of overlapping windows (see WindowGeometry at the boundary): a window's channels,
+// the windows of a row, rows, images.
+static void window_map(const GemmProblem &g, MapSpec &s) {
+  s.dims[0] = (cuuint64_t)g.win_chans;
+  s.strides[0] = (cuuint64_t)g.win_sw;
+  s.strides[1] = (cuuint64_t)g.win_sh;
+  s.strides[2] = (cuuint64_t)g.win_sh * g.H;
+}
+
 static int round_up32(long long n) { return (int)((n + 31) / 32 * 32); }
 
+// Width of a column tile: the fewest tiles of at most 256 columns, all of about the same width.
+static int pick_bn(long long gn) {
+  const long long tiles = (gn + 255) / 256;
+  return round_up32((gn + tiles - 1) / tiles);
+}
+
 // Builds params and maps; returns false if the shape is not eligible for this engine.
-static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, TcParams &p, CUtensorMap &ma,
+// `aligned`: output (and mask) pointers and rows are 32-byte aligned.
+// want: ANY, or only a plan in the resident-weights / tap-pair mode (HALO) or the row-batched mode (BATCHED).
+enum PlanWant { PLAN_ANY = 0, PLAN_HALO = 1, PLAN_BATCHED = 2 };
+static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, TcParams &p, CUtensorMap &ma,
                  CUtensorMap &mb) {
   memset(&p, 0, sizeof(p));
   p.ctas = ctas;
@@ -1840,21 +2062,27 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
   p.gm = g.gm;
   p.gn = g.gn;
   p.splits = 1;
+  p.mode = aligned ? 0 : 1;
   MapSpec sa, sb;
   memset(&sa, 0, sizeof(sa));
   memset(&sb, 0, sizeof(sb));
   int a_mn = 0, b_mn = 0;        // 1 = MN-major operand
   int a_sw = 0, b_sw = 0;
+  int tail = 0;                  // contraction elements of the last chunk of c_chunks when it is not a whole one
   long long m_tiles = 0;
   if (g.gm * g.gn >= (1LL << 31)) return false;
+  // operands as they are copied: padded where the caller's rows are no multiple of 16 bytes
+  const int8_t *q0 = g.q0 ? g.q0 : g.p0, *q1 = g.q1 ? g.q1 : g.p1;
+  if (g.kind == GK_FC_DGRAD && g.gk < 32) return false;            // (10-class heads: the CUDA-core engine is faster)
+  if (g.kind == GK_FC_WGRAD && (g.gm < 32 || g.gk < 32)) return false;
   switch (g.kind) {
     case GK_FC_FWD: {
       p.kdepth = pick_swizzle(g.gk);
-      if (!p.kdepth) return false;
-      p.bn = g.gn >= 256 ? 256 : round_up32(g.gn);
+      p.bn = pick_bn(g.gn);
       a_sw = b_sw = p.kdepth;
-      sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {(cuuint64_t)g.gk}, {(cuuint32_t)p.kdepth, BM}, a_sw, g.p0};
-      sb = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gn}, {(cuuint64_t)g.gk}, {(cuuint32_t)p.kdepth, (cuuint32_t)(p.bn / ctas)}, b_sw, g.p1};
+      const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gk);
+      sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {ld0}, {(cuuint32_t)p.kdepth, BM}, a_sw, q0};
+      sb = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gn}, {ld1}, {(cuuint32_t)p.kdepth, (cuuint32_t)(p.bn / ctas)}, b_sw, q1};
       p.kb_total = (int)((g.gk + p.kdepth - 1) / p.kdepth);
       m_tiles = (g.gm + BM - 1) / BM;
       p.n_tiles_n = (int)((g.gn + p.bn - 1) / p.bn);
@@ -1862,15 +2090,13 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
     }
     case GK_FC_DGRAD: {   // out [M][K'], contraction over N
       p.kdepth = pick_swizzle(g.gk);
-      if (!p.kdepth) return false;
       b_mn = 1;
-      b_sw = pick_swizzle(g.gn);
-      if (!b_sw) return false;
-      p.bn = g.gn >= 256 ? 256 : (int)((g.gn + b_sw - 1) / b_sw * b_sw);
-      if (p.bn % 32) return false;
+      p.bn = pick_bn(g.gn);
+      b_sw = pick_swizzle_mn(p.bn / ctas);
       a_sw = p.kdepth;
-      sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {(cuuint64_t)(g.ld0 ? g.ld0 : g.gk)}, {(cuuint32_t)p.kdepth, BM}, a_sw, g.p0};
-      sb = {2, {(cuuint64_t)g.gn, (cuuint64_t)g.gk}, {(cuuint64_t)g.gn}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, g.p1};
+      const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
+      sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {ld0}, {(cuuint32_t)p.kdepth, BM}, a_sw, q0};
+      sb = {2, {(cuuint64_t)g.gn, (cuuint64_t)g.gk}, {ld1}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, q1};
       p.kb_total = (int)((g.gk + p.kdepth - 1) / p.kdepth);
       m_tiles = (g.gm + BM - 1) / BM;
       p.n_tiles_n = (int)((g.gn + p.bn - 1) / p.bn);
@@ -1879,13 +2105,12 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
     case GK_FC_WGRAD: {   // out [N][K'], contraction over M (rows of both operands)
       a_mn = b_mn = 1;
       a_sw = pick_swizzle(g.gm);
-      b_sw = pick_swizzle(g.gn);
-      if (!a_sw || !b_sw || g.gk < 32) return false;
-      p.kdepth = g.gk >= 128 ? 128 : (g.gk >= 64 ? 64 : 32);
-      p.bn = g.gn >= 256 ? 256 : (int)((g.gn + b_sw - 1) / b_sw * b_sw);
-      if (p.bn % 32) return false;
-      sa = {2, {(cuuint64_t)g.gm, (cuuint64_t)g.gk}, {(cuuint64_t)(g.ld0 ? g.ld0 : g.gm)}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, g.p0};
-      sb = {2, {(cuuint64_t)g.gn, (cuuint64_t)g.gk}, {(cuuint64_t)g.gn}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, g.p1};
+      p.kdepth = pick_swizzle(g.gk);
+      p.bn = pick_bn(g.gn);
+      b_sw = pick_swizzle_mn(p.bn / ctas);
+      const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gm), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
+      sa = {2, {(cuuint64_t)g.gm, (cuuint64_t)g.gk}, {ld0}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, q0};
+      sb = {2, {(cuuint64_t)g.gn, (cuuint64_t)g.gk}, {ld1}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, q1};
       p.kb_total = (int)((g.gk + p.kdepth - 1) / p.kdepth);
       m_tiles = (g.gm + BM - 1) / BM;
       p.n_tiles_n = (int)((g.gn + p.bn - 1) / p.bn);
@@ -1900,72 +2125,124 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
       // copies.  The error of a strided convolution is left to the CUDA-core engine.
       const bool fwd = g.kind == GK_CONV_FWD;
       const int st = g.stride > 1 ? g.stride : 1;
-      if (!fwd && st != 1) return false;
       const int RW = fwd ? g.Wo : g.W, RH = fwd ? g.Ho : g.H;      // pixel grid of the rows
       const int OW = fwd ? g.W : g.Wo, OH = fwd ? g.H : g.Ho;      // pixel grid of the shifted operand
       const bool same = g.Ho == g.H && g.Wo == g.W && st == 1;
       const int Cc = fwd ? g.Ci : g.Co;        // contraction channels
       const int Cn = fwd ? g.Co : g.Ci;        // output channels of this multiply
+      const long long ld0 = g.ld0 ? g.ld0 : Cc, ld1 = g.ld1 ? g.ld1 : g.Ci;       // pixel pitch, tap pitch of w
       p.kdepth = pick_swizzle(Cc);
-      if (!p.kdepth || Cc % p.kdepth) return false;
-      if (!pick_pixel_box(RW, RH, g.B, p.Wt, p.Ht, p.Bt)) return false;
-      if (p.Wt * st > 256 || p.Ht * st > 256) return false;
-      p.w_tiles = (RW + p.Wt - 1) / p.Wt;
-      p.h_tiles = (RH + p.Ht - 1) / p.Ht;
-      p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
-      p.PW = RW; p.PH = RH; p.PB = g.B;
+      tail = Cc % p.kdepth;
+      const int pad_w = g.win_chans ? 0 : g.pad;
       p.R = g.R; p.S = g.S; p.pad = g.pad;
-      p.stride = st;
-      p.c_chunks = Cc / p.kdepth;
+      p.stride = fwd ? st : 1;
+      p.stride_w = g.win_chans ? 1 : p.stride;
+      p.dstride = fwd ? 1 : st;
+      p.c_chunks = (Cc + p.kdepth - 1) / p.kdepth;
       p.Cn = Cn;
       a_sw = p.kdepth;
+      // Pixel rows.  Where a pixel box of 128 tiles the image exactly (and no stride is involved) a tile of output
+      // rows is such a box: it allows the fused 2 x 2 pooling.  Everywhere else (odd image sides, strides) the
+      // rows of a tile are 128 consecutive pixels of the flattened grid, copied in im2col mode, which walks the
+      // grid pixel by pixel, image after image, with the convolution's stride and zero padding.
+      p.i2c = (st > 1 || g.win_chans || !pick_pixel_box(RW, RH, g.B, p.Wt, p.Ht, p.Bt)) ? 1 : 0;
       sa = {4, {(cuuint64_t)Cc, (cuuint64_t)OW, (cuuint64_t)OH, (cuuint64_t)g.B},
-            {(cuuint64_t)Cc, (cuuint64_t)Cc * OW, (cuuint64_t)Cc * OW * OH},
-            {(cuuint32_t)p.kdepth, (cuuint32_t)(p.Wt * st), (cuuint32_t)(p.Ht * st), (cuuint32_t)p.Bt}, a_sw, g.p0,
-            {1, (cuuint32_t)st, (cuuint32_t)st, 1}};
-      if (fwd) {
-        p.bn = Cn >= 256 ? 256 : round_up32(Cn);
-        if (ctas == 2 && Cn > 256) {
-          // Whole waves: with 256-wide tiles the 14 x 14 layers are 98 tile pairs on 74 pairs of SMs, two
-          // waves of which the second is a third full; 192-wide tiles make 147 items, two full waves.
-          // (A 192-wide MMA takes as long as a 256-wide one, so an item is not shorter; it moves three
-          // quarters of the weights.  Measured 31.0 against 31.5 us; 128-wide tiles, three waves of
-          // half the math each, are bound by the shared-memory traffic of their operands: 38.4 us.)
-          const long long mu = ((long long)p.w_tiles * p.h_tiles * p.b_tiles + 1) / 2, units = ctx->sm_count / 2;
-          const long long w256 = (mu * ((Cn + 255) / 256) + units - 1) / units;
-          const long long w192 = (mu * ((Cn + 191) / 192) + units - 1) / units;
-          if (w192 * 192 * 10 < w256 * 256 * 9) p.bn = 192;
+            {(cuuint64_t)ld0, (cuuint64_t)ld0 * OW, (cuuint64_t)ld0 * OW * OH},
+            {(cuuint32_t)p.kdepth, (cuuint32_t)p.Wt, (cuuint32_t)p.Ht, (cuuint32_t)p.Bt}, a_sw, q0};
+      if (g.win_chans) window_map(g, sa);
+      p.PW = RW; p.PH = RH; p.PB = g.B;
+      p.T_r = g.R; p.T_s = g.S;
+      if (p.i2c) {
+        if (g.R > 256 || g.S > 256) return false;
+        p.Wt = p.Ht = p.Bt = 1;
+        sa.im2col = 1;
+        sa.box[1] = BM;
+        if (fwd) {
+          p.i2c_w0 = -pad_w; p.i2c_h0 = -g.pad;
+          sa.estr[1] = (cuuint32_t)p.stride_w; sa.estr[2] = (cuuint32_t)st;
+          sa.hi[0] = pad_w - (g.S - 1); sa.hi[1] = g.pad - (g.R - 1);
+        } else {
+          // phases of the input grid (a single one without a stride): grid position u of phase f is input row
+          // st * (u + u0) + f - pad and collects e[u + u0 - t] for the taps f + st * t.  All phases share the grid
+          // of the widest one; positions outside the tensor are masked.
+          p.nph_r = st < g.R ? st : g.R; p.nph_s = st < g.S ? st : g.S;
+          p.T_r = (g.R + st - 1) / st; p.T_s = (g.S + st - 1) / st;
+          const int fr = g.pad - (p.nph_r - 1), fs = g.pad - (p.nph_s - 1);
+          p.u0_r = fr > 0 ? (fr + st - 1) / st : 0; p.u0_s = fs > 0 ? (fs + st - 1) / st : 0;
+          const int u1_r = (g.H - 1 + g.pad) / st, u1_s = (g.W - 1 + g.pad) / st;
+          p.PH = u1_r - p.u0_r + 1; p.PW = u1_s - p.u0_s + 1;
+          p.i2c_h0 = p.u0_r - (p.T_r - 1); p.i2c_w0 = p.u0_s - (p.T_s - 1);
+          sa.hi[0] = p.i2c_w0 + p.PW - 1 - (OW - 1); sa.hi[1] = p.i2c_h0 + p.PH - 1 - (OH - 1);
+          p.OH = g.H; p.OW = g.W;
         }
-        b_sw = p.kdepth;
-        sb = {2, {(cuuint64_t)g.gk, (cuuint64_t)Cn}, {(cuuint64_t)g.gk}, {(cuuint32_t)p.kdepth, (cuuint32_t)(p.bn / ctas)}, b_sw, g.p1};
-      } else {
+        sa.lo[0] = p.i2c_w0; sa.lo[1] = p.i2c_h0;
+        if ((long long)p.PB * p.PH * p.PW >= (1LL << 31) - 512) return false;
+      }
+      p.w_tiles = (p.PW + p.Wt - 1) / p.Wt;
+      p.h_tiles = (p.PH + p.Ht - 1) / p.Ht;
+      p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
+      m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
+      if (p.i2c) m_tiles = (m_tiles + BM - 1) / BM;
+      p.bn = pick_bn(Cn);
+      if (fwd && ctas == 2 && Cn > 256) {
+        // Whole waves: with 256-wide tiles the 14 x 14 layers are 98 tile pairs on 74 pairs of SMs, two
+        // waves of which the second is a third full; 192-wide tiles make 147 items, two full waves.
+        // (A 192-wide MMA takes as long as a 256-wide one, so an item is not shorter; it moves three
+        // quarters of the weights.  Measured 31.0 against 31.5 us; 128-wide tiles, three waves of
+        // half the math each, are bound by the shared-memory traffic of their operands: 38.4 us.)
+        const long long mu = (m_tiles + 1) / 2, units = ctx->sm_count / 2;
+        const long long w256 = (mu * ((Cn + 255) / 256) + units - 1) / units;
+        const long long w192 = (mu * ((Cn + 191) / 192) + units - 1) / units;
+        if (w192 * 192 * 10 < w256 * 256 * 9) p.bn = 192;
+      }
+      if (p.i2c || tail || g.q0 || g.q1 || g.Ci % 32 != 0) p.mode = 1;
+      // (a copy of w may reach into the next tap's columns only where those are not multiplied)
+      if (!fwd && Cn % pick_swizzle_mn(p.bn / ctas) != 0) p.mode = 1;
+      if (p.dstride > 1) p.mode = 2;
+      // w viewed as [Co][R*S][Ci]
+      sb = {3, {(cuuint64_t)g.Ci, (cuuint64_t)g.R * g.S, (cuuint64_t)g.Co},
+            {(cuuint64_t)ld1, (cuuint64_t)ld1 * g.R * g.S}, {(cuuint32_t)p.kdepth, 1, (cuuint32_t)(p.bn / ctas)}, p.kdepth, q1};
+      if (!fwd) {
         b_mn = 1;
-        b_sw = pick_swizzle(Cn);
-        if (!b_sw || Cn % b_sw) return false;
-        p.bn = Cn >= 256 ? 256 : Cn;
-        if (p.bn % 32 || Cn % p.bn) return false;
-        // w viewed as [Co rows][R*S*Ci]: column = tap * Ci + ci
-        sb = {2, {(cuuint64_t)g.R * g.S * g.Ci, (cuuint64_t)g.Co}, {(cuuint64_t)g.R * g.S * g.Ci},
-              {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, g.p1};
+        sb.swizzle = pick_swizzle_mn(p.bn / ctas);
+        sb.box[0] = (cuuint32_t)sb.swizzle;
+        sb.box[2] = (cuuint32_t)p.kdepth;
+      }
+      b_sw = sb.swizzle;
+      if (p.mode == 0) {       // (plain matrices: [Cn][R*S*Ci], and [Co][R*S*Ci] with column tap * Ci + ci)
+        const cuuint64_t row = (cuuint64_t)g.R * g.S * g.Ci;
+        sb.nd = 2;
+        sb.dims[0] = row; sb.dims[1] = (cuuint64_t)g.Co;
+        sb.strides[0] = row;
+        sb.box[1] = sb.box[2];
       }
       p.kb_total = g.R * g.S * p.c_chunks;
-      m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
       p.n_tiles_n = (Cn + p.bn - 1) / p.bn;
+      if (p.dstride > 1) p.kb_total = p.T_r * p.T_s * p.c_chunks;                 // (of the longest phase)
       // halo mode: one channel chunk, one column tile, weights of all taps fit beside >= 3 patches
-      if (want_halo && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && p.c_chunks == 1 && p.n_tiles_n == 1 &&
-          g.W >= 10 && g.H >= 18) {
+      if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && p.c_chunks == 1 && !tail &&
+          p.n_tiles_n == 1 && g.W >= 10 && g.H >= 18 && !g.q0 && !g.q1 && (fwd ? Cn % 8 == 0 : Cn % 32 == 0)) {
         const int a_stage = (180 * p.kdepth + 1023) / 1024 * 1024;
-        const int b_res = (9 * p.bn * p.kdepth + 1023) / 1024 * 1024;
+        const int tap_cols = fwd ? p.bn : (p.bn + b_sw - 1) / b_sw * b_sw;        // (columns past Cn are not multiplied)
+        const int b_res = (9 * tap_cols * p.kdepth + 1023) / 1024 * 1024;
         if (b_res + 3 * a_stage <= 224 * 1024) {
           p.halo = 1;
+          p.i2c = 0;
+          p.mode = aligned ? 0 : 1;
+          sa.im2col = 0;
+          p.PW = g.W; p.PH = g.H;
           p.Wt = 8; p.Ht = 16; p.Bt = 1;
           p.w_tiles = (g.W + 7) / 8;
           p.h_tiles = (g.H + 15) / 16;
           p.b_tiles = g.B;
           m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
           sa.box[1] = 10; sa.box[2] = 18; sa.box[3] = 1;
-          if (fwd) sb.box[1] = (cuuint32_t)p.bn;
-          p.b_tile_bytes = p.bn * p.kdepth;
+          if (fwd) {
+            sb = {2, {(cuuint64_t)g.gk, (cuuint64_t)Cn}, {(cuuint64_t)g.gk}, {(cuuint32_t)p.kdepth, (cuuint32_t)p.bn}, b_sw, q1};
+          } else {       // w viewed as [Co rows][9 * Ci]: column = tap * Ci + ci
+            sb = {2, {(cuuint64_t)9 * g.Ci, (cuuint64_t)g.Co}, {(cuuint64_t)9 * g.Ci}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, q1};
+          }
+          p.b_tile_bytes = tap_cols * p.kdepth;
           p.b_res_bytes = b_res;
         }
       }
@@ -1979,8 +2256,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
       p.stride = st;
       // (64 x 64)-channel blocks re-read the activations once per block of the other operand, so this
       // mode is kept for layers with few blocks; wide layers use the per-tap tiles below
-      if (want_halo && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && g.Ci % 64 == 0 && g.Co % 64 == 0 &&
-          g.W >= 10 && g.H >= 18 && (long long)g.Ci * g.Co <= 32768) {
+      if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && g.Ci % 64 == 0 && g.Co % 64 == 0 &&
+          g.W >= 10 && g.H >= 18 && (long long)g.Ci * g.Co <= 32768 && !g.q0 && !g.q1) {
         p.halo = 2;
         p.kdepth = 128;
         p.bn = 64;
@@ -2035,30 +2312,50 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
         if (!encode(ctx, &ma, sa) || !encode(ctx, &mb, sb)) return false;
         return true;
       }
+      if (want == PLAN_HALO) return false;
       a_mn = b_mn = 1;
+      const long long ld0 = g.ld0 ? g.ld0 : g.Co, ld1 = g.ld1 ? g.ld1 : g.Ci;     // pixel pitches of e and x
       a_sw = pick_swizzle(g.Co);
-      b_sw = pick_swizzle(g.Ci);
-      if (!a_sw || !b_sw || g.Co % a_sw || g.Ci % b_sw) return false;
-      if (!pick_pixel_box(g.Wo, g.Ho, g.B, p.Wt, p.Ht, p.Bt)) return false;
-      if (p.Wt * st > 256 || p.Ht * st > 256) return false;
       p.kdepth = 128;
-      p.w_tiles = (g.Wo + p.Wt - 1) / p.Wt;
-      p.h_tiles = (g.Ho + p.Ht - 1) / p.Ht;
-      p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
       p.PW = g.Wo; p.PH = g.Ho; p.PB = g.B;
       p.R = g.R; p.S = g.S; p.pad = g.pad;
       p.Cn = g.Ci;
-      p.bn = g.Ci >= 256 ? 256 : g.Ci;
-      if (p.bn % 32 || g.Ci % p.bn) return false;
-      p.n_chunks = g.Ci / p.bn;
-      sa = {4, {(cuuint64_t)g.Co, (cuuint64_t)g.Wo, (cuuint64_t)g.Ho, (cuuint64_t)g.B},
-            {(cuuint64_t)g.Co, (cuuint64_t)g.Co * g.Wo, (cuuint64_t)g.Co * g.Wo * g.Ho},
-            {(cuuint32_t)a_sw, (cuuint32_t)p.Wt, (cuuint32_t)p.Ht, (cuuint32_t)p.Bt}, a_sw, g.p0};
+      p.bn = pick_bn(g.Ci);
+      b_sw = pick_swizzle_mn(p.bn / ctas);
+      p.n_chunks = (g.Ci + p.bn - 1) / p.bn;
+      // (pixel boxes or runs of consecutive pixels: see "Pixel rows" above; a run of e is a piece of a matrix)
+      p.stride_w = g.win_chans ? 1 : st;
+      p.i2c = (st > 1 || g.win_chans || !pick_pixel_box(g.Wo, g.Ho, g.B, p.Wt, p.Ht, p.Bt)) ? 1 : 0;
+      if (p.i2c) p.mode = 1;
       sb = {4, {(cuuint64_t)g.Ci, (cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)g.B},
-            {(cuuint64_t)g.Ci, (cuuint64_t)g.Ci * g.W, (cuuint64_t)g.Ci * g.W * g.H},
-            {(cuuint32_t)b_sw, (cuuint32_t)(p.Wt * st), (cuuint32_t)(p.Ht * st), (cuuint32_t)p.Bt}, b_sw, g.p1,
-            {1, (cuuint32_t)st, (cuuint32_t)st, 1}};
+            {(cuuint64_t)ld1, (cuuint64_t)ld1 * g.W, (cuuint64_t)ld1 * g.W * g.H},
+            {(cuuint32_t)b_sw, (cuuint32_t)p.Wt, (cuuint32_t)p.Ht, (cuuint32_t)p.Bt}, b_sw, q1};
+      if (g.win_chans) window_map(g, sb);
+      if (p.i2c) {
+        if (g.R > 256 || g.S > 256) return false;
+        p.Wt = p.Ht = p.Bt = 1;
+        const int pad_w = g.win_chans ? 0 : g.pad;
+        p.i2c_w0 = -pad_w; p.i2c_h0 = -g.pad;
+        p.i2c_dj = BM % g.Wo;
+        p.i2c_di = BM / g.Wo % g.Ho;
+        p.i2c_db = BM / g.Wo / g.Ho;
+        sa = {2, {(cuuint64_t)g.Co, (cuuint64_t)g.gk}, {(cuuint64_t)ld0}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, q0};
+        sb.im2col = 1;
+        sb.box[1] = (cuuint32_t)p.kdepth;
+        sb.estr[1] = (cuuint32_t)p.stride_w; sb.estr[2] = (cuuint32_t)st;
+        sb.lo[0] = -pad_w; sb.lo[1] = -g.pad;
+        sb.hi[0] = pad_w - (g.S - 1); sb.hi[1] = g.pad - (g.R - 1);
+        if (g.gk >= (1LL << 31) - 512) return false;
+      } else {
+        sa = {4, {(cuuint64_t)g.Co, (cuuint64_t)g.Wo, (cuuint64_t)g.Ho, (cuuint64_t)g.B},
+              {(cuuint64_t)ld0, (cuuint64_t)ld0 * g.Wo, (cuuint64_t)ld0 * g.Wo * g.Ho},
+              {(cuuint32_t)a_sw, (cuuint32_t)p.Wt, (cuuint32_t)p.Ht, (cuuint32_t)p.Bt}, a_sw, q0};
+      }
+      p.w_tiles = (g.Wo + p.Wt - 1) / p.Wt;
+      p.h_tiles = (g.Ho + p.Ht - 1) / p.Ht;
+      p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
       p.kb_total = p.w_tiles * p.h_tiles * p.b_tiles;
+      if (p.i2c) p.kb_total = (int)((g.gk + p.kdepth - 1) / p.kdepth);
       m_tiles = (g.Co + BM - 1) / BM;
       p.n_tiles_n = g.R * g.S * p.n_chunks;
       break;
@@ -2066,7 +2363,12 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
     default:
       return false;
   }
+  if (want == PLAN_HALO && !p.halo) return false;
   p.ksteps = p.kdepth / 32;
+  if (tail && (tail + 31) / 32 < p.ksteps) {
+    p.tail_ks = (tail + 31) / 32;
+    if (p.c_chunks == 1) { p.ksteps = p.tail_ks; p.tail_ks = 0; }                // every chunk is the short one
+  }
   // operand staging
   if (a_mn) {
     p.a_boxes = BM / a_sw;
@@ -2095,11 +2397,11 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
     p.a_bytes = p.mrep * p.a_box_bytes;
     m_tiles = (m_tiles + p.mrep - 1) / p.mrep;
   }
+  if (want == PLAN_BATCHED && p.mrep == 1) return false;
   const int bn_cta = p.bn / ctas;               // output columns staged by each CTA
   if (bn_cta % 16) return false;
   if (b_mn) {
-    if (bn_cta % b_sw) return false;
-    p.b_boxes = bn_cta / b_sw;
+    p.b_boxes = (bn_cta + b_sw - 1) / b_sw;
     p.b_box_bytes = p.kdepth * b_sw;
     p.b_box_step = b_sw;
     p.b_bytes = p.b_boxes * p.b_box_bytes;
@@ -2140,7 +2442,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
   if ((g.kind == GK_FC_FWD || g.kind == GK_FC_DGRAD || g.kind == GK_FC_WGRAD) && p.n_tiles_n > 1 && p.m_units > 1)
     p.raster_g = ctas == 2 ? 8 : 12;
   // split the contraction when the tiles alone cannot fill the SMs
-  if (tiles < units && p.kb_total >= 8) {
+  if (tiles < units && p.kb_total >= 8 && p.dstride <= 1) {
     // pick the split count with the least modelled time: waves of items, each item running its
     // share of the k-blocks plus a fixed cost (pipeline fill and the atomic epilogue) of about
     // four k-blocks
@@ -2164,14 +2466,14 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
     const int max_kb = NITI_SPLIT_MAX_K / p.kdepth;
     const int min_splits = (p.kb_total + max_kb - 1) / max_kb;
     if (p.splits < min_splits) p.splits = min_splits;
-    if (p.splits > NITI_MAX_SPLITS) return false;
+    if (p.splits > NITI_MAX_SPLITS || (p.splits > 1 && p.dstride > 1)) return false;
   }
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
   p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;
   // split contractions add their partial sums atomically: room for the epilogue warps' transpose
   // buffers (consecutive output rows only: every multiply but the pixel-box convolutions)
   p.stg_off = 0;
-  if (p.splits > 1 && !p.halo && g.kind != GK_CONV_FWD && g.kind != GK_CONV_DGRAD) {
+  if (p.splits > 1 && !p.halo && (p.i2c || (g.kind != GK_CONV_FWD && g.kind != GK_CONV_DGRAD))) {
     const int stg_bytes = EPI_WARPS * 32 * 33 * 4;
     int st = (200 * 1024 - stg_bytes) / stage_bytes;
     if (st > MAX_STAGES) st = MAX_STAGES;
@@ -2179,6 +2481,15 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
       p.stages = st;
       p.stg_off = st * stage_bytes;
     }
+  }
+  // rows with a pitch that is no multiple of 8: staging buffers of the fused epilogue's stores
+  p.nstg_off = 0;
+  if (p.splits == 1 && !p.halo && ((g.gn & 7) != 0 || (g.kind == GK_CONV_WGRAD && (p.Cn & 7) != 0))) {
+    int st = (200 * 1024 - EPI_WARPS * 32 * 36) / stage_bytes;
+    if (st > MAX_STAGES) st = MAX_STAGES;
+    if (st < 2) return false;
+    p.stages = st;
+    p.nstg_off = st * stage_bytes;
   }
   if (p.halo) {
     p.splits = 1;
@@ -2208,15 +2519,20 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, bool want_halo, 
   // convolution outputs are spatially structured (borders, images): contiguous item ranges make the
   // first tile of every CTA an even sample of the tensor for the speculative shift
   p.blocked = (g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD) ? 1 : 0;
-  p.items = tiles * p.splits;
+  p.items = tiles * p.splits * (p.dstride > 1 ? p.nph_r * p.nph_s : 1);
   if (p.items >= (1LL << 30)) return false;      // the kernel counts items in 32 bits
+  // the copies an instance issues have the rank and mode of its maps: anything else is a planning error
+  if (!p.halo && (g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD) &&
+      (sb.nd != (p.mode >= 1 ? 3 : 2) || sa.nd != 4 || sa.im2col != p.i2c))
+    return false;
+  if (!p.halo && g.kind == GK_CONV_WGRAD && (sa.nd != (p.i2c ? 2 : 4) || sb.nd != 4 || sb.im2col != p.i2c)) return false;
+  if (p.i2c && p.mode < 1) return false;
   if (!encode(ctx, &ma, sa) || !encode(ctx, &mb, sb)) return false;
   return true;
 }
 
 }  // namespace
 
-size_t niti_tc_scratch_bytes(const GemmProblem &) { return 0; }
 
 int niti_tc_timeout_probe(niti_ctx *ctx, cudaStream_t st) {
   timeout_probe_kernel<<<1, 32, 0, st>>>(ctx->d_status);
@@ -2230,13 +2546,13 @@ int niti_tc_timeout_probe(niti_ctx *ctx, cudaStream_t st) {
 // a second, short wave.
 // Dynamic shared-memory limit of the kernel: once per context, and always the most the device allows
 // beside the kernel's static shared memory (see niti_ctx::smem_optin for why not "what this launch needs").
-template <int CTAS>
+template <int CTAS, int MODE>
 static int tc_set_smem_limit(niti_ctx *ctx) {
   cudaFuncAttributes fa;
-  NITI_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, tc_gemm_kernel<CTAS>));
+  NITI_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, tc_gemm_kernel<CTAS, MODE>));
   const size_t limit = ctx->smem_optin > fa.sharedSizeBytes ? ctx->smem_optin - fa.sharedSizeBytes : 0;
-  NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(tc_gemm_kernel<CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
-  ctx->tc_attr_smem[CTAS] = limit;
+  NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(tc_gemm_kernel<CTAS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  ctx->tc_attr_smem[CTAS + 2 * MODE] = limit;
   return NITI_OK;
 }
 
@@ -2258,22 +2574,23 @@ static int tc_units(niti_ctx *ctx) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    (void)tc_set_smem_limit<2>(ctx);
+    (void)tc_set_smem_limit<2, 0>(ctx);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2>, &cfg) == cudaSuccess && n > 0 && n < cached) cached = n;
+    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2, 0>, &cfg) == cudaSuccess && n > 0 && n < cached) cached = n;
     else (void)cudaGetLastError();
   }
   return cached;
 }
 
-template <int CTAS>
-static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb,
+template <int CTAS, int MODE>
+static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb,
                      int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
   size_t smem = (size_t)p.stages * (p.a_bytes + p.b_bytes) + (size_t)p.b_res_bytes + 1024;
   if (p.stg_off > 0) smem = (size_t)p.stg_off + (size_t)EPI_WARPS * 32 * 33 * 4 + 1024;
-  size_t &attr_smem = ctx->tc_attr_smem[CTAS];
+  if (p.nstg_off > 0) smem = (size_t)p.nstg_off + (size_t)EPI_WARPS * 32 * 36 + 1024;
+  size_t &attr_smem = ctx->tc_attr_smem[CTAS + 2 * MODE];
   if (!attr_smem) {
-    const int rcs = tc_set_smem_limit<CTAS>(ctx);
+    const int rcs = tc_set_smem_limit<CTAS, MODE>(ctx);
     if (rcs != NITI_OK) return rcs;
   }
   if (smem > attr_smem) return niti_fail(ctx, NITI_ERR_SHAPE, "tensor-core kernel: stage buffers exceed the shared memory of an SM");
@@ -2314,7 +2631,7 @@ static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CU
     q.k_tmem_cols = cols;
     // reciprocals for tile index -> coordinates; dividends stay below the tile count
     const unsigned long long n_max = (unsigned long long)(p.w_tiles > 0 ? p.w_tiles : 1) * (p.h_tiles > 0 ? p.h_tiles : 1) *
-                                     (p.b_tiles > 0 ? p.b_tiles : 1) + 2;
+                                     (p.b_tiles > 0 ? p.b_tiles : 1) + 512;
     q.magic_w = (p.w_tiles > 1 && n_max * p.w_tiles < (1ull << 32)) ? (unsigned)((1ull << 32) / p.w_tiles + 1) : 0u;
     q.magic_h = (p.h_tiles > 1 && n_max * p.h_tiles < (1ull << 32)) ? (unsigned)((1ull << 32) / p.h_tiles + 1) : 0u;
   }
@@ -2325,12 +2642,23 @@ static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CU
     slot = ctx->d_spec_tab + 2 * (size_t)((key ^ (key >> 13)) % NITI_SPEC_SLOTS);
     q.spec_tag = (int)(unsigned)(key | 1u);
   }
-  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS>, ma, mb, q, acc, hdr, ctx->d_status, r.out, r.mask,
+  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE>, ma, mb, q, acc, hdr, ctx->d_status, r.out, r.mask,
                                         r.s_a, r.s_w, r.s_out, r.b_out, slot, r.pool_out));
   ctx->launches++;
-  ctx->tc_launches++;
-  if (CTAS == 2) ctx->tc2_launches++;
+  if (MODE != 2) {                   // (the counters of the header cover the kernel without its strided form)
+    ctx->tc_launches++;
+    if (CTAS == 2) ctx->tc2_launches++;
+  }
   return NITI_OK;
+}
+
+static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb,
+                     int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
+  if (p.mode == 2)
+    return p.ctas == 2 ? launch_tc_as<2, 2>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 2>(ctx, st, p, ma, mb, acc, hdr, r);
+  if (p.mode == 1)
+    return p.ctas == 2 ? launch_tc_as<2, 1>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 1>(ctx, st, p, ma, mb, acc, hdr, r);
+  return p.ctas == 2 ? launch_tc_as<2, 0>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 0>(ctx, st, p, ma, mb, acc, hdr, r);
 }
 
 // Profiling event of a launch.  On a stream that is being captured the record becomes an event-record
@@ -2355,21 +2683,24 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   // engine 0: pairs of CTAs (cta_group::2) when there are enough 256-row tiles to fill the GPU.
   // Test switches: 2 / 3 force the single-CTA / paired kernel, 4 keeps the int32 spill epilogue.
   // Test switches: 5 disables the halo mode of small-channel convolutions.
+  // (columns of one tap of a convolution's weight gradient start at multiples of the channel count)
+  const bool aligned = (g.gn & 31) == 0 && ((uintptr_t)r.out & 31) == 0 && ((uintptr_t)r.mask & 31) == 0 &&
+                       (g.kind != GK_CONV_WGRAD || (g.Ci & 31) == 0);
   bool planned = false;
   if ((g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD || g.kind == GK_CONV_WGRAD) && ctx->engine != 3 &&
       ctx->engine != 5)
-    planned = plan(ctx, g, 1, true, p, ma, mb) && p.halo;
+    planned = plan(ctx, g, 1, PLAN_HALO, aligned, p, ma, mb);
   if (!planned && g.kind == GK_FC_FWD && ctx->engine != 3)      // row-batched mode of short contractions
-    planned = plan(ctx, g, 1, false, p, ma, mb) && p.mrep > 1;
+    planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, p, ma, mb);
   if (!planned && ctx->engine != 2 && g.gm >= 2 * BM) {
-    planned = plan(ctx, g, 2, false, p, ma, mb);
+    planned = plan(ctx, g, 2, PLAN_ANY, aligned, p, ma, mb);
     // (pairs halve the operand traffic per MMA; they are kept unless they would leave more than a
     // third of the GPU idle)
     if (planned && ctx->engine != 3 && p.items * 3 < (long long)(ctx->sm_count / 2) * 2) planned = false;
   }
   if (!planned) {
     if (ctx->engine == 3) return NITI_ERR_SHAPE;
-    if (!plan(ctx, g, 1, false, p, ma, mb)) return NITI_ERR_SHAPE;
+    if (!plan(ctx, g, 1, PLAN_ANY, aligned, p, ma, mb)) return NITI_ERR_SHAPE;
   }
   {
     // expected ratio between the max of the whole tensor (N values) and the max of the first tile of
@@ -2395,10 +2726,16 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   p.mbits = r.mbits;
   p.round_mode = r.round_mode;
   p.relu = r.relu;
-  p.epi_mode = (p.splits > 1 || p.halo == 2) ? EPI_ATOMIC : ((ctx->engine == 4 || dp_sum) ? EPI_SPILL : EPI_SPECULATE);
+  p.epi_mode = (p.splits > 1 || p.halo == 2) ? EPI_ATOMIC : ((ctx->engine == 4 || dp_sum || !r.out) ? EPI_SPILL : EPI_SPECULATE);
   if (p.epi_mode == EPI_ATOMIC && niti_partial_slices(g.kind, g.gm) > 1 && p.splits <= niti_partial_slices(g.kind, g.gm) &&
       !p.halo && p.mrep == 1)
     p.epi_mode = EPI_PARTIAL;
+  if (p.dstride > 1 && (p.nph_r < p.dstride || p.nph_s < p.dstride)) {
+    // filter smaller than the stride: no window reaches the input pixels of the other phases
+    if (p.epi_mode == EPI_SPILL) NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(g.gm * g.gn), st));
+    else NITI_CUDA_TRY(ctx, cudaMemsetAsync(r.out, 0, (size_t)(g.gm * g.gn), st));
+    ctx->launches++;
+  }
   if (p.epi_mode == EPI_ATOMIC) {
     NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(g.gm * g.gn), st));
     ctx->launches++;
@@ -2430,7 +2767,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   }
   const bool prof = ctx->profile_on && ctx->prof_ev && ctx->prof_used < NITI_PROF_MAX;
   if (prof) prof_record(ctx->prof_ev[2 * ctx->prof_used], st);
-  int rc = p.ctas == 2 ? launch_tc<2>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc<1>(ctx, st, p, ma, mb, acc, hdr, r);
+  int rc = launch_tc(ctx, st, p, ma, mb, acc, hdr, r);
   if (rc != NITI_OK) return rc;
   if (p.epi_mode == EPI_SPECULATE && p.single_wave) {
     *fused = true;                     // exact shift, scalars published by the last CTA: no second launch
@@ -2441,7 +2778,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
       if (rc != NITI_OK) return rc;
     }
     p.epi_mode = EPI_KNOWN_B;
-    rc = p.ctas == 2 ? launch_tc<2>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc<1>(ctx, st, p, ma, mb, acc, hdr, r);
+    rc = launch_tc(ctx, st, p, ma, mb, acc, hdr, r);
     if (rc != NITI_OK) return rc;
     *fused = true;
   }
