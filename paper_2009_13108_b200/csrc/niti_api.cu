@@ -297,9 +297,9 @@ static bool fill_conv(GemmProblem &p, int kind, int B, int H, int W, int Ci, int
 }
 
 // int32 elements of the accumulator scratch of a fully connected backward call: the larger of the weight
-// gradient [N][K] and the error [M][K] (times its partial slices when the batch is small)
+// gradient [N][K] and the error [M][K]
 static size_t linear_bwd_acc_elems(long long M, long long N, long long K) {
-  const size_t a = (size_t)(M * K) * (size_t)niti_partial_slices(GK_FC_DGRAD, M), b = (size_t)(N * K);
+  const size_t a = (size_t)(M * K), b = (size_t)(N * K);
   return a > b ? a : b;
 }
 
@@ -321,7 +321,7 @@ extern "C" size_t niti_workspace_bytes(int op, const int64_t *d, int nd) {
     case NITI_OP_LINEAR_FWD:
       if (nd != 3 || d[0] <= 0 || d[1] <= 0 || d[2] <= 0) return 0;
       fill_fc(p, GK_FC_FWD, (int)d[0], (int)d[1], (int)d[2]);
-      outs = (size_t)(d[0] * d[1]) * (size_t)niti_partial_slices(GK_FC_FWD, d[0]);
+      outs = (size_t)(d[0] * d[1]);
       extra = pad_bytes(p);
       break;
     case NITI_OP_LINEAR_BWD_UPDATE:
@@ -481,7 +481,7 @@ extern "C" int niti_linear_fwd(niti_ctx *ctx, void *stream, const int8_t *a, con
   fill_fc(p, GK_FC_FWD, M, N, K);
   p.p0 = a; p.p1 = w;
   int64_t dims[3] = {M, N, K};
-  char *pad_mem = (char *)ws + NITI_WS_HEADER + round_up((size_t)M * N * niti_partial_slices(GK_FC_FWD, M) * 4, 256);
+  char *pad_mem = (char *)ws + NITI_WS_HEADER + round_up((size_t)M * N * 4, 256);
   return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes,
                         niti_workspace_bytes(NITI_OP_LINEAR_FWD, dims, 3), pad_mem, out, 7, round_mode, relu,
                         nullptr, s_a, s_w, s_out, b_out);

@@ -190,16 +190,6 @@ struct GemmProblem {
   int win_chans, win_sw, win_sh;
 };
 
-// Fully connected forward / error multiplies with at most 128 output rows (weight streaming: the
-// contraction is split over the SMs) keep up to this many int32 partial tensors in the scratch, one
-// per split; 1 for every other multiply.  The workspace query reserves room accordingly.
-#define NITI_PARTIAL_SLICES 16
-static inline int niti_partial_slices(int kind, long long gm) {
-  return ((kind == 0 || kind == 1) && gm <= 128) ? NITI_PARTIAL_SLICES : 1;   // GK_FC_FWD, GK_FC_DGRAD
-}
-// acc holds `splits` partial tensors of n int32 each: adds them into the first, takes max |sum| into
-// hdr->maxabs32 and raises NITI_DEV_ACC_RANGE when the magnitudes of an element's partial sums add up to 2^31
-int niti_launch_sum_partials(niti_ctx *ctx, cudaStream_t st, int32_t *acc, int splits, long long n, WsHeader *hdr);
 // shard_ok: the caller rounds only this rank's shard afterwards (niti_dp_shard) and all-gathers the result
 int niti_reduce_after_gemm(niti_ctx *ctx, cudaStream_t st, int kind, int32_t *acc, long long n, WsHeader *hdr,
                            bool shard_ok = false);

@@ -51,8 +51,8 @@ struct TcParams {
                                 // weights takes every other tile)
   int one_commit;               // resident-weights mode with as many patch stages as accumulator buffers:
                                 // stage and buffer advance together, one barrier per tile serves both
-  int stg_off;                  // > 0: byte offset (from the aligned base) of the epilogue warps' transpose
-                                // buffers for coalesced atomic adds, 32 x 33 words per warp
+  int red;                      // split contraction whose partial sums are added by TMA reduce copies (map_c)
+  int red_off;                  // byte offset (from the aligned base) of the epilogue warps' 4 KB buffers for them
   int nstg_off;                 // byte offset of the staging buffers for rows with a pitch that is no multiple of 8
   int mrep;                     // 128-row tiles per item (row-batched mode of short contractions), else 1
   int bn_mma;                   // N of one MMA; bn = mrep * bn_mma accumulator columns per item
@@ -131,7 +131,9 @@ struct TcParams {
 // Epilogue modes.  The shift of Algorithm 2 needs the bit-width of the WHOLE accumulator tensor:
 //  EPI_SPILL      store int32 accumulators + max; a second kernel rounds (always exact, 8 B / output
 //                 of extra traffic)
-//  EPI_ATOMIC     split contraction: add partial sums into a zeroed int32 tensor
+//  EPI_ATOMIC     split contraction: add partial sums into a zeroed int32 tensor, 32 x 32 values per TMA reduce copy.
+//                 (An SM retires only about 1.6 atomic additions per cycle from registers, 4.9 us for a 64 x 256 tile
+//                 and 11 us for a 128 x 256 one; the reduce copies add at L2 in whole lines.)
 //  EPI_SPECULATE  every CTA computes its first tile, the grid agrees on the max over those tiles
 //                 (one bounded grid-wide wait), and all tiles are rounded and stored as int8 with the
 //                 shift that max implies, while the true max is tracked.  If the true bit-width turns
@@ -139,13 +141,7 @@ struct TcParams {
 //                 the common case costs one multiply and no int32 traffic)
 //  EPI_KNOWN_B    bit-width known (hdr->maxabs32): round and store directly.  The kernel returns at
 //                 once when the speculative pass was right.
-//  EPI_PARTIAL    split contraction of a multiply with few output rows (fully connected layers at batch
-//                 <= 128): every split stores its int32 partial tile to its own slice of the scratch
-//                 (plain 16-byte stores) and a small kernel adds the slices and takes the max.  An SM
-//                 retires only about 1.6 atomic additions per cycle, so the 64 x 256 partial tile of a
-//                 weight-streaming multiply took 5 us to add atomically, as long as a 4 MB layer takes
-//                 to stream.
-enum { EPI_SPILL = 0, EPI_ATOMIC = 1, EPI_SPECULATE = 2, EPI_KNOWN_B = 3, EPI_PARTIAL = 4 };
+enum { EPI_SPILL = 0, EPI_ATOMIC = 1, EPI_SPECULATE = 2, EPI_KNOWN_B = 3 };
 
 
 // ------------------------------------------------------------------------------------------
@@ -282,6 +278,38 @@ __device__ __forceinline__ void tma_load_im2col(unsigned dst, const CUtensorMap 
       "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(ow), "h"(oh)
       : "memory");
+}
+// Adds a 32 x 32 int32 tile from shared memory (rows of 128 bytes, 128-byte swizzle) into the accumulator tensor;
+// elements outside the tensor are left out.
+__device__ __forceinline__ void tma_reduce_add_4d(const CUtensorMap *map, unsigned src, int c0, int c1, int c2, int c3) {
+  asm volatile(
+      "cp.reduce.async.bulk.tensor.4d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n\t"
+      "cp.async.bulk.commit_group;"
+      ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
+}
+// this thread's reduce copies have read their source / are complete
+__device__ __forceinline__ void tma_reduce_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_reduce_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void st_shared_v4(unsigned addr, int a, int b, int c, int d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void st_shared_b32(unsigned addr, int a) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
+}
+// One lane's 32 values as row `lane` (or, TRANSPOSED, as column `lane`) of the swizzled tile at `buf`.
+template <bool TRANSPOSED>
+__device__ __forceinline__ void stage_tile32(unsigned buf, int lane, const int (&v)[32]) {
+  if (TRANSPOSED) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      st_shared_b32(buf + (unsigned)(j * 128 + ((((lane >> 2) ^ (j & 7)) << 4) | ((lane & 3) << 2))), v[j]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      st_shared_v4(buf + (unsigned)(lane * 128 + ((j ^ (lane & 7)) << 4)), v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+  }
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -857,7 +885,7 @@ __device__ __forceinline__ void halo_mma_loop(const TcParams &p, int issuer, int
 template <int CTAS, int MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const TcParams p, int32_t *__restrict__ acc, WsHeader *hdr, uint32_t *status,
+               const __grid_constant__ CUtensorMap map_c, const TcParams p, int32_t *__restrict__ acc, WsHeader *hdr, uint32_t *status,
                int8_t *__restrict__ out8, const int8_t *__restrict__ mask8, const int32_t *s_a,
                const int32_t *s_w, int32_t *s_out, int32_t *b_out, int32_t *spec_slot, int8_t *__restrict__ pool8) {
   constexpr bool I2C = MODE >= 1, STRIDED = MODE == 2, GENERAL = MODE >= 1;
@@ -938,6 +966,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (threadIdx.x == 32) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
+    if (p.red) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
   }
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -1322,6 +1351,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       bp = b > p.mbits ? b - p.mbits : 0;
     }
     bool ok = true;
+    const unsigned red_buf = smem_base + (unsigned)p.red_off + (unsigned)(warp - EPI_WARP0) * 4096u;
     if (p.halo == 2) {
       // lane = (tap of the pair, input channel), column = output channel; partial sums of this
       // CTA's pixel range are added to g32[co][tap][ci]
@@ -1337,13 +1367,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           const int tap = 2 * pi + which;
           int v[32];
           tc_ld32(tmem_base + ((unsigned)(quarter * 32) << 16) + 64u * pi + (unsigned)c0, v);
-          if (tap < 9) {
-            int32_t *dst = acc + (long long)(co0 + c0) * p.gn + (long long)tap * p.Cn + ci0 + ci;
+          if (tap < 9) {                        // (a warp's 32 rows belong to one tap)
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              pmx = max(pmx, (unsigned)abs(v[j]));
-              if (v[j] != 0) atomicAdd(dst + (long long)j * p.gn, v[j]);
-            }
+            for (int j = 0; j < 32; ++j) pmx = max(pmx, (unsigned)abs(v[j]));
+            if (lane == 0) tma_reduce_wait_read();
+            __syncwarp();
+            stage_tile32<true>(red_buf, lane, v);
+            fence_async_shared();
+            __syncwarp();
+            if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, ci0 + (ci & ~31), tap, co0 + c0, 0);
           }
         }
         pmx = __reduce_max_sync(0xffffffffu, pmx);
@@ -1451,38 +1483,46 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
       tc_fence_after();
       const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)p.bn;
-      if (p.epi_mode == EPI_ATOMIC && p.stg_off > 0) {
-        // Partial sums of a split contraction.  A lane holds one row of the chunk, so an atomic add
-        // issued straight from the registers touches 32 different lines; the chunk is transposed
-        // through shared memory instead and every add instruction covers 32 consecutive columns of
-        // one row (one 128-byte line).  Output rows are consecutive here (no pixel-box mapping).
-        int *stg = reinterpret_cast<int *>(smem_raw + (smem_base - smem_u32(smem_raw)) + p.stg_off) +
-                   (warp - EPI_WARP0) * (32 * 33);
-        const long long row0 = out_row - lane;                 // output row of lane 0 of this warp
+      if (p.epi_mode == EPI_ATOMIC && p.red) {
+        // partial sums of a split contraction: every chunk is staged and added by one copy
         unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
-        for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
+        int x0, x1, x2 = 0, x3 = 0;                            // tensor coordinates of the chunk at column 0
+        if (p.kind == GK_CONV_WGRAD) {
+          const int tap = nt / p.n_chunks;
+          x0 = (nt - tap * p.n_chunks) * p.bn;
+          x1 = tap;
+          x2 = mt * BM + quarter * 32;
+        } else if (p.red == 2) {                               // pixel boxes
+          x0 = (int)col0;
+          int w0, h0, b0;
+          pixel_box(p, mt, w0, h0, b0);
+          x1 = __shfl_sync(0xffffffffu, w0 + r_ww, 0);
+          x2 = __shfl_sync(0xffffffffu, h0 + r_hh, 0);
+          x3 = __shfl_sync(0xffffffffu, b0 + r_bb, 0);
+        } else {
+          x0 = (int)col0;
+          x1 = mt * BM + quarter * 32;
+        }
+        const bool any_row = __any_sync(0xffffffffu, row_ok);
+        for (int c = 32 * chunk_phase; c < p.bn && c < ncols_valid && any_row; c += 32 * wpq) {
           int v[32];
           tc_ld32(tm_row + (unsigned)c, v);
-          if (c < ncols_valid) {                               // (uniform across the warp)
+          // (rows and columns outside the matrix are clipped by the copy; they may hold anything)
+          if (row_ok) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { stg[lane * 33 + j] = v[j]; pmx = max(pmx, (unsigned)abs(v[j])); }
-            __syncwarp();
-            const bool col_ok = c + lane < ncols_valid;
-            int32_t *dcol = acc + row0 * p.gn + col0 + c + lane;
-            long long rows_left = p.gm - row0;
-            if (rows_left > 32) rows_left = 32;
-            for (int rr = 0; rr < (int)rows_left; ++rr) {
-              const int val = stg[rr * 33 + lane];
-              if (col_ok && val != 0) atomicAdd(dcol + (long long)rr * p.gn, val);
-            }
-            __syncwarp();
+            for (int j = 0; j < 32; ++j) pmx = max(pmx, (unsigned)abs(v[j]));
           }
+          if (lane == 0) tma_reduce_wait_read();
+          __syncwarp();
+          stage_tile32<false>(red_buf, lane, v);
+          fence_async_shared();
+          __syncwarp();
+          if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, x0 + c, x1, x2, x3);
         }
         pmx = __reduce_max_sync(0xffffffffu, pmx);
         if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
-      } else if (p.epi_mode <= EPI_ATOMIC || p.epi_mode == EPI_PARTIAL) {
+      } else if (p.epi_mode <= EPI_ATOMIC) {
         int32_t *dst = acc + out_row * p.gn + col0;
-        if (p.epi_mode == EPI_PARTIAL) dst += (long long)split * p.gm * p.gn;      // this split's slice
         const bool vec_ok = ((p.gn & 3) == 0) && ((col0 & 3) == 0);
         unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
         for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
@@ -1878,6 +1918,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       if (lane == 0 && mx) atomicMax(&cta_max, mx);     // (one global atomic per CTA, below)
     }
+    if (p.red && lane == 0) tma_reduce_wait_all();      // (shared memory stays valid until the copies are done)
   }
 
   // ================= common exit =================
@@ -2033,6 +2074,41 @@ static bool pick_pixel_box(int W, int H, int B, int &Wt, int &Ht, int &Bt) {
   return Wt <= W && Ht <= H && Bt <= B;
 }
 
+constexpr size_t SMEM_BUDGET = 225 * 1024;            // dynamic shared memory beside the kernel's static arrays and alignment
+constexpr size_t RED_BYTES = (size_t)EPI_WARPS * 4096;
+
+// Map of the int32 accumulators for the reduce copies of a split contraction: 32 columns x 32 rows per copy, where
+// the rows are consecutive rows, or one tap's rows of 32 output channels, or 32 pixels of a box.  Rows of a pitch
+// that is no multiple of 16 bytes have no map (the epilogue then adds from registers).
+static bool reduce_map(niti_ctx *ctx, const GemmProblem &g, TcParams &p, int32_t *acc, CUtensorMap &mc) {
+  if (!ctx->encode_tiled || ((uintptr_t)acc & 15)) return false;
+  const cuuint64_t row = (cuuint64_t)g.gn * 4;
+  cuuint64_t dims[4] = {(cuuint64_t)g.gn, (cuuint64_t)g.gm, 1, 1};
+  cuuint64_t strides[3] = {row, row * (cuuint64_t)g.gm, row * (cuuint64_t)g.gm};
+  cuuint32_t box[4] = {32, 32, 1, 1};
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  int red = 1;
+  if (g.kind == GK_CONV_WGRAD) {
+    dims[0] = (cuuint64_t)p.Cn; dims[1] = (cuuint64_t)g.R * g.S; dims[2] = (cuuint64_t)g.Co;
+    strides[0] = (cuuint64_t)p.Cn * 4; strides[1] = row; strides[2] = row * (cuuint64_t)g.Co;
+    box[1] = 1; box[2] = 32;
+  } else if ((g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD) && !p.i2c) {
+    red = 2;
+    dims[1] = (cuuint64_t)p.PW; dims[2] = (cuuint64_t)p.PH; dims[3] = (cuuint64_t)p.PB;
+    strides[1] = row * p.PW; strides[2] = row * p.PW * p.PH;
+    box[1] = p.Wt < 32 ? p.Wt : 32;
+    box[2] = p.Ht < 32 / (int)box[1] ? p.Ht : 32 / box[1];
+    box[3] = 32 / (box[1] * box[2]);
+  }
+  if ((strides[0] & 15) || (strides[1] & 15) || strides[2] >= (1ull << 40)) return false;
+  if (((EncodeTiledFn)ctx->encode_tiled)(&mc, CU_TENSOR_MAP_DATA_TYPE_INT32, 4, acc, dims, strides, box, es,
+                                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                         CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return false;
+  p.red = red;
+  return true;
+}
+
 // Extents and strides of a tensor of overlapping windows (see WindowGeometry at the boundary): a window's channels,
 // the windows of a row, rows, images.
 static void window_map(const GemmProblem &g, MapSpec &s) {
@@ -2054,8 +2130,8 @@ static int pick_bn(long long gn) {
 // `aligned`: output (and mask) pointers and rows are 32-byte aligned.
 // want: ANY, or only a plan in the resident-weights / tap-pair mode (HALO) or the row-batched mode (BATCHED).
 enum PlanWant { PLAN_ANY = 0, PLAN_HALO = 1, PLAN_BATCHED = 2 };
-static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, TcParams &p, CUtensorMap &ma,
-                 CUtensorMap &mb) {
+static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, int32_t *acc, TcParams &p, CUtensorMap &ma,
+                 CUtensorMap &mb, CUtensorMap &mc) {
   memset(&p, 0, sizeof(p));
   p.ctas = ctas;
   p.kind = g.kind;
@@ -2309,6 +2385,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
         p.items = blocks * p.splits;
         p.m_units = 1;
         p.n_tiles_n = 1;
+        if (!reduce_map(ctx, g, p, acc, mc)) return false;
+        p.red_off = p.stages * (p.a_bytes + p.b_bytes);
         if (!encode(ctx, &ma, sa) || !encode(ctx, &mb, sb)) return false;
         return true;
       }
@@ -2449,9 +2527,6 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     double best = 1e30;
     int best_s = 1;
     int max_s = p.kb_total / 4;
-    // (multiplies with few output rows keep their splits' partial tiles in separate slices of the scratch)
-    const int slices = niti_partial_slices(g.kind, g.gm);
-    if (slices > 1 && max_s > slices) max_s = slices;
     for (int sp = 1; sp <= max_s && sp <= 4 * units; ++sp) {
       const long long it = tiles * sp;
       const long long waves = (it + units - 1) / units;
@@ -2470,16 +2545,14 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   }
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
   p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;
-  // split contractions add their partial sums atomically: room for the epilogue warps' transpose
-  // buffers (consecutive output rows only: every multiply but the pixel-box convolutions)
-  p.stg_off = 0;
-  if (p.splits > 1 && !p.halo && (p.i2c || (g.kind != GK_CONV_FWD && g.kind != GK_CONV_DGRAD))) {
-    const int stg_bytes = EPI_WARPS * 32 * 33 * 4;
-    int st = (200 * 1024 - stg_bytes) / stage_bytes;
+  if (p.splits > 1 && !p.halo && reduce_map(ctx, g, p, acc, mc)) {
+    int st = (int)(SMEM_BUDGET - RED_BYTES) / stage_bytes;
     if (st > MAX_STAGES) st = MAX_STAGES;
     if (st >= 2) {
       p.stages = st;
-      p.stg_off = st * stage_bytes;
+      p.red_off = st * stage_bytes;
+    } else {
+      p.red = 0;
     }
   }
   // rows with a pitch that is no multiple of 8: staging buffers of the fused epilogue's stores
@@ -2583,10 +2656,10 @@ static int tc_units(niti_ctx *ctx) {
 }
 
 template <int CTAS, int MODE>
-static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb,
+static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                      int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
   size_t smem = (size_t)p.stages * (p.a_bytes + p.b_bytes) + (size_t)p.b_res_bytes + 1024;
-  if (p.stg_off > 0) smem = (size_t)p.stg_off + (size_t)EPI_WARPS * 32 * 33 * 4 + 1024;
+  if (p.red) smem = (size_t)p.red_off + RED_BYTES + 1024;
   if (p.nstg_off > 0) smem = (size_t)p.nstg_off + (size_t)EPI_WARPS * 32 * 36 + 1024;
   size_t &attr_smem = ctx->tc_attr_smem[CTAS + 2 * MODE];
   if (!attr_smem) {
@@ -2642,7 +2715,7 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
     slot = ctx->d_spec_tab + 2 * (size_t)((key ^ (key >> 13)) % NITI_SPEC_SLOTS);
     q.spec_tag = (int)(unsigned)(key | 1u);
   }
-  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE>, ma, mb, q, acc, hdr, ctx->d_status, r.out, r.mask,
+  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE>, ma, mb, mc, q, acc, hdr, ctx->d_status, r.out, r.mask,
                                         r.s_a, r.s_w, r.s_out, r.b_out, slot, r.pool_out));
   ctx->launches++;
   if (MODE != 2) {                   // (the counters of the header cover the kernel without its strided form)
@@ -2652,13 +2725,13 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
   return NITI_OK;
 }
 
-static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb,
+static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                      int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
   if (p.mode == 2)
-    return p.ctas == 2 ? launch_tc_as<2, 2>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 2>(ctx, st, p, ma, mb, acc, hdr, r);
+    return p.ctas == 2 ? launch_tc_as<2, 2>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 2>(ctx, st, p, ma, mb, mc, acc, hdr, r);
   if (p.mode == 1)
-    return p.ctas == 2 ? launch_tc_as<2, 1>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 1>(ctx, st, p, ma, mb, acc, hdr, r);
-  return p.ctas == 2 ? launch_tc_as<2, 0>(ctx, st, p, ma, mb, acc, hdr, r) : launch_tc_as<1, 0>(ctx, st, p, ma, mb, acc, hdr, r);
+    return p.ctas == 2 ? launch_tc_as<2, 1>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 1>(ctx, st, p, ma, mb, mc, acc, hdr, r);
+  return p.ctas == 2 ? launch_tc_as<2, 0>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 0>(ctx, st, p, ma, mb, mc, acc, hdr, r);
 }
 
 // Profiling event of a launch.  On a stream that is being captured the record becomes an event-record
@@ -2675,7 +2748,8 @@ static void prof_record(cudaEvent_t ev, cudaStream_t st) {
 int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const RoundSpec &r_in, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled, bool shard_ok, bool *updated) {
   TcParams p;
-  CUtensorMap ma, mb;
+  CUtensorMap ma, mb, mc;
+  memset(&mc, 0, sizeof(mc));
   RoundSpec r = r_in;
   *fused = false;
   if (pooled) *pooled = false;
@@ -2689,18 +2763,18 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   bool planned = false;
   if ((g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD || g.kind == GK_CONV_WGRAD) && ctx->engine != 3 &&
       ctx->engine != 5)
-    planned = plan(ctx, g, 1, PLAN_HALO, aligned, p, ma, mb);
+    planned = plan(ctx, g, 1, PLAN_HALO, aligned, acc, p, ma, mb, mc);
   if (!planned && g.kind == GK_FC_FWD && ctx->engine != 3)      // row-batched mode of short contractions
-    planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, p, ma, mb);
+    planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, acc, p, ma, mb, mc);
   if (!planned && ctx->engine != 2 && g.gm >= 2 * BM) {
-    planned = plan(ctx, g, 2, PLAN_ANY, aligned, p, ma, mb);
+    planned = plan(ctx, g, 2, PLAN_ANY, aligned, acc, p, ma, mb, mc);
     // (pairs halve the operand traffic per MMA; they are kept unless they would leave more than a
     // third of the GPU idle)
     if (planned && ctx->engine != 3 && p.items * 3 < (long long)(ctx->sm_count / 2) * 2) planned = false;
   }
   if (!planned) {
     if (ctx->engine == 3) return NITI_ERR_SHAPE;
-    if (!plan(ctx, g, 1, PLAN_ANY, aligned, p, ma, mb)) return NITI_ERR_SHAPE;
+    if (!plan(ctx, g, 1, PLAN_ANY, aligned, acc, p, ma, mb, mc)) return NITI_ERR_SHAPE;
   }
   {
     // expected ratio between the max of the whole tensor (N values) and the max of the first tile of
@@ -2727,9 +2801,6 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   p.round_mode = r.round_mode;
   p.relu = r.relu;
   p.epi_mode = (p.splits > 1 || p.halo == 2) ? EPI_ATOMIC : ((ctx->engine == 4 || dp_sum || !r.out) ? EPI_SPILL : EPI_SPECULATE);
-  if (p.epi_mode == EPI_ATOMIC && niti_partial_slices(g.kind, g.gm) > 1 && p.splits <= niti_partial_slices(g.kind, g.gm) &&
-      !p.halo && p.mrep == 1)
-    p.epi_mode = EPI_PARTIAL;
   if (p.dstride > 1 && (p.nph_r < p.dstride || p.nph_s < p.dstride)) {
     // filter smaller than the stride: no window reaches the input pixels of the other phases
     if (p.epi_mode == EPI_SPILL) NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(g.gm * g.gn), st));
@@ -2767,7 +2838,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   }
   const bool prof = ctx->profile_on && ctx->prof_ev && ctx->prof_used < NITI_PROF_MAX;
   if (prof) prof_record(ctx->prof_ev[2 * ctx->prof_used], st);
-  int rc = launch_tc(ctx, st, p, ma, mb, acc, hdr, r);
+  int rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
   if (rc != NITI_OK) return rc;
   if (p.epi_mode == EPI_SPECULATE && p.single_wave) {
     *fused = true;                     // exact shift, scalars published by the last CTA: no second launch
@@ -2778,7 +2849,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
       if (rc != NITI_OK) return rc;
     }
     p.epi_mode = EPI_KNOWN_B;
-    rc = launch_tc(ctx, st, p, ma, mb, acc, hdr, r);
+    rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
     if (rc != NITI_OK) return rc;
     *fused = true;
   }
@@ -2786,11 +2857,6 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     prof_record(ctx->prof_ev[2 * ctx->prof_used + 1], st);
     ctx->prof_ops[ctx->prof_used] = 2.0 * (double)g.gm * (double)g.gn * (double)g.gk;
     ctx->prof_used++;
-  }
-  if (p.epi_mode == EPI_PARTIAL) {     // adds the splits' slices into the first one and takes the max magnitude
-    rc = niti_launch_sum_partials(ctx, st, acc, p.splits, g.gm * g.gn, hdr);
-    if (rc != NITI_OK || !dp) return rc;
-    return niti_reduce(ctx, st, &hdr->maxabs32, 1, NITI_REDUCE_MAX_U32);
   }
   if (p.epi_mode == EPI_ATOMIC) {
     // (weight gradients under data parallelism: the sums over the ranks first, then their max)
