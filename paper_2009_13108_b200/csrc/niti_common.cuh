@@ -77,7 +77,7 @@ struct niti_ctx {
 // Scalars at the start of a workspace.
 struct WsHeader {
   unsigned int maxabs32;            // a value with the bit length of max |acc| (a max, or an OR of magnitudes)
-  unsigned int done_ctas;           // CTAs that have finished (single-wave launches publish b themselves)
+  unsigned int unused;
   unsigned long long maxabs64;      // same for the 64-bit loss accumulators
   // the three words of the speculative agreement share one 16-byte line so that one load polls them all
   unsigned int est_max;             // max |acc| over the first tile of the CTAs that have reported

@@ -46,7 +46,7 @@ struct TcParams {
   unsigned magic_w, magic_h;    // floor(2^32 / tiles) + 1 for w_tiles, h_tiles: n / d = umulhi(n, magic) while
                                 // n * d < 2^32 (0: divide)
   int quorum;                   // CTAs whose first tile must have reported before the speculative bit-width
-                                // is fixed (all of them when the sample is the whole tensor)
+                                // is fixed (launches that are not single-wave)
   int nissue;                   // resident-weights mode: warps that issue MMAs (2: the warp that loaded the
                                 // weights takes every other tile)
   int one_commit;               // resident-weights mode with as many patch stages as accumulator buffers:
@@ -125,7 +125,7 @@ struct TcParams {
   int pool;                     // 1: the epilogue also stores the 2 x 2 max-pool of the (ReLU'd) output tile
   int pool_xh;                  // lane distance of the pixel one image row below (the pixel to the right is lane ^ 1)
   int single_wave;              // every CTA has at most one tile: the sample is the whole tensor, the shift
-                                // is exact, and the last CTA to finish publishes b and the exponent
+                                // is exact, and the first CTA publishes b and the exponent
 };
 
 // Epilogue modes.  The shift of Algorithm 2 needs the bit-width of the WHOLE accumulator tensor:
@@ -1581,38 +1581,76 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         if (p.epi_mode == EPI_SPECULATE && use == 0) {
           // first tile of this CTA: max only, then agree on the estimate with the whole grid
-          unsigned m0 = 0;
-          for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
+          // (columns of a partly filled chunk beyond the matrix accumulate zeros; whole chunks beyond it are left out)
+          const int cend0 = p.mrep > 1 ? p.bn : (ncols_valid < p.bn ? ncols_valid : p.bn);
+          int hi0 = 0, lo0 = 0;
+          for (int c = 32 * chunk_phase; c < cend0; c += 32 * wpq) {
             int v[32];
             tc_ld32(tm_row + (unsigned)c, v);
-            int cc = c;
             bool rok = row_ok;
-            if (p.mrep > 1) {
-              const int jt = c / p.bn_mma;
-              cc = c - jt * p.bn_mma;
-              rok = out_row + (long long)jt * BM < p.gm;
-            }
+            if (p.mrep > 1) rok = out_row + (long long)(c / p.bn_mma) * BM < p.gm;
             if (rok) {
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (cc + j < ncols_valid) {
-                  unsigned a = v[j] < 0 ? 0u - (unsigned)v[j] : (unsigned)v[j];
-                  m0 = a > m0 ? a : m0;
-                }
+              for (int j = 0; j < 32; j += 2) {
+                hi0 = __vimax3_s32(hi0, v[j], v[j + 1]);
+                lo0 = __vimin3_s32(lo0, v[j], v[j + 1]);
+              }
             }
           }
-          for (int o = 16; o > 0; o >>= 1) {
-            unsigned u = __shfl_xor_sync(0xffffffffu, m0, o);
-            m0 = u > m0 ? u : m0;
-          }
+          unsigned m0 = max((unsigned)hi0, 0u - (unsigned)lo0);
+          m0 = __reduce_max_sync(0xffffffffu, m0);
           // The warps of this CTA combine their maxima in shared memory; the last one to report speaks
           // for the CTA in the grid-wide agreement (one atomic and one poller per CTA: with every warp
           // of every CTA polling the same word the wait itself took microseconds) and publishes the
           // shift to the others through shared memory.
+          unsigned last = 0;
           if (lane == 0) {
             if (m0) atomicMax(&first_max, m0);
             __threadfence_block();
-            if (atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active) {
+            last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
+          }
+          if (p.single_wave) {
+            // Every CTA has one tile: the sample is the whole tensor.  Each CTA posts its maximum in a word of its
+            // own and reads everybody's, one store and one round of loads apart (through a shared maximum, a counter
+            // and a published word the same agreement was a chain of five L2 round trips); the words carry the data
+            // themselves, so nothing has to be fenced, and the shift is exact.
+            if (__shfl_sync(0xffffffffu, last, 0)) {
+              unsigned *words = niti_split_max(hdr);
+              if (lane == 0) *(volatile unsigned *)(words + blockIdx.x) = *(volatile unsigned *)&first_max + 1u;
+              unsigned all_max = 0;
+              const long long t0 = clock64();
+              while (true) {
+                bool seen = true;
+                all_max = 0;
+                for (unsigned i = (unsigned)lane; i < gridDim.x; i += 32) {
+                  const unsigned w = *(volatile unsigned *)(words + i);
+                  seen = seen && w != 0;
+                  all_max = max(all_max, w);
+                }
+                if (__all_sync(0xffffffffu, seen)) break;
+                if (__any_sync(0xffffffffu, abort_flag != 0)) break;
+                if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES)) {
+                  abort_flag = 1;
+                  atomicOr(status, NITI_DEV_TIMEOUT);
+                  break;
+                }
+              }
+              all_max = __reduce_max_sync(0xffffffffu, all_max);
+              if (lane == 0 && all_max) {
+                const int b = niti_bitlen32(all_max - 1u), bpf = b > p.mbits ? b - p.mbits : 0;
+                spec_bp_ready = bpf + 1;
+                if (blockIdx.x == 0) {                       // (no second launch publishes the scalars)
+                  if (b_out) *b_out = b;
+                  if (s_out) {
+                    const int sv = bpf + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
+                    *s_out = sv;
+                    if (sv < -128 || sv > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
+                  }
+                }
+              }
+            }
+          } else if (lane == 0) {
+            if (last) {
               const unsigned cm = *(volatile unsigned *)&first_max;
               if (cm) atomicMax(&hdr->est_max, cm);
               __threadfence();
@@ -1664,6 +1702,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               const int b = (int)pub - 1;
               spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
             }
+          }
+          if (lane == 0) {
             long long t1 = clock64();
             while (spec_bp_ready == 0) {
               if (abort_flag) break;
@@ -1924,30 +1964,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // ================= common exit =================
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && cta_max) atomicMax(&hdr->maxabs32, cta_max);
+  if (threadIdx.x == 0 && cta_max && !(p.single_wave && p.epi_mode == EPI_SPECULATE)) atomicMax(&hdr->maxabs32, cta_max);
   if (abort_flag) {
     // give copies and MMAs still in flight time to land before shared and tensor memory go away
     long long t0 = clock64();
     while (clock64() - t0 < 20000000LL) {
     }
     __syncthreads();
-  }
-  if (p.single_wave && p.epi_mode == EPI_SPECULATE && threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(&hdr->done_ctas, 1u) == gridDim.x - 1) {
-      __threadfence();
-      const int b_true = niti_bitlen32(*(volatile unsigned *)&hdr->maxabs32);
-      const int bpf = b_true > p.mbits ? b_true - p.mbits : 0;
-      // the shift every CTA rounded with came from the agreed maximum over ALL tiles, so it must be the
-      // true one; anything else means the agreement was broken and the stored int8 values are not exact
-      if (b_true != (int)(*(volatile unsigned *)&hdr->spec_b) - 1) atomicOr(status, NITI_DEV_INTERNAL);
-      if (b_out) *b_out = b_true;
-      if (s_out) {
-        int sv = bpf + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
-        *s_out = sv;
-        if (sv < -128 || sv > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
-      }
-    }
   }
   if (CTAS == 2) cluster_sync_all();   // nobody leaves while the peer may still touch this CTA
   if (warp == MMA_WARP) {
@@ -2795,7 +2818,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   {
     const long long units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
     const long long grid = (p.items < units ? p.items : units) * p.ctas;
-    p.quorum = (int)(p.single_wave ? grid : (grid + 1) / 2);
+    p.quorum = (int)((grid + 1) / 2);
   }
   p.mbits = r.mbits;
   p.round_mode = r.round_mode;
