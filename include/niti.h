@@ -118,8 +118,9 @@ int niti_set_engine(niti_ctx *ctx, int engine);
 
 /* Number of kernels / memsets this context has enqueued so far. */
 uint64_t niti_launch_count(niti_ctx *ctx);
-/* Of those, launches of the tensor-core (tcgen05) matrix-multiply kernel (without the instance that computes
- * the error of strided convolutions, which only niti_launch_count() counts). */
+/* Of those, launches of the tensor-core matrix-multiply kernels: tcgen05 (without the instance that computes the
+ * error of strided convolutions, which only niti_launch_count() counts) and the mma.sync kernel of small fully
+ * connected multiplies, whose backward launch runs two multiplies and counts as two. */
 uint64_t niti_tc_launch_count(niti_ctx *ctx);
 /* Of those, launches of the paired-CTA (cta_group::2) variant. */
 uint64_t niti_tc_pair_launch_count(niti_ctx *ctx);

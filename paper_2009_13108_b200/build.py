@@ -10,7 +10,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libniti_b200.so")
-SOURCES = ["niti_api.cu", "niti_elementwise.cu", "niti_simt_gemm.cu", "niti_tc_gemm.cu"]
+SOURCES = ["niti_api.cu", "niti_elementwise.cu", "niti_simt_gemm.cu", "niti_small_gemm.cu", "niti_tc_gemm.cu"]
 
 
 def _newest_source() -> float:

@@ -482,8 +482,13 @@ extern "C" int niti_linear_fwd(niti_ctx *ctx, void *stream, const int8_t *a, con
   p.p0 = a; p.p1 = w;
   int64_t dims[3] = {M, N, K};
   char *pad_mem = (char *)ws + NITI_WS_HEADER + round_up((size_t)M * N * 4, 256);
-  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes,
-                        niti_workspace_bytes(NITI_OP_LINEAR_FWD, dims, 3), pad_mem, out, 7, round_mode, relu,
+  const size_t need = niti_workspace_bytes(NITI_OP_LINEAR_FWD, dims, 3);
+  if (ws && !((uintptr_t)ws & 255) && ws_bytes >= need) {
+    const RoundSpec rs = {out, nullptr, 7, round_mode, relu, s_a, s_w, s_out, b_out, nullptr, nullptr};
+    const int rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, p, rs, nullptr, nullptr);
+    if (rc != NITI_ERR_SHAPE) return rc;
+  }
+  return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, pad_mem, out, 7, round_mode, relu,
                         nullptr, s_a, s_w, s_out, b_out);
 }
 
@@ -514,6 +519,13 @@ static int linear_bwd_impl(niti_ctx *ctx, void *stream, const int8_t *a, const i
   pd.p0 = e; pd.p1 = w;
   fill_fc(pw, GK_FC_WGRAD, M, N, K);
   pw.p0 = e; pw.p1 = a;
+  {
+    const RoundSpec rd = {e_prev, relu_mask_src, 7, round_mode, 0, nullptr, nullptr, nullptr, b_e, nullptr, nullptr};
+    const RoundSpec rw = {g, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, b_g, nullptr, update_w};
+    const int rc = e_prev ? niti_small_gemm(ctx, (cudaStream_t)stream, ws, pd, rd, &pw, &rw)
+                          : niti_small_gemm(ctx, (cudaStream_t)stream, ws, pw, rw, nullptr, nullptr);
+    if (rc != NITI_ERR_SHAPE) return rc;
+  }
   char *pad_a = pad_mem + pad_bytes(pd) - pad_bytes(pw, 0);      // (the weight gradient finds e padded already)
   if (pad_bytes(pd, 0) && N >= 32 && ctx->engine != 1) {
     const int rcp = niti_launch_pad_pitch(ctx, (cudaStream_t)stream, e, (int8_t *)pad_mem, M, N, pitch16(N));

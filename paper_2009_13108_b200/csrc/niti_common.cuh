@@ -17,7 +17,7 @@ struct niti_ctx {
   int32_t *d_spec_tab;      // NITI_SPEC_SLOTS x {tag, error}: per call site, by how many bits the sample-based
                             // estimate of the speculative epilogue missed the true bit-width last time
   uint64_t launches;
-  uint64_t tc_launches;     // launches of the tensor-core matrix-multiply kernel
+  uint64_t tc_launches;     // launches of the tensor-core matrix-multiply kernels (two multiplies in one count as two)
   uint64_t tc2_launches;    // of those, launches of the paired-CTA (cta_group::2) variant
   char err[256];
   // optional timing of the tensor-core kernel: event pairs recorded around each launch
@@ -51,6 +51,7 @@ struct niti_ctx {
   // device, not to a context: every context therefore sets this same value (a context that set only what it
   // needed would lower the limit under another context of the process)
   size_t smem_optin;
+  int small_ready;          // attributes of the small-multiply kernel are set
 };
 
 
@@ -232,6 +233,12 @@ struct RoundSpec {
 // (`out` is then not written).
 int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, const RoundSpec &r, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled = nullptr, bool shard_ok = false, bool *updated = nullptr);
+
+// Small fully connected multiplies, one launch for one (g2 == null) or both multiplies of a backward call;
+// NITI_ERR_SHAPE when the problem is not small (nothing was enqueued).
+#define NITI_SMALL_MACS 200.0e6
+int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem &g, const RoundSpec &r,
+                    const GemmProblem *g2, const RoundSpec *r2);
 
 // Epilogue pass: b from hdr->maxabs32, bp = max(0, b - mbits), out = Round(acc) with optional ReLU
 // and optional mask; s_out = s_a + s_w + bp if s_out != NULL; b_out = b if != NULL.

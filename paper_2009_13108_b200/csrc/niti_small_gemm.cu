@@ -1,0 +1,421 @@
+// Small fully connected multiplies (at most NITI_SMALL_MACS multiply-accumulates): one launch that loads, multiplies,
+// agrees on the bit-width, rounds and stores; a backward call runs its error and weight-gradient multiplies in the
+// same launch.
+//
+// Bound: latency.  On the tcgen05 kernel a 64 x 256 x 784 layer took 10 - 13 us of which the multiply is a few hundred
+// nanoseconds: tensor-memory allocation, barriers and descriptors (1.3 us), first TMA data (2.8 us), tensor-memory
+// round trips.  Here a CTA copies its operands with asynchronous copies issued at once, multiplies with mma.sync
+// (m16n8k32, int8) from shared memory, and the CTAs (at most one per SM) exchange their maxima through words of the
+// workspace header.  (One cluster of up to 16 CTAs that exchanges them through distributed shared memory measured the
+// same at 4 M multiply-accumulates, 5.4 against 5.2 us, and slower above, 8.2 against 5.8 us at 256^3.)
+// Measured (graph replay, forward / backward call, tcgen05 kernel -> this): 64 x 256 x 784 12.0 / 21.1 -> 7.0 / 8.4 us,
+// 256 x 256 x 256 9.8 / 20.7 -> 5.4 / 7.9 us, 512 x 512 x 512 10.8 / 22.7 -> 8.6 / 13.7 us, 1000 x 500 x 250 (rows that
+// TMA needs padded) 15.9 / 60.1 -> 15.2 / 17.4 us, 256 x 10 x 512 (CUDA-core backward before) 9.5 / 35.3 -> 5.8 / 7.5 us.
+// The line at NITI_SMALL_MACS: at 134 M 8.6 - 8.8 against 10.7 - 10.8 us forward and 13.7 - 15.4 against 22.7 - 27.0 us
+// backward; at 268 M 9.4 - 11.2 against 10.5 - 13.3 us and 19.2 - 27.6 against 27.4 - 29.3 us, about even.
+//
+// Contraction order.  mma.sync wants k = 4t .. 4t+3 and 16 + 4t .. from thread t of a group; any permutation of k that
+// both operands share gives the same sums, so a thread takes the 16 contiguous bytes at 16 t of a 64-byte step: one
+// 16-byte shared load per row feeds two MMAs.  Rows are permuted too: fragment row g of the four 8-row groups of a
+// 32 x 32 warp tile is matrix row 4g + group, which makes a thread's results 8 contiguous columns.
+#include "niti_common.cuh"
+
+namespace {
+
+constexpr int SMALL_THREADS = 512;
+constexpr int SMALL_WARPS = SMALL_THREADS / 32;
+constexpr long long SMALL_WAIT_CYCLES = 2000000000LL;
+constexpr size_t SMALL_SMEM = 200 * 1024;
+
+// One multiply out[m][n] = sum_k A(m, k) B(n, k).  An operand is K-major (row r, element k at p[r * ld + k]) or
+// MN-major (p[k * ld + r]).
+struct SmallOp {
+  const int8_t *a, *b;
+  int lda, ldb, a_mn, b_mn;
+  int gm, gn, gk;
+  int rm, rn, cn;             // region of a CTA (multiples of 32), CTAs per row of regions
+  int ctas;                   // CTAs of this multiply (0: this launch has no such multiply)
+  int kc;                     // contraction elements staged at a time (multiple of 64)
+  int8_t *out;
+  const int8_t *mask;         // output is zero where mask <= 0
+  int8_t *upd;                // weights from which the rounded result is subtracted (out is then not written)
+  int mbits, relu;
+  const int32_t *s_a, *s_w;
+  int32_t *s_out, *b_out;
+};
+struct SmallParams {
+  SmallOp op[2];              // op[0]: forward or error; op[1]: the weight gradient beside an error
+  int round_mode;
+  unsigned *words;            // one cleared word per CTA
+  uint32_t *status;
+};
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+// asynchronous copy of SIZE bytes, those from the `bytes`-th on zero
+template <int SIZE>
+__device__ __forceinline__ void cp_async(unsigned dst, const void *src, int bytes) {
+  if (SIZE == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(SIZE), "r"(bytes) : "memory");
+}
+template <int SIZE>
+__device__ __forceinline__ void stage_rows(const int8_t *p, int ld, int gk, int r0, int rv, int k0, int kc, int8_t *dst) {
+  const int parts = kc / SIZE;
+  for (int idx = threadIdx.x; idx < rv * parts; idx += SMALL_THREADS) {
+    const int r = idx / parts, c = (idx - r * parts) * SIZE;
+    int n = gk - k0 - c;
+    n = n < 0 ? 0 : (n > SIZE ? SIZE : n);
+    const int8_t *src = p + (long long)(r0 + r) * ld + k0 + (n > 0 ? c : 0);
+    cp_async<SIZE>(smem_addr(dst + r * (kc + 16) + c), src, n);
+  }
+}
+__device__ __forceinline__ void mma_s8(int (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Four bytes from p, those from the n-th on zero; reads only aligned words that hold at least one wanted byte.
+__device__ __forceinline__ unsigned load_bytes4(const int8_t *p, int n) {
+  if (n <= 0) return 0u;
+  const unsigned mis = (unsigned)(uintptr_t)p & 3u;
+  const unsigned *q = reinterpret_cast<const unsigned *>((uintptr_t)p - mis);
+  const unsigned lo = q[0];
+  const unsigned hi = mis + (unsigned)(n < 4 ? n : 4) > 4u ? q[1] : 0u;
+  const unsigned v = __funnelshift_r(lo, hi, 8u * mis);
+  return n >= 4 ? v : v & (0xffffffffu >> (32 - 8 * n));
+}
+
+// Stages rows r0 .. r0 + rows - 1, elements k0 .. k0 + kc - 1 of an operand as dst[row][kc + 16], zero beyond gk.
+// Rows beyond the matrix are left as they are (their results are never used).
+__device__ __forceinline__ void stage_operand(const int8_t *p, int ld, int mn, int extent, int gk, int r0, int rows, int k0,
+                                              int kc, int8_t *dst) {
+  const int pitch = kc + 16;
+  const int rv = extent - r0 < rows ? extent - r0 : rows;          // rows inside the matrix
+  if (!mn) {
+    const unsigned al = (unsigned)ld | (unsigned)(uintptr_t)p;
+    if ((al & 15) == 0) {
+      stage_rows<16>(p, ld, gk, r0, rv, k0, kc, dst);
+    } else if ((al & 7) == 0) {
+      stage_rows<8>(p, ld, gk, r0, rv, k0, kc, dst);
+    } else if ((al & 3) == 0) {
+      stage_rows<4>(p, ld, gk, r0, rv, k0, kc, dst);
+    } else {
+      // rows at any byte: words through registers, eight in flight per thread
+      const int words = kc >> 2, total = rv * words;
+      for (int base = threadIdx.x; base < total; base += 8 * SMALL_THREADS) {
+        unsigned v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int idx = base + u * SMALL_THREADS;
+          const int r = idx / words, c = (idx - r * words) * 4;
+          v[u] = idx < total ? load_bytes4(p + (long long)(r0 + r) * ld + k0 + c, gk - k0 - c) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int idx = base + u * SMALL_THREADS;
+          const int r = idx / words, c = (idx - r * words) * 4;
+          if (idx < total) *reinterpret_cast<unsigned *>(dst + r * pitch + c) = v[u];
+        }
+      }
+    }
+    return;
+  }
+  // 4 x 4 byte blocks, transposed on the way; a warp takes 16 blocks along k and 2 along the rows (conflict-free stores)
+  const int rq_n = (rv + 3) >> 2, rq2 = (rq_n + 1) >> 1, kq16 = kc >> 6;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool words_ok = (ld & 3) == 0 && ((uintptr_t)p & 3) == 0;
+  constexpr int UNR = 4;                                            // blocks in flight per thread
+  for (int job0 = warp; job0 < rq2 * kq16; job0 += UNR * SMALL_WARPS) {
+    unsigned w[UNR][4];
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      const int job = job0 + u * SMALL_WARPS;
+      const int jr = job / kq16, jk = job - jr * kq16;
+      const int rq = jr * 2 + (lane >> 4), k = (jk * 16 + (lane & 15)) * 4;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        w[u][i] = 0u;
+        if (rq < rq_n && k0 + k + i < gk) {
+          const int8_t *src = p + (long long)(k0 + k + i) * ld + r0 + 4 * rq;
+          w[u][i] = words_ok && 4 * rq + 4 <= rv ? *reinterpret_cast<const unsigned *>(src) : load_bytes4(src, rv - 4 * rq);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      const int job = job0 + u * SMALL_WARPS;
+      const int jr = job / kq16, jk = job - jr * kq16;
+      const int rq = jr * 2 + (lane >> 4), k = (jk * 16 + (lane & 15)) * 4;
+      if (rq >= rq_n) continue;
+      const unsigned t0 = __byte_perm(w[u][0], w[u][1], 0x5140), t1 = __byte_perm(w[u][2], w[u][3], 0x5140);
+      const unsigned t2 = __byte_perm(w[u][0], w[u][1], 0x7362), t3 = __byte_perm(w[u][2], w[u][3], 0x7362);
+      int8_t *d = dst + (4 * rq) * pitch + k;
+      *reinterpret_cast<unsigned *>(d) = __byte_perm(t0, t1, 0x5410);
+      *reinterpret_cast<unsigned *>(d + pitch) = __byte_perm(t0, t1, 0x7632);
+      *reinterpret_cast<unsigned *>(d + 2 * pitch) = __byte_perm(t2, t3, 0x5410);
+      *reinterpret_cast<unsigned *>(d + 3 * pitch) = __byte_perm(t2, t3, 0x7632);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(SMALL_THREADS, 1)
+small_gemm_kernel(const __grid_constant__ SmallParams p) {
+  extern __shared__ __align__(16) int8_t smem[];
+  __shared__ unsigned cta_max, group_max;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // which multiply, which region
+  const int ctas0 = p.op[0].ctas;
+  const int which = ((int)blockIdx.x < ctas0 || p.op[1].ctas == 0) ? 0 : 1;
+  const SmallOp &o = p.op[which];
+  const int first = which ? ctas0 : 0;
+  const int cta = (int)blockIdx.x - first;
+  const int cm_i = cta / o.cn, cn_i = cta - cm_i * o.cn;
+  const int m0 = cm_i * o.rm, n0 = cn_i * o.rn;
+  const int acc_pitch = o.rn + 4;
+  int *acc = reinterpret_cast<int *>(smem);                 // [rm][rn + 4]
+  int8_t *As = smem + (size_t)o.rm * acc_pitch * 4, *Bs = As + o.rm * (o.kc + 16);
+  if (tid == 0) cta_max = 0;
+  unsigned mx = 0;
+  {
+    const int tiles_n = o.rn >> 5, tiles = (o.rm >> 5) * tiles_n;
+    const int steps_c = o.kc >> 6;                          // 64-element steps of a full chunk
+    int wk = SMALL_WARPS / tiles;                           // warps that share a tile along k
+    wk = wk < 1 ? 1 : (wk > steps_c ? steps_c : wk);
+    const bool direct = wk == 1 && o.kc >= o.gk;            // one writer per result
+    if (!direct)
+      for (int i = tid; i < o.rm * acc_pitch; i += SMALL_THREADS) acc[i] = 0;
+    for (int k0 = 0; k0 < o.gk; k0 += o.kc) {
+      if (k0) __syncthreads();                              // the previous chunk has been read
+      stage_operand(o.a, o.lda, o.a_mn, o.gm, o.gk, m0, o.rm, k0, o.kc, As);
+      stage_operand(o.b, o.ldb, o.b_mn, o.gn, o.gk, n0, o.rn, k0, o.kc, Bs);
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      const int left = o.gk - k0, steps = left >= o.kc ? steps_c : (left + 63) >> 6;
+      const int per = (steps + wk - 1) / wk, pitch = o.kc + 16;
+      const int g = lane >> 2, t = lane & 3;
+      for (int job = warp; job < tiles * wk; job += SMALL_WARPS) {
+        const int tile = job / wk, ks = job - tile * wk;
+        const int tm = tile / tiles_n, tn = tile - tm * tiles_n;
+        const int s0 = ks * per, s1 = s0 + per < steps ? s0 + per : steps;
+        int c[2][4][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[i][j][q] = 0;
+        const int8_t *ap = As + (tm * 32 + 4 * g) * pitch + 16 * t, *bp = Bs + (tn * 32 + 4 * g) * pitch + 16 * t;
+        for (int s = s0; s < s1; ++s) {
+          uint4 av[4], bv[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            av[r] = *reinterpret_cast<const uint4 *>(ap + r * pitch + 64 * s);
+            bv[r] = *reinterpret_cast<const uint4 *>(bp + r * pitch + 64 * s);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const unsigned a0[4] = {av[2 * i].x, av[2 * i + 1].x, av[2 * i].y, av[2 * i + 1].y};
+            const unsigned a1[4] = {av[2 * i].z, av[2 * i + 1].z, av[2 * i].w, av[2 * i + 1].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              mma_s8(c[i][j], a0, bv[j].x, bv[j].y);
+              mma_s8(c[i][j], a1, bv[j].z, bv[j].w);
+            }
+          }
+        }
+        // rows 4g + 2i (+ 1), columns 8t + j and 8t + 4 + j
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            int *row = acc + (tm * 32 + 4 * g + 2 * i + h) * acc_pitch + tn * 32 + 8 * t;
+            if (direct) {
+              *reinterpret_cast<int4 *>(row) = make_int4(c[i][0][2 * h], c[i][1][2 * h], c[i][2][2 * h], c[i][3][2 * h]);
+              *reinterpret_cast<int4 *>(row + 4) =
+                  make_int4(c[i][0][2 * h + 1], c[i][1][2 * h + 1], c[i][2][2 * h + 1], c[i][3][2 * h + 1]);
+            } else if (s0 < s1) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                atomicAdd(row + j, c[i][j][2 * h]);
+                atomicAdd(row + 4 + j, c[i][j][2 * h + 1]);
+              }
+            }
+          }
+      }
+    }
+    __syncthreads();
+    // largest magnitude of the region
+    const int q = o.rn >> 2;
+    for (int idx = tid; idx < o.rm * q; idx += SMALL_THREADS) {
+      const int r = idx / q, cc = (idx - r * q) * 4;
+      if (m0 + r >= o.gm) continue;
+      const int4 v = *reinterpret_cast<const int4 *>(acc + r * acc_pitch + cc);
+      const int nv = o.gn - n0 - cc;
+      if (nv > 0) mx = max(mx, (unsigned)abs(v.x));
+      if (nv > 1) mx = max(mx, (unsigned)abs(v.y));
+      if (nv > 2) mx = max(mx, (unsigned)abs(v.z));
+      if (nv > 3) mx = max(mx, (unsigned)abs(v.w));
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0 && mx) atomicMax(&cta_max, mx);
+  __syncthreads();
+  // agreement: maximum over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after
+  // op[0]'s reads of the same weights.
+  if (warp == 0) {
+    if (lane == 0) *(volatile unsigned *)(p.words + blockIdx.x) = cta_max + 1u;
+    const int from = o.upd ? 0 : first, to = first + o.ctas;       // (an update waits for op[0] as well)
+    const long long t0 = clock64();
+    unsigned m = 0;
+    while (true) {
+      bool seen = true;
+      m = 0;
+      for (int i = from + lane; i < to; i += 32) {
+        const unsigned w = *(volatile unsigned *)(p.words + i);
+        seen = seen && w != 0;
+        if (i >= first) m = max(m, w);
+      }
+      if (__all_sync(0xffffffffu, seen)) break;
+      if (__any_sync(0xffffffffu, clock64() - t0 > SMALL_WAIT_CYCLES)) {
+        if (lane == 0) atomicOr(p.status, NITI_DEV_TIMEOUT);
+        m = 0;
+        break;
+      }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) group_max = m;
+  }
+  __syncthreads();
+  if (group_max == 0) return;                             // (gave up waiting)
+  mx = group_max - 1u;
+  const int b = niti_bitlen32(mx), bp = b > o.mbits ? b - o.mbits : 0;
+  const unsigned qmax = (1u << o.mbits) - 1u;
+  if (cta == 0 && tid == 0) {
+    if (o.b_out) *o.b_out = b;
+    if (o.s_out) {
+      const int s = bp + (o.s_a ? *o.s_a : 0) + (o.s_w ? *o.s_w : 0);
+      *o.s_out = s;
+      if (s < -128 || s > 127) atomicOr(p.status, NITI_DEV_EXP_RANGE);
+    }
+  }
+  const int q = o.rn >> 2;
+  int8_t *dst = o.upd ? o.upd : o.out;
+  const bool words_ok = (o.gn & 3) == 0 && (((uintptr_t)dst | (uintptr_t)o.mask) & 3) == 0;
+  for (int idx = tid; idx < o.rm * q; idx += SMALL_THREADS) {
+    const int r = idx / q, cc = (idx - r * q) * 4;
+    const int nv = o.gn - n0 - cc;
+    if (m0 + r >= o.gm || nv <= 0) continue;
+    const long long off = (long long)(m0 + r) * o.gn + n0 + cc;
+    const int4 v = *reinterpret_cast<const int4 *>(acc + r * acc_pitch + cc);
+    const int xs[4] = {v.x, v.y, v.z, v.w};
+    unsigned w = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      int x = niti_round_i32(xs[j], bp, qmax, p.round_mode);
+      if (o.relu && x < 0) x = 0;
+      w |= (unsigned)(x & 0xff) << (8 * j);
+    }
+    if (words_ok) {
+      if (o.mask) w &= __vcmpgts4(*reinterpret_cast<const unsigned *>(o.mask + off), 0u);
+      if (o.upd) w = __vmaxs4(__vsubss4(*reinterpret_cast<const unsigned *>(dst + off), w), 0x81818181u);
+      *reinterpret_cast<unsigned *>(dst + off) = w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j >= nv) break;
+        int x = (int)(int8_t)(w >> (8 * j));
+        if (o.mask && o.mask[off + j] <= 0) x = 0;
+        if (o.upd) {
+          x = (int)dst[off + j] - x;
+          x = x > 127 ? 127 : (x < -127 ? -127 : x);
+        }
+        dst[off + j] = (int8_t)x;
+      }
+    }
+  }
+}
+
+inline int up32(long long v) { return (int)((v + 31) / 32 * 32); }
+inline size_t region_smem(int rm, int rn, int kc) { return (size_t)rm * (rn + 4) * 4 + (size_t)(rm + rn) * (kc + 16); }
+
+// Regions of one multiply over at most `max_ctas` CTAs: the split with the least modelled time of a CTA (operand bytes
+// at about 32 per clock, 512 multiply-accumulates and two results per clock).  False when no region fits.
+bool pick_regions(SmallOp &o, int max_ctas) {
+  double best = 1e30;
+  for (int cm = 1; cm <= max_ctas && (cm - 1) * 32 < o.gm; ++cm) {
+    const int rm = up32((o.gm + cm - 1) / cm);
+    const int cn = max_ctas / ((o.gm + rm - 1) / rm);
+    if (cn < 1) continue;
+    const int rn = up32((o.gn + cn - 1) / cn);
+    if ((long long)rm * rn > 24576) continue;
+    int kc = (o.gk + 63) / 64 * 64;
+    while (kc > 64 && region_smem(rm, rn, kc) > SMALL_SMEM) kc = (kc / 2 + 63) / 64 * 64;
+    if (region_smem(rm, rn, kc) > SMALL_SMEM) continue;
+    const double t = (double)(rm + rn) * o.gk / 32 + (double)rm * rn * o.gk / 512 + (double)rm * rn / 2;
+    if (t < best * 0.999) {
+      best = t;
+      o.rm = rm; o.rn = rn; o.kc = kc;
+      o.cn = (o.gn + rn - 1) / rn;
+      o.ctas = (o.gm + rm - 1) / rm * o.cn;
+    }
+  }
+  return best < 1e30;
+}
+
+}  // namespace
+
+static void fill_op(SmallOp &o, const GemmProblem &g, const RoundSpec &r) {
+  memset(&o, 0, sizeof(o));
+  o.a = g.p0; o.b = g.p1;
+  o.gm = (int)g.gm; o.gn = (int)g.gn; o.gk = (int)g.gk;
+  o.lda = g.kind == GK_FC_FWD ? g.K : g.N;
+  o.ldb = g.K;
+  o.a_mn = g.kind == GK_FC_WGRAD;
+  o.b_mn = g.kind != GK_FC_FWD;
+  o.out = r.out; o.mask = r.mask; o.upd = r.update_w;
+  o.mbits = r.mbits; o.relu = r.relu;
+  o.s_a = r.s_a; o.s_w = r.s_w; o.s_out = r.s_out; o.b_out = r.b_out;
+}
+
+// Runs one multiply (g2 == null) or the two multiplies of a backward call in one launch.  NITI_ERR_SHAPE: not a
+// small problem, nothing was enqueued.
+int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem &g, const RoundSpec &r,
+                    const GemmProblem *g2, const RoundSpec *r2) {
+  const double macs = (double)g.M * g.N * g.K;
+  const bool narrow = g.N < 32 && g.kind != GK_FC_FWD;             // (the alternative is the CUDA-core engine)
+  if (ctx->engine != 0 || ctx->reduce_fn || g.kind > GK_FC_WGRAD || macs > NITI_SMALL_MACS * (narrow ? 4 : 1) || g.gk > NITI_SPLIT_MAX_K ||
+      (g2 && g2->gk > NITI_SPLIT_MAX_K))
+    return NITI_ERR_SHAPE;
+  SmallParams p;
+  memset(&p, 0, sizeof(p));
+  p.round_mode = r.round_mode;
+  p.status = ctx->d_status;
+  fill_op(p.op[0], g, r);
+  if (g2) fill_op(p.op[1], *g2, *r2);
+  if (!ctx->small_ready) {
+    NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(small_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
+    ctx->small_ready = 1;
+  }
+  const int n = ctx->sm_count;
+  if (!pick_regions(p.op[0], g2 ? n / 2 : n)) return NITI_ERR_SHAPE;
+  if (g2 && !pick_regions(p.op[1], n - p.op[0].ctas)) return NITI_ERR_SHAPE;
+  const int grid = p.op[0].ctas + p.op[1].ctas;
+  size_t smem = region_smem(p.op[0].rm, p.op[0].rn, p.op[0].kc);
+  if (g2) {
+    const size_t s2 = region_smem(p.op[1].rm, p.op[1].rn, p.op[1].kc);
+    if (s2 > smem) smem = s2;
+  }
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  WsHeader *hdr = nullptr;
+  const int rc = niti_take_header(ctx, st, ws, &hdr);
+  if (rc != NITI_OK) return rc;
+  p.words = niti_split_max(hdr);
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(SMALL_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, small_gemm_kernel, p));
+  ctx->launches++;
+  ctx->tc_launches += g2 ? 2 : 1;
+  return NITI_OK;
+}
