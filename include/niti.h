@@ -356,6 +356,10 @@ int niti_int_xent_noalloc(void *stream, const int8_t *a, const int32_t *s_a, con
 /* Weight update (Algorithm 1 last line; Section 3.3): w <- clamp(w - g, -127, 127), in place. */
 int niti_int_sgd_update(niti_ctx *ctx, void *stream, int8_t *w, const int8_t *g, int64_t n);
 
+/* Copies n tensors (bytes[i] bytes from src[i] to dst[i]; 16-byte aligned device pointers in host arrays, no two
+ * overlapping) with one launch per 32 tensors: the restore of a network's weights from a snapshot. */
+int niti_copy_tensors(niti_ctx *ctx, void *stream, int n, void *const *dst, const void *const *src, const int64_t *bytes);
+
 /* Support ops on int8 tensors between the layers (implied by the paper's
  * networks, Section 4); exponents are unchanged.
  *   relu_fwd: y = max(x, 0) (y may alias x).

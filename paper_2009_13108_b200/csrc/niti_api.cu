@@ -425,9 +425,9 @@ static int run_gemm_round(niti_ctx *ctx, cudaStream_t st, GemmProblem p, void *w
                           const GemmProblem *tc_form = nullptr) {
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
-  WsHeader *hdr = nullptr;
+  WsHeader *hdr = niti_take_header(ctx, ws);
   int32_t *acc = (int32_t *)((char *)ws + NITI_WS_HEADER);
-  int rc = niti_take_header(ctx, st, ws, &hdr);                            // zeroed reduction scalars and split maxima
+  int rc = NITI_OK;
   const bool narrow = p.kind <= GK_FC_WGRAD && p.N < 32 && p.kind != GK_FC_FWD;       // (the CUDA-core engine's)
   if (rc == NITI_OK && ctx->engine != 1 && !narrow && !tc_form) rc = pad_operands(ctx, st, p, pad_mem);
   if (rc != NITI_OK) return rc;
@@ -708,9 +708,8 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
     // columns that are taps are then rounded into g, or subtracted from the weights
     cudaStream_t st = (cudaStream_t)stream;
     const size_t M = (size_t)B * p.Ho * p.Wo;
-    WsHeader *hdr = nullptr;
-    int rc = niti_take_header(ctx, st, ws, &hdr);
-    if (rc != NITI_OK) return rc;
+    WsHeader *hdr = niti_take_header(ctx, ws);
+    int rc = NITI_OK;
     int8_t *xcol = (int8_t *)conv_pad_mem(p, ws);
     const size_t x_bytes = wg.Cp ? wg.x_bytes + wg.w_bytes : round_up(M * 32, 256) + round_up((size_t)Cout * 32, 256);
     int32_t *acc = (int32_t *)(xcol + x_bytes);

@@ -41,6 +41,7 @@ struct niti_ctx {
   // niti_begin_step: workspace whose headers were cleared in one go, and how many of them are used up
   void *step_ws;
   int step_slot;
+  struct WsHeader *dirty_hdr;   // header of the call being enqueued that has not been cleared yet, or null
   int dp_rank, dp_world;    // niti_set_dp_shard: > 1 ranks = weight gradients are reduce-scattered, rounded per
                             // shard and all-gathered as int8 (5 bytes per weight on the wire instead of 8)
   // per-device facts of the tensor-core kernel, indexed by CTAs per tile (1 or 2): co-resident CTAs /
@@ -60,7 +61,7 @@ struct niti_ctx {
 #define NITI_SPEC_SLOTS 4096
 // Every workspace starts with NITI_HDR_SLOTS headers of NITI_HDR_SLOT_BYTES each (reduction scalars, the
 // words of the speculative agreement, split maxima).  A call needs a zeroed header.  Without further
-// notice it clears and uses the first one.  After niti_begin_step() has cleared all of them with one
+// notice it clears and uses the last one.  After niti_begin_step() has cleared all of them with one
 // memset, the following calls on that workspace take one header each, in order, without clearing (a
 // cleared-per-call header costs a memset node of about 2 us in front of every multiply of a step).
 #define NITI_HDR_SLOTS 64
@@ -102,20 +103,33 @@ __host__ __device__ __forceinline__ unsigned int *niti_split_max(WsHeader *hdr) 
     }                                                                                   \
   } while (0)
 
-// A zeroed header for the call that is being enqueued: the next unused one of a workspace prepared by
-// niti_begin_step(), else the first one, cleared here.
-static inline int niti_take_header(niti_ctx *ctx, cudaStream_t st, void *ws, WsHeader **hdr) {
+// A header for the call that is being enqueued: the next unused one of a workspace prepared by niti_begin_step()
+// (zeroed already), else the last one, which niti_clear() has to clear before the call's first kernel.  The last one
+// ends where the accumulators begin, so that a split contraction clears both with one memset.
+static inline WsHeader *niti_take_header(niti_ctx *ctx, void *ws) {
+  char *base = reinterpret_cast<char *>(ws);
   if (ws == ctx->step_ws && ctx->step_slot < NITI_HDR_SLOTS) {
-    *hdr = reinterpret_cast<WsHeader *>(reinterpret_cast<char *>(ws) + (size_t)NITI_HDR_SLOT_BYTES * ctx->step_slot++);
-    return NITI_OK;
+    ctx->dirty_hdr = nullptr;
+    return reinterpret_cast<WsHeader *>(base + (size_t)NITI_HDR_SLOT_BYTES * ctx->step_slot++);
   }
-  *hdr = reinterpret_cast<WsHeader *>(ws);
+  ctx->dirty_hdr = reinterpret_cast<WsHeader *>(base + (size_t)NITI_HDR_SLOT_BYTES * (NITI_HDR_SLOTS - 1));
+  return ctx->dirty_hdr;
+}
+static inline int niti_memset0(niti_ctx *ctx, cudaStream_t st, void *p, size_t bytes) {
   ctx->launches++;
-  if (cudaMemsetAsync(ws, 0, NITI_HDR_SLOT_BYTES, st) != cudaSuccess) {
-    snprintf(ctx->err, sizeof(ctx->err), "clearing the workspace header failed");
-    return NITI_ERR_CUDA;
-  }
+  NITI_CUDA_TRY(ctx, cudaMemsetAsync(p, 0, bytes, st));
   return NITI_OK;
+}
+// Clears the header taken last if that is still to be done, and the accumulators (acc may be null).
+static inline int niti_clear(niti_ctx *ctx, cudaStream_t st, int32_t *acc = nullptr, size_t acc_bytes = 0) {
+  char *hdr = reinterpret_cast<char *>(ctx->dirty_hdr);
+  ctx->dirty_hdr = nullptr;
+  if (hdr && acc && hdr + NITI_HDR_SLOT_BYTES == reinterpret_cast<char *>(acc))
+    return niti_memset0(ctx, st, hdr, NITI_HDR_SLOT_BYTES + acc_bytes);
+  int rc = NITI_OK;
+  if (hdr) rc = niti_memset0(ctx, st, hdr, NITI_HDR_SLOT_BYTES);
+  if (rc == NITI_OK && acc) rc = niti_memset0(ctx, st, acc, acc_bytes);
+  return rc;
 }
 
 static inline int niti_fail(niti_ctx *ctx, int code, const char *msg) {

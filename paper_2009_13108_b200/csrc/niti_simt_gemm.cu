@@ -258,13 +258,15 @@ int niti_simt_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, int32_t
   splits = (p.gk + kps - 1) / kps;
   dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)splits);
   if (splits > 1) {
-    NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(p.gm * p.gn), st));
-    ctx->launches++;
+    const int rc = niti_clear(ctx, st, acc, sizeof(int32_t) * (size_t)(p.gm * p.gn));
+    if (rc != NITI_OK) return rc;
     simt_gemm_kernel<true><<<grid, 256, 0, st>>>(q, acc, hdr, kps);
     ctx->launches++;
     NITI_CUDA_TRY(ctx, cudaGetLastError());
     return niti_launch_maxabs(ctx, st, acc, p.gm * p.gn, hdr, (int)splits);
   }
+  const int rc = niti_clear(ctx, st);
+  if (rc != NITI_OK) return rc;
   simt_gemm_kernel<false><<<grid, 256, 0, st>>>(q, acc, hdr, kps);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());

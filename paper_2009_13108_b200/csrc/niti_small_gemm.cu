@@ -406,8 +406,8 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
   }
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  WsHeader *hdr = nullptr;
-  const int rc = niti_take_header(ctx, st, ws, &hdr);
+  WsHeader *hdr = niti_take_header(ctx, ws);
+  const int rc = niti_clear(ctx, st);
   if (rc != NITI_OK) return rc;
   p.words = niti_split_max(hdr);
   cfg.gridDim = dim3((unsigned)grid, 1, 1);

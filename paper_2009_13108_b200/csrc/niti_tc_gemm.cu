@@ -2392,9 +2392,9 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
         int best_s = 1;
         double best_eff = 0;
         const int max_s = p.kb_total / 4 > 0 ? p.kb_total / 4 : 1;
-        for (int sp = 1; sp <= max_s && sp <= 4 * ctx->sm_count; ++sp) {
-          const long long it = blocks * sp;
-          const long long waves = (it + ctx->sm_count - 1) / ctx->sm_count;
+        for (int sp = 1; sp <= max_s && sp <= 4 * ctx->sm_count && best_eff < 0.98; ++sp) {
+          const int it = (int)blocks * sp;
+          const int waves = (it + ctx->sm_count - 1) / ctx->sm_count;
           const double eff = (double)it / (double)(waves * ctx->sm_count);
           if (eff > best_eff + 0.02) { best_eff = eff; best_s = sp; }
         }
@@ -2551,8 +2551,10 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     int best_s = 1;
     int max_s = p.kb_total / 4;
     for (int sp = 1; sp <= max_s && sp <= 4 * units; ++sp) {
-      const long long it = tiles * sp;
-      const long long waves = (it + units - 1) / units;
+      const int it = (int)tiles * sp;
+      const int waves = (it + units - 1) / units;
+      // (no later split count can cost less than this: the host time of the search counts in short calls)
+      if ((double)tiles * p.kb_total / units + 4.0 * waves >= best * 0.98) break;
       const double cost = (double)waves * ((double)((p.kb_total + sp - 1) / sp) + 4.0);
       if (cost < best * 0.98) { best = cost; best_s = sp; }
     }
@@ -2830,10 +2832,8 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     else NITI_CUDA_TRY(ctx, cudaMemsetAsync(r.out, 0, (size_t)(g.gm * g.gn), st));
     ctx->launches++;
   }
-  if (p.epi_mode == EPI_ATOMIC) {
-    NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(g.gm * g.gn), st));
-    ctx->launches++;
-  }
+  int rc = p.epi_mode == EPI_ATOMIC ? niti_clear(ctx, st, acc, sizeof(int32_t) * (size_t)(g.gm * g.gn)) : niti_clear(ctx, st);
+  if (rc != NITI_OK) return rc;
   // Fused 2 x 2 max-pool: the fused epilogue of a forward convolution with ReLU also stores the pooled
   // tile when every pooling window lies inside one warp's 32 pixels (8 x 16 pixel tiles of the
   // resident-weights mode, or pixel boxes at most 16 wide and at least 2 high) and the rows are whole,
@@ -2861,7 +2861,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   }
   const bool prof = ctx->profile_on && ctx->prof_ev && ctx->prof_used < NITI_PROF_MAX;
   if (prof) prof_record(ctx->prof_ev[2 * ctx->prof_used], st);
-  int rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
+  rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
   if (rc != NITI_OK) return rc;
   if (p.epi_mode == EPI_SPECULATE && p.single_wave) {
     *fused = true;                     // exact shift, scalars published by the last CTA: no second launch

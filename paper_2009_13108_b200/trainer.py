@@ -104,9 +104,8 @@ class NitiTrainer:
         self._initial = [w.clone() for w in self.weights]
 
     def reset_weights(self):
-        """Restores the snapshot (device-to-device copies on the current stream)."""
-        for w, w0 in zip(self.weights, self._initial):
-            w.copy_(w0, non_blocking=True)
+        """Restores the snapshot (one device-to-device copy launch on the current stream)."""
+        self.n.copy_tensors(self.weights, self._initial)
 
     def capture(self, with_reset: bool = False):
         """Captures one step (optionally preceded by reset_weights) into a CUDA graph; returns a
