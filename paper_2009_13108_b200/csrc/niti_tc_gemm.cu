@@ -2151,9 +2151,10 @@ static int pick_bn(long long gn) {
 
 // Builds params and maps; returns false if the shape is not eligible for this engine.
 // `aligned`: output (and mask) pointers and rows are 32-byte aligned.
+// force_bn: column tile of an unsplit one-wave plan (see pick_one_wave), 0 for the planner's own choice.
 // want: ANY, or only a plan in the resident-weights / tap-pair mode (HALO) or the row-batched mode (BATCHED).
 enum PlanWant { PLAN_ANY = 0, PLAN_HALO = 1, PLAN_BATCHED = 2 };
-static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, int32_t *acc, TcParams &p, CUtensorMap &ma,
+static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, int force_bn, int32_t *acc, TcParams &p, CUtensorMap &ma,
                  CUtensorMap &mb, CUtensorMap &mc) {
   memset(&p, 0, sizeof(p));
   p.ctas = ctas;
@@ -2177,7 +2178,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   switch (g.kind) {
     case GK_FC_FWD: {
       p.kdepth = pick_swizzle(g.gk);
-      p.bn = pick_bn(g.gn);
+      p.bn = force_bn ? force_bn : pick_bn(g.gn);
       a_sw = b_sw = p.kdepth;
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gk);
       sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {ld0}, {(cuuint32_t)p.kdepth, BM}, a_sw, q0};
@@ -2190,7 +2191,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     case GK_FC_DGRAD: {   // out [M][K'], contraction over N
       p.kdepth = pick_swizzle(g.gk);
       b_mn = 1;
-      p.bn = pick_bn(g.gn);
+      p.bn = force_bn ? force_bn : pick_bn(g.gn);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       a_sw = p.kdepth;
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
@@ -2205,7 +2206,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       a_mn = b_mn = 1;
       a_sw = pick_swizzle(g.gm);
       p.kdepth = pick_swizzle(g.gk);
-      p.bn = pick_bn(g.gn);
+      p.bn = force_bn ? force_bn : pick_bn(g.gn);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gm), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
       sa = {2, {(cuuint64_t)g.gm, (cuuint64_t)g.gk}, {ld0}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, q0};
@@ -2282,8 +2283,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
       m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
       if (p.i2c) m_tiles = (m_tiles + BM - 1) / BM;
-      p.bn = pick_bn(Cn);
-      if (fwd && ctas == 2 && Cn > 256) {
+      p.bn = force_bn ? force_bn : pick_bn(Cn);
+      if (fwd && ctas == 2 && Cn > 256 && !force_bn) {
         // Whole waves: with 256-wide tiles the 14 x 14 layers are 98 tile pairs on 74 pairs of SMs, two
         // waves of which the second is a third full; 192-wide tiles make 147 items, two full waves.
         // (A 192-wide MMA takes as long as a 256-wide one, so an item is not shorter; it moves three
@@ -2421,7 +2422,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.PW = g.Wo; p.PH = g.Ho; p.PB = g.B;
       p.R = g.R; p.S = g.S; p.pad = g.pad;
       p.Cn = g.Ci;
-      p.bn = pick_bn(g.Ci);
+      p.bn = force_bn ? force_bn : pick_bn(g.Ci);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       p.n_chunks = (g.Ci + p.bn - 1) / p.bn;
       // (pixel boxes or runs of consecutive pixels: see "Pixel rows" above; a run of e is a piece of a matrix)
@@ -2543,7 +2544,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   if ((g.kind == GK_FC_FWD || g.kind == GK_FC_DGRAD || g.kind == GK_FC_WGRAD) && p.n_tiles_n > 1 && p.m_units > 1)
     p.raster_g = ctas == 2 ? 8 : 12;
   // split the contraction when the tiles alone cannot fill the SMs
-  if (tiles < units && p.kb_total >= 8 && p.dstride <= 1) {
+  if (tiles < units && p.kb_total >= 8 && p.dstride <= 1 && !force_bn) {
     // pick the split count with the least modelled time: waves of items, each item running its
     // share of the k-blocks plus a fixed cost (pipeline fill and the atomic epilogue) of about
     // four k-blocks
@@ -2566,6 +2567,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     const int max_kb = NITI_SPLIT_MAX_K / p.kdepth;
     const int min_splits = (p.kb_total + max_kb - 1) / max_kb;
     if (p.splits < min_splits) p.splits = min_splits;
+    if (force_bn && p.splits > 1) return false;
     if (p.splits > NITI_MAX_SPLITS || (p.splits > 1 && p.dstride > 1)) return false;
   }
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
@@ -2770,6 +2772,50 @@ static void prof_record(cudaEvent_t ev, cudaStream_t st) {
     cudaEventRecord(ev, st);
 }
 
+// Cycles of one k-block of a tile: the MMAs (bound by their math or by the shared-memory reads of their operands) or
+// the operand copies (measured: about 84 bytes per clock into one SM, 9000 into all of them; never below 400 cycles for
+// 128 contraction elements however narrow the tile).
+static double kblock_cycles(const TcParams &p, int ctas, int bn, long long ctas_running) {
+  const double mma = bn / 2.0, smem = 32.0 + bn / (4.0 * ctas), bytes = (128.0 + (double)bn / ctas) * p.kdepth;
+  double c = p.ksteps * (mma > smem ? mma : smem);
+  if (c < bytes / 84.0) c = bytes / 84.0;
+  if (c < bytes * ctas_running / 9000.0) c = bytes * ctas_running / 9000.0;
+  return c < 100.0 * p.ksteps ? 100.0 * p.ksteps : c;
+}
+// A multiply of at most one tile per SM: an unsplit plan whose every CTA (pair) has one tile rounds in its own epilogue
+// with an exact shift, in one launch.  Splitting the contraction shortens the main loop but costs a zeroed scratch, the
+// reduce copies and two passes over the int32 sums (measured 3.5 us + 5 us per million outputs); pairs of CTAs cost
+// 0.8 us more set-up than single ones.  Measured (graph replay, the former plan -> this one): 256 images of 4 x 4, 512
+// -> 512 channels, forward 33.3 -> 20.7, error 29.7 -> 21.7, weight gradient 30.3 -> 21.2 us; 100 images of 9 x 9, 96 ->
+// 160 channels, forward 21.5 -> 13.2, error 20.0 -> 14.2 us, but its weight gradient (64 k-blocks over 18 tiles) 16.4 us
+// split against 28.3 us unsplit: the model below draws that line.  (Splits that form a cluster and add their partial
+// tiles through distributed shared memory were built and measured: 24.3 - 25.0 us against 20.7 us unsplit on the first
+// of these; the agreement over twice as many CTAs and the exchange cost what the shorter main loop saves.)
+static bool pick_one_wave(niti_ctx *ctx, const GemmProblem &g, const TcParams &p, int &ctas, int &bn) {
+  const int units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
+  if (p.halo || p.mrep > 1 || p.dstride > 1 || p.items > 4LL * units) return false;
+  const long long waves = (p.items + units - 1) / units, running = (p.items < units ? p.items : units) * p.ctas;
+  double best = (double)waves * (p.kb_per_split * kblock_cycles(p, p.ctas, p.bn, running) + (waves > 1 ? 3000.0 : 0.0)) +
+                (p.ctas == 2 ? 1500.0 : 0.0) +
+                (p.splits > 1 ? 6500.0 + 0.0095 * (double)g.gm * (double)g.gn : (waves > 1 ? 3500.0 : 0.0));
+  best *= 0.97;
+  const int cols = g.kind == GK_CONV_WGRAD ? p.Cn : (int)g.gn, taps = g.kind == GK_CONV_WGRAD ? g.R * g.S : 1;
+  const bool boxes = (g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD) && !p.i2c;
+  const long long m128 = boxes ? (long long)p.w_tiles * p.h_tiles * p.b_tiles : (g.gm + BM - 1) / BM;
+  bool found = false;
+  for (int c = 1; c <= 2; ++c) {
+    if (c == 2 && g.gm < 2 * BM) break;
+    const long long mu = (m128 + c - 1) / c, cap = c == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
+    for (int nt = (cols + 255) / 256; nt <= (cols + 31) / 32 && mu * nt * taps <= cap; ++nt) {
+      const int w = round_up32((cols + nt - 1) / nt);
+      if ((cols + w - 1) / w != nt) continue;
+      const double t = p.kb_total * kblock_cycles(p, c, w, mu * nt * taps * c) + (c == 2 ? 1500.0 : 0.0);
+      if (t < best) { best = t * 0.99; ctas = c; bn = w; found = true; }
+    }
+  }
+  return found;
+}
+
 int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const RoundSpec &r_in, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled, bool shard_ok, bool *updated) {
   TcParams p;
@@ -2788,18 +2834,30 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   bool planned = false;
   if ((g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD || g.kind == GK_CONV_WGRAD) && ctx->engine != 3 &&
       ctx->engine != 5)
-    planned = plan(ctx, g, 1, PLAN_HALO, aligned, acc, p, ma, mb, mc);
+    planned = plan(ctx, g, 1, PLAN_HALO, aligned, 0, acc, p, ma, mb, mc);
   if (!planned && g.kind == GK_FC_FWD && ctx->engine != 3)      // row-batched mode of short contractions
-    planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, acc, p, ma, mb, mc);
+    planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, 0, acc, p, ma, mb, mc);
   if (!planned && ctx->engine != 2 && g.gm >= 2 * BM) {
-    planned = plan(ctx, g, 2, PLAN_ANY, aligned, acc, p, ma, mb, mc);
+    planned = plan(ctx, g, 2, PLAN_ANY, aligned, 0, acc, p, ma, mb, mc);
     // (pairs halve the operand traffic per MMA; they are kept unless they would leave more than a
     // third of the GPU idle)
     if (planned && ctx->engine != 3 && p.items * 3 < (long long)(ctx->sm_count / 2) * 2) planned = false;
   }
   if (!planned) {
     if (ctx->engine == 3) return NITI_ERR_SHAPE;
-    if (!plan(ctx, g, 1, PLAN_ANY, aligned, acc, p, ma, mb, mc)) return NITI_ERR_SHAPE;
+    if (!plan(ctx, g, 1, PLAN_ANY, aligned, 0, acc, p, ma, mb, mc)) return NITI_ERR_SHAPE;
+  }
+  if (ctx->engine == 0 && !ctx->reduce_fn && r.out) {
+    int c = 0, w = 0;
+    if (pick_one_wave(ctx, g, p, c, w)) {
+      TcParams p1;
+      CUtensorMap a1, b1, c1;
+      if (plan(ctx, g, c, PLAN_ANY, aligned, w, acc, p1, a1, b1, c1)) {
+        p = p1;
+        ma = a1;
+        mb = b1;
+      }
+    }
   }
   {
     // expected ratio between the max of the whole tensor (N values) and the max of the first tile of
@@ -2846,15 +2904,16 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     else if (!p.halo && p.Wt >= 2 && p.Wt <= 16 && p.Ht >= 2) { p.pool = 1; p.pool_xh = p.Wt; }
     *pooled = p.pool != 0;
   }
-  // Weight update inside the epilogue (Section 3.3): a fully connected weight gradient whose epilogue
+  // Weight update inside the epilogue (Section 3.3): a weight gradient whose epilogue
   // rounds by itself subtracts the rounded values from the weights in place of storing them.  A
   // speculative pass must not touch the weights (a wrong guess could not be taken back), so the update
   // is fused only where the shift is exact when the stores happen: single-wave launches.  (Measured
   // and not kept for the other launches: a first pass for the bit-width alone followed by a rounding
   // pass that updates, 198 us against 185 us for the 4096 x 25088 layer at batch 64.)
   p.update = 0;
-  if (updated && r.update_w && g.kind == GK_FC_WGRAD && p.epi_mode == EPI_SPECULATE && p.single_wave && p.mrep == 1 &&
-      !p.halo && !r.mask && !r.relu && (g.gn % 32) == 0 && ((uintptr_t)r.update_w & 31) == 0) {
+  if (updated && r.update_w && (g.kind == GK_FC_WGRAD || (g.kind == GK_CONV_WGRAD && (g.Ci & 31) == 0)) &&
+      p.epi_mode == EPI_SPECULATE && p.single_wave && p.mrep == 1 && !p.halo && !r.mask && !r.relu && (g.gn % 32) == 0 &&
+      ((uintptr_t)r.update_w & 31) == 0) {
     p.update = 1;
     r.out = r.update_w;
     *updated = true;
