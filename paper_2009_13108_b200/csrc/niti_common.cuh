@@ -173,6 +173,17 @@ __device__ __forceinline__ int niti_round_i32(int x, int bp, unsigned qmax, int 
 
 __device__ __forceinline__ int niti_bitlen32(unsigned v) { return 32 - __clz(v); }
 
+// Four bytes from p, those from the n-th on zero; reads only aligned words that hold at least one wanted byte.
+__device__ __forceinline__ unsigned niti_load_bytes4(const int8_t *p, int n) {
+  if (n <= 0) return 0u;
+  const unsigned mis = (unsigned)(uintptr_t)p & 3u;
+  const unsigned *q = reinterpret_cast<const unsigned *>((uintptr_t)p - mis);
+  const unsigned lo = q[0];
+  const unsigned hi = mis + (unsigned)(n < 4 ? n : 4) > 4u ? q[1] : 0u;
+  const unsigned v = __funnelshift_r(lo, hi, 8u * mis);
+  return n >= 4 ? v : v & (0xffffffffu >> (32 - 8 * n));
+}
+
 // ---- internal launchers (defined across the .cu files) ----------------------------------------
 // Shape of one matrix multiply D[m][n] = sum_k A(m,k) * B(n,k) with implicit operand addressing.
 enum NitiGemmKind {

@@ -253,25 +253,23 @@ round_compact_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict
 
 // Few-channel convolutions with more than 32 taps ("windows", see window_geometry): image rows with `pad` zero
 // pixels on the left, enough on the right for the last window, and every pixel widened from Ci to Cp bytes (4, 8 or
-// 16).  One word of the widened row per thread (bound: memory; the taps are not copied, so 224 x 224 x 3 images
-// become 13 MB for an 11 x 11 stride-4 layer where gathered rows were 74 MB and took 80 us to write).
+// 16).  Bound: memory (the taps are not copied, so 224 x 224 x 3 images become 13 MB for an 11 x 11 stride-4 layer where
+// gathered rows were 74 MB and took 80 us to write).  A thread writes 16 bytes, 16 / Cp pixels, from unaligned words
+// (with a byte per load and a 64-bit division per word the pass took 20 us).
 __global__ void __launch_bounds__(256)
-widen_pixels_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xw, int rows, int W, int Ci, int Cp, int pad,
-                    int row_words) {
-  const int wpp = Cp >> 2;                                 // words per pixel
-  const long long total = (long long)rows * row_words;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(idx / row_words), wd = (int)(idx - (long long)r * row_words);
-    const int px = wd / wpp - pad, c0 = 4 * (wd - (wd / wpp) * wpp);
-    unsigned v = 0;
-    if (px >= 0 && px < W && c0 < Ci) {
-      const int8_t *src = x + ((long long)r * W + px) * Ci + c0;
+widen_pixels_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xw, unsigned rows, int W, int Ci, int cp_shift, int pad,
+                    unsigned row_parts) {
+  const unsigned total = rows * row_parts, stride = gridDim.x * blockDim.x;
+  for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride) {
+    const unsigned r = idx / row_parts, part = idx - r * row_parts;
+    const int8_t *row = x + (long long)r * W * Ci;
+    unsigned v[4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c0 + c < Ci) v |= (unsigned)(uint8_t)src[c] << (8 * c);
+    for (int j = 0; j < 4; ++j) {
+      const int byte = (int)part * 16 + 4 * j, px = (byte >> cp_shift) - pad, c0 = byte & ((1 << cp_shift) - 1);
+      v[j] = px >= 0 && px < W ? niti_load_bytes4(row + px * Ci + c0, Ci - c0) : 0u;
     }
-    reinterpret_cast<unsigned *>(xw)[idx] = v;
+    reinterpret_cast<uint4 *>(xw)[idx] = make_uint4(v[0], v[1], v[2], v[3]);
   }
 }
 // weights [Cout][R][S][Ci] -> [Cout][R][pitch], tap column s in bytes s * Cp .. s * Cp + Ci - 1, zero elsewhere
@@ -286,10 +284,12 @@ widen_weights_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ ww, int 
 }
 int niti_launch_widen(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *xw, int rows, int W, int Ci, int Cp, int pad,
                       int row_bytes, const int8_t *w, int8_t *ww, int wrows, int S, int pitch) {
-  const long long words = (long long)rows * (row_bytes / 4);
-  long long blocks = (words + 255) / 256;
+  const long long parts = (long long)rows * (row_bytes / 16);
+  if (parts >= (1LL << 31)) return niti_fail(ctx, NITI_ERR_SHAPE, "few-channel convolution: image too large");
+  long long blocks = (parts + 255) / 256;
   if (blocks > (long long)ctx->sm_count * 64) blocks = (long long)ctx->sm_count * 64;
-  widen_pixels_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, xw, rows, W, Ci, Cp, pad, row_bytes / 4);
+  const int cp_shift = Cp == 4 ? 2 : (Cp == 8 ? 3 : 4);
+  widen_pixels_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, xw, (unsigned)rows, W, Ci, cp_shift, pad, (unsigned)(row_bytes / 16));
   ctx->launches++;
   if (w) {
     widen_weights_kernel<<<(unsigned)(((long long)wrows * pitch + 255) / 256), 256, 0, st>>>(w, ww, wrows, S, Ci, Cp, pitch);

@@ -73,17 +73,6 @@ __device__ __forceinline__ void mma_s8(int (&c)[4], const unsigned (&a)[4], unsi
                : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// Four bytes from p, those from the n-th on zero; reads only aligned words that hold at least one wanted byte.
-__device__ __forceinline__ unsigned load_bytes4(const int8_t *p, int n) {
-  if (n <= 0) return 0u;
-  const unsigned mis = (unsigned)(uintptr_t)p & 3u;
-  const unsigned *q = reinterpret_cast<const unsigned *>((uintptr_t)p - mis);
-  const unsigned lo = q[0];
-  const unsigned hi = mis + (unsigned)(n < 4 ? n : 4) > 4u ? q[1] : 0u;
-  const unsigned v = __funnelshift_r(lo, hi, 8u * mis);
-  return n >= 4 ? v : v & (0xffffffffu >> (32 - 8 * n));
-}
-
 // Stages rows r0 .. r0 + rows - 1, elements k0 .. k0 + kc - 1 of an operand as dst[row][kc + 16], zero beyond gk.
 // Rows beyond the matrix are left as they are (their results are never used).
 __device__ __forceinline__ void stage_operand(const int8_t *p, int ld, int mn, int extent, int gk, int r0, int rows, int k0,
@@ -107,7 +96,7 @@ __device__ __forceinline__ void stage_operand(const int8_t *p, int ld, int mn, i
         for (int u = 0; u < 8; ++u) {
           const int idx = base + u * SMALL_THREADS;
           const int r = idx / words, c = (idx - r * words) * 4;
-          v[u] = idx < total ? load_bytes4(p + (long long)(r0 + r) * ld + k0 + c, gk - k0 - c) : 0u;
+          v[u] = idx < total ? niti_load_bytes4(p + (long long)(r0 + r) * ld + k0 + c, gk - k0 - c) : 0u;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -136,7 +125,7 @@ __device__ __forceinline__ void stage_operand(const int8_t *p, int ld, int mn, i
         w[u][i] = 0u;
         if (rq < rq_n && k0 + k + i < gk) {
           const int8_t *src = p + (long long)(k0 + k + i) * ld + r0 + 4 * rq;
-          w[u][i] = words_ok && 4 * rq + 4 <= rv ? *reinterpret_cast<const unsigned *>(src) : load_bytes4(src, rv - 4 * rq);
+          w[u][i] = words_ok && 4 * rq + 4 <= rv ? *reinterpret_cast<const unsigned *>(src) : niti_load_bytes4(src, rv - 4 * rq);
         }
       }
     }
