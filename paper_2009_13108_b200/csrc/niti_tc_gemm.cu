@@ -95,6 +95,7 @@ struct TcParams {
   int OH, OW;                   // extent of the tensor the output rows are written to
   int Cn;                       // wgrad: input channels Ci (columns per tap)
   int n_chunks;                 // wgrad: column chunks per tap
+  int tg, tg_cols, tg_boxes;    // wgrad: taps per column tile (tap groups), columns and copies (per CTA) of one tap
   int ctas;                     // CTAs per tile: 1, or 2 (cta_group::2, 256-row tiles)
   int m_units;                  // row units: 128-row tiles (ctas = 1) or 256-row pairs (ctas = 2)
   int raster_g;                 // row units per rasterisation group (0: row-major order)
@@ -786,6 +787,15 @@ __device__ __forceinline__ void load_im2col(unsigned dst, const CUtensorMap *m, 
   else tma_load_im2col(dst, m, bar, c, w, h, n, (unsigned short)ow, (unsigned short)oh);
 }
 
+// Next tap of a tap group; beyond the last one it is repeated (the filler's results are not used).
+__device__ __forceinline__ void next_tap(const TcParams &p, int &jb, int &r, int &s) {
+  jb = 0;
+  if (++s == p.S) {
+    s = 0;
+    if (++r == p.R) { r = p.R - 1; s = p.S - 1; }
+  }
+}
+
 // item -> (row unit, column tile, split).  Row units (one CTA's 128 rows, or a pair's 256) are
 // visited in groups of raster_g so that the CTAs running at the same time share operand tiles in L2.
 // (32-bit arithmetic throughout: one thread of the producer, issuer and epilogue warps runs this per
@@ -865,6 +875,7 @@ __device__ __forceinline__ void halo_mma_loop(const TcParams &p, int issuer, int
     const unsigned a_lo = a_stage_lo + (unsigned)stage * a_stage16;
     if (leader) {
       if (ksteps == 2) halo_issue_tile<2>(tmem_d, a_lo, a_hi, a_off, b_hi, b_tap, b_kstep16, idesc);
+      else if (ksteps == 3) halo_issue_tile<3>(tmem_d, a_lo, a_hi, a_off, b_hi, b_tap, b_kstep16, idesc);
       else if (ksteps == 4) halo_issue_tile<4>(tmem_d, a_lo, a_hi, a_off, b_hi, b_tap, b_kstep16, idesc);
       else halo_issue_tile<1>(tmem_d, a_lo, a_hi, a_off, b_hi, b_tap, b_kstep16, idesc);
       if (!one_commit) tc_commit(empty0 + 8 * stage);
@@ -1048,10 +1059,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         for (int tap = 0; warp == PROD_WARPS - 1 && leader && tap < 9; ++tap) {
           const unsigned dst = smem_base + tap * p.b_tile_bytes;
           if (p.kind == GK_CONV_FWD) {
-            tma_load_2d(dst, &map_b, bres_bar, tap * p.kdepth, 0);
+            if (GENERAL) tma_load_3d(dst, &map_b, bres_bar, 0, tap, 0);
+            else tma_load_2d(dst, &map_b, bres_bar, tap * p.kdepth, 0);
           } else {
-            for (int j = 0; j < p.b_boxes; ++j)
-              tma_load_2d(dst + j * p.b_box_bytes, &map_b, bres_bar, tap * p.Cn + j * p.b_box_step, 0);
+            for (int j = 0; j < p.b_boxes; ++j) {
+              if (GENERAL) tma_load_3d(dst + j * p.b_box_bytes, &map_b, bres_bar, j * p.b_box_step, tap, 0);
+              else tma_load_2d(dst + j * p.b_box_bytes, &map_b, bres_bar, tap * p.Cn + j * p.b_box_step, 0);
+            }
           }
         }
         if (p.nissue == 2 && warp == PROD_WARPS - 1) {
@@ -1124,8 +1138,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (kb1 > p.kb_total) kb1 = p.kb_total;
         if (STRIDED) kb1 = phq.n_r * phq.n_s * p.c_chunks;
         if (p.kind == GK_CONV_WGRAD) {
-          tap_n = nt / p.n_chunks;
-          ci0 = (nt % p.n_chunks) * p.bn + (int)rank * bn_cta;
+          if (p.tg > 1) {
+            tap_n = nt * p.tg + (int)rank * (p.tg / CTAS);
+          } else {
+            tap_n = nt / p.n_chunks;
+            ci0 = (nt % p.n_chunks) * p.bn + (int)rank * bn_cta;
+          }
         }
         // k-block counters, stepped instead of divided inside the loop (one thread issues all copies,
         // so every scalar instruction here is on the critical path):
@@ -1141,7 +1159,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
         }
         int wg_r = 0, wg_s = 0;
-        if (p.kind == GK_CONV_WGRAD) { wg_r = tap_n / p.S; wg_s = tap_n % p.S; }
+        if (p.kind == GK_CONV_WGRAD) {
+          if (tap_n >= p.R * p.S) tap_n = p.R * p.S - 1;          // (filler of a last, short tap group)
+          wg_r = tap_n / p.S; wg_s = tap_n % p.S;
+        }
         const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + p.b_boxes * p.b_box_bytes));
         for (int kb = kb0; kb < kb1; ++kb) {
          if (owner == warp) {
@@ -1192,16 +1213,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               if (I2C && p.i2c) {        // consecutive pixels: e as a plain matrix, x as im2col rows of the same pixels
                 for (int j = 0; j < p.a_boxes; ++j)
                   load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * BM);
-                for (int j = 0; j < p.b_boxes; ++j)
-                  load_im2col<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + j * p.b_box_step,
-                                    kwt * p.stride_w + p.i2c_w0, kht * p.stride + p.i2c_h0, kbt, wg_s, wg_r);
+                for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
+                  load_im2col<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step,
+                                    kwt * p.stride_w + p.i2c_w0, kht * p.stride + p.i2c_h0, kbt, ts2, tr2);
+                  if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
+                }
                 break;
               }
               for (int j = 0; j < p.a_boxes; ++j)
                 load4<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kw0, kh0, kbb0);
-              for (int j = 0; j < p.b_boxes; ++j)
-                load4<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + j * p.b_box_step, kw0 * p.stride + wg_s - p.pad,
-                            kh0 * p.stride + wg_r - p.pad, kbb0);
+              for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
+                load4<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step, kw0 * p.stride + ts2 - p.pad,
+                            kh0 * p.stride + tr2 - p.pad, kbb0);
+                if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
+              }
               break;
             }
           }
@@ -1463,7 +1488,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         int tap = nt / p.n_chunks, ci0 = (nt % p.n_chunks) * p.bn;
         col0 = (long long)tap * p.Cn + ci0;
         int rem = p.Cn - ci0;
-        ncols_valid = rem < p.bn ? rem : p.bn;
+        ncols_valid = rem < p.bn && p.tg <= 1 ? rem : p.bn;
       } else {
         // (row-batched mode: the row of the first of the item's mrep tiles; column chunk c of the
         // accumulator then belongs to tile c / bn_mma)
@@ -1505,6 +1530,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         const bool any_row = __any_sync(0xffffffffu, row_ok);
         for (int c = 32 * chunk_phase; c < p.bn && c < ncols_valid && any_row; c += 32 * wpq) {
+          int xc = x0 + c, xt = x1;
+          if (p.kind == GK_CONV_WGRAD && p.tg > 1) {           // tap group: tg_cols (a power of two) columns per tap
+            xt = nt * p.tg + c / p.tg_cols;
+            xc = c & (p.tg_cols - 1);
+            if (xt >= p.R * p.S || xc >= p.Cn) continue;
+          }
           int v[32];
           tc_ld32(tm_row + (unsigned)c, v);
           // (rows and columns outside the matrix are clipped by the copy; they may hold anything)
@@ -1517,7 +1548,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           stage_tile32<false>(red_buf, lane, v);
           fence_async_shared();
           __syncwarp();
-          if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, x0 + c, x1, x2, x3);
+          if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, xc, xt, x2, x3);
         }
         pmx = __reduce_max_sync(0xffffffffu, pmx);
         if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
@@ -2097,6 +2128,32 @@ static bool pick_pixel_box(int W, int H, int B, int &Wt, int &Ht, int &Bt) {
   return Wt <= W && Ht <= H && Bt <= B;
 }
 
+// Tap groups of a weight gradient with few input channels.  With one tap per column tile every tap reads the error
+// tensor again and a k-block's MMAs are shorter than its copies and barriers (about 400 cycles); a tile of several taps
+// reads the error once for all of them.  The modelled cycles of all taps' k-blocks decide: MMAs (math or shared-memory
+// reads), operand copies, or that floor.  Pairs of CTAs hold half of the taps each.  Measured, weight gradient with
+// update: 5 x 5, 96 -> 256 channels, 27 x 27, batch 128 91.7 -> 60.5 us; 3 x 3, 24 -> 72, 64 x 64, batch 64 99.7 -> 60.6 us;
+// 48 -> 96, 36 x 36, batch 100 37.9 -> 31.7 us; 32 -> 64, 28 x 28, batch 256 36.6 -> 26.6 us.
+static int pick_tap_group(const GemmProblem &g, int ctas, int &cols) {
+  cols = g.Ci <= 32 ? 32 : (g.Ci <= 64 ? 64 : 128);
+  if (g.Ci > 128 || g.gk < 160 * 128) return 1;         // (few k-blocks: 96 -> 160 at 9 x 9, 64 k-blocks, 16.2 single, 17.9 grouped)
+  const int taps = g.R * g.S;
+  const double arows = g.Co / ctas < 128 ? (g.Co + ctas - 1) / ctas : 128;
+  auto cost = [&](int t, int n) {
+    const double mma = n / 2.0, smem = 32.0 + n / (4.0 * ctas);
+    double c = 4.0 * (mma > smem ? mma : smem);
+    const double copies = (arows + (double)n / ctas) * 128.0 / 84.0;
+    if (c < copies) c = copies;
+    if (c < 400.0) c = 400.0;
+    return (double)((taps + t - 1) / t) * c;
+  };
+  int best_t = 1;
+  double best = 0.95 * cost(1, (g.Ci + 31) / 32 * 32);
+  for (int t = 2; t <= taps && t * cols <= 256; t += ctas)
+    if (cost(t, t * cols) < best) { best = cost(t, t * cols); best_t = t; }
+  return best_t;
+}
+
 constexpr size_t SMEM_BUDGET = 225 * 1024;            // dynamic shared memory beside the kernel's static arrays and alignment
 constexpr size_t RED_BYTES = (size_t)EPI_WARPS * 4096;
 
@@ -2141,6 +2198,13 @@ static void window_map(const GemmProblem &g, MapSpec &s) {
   s.strides[2] = (cuuint64_t)g.win_sh * g.H;
 }
 
+// The patches of the resident-weights mode cover 8 x 16 pixels: images that fill at least
+// three quarters of them, or are large enough.
+static bool halo_fits(int W, int H) {
+  const int cover = (W + 7) / 8 * 8 * ((H + 15) / 16 * 16);
+  return (W >= 10 && H >= 18) || 4 * W * H >= 3 * cover;
+}
+
 static int round_up32(long long n) { return (int)((n + 31) / 32 * 32); }
 
 // Width of a column tile: the fewest tiles of at most 256 columns, all of about the same width.
@@ -2151,7 +2215,8 @@ static int pick_bn(long long gn) {
 
 // Builds params and maps; returns false if the shape is not eligible for this engine.
 // `aligned`: output (and mask) pointers and rows are 32-byte aligned.
-// force_bn: column tile of an unsplit one-wave plan (see pick_one_wave), 0 for the planner's own choice.
+// force_bn: column tile of an unsplit one-wave plan (see pick_one_wave), 0 for the planner's own choice, -1 for that
+// without tap groups.
 // want: ANY, or only a plan in the resident-weights / tap-pair mode (HALO) or the row-batched mode (BATCHED).
 enum PlanWant { PLAN_ANY = 0, PLAN_HALO = 1, PLAN_BATCHED = 2 };
 static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, bool aligned, int force_bn, int32_t *acc, TcParams &p, CUtensorMap &ma,
@@ -2178,7 +2243,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   switch (g.kind) {
     case GK_FC_FWD: {
       p.kdepth = pick_swizzle(g.gk);
-      p.bn = force_bn ? force_bn : pick_bn(g.gn);
+      p.bn = force_bn > 0 ? force_bn : pick_bn(g.gn);
       a_sw = b_sw = p.kdepth;
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gk);
       sa = {2, {(cuuint64_t)g.gk, (cuuint64_t)g.gm}, {ld0}, {(cuuint32_t)p.kdepth, BM}, a_sw, q0};
@@ -2191,7 +2256,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     case GK_FC_DGRAD: {   // out [M][K'], contraction over N
       p.kdepth = pick_swizzle(g.gk);
       b_mn = 1;
-      p.bn = force_bn ? force_bn : pick_bn(g.gn);
+      p.bn = force_bn > 0 ? force_bn : pick_bn(g.gn);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       a_sw = p.kdepth;
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
@@ -2206,7 +2271,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       a_mn = b_mn = 1;
       a_sw = pick_swizzle(g.gm);
       p.kdepth = pick_swizzle(g.gk);
-      p.bn = force_bn ? force_bn : pick_bn(g.gn);
+      p.bn = force_bn > 0 ? force_bn : pick_bn(g.gn);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gm), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
       sa = {2, {(cuuint64_t)g.gm, (cuuint64_t)g.gk}, {ld0}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, q0};
@@ -2283,8 +2348,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
       m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
       if (p.i2c) m_tiles = (m_tiles + BM - 1) / BM;
-      p.bn = force_bn ? force_bn : pick_bn(Cn);
-      if (fwd && ctas == 2 && Cn > 256 && !force_bn) {
+      p.bn = force_bn > 0 ? force_bn : pick_bn(Cn);
+      if (fwd && ctas == 2 && Cn > 256 && force_bn <= 0) {
         // Whole waves: with 256-wide tiles the 14 x 14 layers are 98 tile pairs on 74 pairs of SMs, two
         // waves of which the second is a third full; 192-wide tiles make 147 items, two full waves.
         // (A 192-wide MMA takes as long as a 256-wide one, so an item is not shorter; it moves three
@@ -2320,15 +2385,16 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.n_tiles_n = (Cn + p.bn - 1) / p.bn;
       if (p.dstride > 1) p.kb_total = p.T_r * p.T_s * p.c_chunks;                 // (of the longest phase)
       // halo mode: one channel chunk, one column tile, weights of all taps fit beside >= 3 patches
-      if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && p.c_chunks == 1 && !tail &&
-          p.n_tiles_n == 1 && g.W >= 10 && g.H >= 18 && !g.q0 && !g.q1 && (fwd ? Cn % 8 == 0 : Cn % 32 == 0)) {
+      // (short channel chunks and padded operands need the general instance, whose weights come through a 3-D map)
+      if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && p.c_chunks == 1 &&
+          p.n_tiles_n == 1 && halo_fits(g.W, g.H) && Cn % 8 == 0) {
         const int a_stage = (180 * p.kdepth + 1023) / 1024 * 1024;
         const int tap_cols = fwd ? p.bn : (p.bn + b_sw - 1) / b_sw * b_sw;        // (columns past Cn are not multiplied)
         const int b_res = (9 * tap_cols * p.kdepth + 1023) / 1024 * 1024;
         if (b_res + 3 * a_stage <= 224 * 1024) {
           p.halo = 1;
           p.i2c = 0;
-          p.mode = aligned ? 0 : 1;
+          p.mode = aligned && !tail && !g.q0 && !g.q1 && (fwd || Cn % 32 == 0) ? 0 : 1;
           sa.im2col = 0;
           p.PW = g.W; p.PH = g.H;
           p.Wt = 8; p.Ht = 16; p.Bt = 1;
@@ -2337,7 +2403,10 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
           p.b_tiles = g.B;
           m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
           sa.box[1] = 10; sa.box[2] = 18; sa.box[3] = 1;
-          if (fwd) {
+          if (p.mode == 1) {
+            sb = {3, {(cuuint64_t)g.Ci, 9, (cuuint64_t)g.Co}, {(cuuint64_t)ld1, (cuuint64_t)9 * ld1},
+                  {(cuuint32_t)b_sw, 1, (cuuint32_t)(fwd ? p.bn : p.kdepth)}, b_sw, q1};
+          } else if (fwd) {
             sb = {2, {(cuuint64_t)g.gk, (cuuint64_t)Cn}, {(cuuint64_t)g.gk}, {(cuuint32_t)p.kdepth, (cuuint32_t)p.bn}, b_sw, q1};
           } else {       // w viewed as [Co rows][9 * Ci]: column = tap * Ci + ci
             sb = {2, {(cuuint64_t)9 * g.Ci, (cuuint64_t)g.Co}, {(cuuint64_t)9 * g.Ci}, {(cuuint32_t)b_sw, (cuuint32_t)p.kdepth}, b_sw, q1};
@@ -2354,10 +2423,12 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       const int st = g.stride > 1 ? g.stride : 1;
       const bool same = g.Ho == g.H && g.Wo == g.W && st == 1;
       p.stride = st;
-      // (64 x 64)-channel blocks re-read the activations once per block of the other operand, so this
-      // mode is kept for layers with few blocks; wide layers use the per-tap tiles below
+      // (64 x 64)-channel blocks re-read the activations once per block of the other operand and their N = 64 MMAs run
+      // at two thirds of the rate: this mode is kept where the tap groups below would leave half of the MMA's rows
+      // empty (64 output channels: 119 against 203 us at 224 x 224) or spend as much on copies (128 -> 128 channels at
+      // 112 x 112: 115 against 124 us); 64 -> 128 at 56 x 56 30.5 against 26.3 us, 128 -> 256 84 against 62 us
       if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && g.Ci % 64 == 0 && g.Co % 64 == 0 &&
-          g.W >= 10 && g.H >= 18 && (long long)g.Ci * g.Co <= 32768 && !g.q0 && !g.q1) {
+          g.W >= 10 && g.H >= 18 && (long long)g.Ci * g.Co <= 16384 && (g.Co == 64 || g.Ci >= 128) && !g.q0 && !g.q1) {
         p.halo = 2;
         p.kdepth = 128;
         p.bn = 64;
@@ -2422,9 +2493,19 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.PW = g.Wo; p.PH = g.Ho; p.PB = g.B;
       p.R = g.R; p.S = g.S; p.pad = g.pad;
       p.Cn = g.Ci;
-      p.bn = force_bn ? force_bn : pick_bn(g.Ci);
+      p.bn = force_bn > 0 ? force_bn : pick_bn(g.Ci);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       p.n_chunks = (g.Ci + p.bn - 1) / p.bn;
+      p.tg = 1;
+      if (force_bn == 0) {
+        const int t = pick_tap_group(g, ctas, p.tg_cols);
+        if (t > 1) {
+          p.tg = t;
+          p.bn = t * p.tg_cols;
+          p.n_chunks = 1;
+          b_sw = p.tg_cols;                       // (32, 64 or 128: one copy per tap)
+        }
+      }
       // (pixel boxes or runs of consecutive pixels: see "Pixel rows" above; a run of e is a piece of a matrix)
       p.stride_w = g.win_chans ? 1 : st;
       p.i2c = (st > 1 || g.win_chans || !pick_pixel_box(g.Wo, g.Ho, g.B, p.Wt, p.Ht, p.Bt)) ? 1 : 0;
@@ -2459,7 +2540,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.kb_total = p.w_tiles * p.h_tiles * p.b_tiles;
       if (p.i2c) p.kb_total = (int)((g.gk + p.kdepth - 1) / p.kdepth);
       m_tiles = (g.Co + BM - 1) / BM;
-      p.n_tiles_n = g.R * g.S * p.n_chunks;
+      p.n_tiles_n = (g.R * g.S + p.tg - 1) / p.tg * p.n_chunks;
       break;
     }
     default:
@@ -2504,6 +2585,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   if (bn_cta % 16) return false;
   if (b_mn) {
     p.b_boxes = (bn_cta + b_sw - 1) / b_sw;
+    p.tg_boxes = p.tg > 1 ? 1 : p.b_boxes;
     p.b_box_bytes = p.kdepth * b_sw;
     p.b_box_step = b_sw;
     p.b_bytes = p.b_boxes * p.b_box_bytes;
@@ -2544,7 +2626,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   if ((g.kind == GK_FC_FWD || g.kind == GK_FC_DGRAD || g.kind == GK_FC_WGRAD) && p.n_tiles_n > 1 && p.m_units > 1)
     p.raster_g = ctas == 2 ? 8 : 12;
   // split the contraction when the tiles alone cannot fill the SMs
-  if (tiles < units && p.kb_total >= 8 && p.dstride <= 1 && !force_bn) {
+  if (tiles < units && p.kb_total >= 8 && p.dstride <= 1 && force_bn <= 0) {
     // pick the split count with the least modelled time: waves of items, each item running its
     // share of the k-blocks plus a fixed cost (pipeline fill and the atomic epilogue) of about
     // four k-blocks
@@ -2567,7 +2649,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     const int max_kb = NITI_SPLIT_MAX_K / p.kdepth;
     const int min_splits = (p.kb_total + max_kb - 1) / max_kb;
     if (p.splits < min_splits) p.splits = min_splits;
-    if (force_bn && p.splits > 1) return false;
+    if (force_bn > 0 && p.splits > 1) return false;
     if (p.splits > NITI_MAX_SPLITS || (p.splits > 1 && p.dstride > 1)) return false;
   }
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
@@ -2582,6 +2664,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.red = 0;
     }
   }
+  // (tap groups only where the sums leave through reduce copies, which place every tap's columns)
+  if (p.tg > 1 && !(p.splits > 1 && p.red)) return plan(ctx, g, ctas, want, aligned, -1, acc, p, ma, mb, mc);
   // rows with a pitch that is no multiple of 8: staging buffers of the fused epilogue's stores
   p.nstg_off = 0;
   if (p.splits == 1 && !p.halo && ((g.gn & 7) != 0 || (g.kind == GK_CONV_WGRAD && (p.Cn & 7) != 0))) {
@@ -2622,6 +2706,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   p.items = tiles * p.splits * (p.dstride > 1 ? p.nph_r * p.nph_s : 1);
   if (p.items >= (1LL << 30)) return false;      // the kernel counts items in 32 bits
   // the copies an instance issues have the rank and mode of its maps: anything else is a planning error
+  if (p.halo == 1 && (sb.nd != (p.mode >= 1 ? 3 : 2) || sa.nd != 4 || sa.im2col)) return false;
   if (!p.halo && (g.kind == GK_CONV_FWD || g.kind == GK_CONV_DGRAD) &&
       (sb.nd != (p.mode >= 1 ? 3 : 2) || sa.nd != 4 || sa.im2col != p.i2c))
     return false;

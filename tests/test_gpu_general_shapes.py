@@ -18,6 +18,11 @@ CASES = [
     (2, 16, 16, 96, 96, 5, 2, 1),       # exact pixel boxes with short channel chunks
     (2, 16, 16, 256, 96, 3, 1, 1), (4, 16, 8, 160, 256, 3, 1, 1), (2, 16, 32, 48, 128, 3, 1, 1),
     (128, 3, 5, 96, 256, 3, 1, 1),      # pixel boxes of one pixel in 128 images
+    (2, 36, 36, 48, 96, 3, 1, 1),       # resident weights with short channel chunks (48 of 64, 96 of 128)
+    (3, 19, 26, 24, 40, 3, 1, 1), (2, 32, 24, 16, 72, 3, 1, 1), (2, 20, 11, 112, 24, 3, 1, 1),
+    (3, 16, 8, 64, 64, 3, 1, 1), (2, 15, 15, 32, 64, 3, 1, 1), (4, 14, 16, 64, 128, 3, 1, 1),   # one patch high
+    (90, 17, 15, 24, 72, 3, 1, 1), (90, 16, 16, 48, 96, 3, 1, 1), (40, 24, 24, 96, 256, 3, 1, 1),   # tap groups
+    (40, 23, 24, 112, 288, 3, 1, 1), (90, 16, 16, 32, 40, 5, 2, 1), (90, 33, 31, 64, 128, 3, 1, 2),
     (3, 16, 16, 64, 64, 3, 1, 2),       # strided error: four phases of 4, 2, 2 and 1 taps
     (2, 17, 23, 32, 96, 3, 1, 2),
     (2, 19, 13, 64, 32, 5, 2, 3),
