@@ -184,6 +184,53 @@ __device__ __forceinline__ unsigned niti_load_bytes4(const int8_t *p, int n) {
   return n >= 4 ? v : v & (0xffffffffu >> (32 - 8 * n));
 }
 
+// Maximum over n CTAs (at most NITI_AGREE_MAX), plus one, for one converged warp of every CTA; 0: gave up (`late()` said
+// so).  Words [0, n) of the area take what the CTAs post.  Up to NITI_AGREE_DIRECT CTAs all poll all words; with more, the
+// first CTA alone does and answers into a mailbox of 16 bytes per CTA that only that CTA polls, because the reads of a few
+// L2 lines by everybody delay the posts (3100 cycles for 64 CTAs, 6000 - 8000 for 128; one call with 98 CTAs 12.0 -> 10.5
+// us, with 64 14.1 -> 13.0 us, with 144 16.0 -> 13.7 us; with 16 6.9 us directly, 7.5 us through mailboxes).  `extra` more
+// words in front of the area have to be posted first.
+#define NITI_AGREE_MAX 160
+#define NITI_AGREE_DIRECT 48
+#define NITI_AGREE_WORDS (5 * NITI_AGREE_MAX)      // posts, then mailboxes
+template <typename Late>
+__device__ __forceinline__ unsigned niti_agree_max(unsigned *posts, unsigned *mail, unsigned mine, int cta, int n, int extra,
+                                                   int lane, Late late) {
+  if (lane == 0) *(volatile unsigned *)(posts + cta) = mine + 1u;
+  if (cta == 0 || n <= NITI_AGREE_DIRECT) {
+    unsigned m;
+    while (true) {
+      bool seen = true;
+      m = 0;
+      unsigned w[5];
+#pragma unroll
+      for (int u = 0; u < 5; ++u) {
+        const int i = 32 * u + lane - extra;
+        w[u] = i < n ? *(volatile unsigned *)(posts + i) : 1u;
+      }
+#pragma unroll
+      for (int u = 0; u < 5; ++u) {
+        const int i = 32 * u + lane - extra;
+        seen = seen && w[u] != 0;
+        if (i >= 0 && i < n) m = max(m, w[u]);
+      }
+      if (__all_sync(0xffffffffu, seen)) break;
+      if (late()) return 0u;
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (n > NITI_AGREE_DIRECT)
+      for (int i = lane; i < n; i += 32) *(volatile unsigned *)(mail + 4 * i) = m;
+    return m;
+  }
+  unsigned m = 0;
+  while (true) {
+    if (lane == 0) m = *(volatile unsigned *)(mail + 4 * cta);
+    m = __shfl_sync(0xffffffffu, m, 0);
+    if (m) return m;
+    if (late()) return 0u;
+  }
+}
+
 // ---- internal launchers (defined across the .cu files) ----------------------------------------
 // Shape of one matrix multiply D[m][n] = sum_k A(m,k) * B(n,k) with implicit operand addressing.
 enum NitiGemmKind {

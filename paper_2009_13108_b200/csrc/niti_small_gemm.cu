@@ -251,26 +251,14 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   // agreement: maximum over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after
   // op[0]'s reads of the same weights.
   if (warp == 0) {
-    if (lane == 0) *(volatile unsigned *)(p.words + blockIdx.x) = cta_max + 1u;
-    const int from = o.upd ? 0 : first, to = first + o.ctas;       // (an update waits for op[0] as well)
     const long long t0 = clock64();
-    unsigned m = 0;
-    while (true) {
-      bool seen = true;
-      m = 0;
-      for (int i = from + lane; i < to; i += 32) {
-        const unsigned w = *(volatile unsigned *)(p.words + i);
-        seen = seen && w != 0;
-        if (i >= first) m = max(m, w);
-      }
-      if (__all_sync(0xffffffffu, seen)) break;
-      if (__any_sync(0xffffffffu, clock64() - t0 > SMALL_WAIT_CYCLES)) {
-        if (lane == 0) atomicOr(p.status, NITI_DEV_TIMEOUT);
-        m = 0;
-        break;
-      }
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
+    // (an update waits for op[0] as well)
+    const unsigned m = niti_agree_max(p.words + first, p.words + NITI_AGREE_MAX + 4 * first, cta_max, cta, o.ctas,
+                                      o.upd ? first : 0, lane, [&]() {
+                                        const bool out = __any_sync(0xffffffffu, clock64() - t0 > SMALL_WAIT_CYCLES);
+                                        if (out && lane == 0) atomicOr(p.status, NITI_DEV_TIMEOUT);
+                                        return out;
+                                      });
     if (lane == 0) group_max = m;
   }
   __syncthreads();
@@ -384,7 +372,7 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
     NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(small_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
     ctx->small_ready = 1;
   }
-  const int n = ctx->sm_count;
+  const int n = ctx->sm_count < NITI_AGREE_MAX ? ctx->sm_count : NITI_AGREE_MAX;
   if (!pick_regions(p.op[0], g2 ? n / 2 : n)) return NITI_ERR_SHAPE;
   if (g2 && !pick_regions(p.op[1], n - p.op[0].ctas)) return NITI_ERR_SHAPE;
   const int grid = p.op[0].ctas + p.op[1].ctas;

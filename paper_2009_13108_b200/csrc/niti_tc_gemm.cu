@@ -1641,32 +1641,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
           }
           if (p.single_wave) {
-            // Every CTA has one tile: the sample is the whole tensor.  Each CTA posts its maximum in a word of its
-            // own and reads everybody's, one store and one round of loads apart (through a shared maximum, a counter
-            // and a published word the same agreement was a chain of five L2 round trips); the words carry the data
-            // themselves, so nothing has to be fenced, and the shift is exact.
+            // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
             if (__shfl_sync(0xffffffffu, last, 0)) {
               unsigned *words = niti_split_max(hdr);
-              if (lane == 0) *(volatile unsigned *)(words + blockIdx.x) = *(volatile unsigned *)&first_max + 1u;
-              unsigned all_max = 0;
               const long long t0 = clock64();
-              while (true) {
-                bool seen = true;
-                all_max = 0;
-                for (unsigned i = (unsigned)lane; i < gridDim.x; i += 32) {
-                  const unsigned w = *(volatile unsigned *)(words + i);
-                  seen = seen && w != 0;
-                  all_max = max(all_max, w);
-                }
-                if (__all_sync(0xffffffffu, seen)) break;
-                if (__any_sync(0xffffffffu, abort_flag != 0)) break;
-                if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES)) {
-                  abort_flag = 1;
-                  atomicOr(status, NITI_DEV_TIMEOUT);
-                  break;
-                }
-              }
-              all_max = __reduce_max_sync(0xffffffffu, all_max);
+              const unsigned all_max = niti_agree_max(
+                  words, words + NITI_AGREE_MAX, *(volatile unsigned *)&first_max, (int)blockIdx.x, (int)gridDim.x, 0, lane, [&]() {
+                    const bool out = __any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES);
+                    if (out && lane == 0) {
+                      abort_flag = 1;
+                      atomicOr(status, NITI_DEV_TIMEOUT);
+                    }
+                    return out || __any_sync(0xffffffffu, abort_flag != 0);
+                  });
               if (lane == 0 && all_max) {
                 const int b = niti_bitlen32(all_max - 1u), bpf = b > p.mbits ? b - p.mbits : 0;
                 spec_bp_ready = bpf + 1;
@@ -2959,7 +2946,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   // data parallelism (niti_set_reduce_hook): the max magnitude is combined over the ranks between the
   // two launches, so there is always a second launch; weight gradients keep their int32 sums
   const bool dp = ctx->reduce_fn != nullptr, dp_sum = dp && niti_is_wgrad(g.kind);
-  p.single_wave = (!dp && p.items <= (p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx)) && p.spec_mul256 == 256) ? 1 : 0;
+  p.single_wave = (!dp && p.items * p.ctas <= NITI_AGREE_MAX && p.items <= (p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx)) && p.spec_mul256 == 256) ? 1 : 0;
   {
     const long long units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
     const long long grid = (p.items < units ? p.items : units) * p.ctas;
