@@ -2275,6 +2275,9 @@ static int pick_bn(long long gn) {
   return round_up32((gn + tiles - 1) / tiles);
 }
 
+// Contractions up to this length run on single CTAs, deeper ones on CTA pairs (see niti_tc_gemm's choice of a plan).
+constexpr long long PAIR_MIN_K = 1152;
+
 // Builds params and maps; returns false if the shape is not eligible for this engine.
 // `aligned`: output (and mask) pointers and rows are 32-byte aligned.
 // force_bn: column tile of an unsplit one-wave plan (see pick_one_wave), 0 for the planner's own choice, -1 for that
@@ -2749,10 +2752,14 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     if (p.stages % d == 0) p.nprod = d;
   p.nbuf = 512 / p.bn;
   if (p.nbuf > MAX_TBUF) p.nbuf = MAX_TBUF;
-  // epilogue groups: as many as leave no warp without a chunk and one spare accumulator buffer
+  // epilogue groups: as many as leave no warp without a chunk and one spare accumulator buffer; without the spare
+  // one where the epilogue of a plain multiply is the bound and no MMA waits for long (single CTAs, 8192 x 8192 at
+  // K = 256 / 512 / 1024 40.5 -> 39.8, 46.3 -> 44.7, 63.3 -> 61.8 us, the gradient above 64.8 -> 59.6 us;
+  // convolutions of the same depth are 1 - 4 % slower that way)
+  const bool short_fc = ctas == 1 && g.kind <= GK_FC_WGRAD && g.gk <= PAIR_MIN_K;
   p.egroups = 1;
   for (int gq = 2; gq <= 4; gq *= 2)
-    if (EPI_PER_Q / gq <= p.bn / 32 && p.nbuf >= gq + 1) p.egroups = gq;
+    if (EPI_PER_Q / gq <= p.bn / 32 && p.nbuf >= gq + (short_fc ? 0 : 1)) p.egroups = gq;
   p.nbuf = p.nbuf / p.egroups * p.egroups;     // a buffer always returns to the same group
   p.one_commit = 0;
   if (p.halo == 1 && p.stages >= p.nbuf) {
@@ -2868,7 +2875,9 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
     const int gunits = (int)(grid / CTAS);
     q.blk_per = (int)(p.items / gunits);
     q.blk_extra = (int)(p.items % gunits);
-    const int eg = p.halo == 2 ? 1 : p.egroups;
+    // (a CTA with a single tile has all its epilogue warps on that tile)
+    if (p.items <= gunits) q.egroups = 1;
+    const int eg = p.halo == 2 ? 1 : q.egroups;
     q.k_wpq = EPI_PER_Q / eg;
     const int chunks_all = p.bn / 32;
     q.k_wpq_active = p.halo == 2 ? EPI_PER_Q : (chunks_all < q.k_wpq ? chunks_all : q.k_wpq);
@@ -3015,7 +3024,13 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     planned = plan(ctx, g, 1, PLAN_HALO, aligned, 0, acc, p, ma, mb, mc);
   if (!planned && g.kind == GK_FC_FWD && ctx->engine != 3)      // row-batched mode of short contractions
     planned = plan(ctx, g, 1, PLAN_BATCHED, aligned, 0, acc, p, ma, mb, mc);
-  if (!planned && ctx->engine != 2 && g.gm >= 2 * BM) {
+  // Pairs halve the operand traffic per MMA, and couple two SMs' epilogues to one accumulator.  With a short
+  // contraction the epilogue is the bound (about 3 - 4 k cycles per tile against 560 per k-block of 128), and two
+  // CTAs that drain their own tiles are ahead: gradient of 4096 x 25088 weights at batch 64 92 -> 65 us, 8192 x 8192
+  // at K = 256 / 512 / 1024 / 2048 54 -> 41, 55 -> 46, 64 -> 63, 90 -> 102 us; convolutions with K = 128 69.5 -> 52.4,
+  // 1152 25.6 -> 23.7, 2304 82 -> 92 us; strided errors (K of one phase) with K = 576 40.1 -> 36.2 us.
+  const long long k_tile = g.gk / (g.kind == GK_CONV_DGRAD ? (long long)g.stride * g.stride : 1);
+  if (!planned && ctx->engine != 2 && g.gm >= 2 * BM && (ctx->engine == 3 || k_tile > PAIR_MIN_K)) {
     planned = plan(ctx, g, 2, PLAN_ANY, aligned, 0, acc, p, ma, mb, mc);
     // (pairs halve the operand traffic per MMA; they are kept unless they would leave more than a
     // third of the GPU idle)
