@@ -337,157 +337,32 @@ int niti_launch_round_compact(niti_ctx *ctx, cudaStream_t st, const int32_t *acc
 // (64-bit) and the arg-max hit.  Pass 2: shared binary point, e32 recomputed and rounded to int8.
 // ---------------------------------------------------------------------------------------------
 // One warp per sample.  Pass 1 keeps two 64-bit scalars per sample (the offset p of Eq. 4 and the
-// sum of the T_i) instead of the T_i themselves; pass 2 recomputes T_i from the logit, which is a few
-// integer operations, so that the only per-element traffic is the logit read twice and the int8
-// result written once.
-__device__ __forceinline__ long long warp_reduce_ll(long long v, int op /*0 sum,1 max,2 min*/) {
-  for (int o = 16; o > 0; o >>= 1) {
-    long long u = __shfl_xor_sync(0xffffffffu, v, o);
-    v = op == 0 ? v + u : (op == 1 ? (u > v ? u : v) : (u < v ? u : v));
-  }
-  return v;
-}
-// x-hat of Eq. 3: (47274 * a) >> (15 - s), a left shift when s > 15
-__device__ __forceinline__ long long xent_xhat(int a, long long sh_amt) {
-  const long long P = 47274LL * (long long)a;
-  return sh_amt >= 0 ? (P >> sh_amt) : P * (1LL << (-sh_amt));
-}
-// T_i of Eq. 2 (s <= -7) or Eq. 4
-__device__ __forceinline__ long long xent_T(int a, int s, long long sh_amt, long long p) {
-  if (s <= -7) {
-    const long long ai = a;
-    return (1LL << (1 - 2 * s)) + ai * (1LL << (1 - s)) + ai * ai;
-  }
-  const long long xt = xent_xhat(a, sh_amt) - p;
-  return 1LL << (xt > 0 ? xt : 0);
+// sum of the T_i) instead of the T_i themselves; pass 2 recomputes T_i from the logit, so that the only
+// per-element traffic is the logit read twice and the int8 result written once.
+//
+// Eq. 3 in 32 bits.  x-hat of a logit is (47274 * a) >> (15 - s), a left shift when s > 15.  Without the left shift
+// two different logits are already 47274 apart, more than the window of 10: every T_i is 1 with it or without it, so
+// s > 15 is computed with no shift at all, and products (at most 23 bits) and thresholds fit 32 bits.  Off the label T_i
+// is a power of two, at most 2^9.
+constexpr int XENT_MUL = 47274;
+__device__ __forceinline__ int xent_shift(int s) { return s < 15 ? 15 - s : 0; }            // (s in -6 .. 24)
+__device__ __forceinline__ int xent_xhat(int a, int sh) { return (XENT_MUL * a) >> sh; }
+// log2 of T_i (Eq. 4); entries above the row's largest logit are never used
+__device__ __forceinline__ int xent_log_T(int a, int sh, int p) { return min(max(xent_xhat(a, sh) - p, 0), 15); }
+// T_i of Eq. 2 (s <= -7)
+__device__ __forceinline__ long long xent_T2(int a, int s) {
+  const long long ai = a;
+  return (1LL << (1 - 2 * s)) + ai * (1LL << (1 - s)) + ai * ai;
 }
 constexpr int XENT_WARPS = 8;
 
-__global__ void __launch_bounds__(32 * XENT_WARPS)
-xent_row_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr,
-                const int32_t *__restrict__ labels, long long *__restrict__ rowinfo, WsHeader *hdr,
-                int B, int N, uint32_t *__restrict__ status) {
-  __shared__ unsigned long long sh_max[XENT_WARPS];
-  __shared__ int sh_hit[XENT_WARPS];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * XENT_WARPS + warp;
-  const int s = *s_a_ptr;
-  unsigned long long row_max = 0;
-  int hit = 0;
-  if (r < B) {
-    const int label = labels[r];
-    const int8_t *row = a + (long long)r * N;
-    if (s < -22 || s > 24 || label < 0 || label >= N) {
-      if (lane == 0) {
-        atomicOr(status, (s < -22 || s > 24) ? NITI_DEV_XENT_RANGE : NITI_DEV_BAD_LABEL);
-        rowinfo[2 * (long long)r] = 0;
-        rowinfo[2 * (long long)r + 1] = 0;
-      }
-    } else {
-      const long long LLMIN = -0x7fffffffffffffffLL - 1, LLMAX = 0x7fffffffffffffffLL;
-      const long long sh_amt = 15 - (long long)s;
-      long long p = 0;
-      if (s > -7) {
-        long long mx = LLMIN;
-        for (int i = lane; i < N; i += 32) {
-          const long long xh = xent_xhat(row[i], sh_amt);
-          mx = xh > mx ? xh : mx;
-        }
-        mx = warp_reduce_ll(mx, 1);
-        p = LLMAX;
-        for (int i = lane; i < N; i += 32) {
-          const long long xh = xent_xhat(row[i], sh_amt);
-          if (xh > mx - 10 && xh < p) p = xh;
-        }
-        p = warp_reduce_ll(p, 2);
-      }
-      // sum of T_i, the largest T_i off the label, and the first arg-max of the row for the hit count
-      long long csum = 0, t_other = 0;
-      int best_v = -1000, best_i = 0x7fffffff;
-      for (int i = lane; i < N; i += 32) {
-        const int ai = row[i];
-        const long long T = xent_T(ai, s, sh_amt, p);
-        csum += T;
-        if (i != label && T > t_other) t_other = T;
-        if (ai > best_v) { best_v = ai; best_i = i; }
-      }
-      csum = warp_reduce_ll(csum, 0);
-      t_other = warp_reduce_ll(t_other, 1);
-      long long key = ((long long)(best_v + 1000) << 32) | (unsigned)(0x7fffffff - best_i);
-      key = warp_reduce_ll(key, 1);
-      // e32 = T_i off the label (positive) and T_label - sum (not positive) on it
-      const long long t_label = xent_T(row[label], s, sh_amt, p);
-      const long long on_label = csum - t_label;
-      row_max = (unsigned long long)(t_other > on_label ? t_other : on_label);
-      hit = (0x7fffffff - (int)(key & 0xffffffffLL)) == label ? 1 : 0;
-      if (lane == 0) {
-        rowinfo[2 * (long long)r] = p;
-        rowinfo[2 * (long long)r + 1] = csum;
-      }
-    }
-  }
-  if (lane == 0) { sh_max[warp] = row_max; sh_hit[warp] = hit; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long m = 0;
-    int h = 0;
-    for (int w = 0; w < XENT_WARPS; ++w) { m = sh_max[w] > m ? sh_max[w] : m; h += sh_hit[w]; }
-    if (m > *(volatile unsigned long long *)&hdr->maxabs64) atomicMax(&hdr->maxabs64, m);
-    if (h) atomicAdd(&hdr->hits, (unsigned)h);
-  }
-}
-
-__global__ void __launch_bounds__(32 * XENT_WARPS)
-xent_round_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr,
-                  const int32_t *__restrict__ labels, const long long *__restrict__ rowinfo,
-                  const WsHeader *__restrict__ hdr, int8_t *__restrict__ out, int B, int N, int round_mode,
-                  int32_t *__restrict__ b_out, int32_t *__restrict__ n_correct) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * XENT_WARPS + warp;
-  const unsigned long long mxv = hdr->maxabs64;
-  const int b = 64 - __clzll((long long)mxv);
-  const int bp = b > 7 ? b - 7 : 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (b_out) *b_out = b;
-    if (n_correct) *n_correct = (int32_t)hdr->hits;
-  }
-  if (r >= B) return;
-  const int s = *s_a_ptr;
-  const int label = labels[r];
-  const int8_t *row = a + (long long)r * N;
-  int8_t *orow = out + (long long)r * N;
-  const bool bad = s < -22 || s > 24 || label < 0 || label >= N;
-  const long long sh_amt = 15 - (long long)s;
-  const long long p = rowinfo[2 * (long long)r], csum = rowinfo[2 * (long long)r + 1];
-  auto one = [&](int i, int ai) -> int {
-    if (bad) return 0;
-    const long long v = xent_T(ai, s, sh_amt, p) - (i == label ? csum : 0);
-    const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    const long long q = (long long)niti_round_mag<unsigned long long>(m, bp, 127ull, round_mode);
-    return (int)(v < 0 ? -q : q);
-  };
-  if ((N & 3) == 0 && (((uintptr_t)a | (uintptr_t)out) & 3) == 0) {
-    // four logits per lane per step: 128 contiguous bytes per warp instruction
-    for (int i = 4 * lane; i < N; i += 128) {
-      const unsigned w = *reinterpret_cast<const unsigned *>(row + i);
-      unsigned o = 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        o |= ((unsigned)one(i + k, (int)(int8_t)(w >> (8 * k))) & 0xffu) << (8 * k);
-      *reinterpret_cast<unsigned *>(orow + i) = o;
-    }
-  } else {
-    for (int i = lane; i < N; i += 32) orow[i] = (int8_t)one(i, row[i]);
-  }
-}
-
-// ---- fast path (N % 4 == 0, 4-byte aligned rows): packed bytes and per-row tables ---------------
-// T_i depends on the logit value alone once the row's offset p is known, and x-hat is monotone in
-// the logit, so a row needs: the maxima of the logits before and after the label (packed byte max;
-// they also decide the arg-max hit), for Eq. 2 the sums of a and a^2 (dp4a), for Eq. 3-4 the smallest
-// logit whose x-hat exceeds max - 10 (a binary search over the 256 logit values gives the threshold,
-// a packed min the logit) and the sum of T over a 256-entry table.  Pass 2 builds a 256-entry table
-// of rounded results per row and looks every logit up; only the label element is computed apart.
+// What a row contributes: offset p of Eq. 4, sum of the T_i, largest magnitude of e32, hit.
+struct XentRow {
+  long long p, csum;
+  unsigned long long top;
+  int hit;
+};
+__device__ __forceinline__ bool xent_bad(int s, int label, int N) { return s < -22 || s > 24 || label < 0 || label >= N; }
 __device__ __forceinline__ int hmax_s8x4(unsigned w) {
   const int b0 = (int)(int8_t)w, b1 = (int)(int8_t)(w >> 8), b2 = (int)(int8_t)(w >> 16), b3 = (int)(int8_t)(w >> 24);
   return max(max(b0, b1), max(b2, b3));
@@ -496,271 +371,386 @@ __device__ __forceinline__ int hmin_s8x4(unsigned w) {
   const int b0 = (int)(int8_t)w, b1 = (int)(int8_t)(w >> 8), b2 = (int)(int8_t)(w >> 16), b3 = (int)(int8_t)(w >> 24);
   return min(min(b0, b1), min(b2, b3));
 }
-__device__ __forceinline__ int warp_max_i(int v) {
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ int warp_min_i(int v) {
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ int warp_sum_i(int v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
-// Tables for many rows (B >= XENT_TAB_MIN_ROWS).  The offset p of Eq. 4 is x-hat of one of the 256
-// logit values, so there are at most 256 different T tables and, once the shared binary point is
-// known, 256 different tables of rounded results: they are computed once per call (two launches of
-// 256 x 256 threads) and a row copies the 512- or 256-byte line it needs instead of evaluating
-// 2 x 256 64-bit expressions of its own.  ttab[i][v] = T(v - 128) with p = x-hat(i - 128) (16 bits:
-// entries a row can use are at most 2^9); thr[t] = 128 + the smallest logit whose x-hat exceeds
-// x-hat(t - 128) - 10; qtab[i][v] = T rounded with the shared binary point.  With tables the first
-// scalar of a row is p * 256 + (index of its line).
-constexpr int XENT_TAB_MIN_ROWS = 1024;
-struct XentTables {
-  unsigned short *ttab;
-  unsigned char *qtab;
-  unsigned char *thr;
+// Units of a row: four logits (whole, aligned words) or one.  Rows of at most xent_held units per lane stay in registers
+// over the sweeps of pass 1: up to 1024 logits in words, 64 as bytes.
+template <bool PACKED>
+constexpr int xent_held = PACKED ? 8 : 2;
+template <bool PACKED>
+__device__ __forceinline__ unsigned xent_unit(const int8_t *row, int i) {
+  return PACKED ? reinterpret_cast<const unsigned *>(row)[i] : (unsigned)(int)row[i];
+}
+template <bool PACKED, bool HELD>
+struct XentSweep {
+  const int8_t *row;
+  int units, lane;
+  unsigned w[HELD ? xent_held<PACKED> : 1];
+  __device__ __forceinline__ XentSweep(const int8_t *r, int n, int l) : row(r), units(n), lane(l) {
+    if (HELD) {
+#pragma unroll
+      for (int j = 0; j < xent_held<PACKED>; ++j) {
+        w[HELD ? j : 0] = 0u;
+        if (lane + 32 * j < units) w[HELD ? j : 0] = xent_unit<PACKED>(row, lane + 32 * j);
+      }
+    }
+  }
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {
+    if (HELD) {
+#pragma unroll
+      for (int j = 0; j < xent_held<PACKED>; ++j)
+        if (lane + 32 * j < units) f(lane + 32 * j, w[HELD ? j : 0]);
+    } else {
+      for (int i = lane; i < units; i += 32) f(i, xent_unit<PACKED>(row, i));
+    }
+  }
+  // logit i of the row (the same i in the whole warp)
+  __device__ __forceinline__ int logit(int i) const {
+    if (!HELD) return (int)row[i];
+    const int u = PACKED ? i >> 2 : i;
+    unsigned x = 0;
+#pragma unroll
+    for (int j = 0; j < xent_held<PACKED>; ++j)
+      x |= w[HELD ? j : 0] & (0u - (unsigned)(j == u >> 5));       // (masks: an index would put the words in local memory)
+    x = __shfl_sync(0xffffffffu, x, u & 31);
+    return PACKED ? (int)(int8_t)(x >> (8 * (i & 3))) : (int)x;
+  }
 };
 
-__global__ void __launch_bounds__(256)
-xent_ttab_kernel(const int32_t *__restrict__ s_a_ptr, XentTables t) {
-  const int s = *s_a_ptr;
-  if (s < -22 || s > 24 || s <= -7) return;             // (Eq. 2 needs no table of T)
-  const long long sh_amt = 15 - (long long)s;
-  const int i = blockIdx.x, v = threadIdx.x;
-  const long long p = xent_xhat(i - 128, sh_amt);
-  t.ttab[i * 256 + v] = (unsigned short)xent_T(v - 128, s, sh_amt, p);
-  if (i == 0) {
-    const long long mx = xent_xhat(v - 128, sh_amt);
-    int lo = -128, hi = v - 128;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (xent_xhat(mid, sh_amt) > mx - 10) hi = mid; else lo = mid + 1;
-    }
-    t.thr[v] = (unsigned char)(lo + 128);
+// Pass 1 of one row by one warp.  x-hat is monotone in the logit, so a row needs: the maxima of the logits before and
+// after the label (they also decide the arg-max hit), for Eq. 2 the sums of a and a^2, for Eq. 3-4 the smallest logit
+// whose x-hat exceeds max - 10 (a division gives the threshold) and the sum of the powers of two.
+// (s and label are in range)
+template <bool PACKED, bool HELD>
+__device__ __forceinline__ XentRow xent_row(const XentSweep<PACKED, HELD> &units, int N, int s, int label) {
+  XentRow out;
+  const int a_label = units.logit(label);
+  const int lw = PACKED ? label >> 2 : label, lb = label & 3;
+  int max_before = -128, max_after = -128, sum_a = 0, sum_q = 0;
+  if (PACKED) {
+    const unsigned low = lb == 0 ? 0u : (0xffffffffu >> (32 - 8 * lb));          // bytes before the label
+    const unsigned high = lb == 3 ? 0u : (0xffffffffu << (8 * (lb + 1)));        // bytes after it
+    unsigned mb = 0x80808080u, ma = 0x80808080u;
+    units.each([&](int i, unsigned w) {
+      sum_a = __dp4a((int)w, 0x01010101, sum_a);
+      sum_q = __dp4a((int)w, (int)w, sum_q);
+      const unsigned kb = i < lw ? 0xffffffffu : (i == lw ? low : 0u), ka = i > lw ? 0xffffffffu : (i == lw ? high : 0u);
+      mb = __vmaxs4(mb, (w & kb) | (0x80808080u & ~kb));
+      ma = __vmaxs4(ma, (w & ka) | (0x80808080u & ~ka));
+    });
+    max_before = hmax_s8x4(mb);
+    max_after = hmax_s8x4(ma);
+  } else {
+    units.each([&](int i, unsigned w) {
+      const int v = (int)w;
+      sum_a += v;
+      sum_q += v * v;
+      if (i < lw) max_before = max(max_before, v);
+      if (i > lw) max_after = max(max_after, v);
+    });
   }
+  max_before = __reduce_max_sync(0xffffffffu, max_before);
+  max_after = __reduce_max_sync(0xffffffffu, max_after);
+  const int max_other = max(max_before, max_after);       // -128 when the row has one element
+  out.hit = (label == 0 || a_label > max_before) && a_label >= max_after ? 1 : 0;   // the first arg-max is the label
+  out.p = 0;
+  long long t_other, t_label;
+  if (s <= -7) {
+    sum_a = __reduce_add_sync(0xffffffffu, sum_a);
+    sum_q = __reduce_add_sync(0xffffffffu, sum_q);
+    out.csum = (long long)N * (1LL << (1 - 2 * s)) + (long long)sum_a * (1LL << (1 - s)) + (long long)sum_q;
+    t_other = N > 1 ? xent_T2(max_other, s) : 0;          // T is increasing in the logit
+    t_label = xent_T2(a_label, s);
+  } else {
+    // smallest logit value whose x-hat exceeds mx - 10: 47274 * a >= (mx - 9) * 2^sh, rounded up
+    const int sh = xent_shift(s), mx = xent_xhat(max(max_other, a_label), sh);
+    const int num = (mx - 9) * (1 << sh);
+    const int lo = max(num > 0 ? (num + XENT_MUL - 1) / XENT_MUL : num / XENT_MUL, -128);
+    // the smallest logit of the row that is at least that value
+    int a_star = 127;
+    if (PACKED) {
+      const unsigned thr4 = (unsigned)(lo & 0xff) * 0x01010101u;
+      unsigned mn = 0x7f7f7f7fu;
+      units.each([&](int, unsigned w) {
+        const unsigned m = __vcmpges4(w, thr4);
+        mn = __vmins4(mn, (w & m) | (0x7f7f7f7fu & ~m));
+      });
+      a_star = hmin_s8x4(mn);
+    } else {
+      units.each([&](int, unsigned w) {
+        if ((int)w >= lo) a_star = min(a_star, (int)w);
+      });
+    }
+    const int p = xent_xhat(__reduce_min_sync(0xffffffffu, a_star), sh);
+    int acc = 0;
+    units.each([&](int, unsigned w) {
+      if (PACKED) {
+        acc += 1 << max(xent_xhat((int)(int8_t)w, sh) - p, 0);
+        acc += 1 << max(xent_xhat((int)(int8_t)(w >> 8), sh) - p, 0);
+        acc += 1 << max(xent_xhat((int)(int8_t)(w >> 16), sh) - p, 0);
+        acc += 1 << max(xent_xhat((int)w >> 24, sh) - p, 0);
+      } else {
+        acc += 1 << max(xent_xhat((int)w, sh) - p, 0);
+      }
+    });
+    out.p = p;
+    out.csum = (long long)__reduce_add_sync(0xffffffffu, acc);
+    t_other = N > 1 ? 1LL << xent_log_T(max_other, sh, p) : 0;
+    t_label = 1LL << xent_log_T(a_label, sh, p);
+  }
+  // e32 = T_i off the label (positive) and T_label - sum (not positive) on it
+  const long long on_label = out.csum - t_label;
+  out.top = (unsigned long long)(t_other > on_label ? t_other : on_label);
+  return out;
 }
 
-__global__ void __launch_bounds__(256)
-xent_qtab_kernel(const int32_t *__restrict__ s_a_ptr, const WsHeader *__restrict__ hdr, XentTables t, int round_mode) {
-  const int s = *s_a_ptr;
-  if (s < -22 || s > 24) return;
-  const unsigned long long mxv = hdr->maxabs64;
-  const int b = 64 - __clzll((long long)mxv);
-  const int bp = b > 7 ? b - 7 : 0;
-  const long long sh_amt = 15 - (long long)s;
-  const int i = blockIdx.x, v = threadIdx.x;
-  const long long p = s <= -7 ? 0 : xent_xhat(i - 128, sh_amt);
-  const unsigned long long T = (unsigned long long)xent_T(v - 128, s, sh_amt, p);
-  t.qtab[i * 256 + v] = (unsigned char)niti_round_mag<unsigned long long>(T, bp, 127ull, round_mode);
+// Pass 2 of one row by one warp: off the label e32 = T(a) > 0, one rounded value per logit value, looked up in 256 bytes:
+// the block's for Eq. 2 (q2), for Eq. 4 this warp's (q4), filled here from the rounded powers of two.
+template <bool PACKED, bool HELD>
+__device__ __forceinline__ void xent_out(const XentSweep<PACKED, HELD> &units, int8_t *__restrict__ out, int N, int s, int label, int bp,
+                                         int round_mode, int p, long long csum, const unsigned char *q2, unsigned char *q4, int lane) {
+  if (xent_bad(s, label, N)) {
+    units.each([&](int i, unsigned) {
+      if (PACKED) reinterpret_cast<unsigned *>(out)[i] = 0u;
+      else out[i] = 0;
+    });
+    return;
+  }
+  const int a_label = units.logit(label), sh = xent_shift(s);
+  long long t_label;
+  if (s > -7) {
+    // (sums of Eq. 4 are below 2^26: bp < 32)
+    const unsigned q_lane = niti_round_mag<unsigned>(1u << (lane & 15), bp, 127u, round_mode);
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < 256; v += 32)
+      q4[v + lane] = (unsigned char)__shfl_sync(0xffffffffu, q_lane, xent_log_T(v + lane - 128, sh, p));
+    __syncwarp();
+    t_label = 1LL << xent_log_T(a_label, sh, p);
+  } else {
+    t_label = xent_T2(a_label, s);
+  }
+  const unsigned char *q = s > -7 ? q4 : q2;
+  // on the label e32 = T - sum <= 0
+  const unsigned q_label =
+      (unsigned)(0 - (int)niti_round_mag<unsigned long long>((unsigned long long)(csum - t_label), bp, 127ull, round_mode)) & 0xffu;
+  const int lw = label >> 2, lb = label & 3;
+  units.each([&](int i, unsigned v) {
+    if (PACKED) {
+      const unsigned w = v ^ 0x80808080u;                                  // logit + 128 per byte
+      unsigned o = (unsigned)q[w & 0xff] | ((unsigned)q[(w >> 8) & 0xff] << 8) | ((unsigned)q[(w >> 16) & 0xff] << 16) |
+                   ((unsigned)q[w >> 24] << 24);
+      if (i == lw) o = (o & ~(0xffu << (8 * lb))) | (q_label << (8 * lb));
+      reinterpret_cast<unsigned *>(out)[i] = o;
+    } else {
+      out[i] = (int8_t)(i == label ? q_label : (unsigned)q[(int)v + 128]);
+    }
+  });
 }
 
-template <bool TAB>
+// The rows of one block.  ONE: a single row per warp, of at most 32 * xent_held units, whose logits, offset and sum stay in
+// registers between the passes; otherwise rows are strided over the warps and two scalars per row go through memory.
+template <bool PACKED, bool ONE>
+struct XentBlock {
+  XentSweep<PACKED, ONE> held;
+  XentRow mine;
+  int label;
+  __device__ __forceinline__ static long long first_row() {
+    return (long long)blockIdx.x * ((int)blockDim.x >> 5) + (threadIdx.x >> 5);
+  }
+  __device__ __forceinline__ XentBlock(const int8_t *__restrict__ a, const int32_t *__restrict__ labels, int B, int N)
+      : held(a + first_row() * N, ONE && first_row() < B ? (PACKED ? N >> 2 : N) : 0, (int)threadIdx.x & 31) {
+    label = ONE && first_row() < B ? labels[first_row()] : 0;
+  }
+  // pass 1: the 64-bit maximum and the hits of the block, in m / h of thread 0
+  __device__ __forceinline__ void stats(const int8_t *__restrict__ a, int s, const int32_t *__restrict__ labels, long long *rowinfo, int B,
+                                        int N, uint32_t *status, unsigned long long *sh_max, int *sh_hit, unsigned long long &m, int &h) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = (int)blockDim.x >> 5;
+    unsigned long long top = 0;
+    int hits = 0;
+    for (long long r = first_row(); r < B; r += (long long)gridDim.x * warps) {
+      if (!ONE) label = labels[r];
+      mine = {0, 0, 0ull, 0};
+      if (xent_bad(s, label, N)) {
+        if (lane == 0) atomicOr(status, (s < -22 || s > 24) ? NITI_DEV_XENT_RANGE : NITI_DEV_BAD_LABEL);
+      } else if (ONE) {
+        mine = xent_row(held, N, s, label);
+      } else {
+        const int units = PACKED ? N >> 2 : N;
+        mine = units <= 32 * xent_held<PACKED> ? xent_row(XentSweep<PACKED, true>(a + r * N, units, lane), N, s, label)
+                                       : xent_row(XentSweep<PACKED, false>(a + r * N, units, lane), N, s, label);
+      }
+      if (!ONE && lane == 0) {
+        rowinfo[2 * r] = mine.p;
+        rowinfo[2 * r + 1] = mine.csum;
+      }
+      top = mine.top > top ? mine.top : top;
+      hits += mine.hit;
+      if (ONE) break;
+    }
+    if (lane == 0) { sh_max[warp] = top; sh_hit[warp] = hits; }
+    __syncthreads();
+    m = 0;
+    h = 0;
+    if (threadIdx.x == 0)
+      for (int w = 0; w < warps; ++w) { m = sh_max[w] > m ? sh_max[w] : m; h += sh_hit[w]; }
+  }
+  // pass 2.  q_tab: 256 bytes of the block, then 256 of every warp
+  __device__ __forceinline__ void outs(const int8_t *__restrict__ a, int s, const int32_t *__restrict__ labels, const long long *rowinfo,
+                                       int8_t *__restrict__ out, int B, int N, int bp, int round_mode, unsigned char *q_tab) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = (int)blockDim.x >> 5;
+    if (s <= -7 && s >= -22) {
+      if (threadIdx.x < 256)
+        q_tab[threadIdx.x] =
+            (unsigned char)niti_round_mag<unsigned long long>((unsigned long long)xent_T2((int)threadIdx.x - 128, s), bp, 127ull, round_mode);
+      __syncthreads();
+    }
+    for (long long r = first_row(); r < B; r += (long long)gridDim.x * warps) {
+      unsigned char *q4 = q_tab + 256 * (warp + 1);
+      if (ONE) {
+        xent_out(held, out + r * N, N, s, label, bp, round_mode, (int)mine.p, mine.csum, q_tab, q4, lane);
+        break;
+      }
+      const int units = PACKED ? N >> 2 : N;
+      const int p = (int)rowinfo[2 * r];
+      const long long csum = rowinfo[2 * r + 1];
+      if (units <= 32 * xent_held<PACKED>)
+        xent_out(XentSweep<PACKED, true>(a + r * N, units, lane), out + r * N, N, s, labels[r], bp, round_mode, p, csum, q_tab, q4, lane);
+      else
+        xent_out(XentSweep<PACKED, false>(a + r * N, units, lane), out + r * N, N, s, labels[r], bp, round_mode, p, csum, q_tab, q4, lane);
+    }
+  }
+};
+
+// Both passes in two launches: the scratch has no room for an agreement (no-allocation variant), or the maximum is
+// combined over the ranks in between.
+template <bool PACKED>
 __global__ void __launch_bounds__(32 * XENT_WARPS)
-xent_row_fast_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr,
-                     const int32_t *__restrict__ labels, long long *__restrict__ rowinfo, WsHeader *hdr,
-                     int B, int N, uint32_t *__restrict__ status, XentTables tabs) {
+xent_row_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
+                long long *rowinfo, WsHeader *hdr, int B, int N, uint32_t *__restrict__ status) {
   __shared__ unsigned long long sh_max[XENT_WARPS];
   __shared__ int sh_hit[XENT_WARPS];
-  __shared__ __align__(16) unsigned short sh_T[XENT_WARPS][256];     // T(a) of Eq. 4 for a = -128 .. 127 (at most 2^9)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * XENT_WARPS + warp;
-  const int s = *s_a_ptr;
-  unsigned long long row_max = 0;
-  int hit = 0;
-  if (r < B) {
-    const int label = labels[r];
-    if (s < -22 || s > 24 || label < 0 || label >= N) {
-      if (lane == 0) {
-        atomicOr(status, (s < -22 || s > 24) ? NITI_DEV_XENT_RANGE : NITI_DEV_BAD_LABEL);
-        rowinfo[2 * (long long)r] = 0;
-        rowinfo[2 * (long long)r + 1] = 0;
-      }
-    } else {
-      const unsigned *row = reinterpret_cast<const unsigned *>(a + (long long)r * N);
-      const int words = N >> 2, lw = label >> 2, lb = label & 3;
-      const long long sh_amt = 15 - (long long)s;
-      const int a_label = (int)a[(long long)r * N + label];
-      // sweep 1: packed maxima before / after the label, sums of a and a^2
-      unsigned mb = 0x80808080u, ma = 0x80808080u;
-      int sum_a = 0, sum_q = 0;
-      for (int wi = lane; wi < words; wi += 32) {
-        const unsigned w = row[wi];
-        sum_a = __dp4a((int)w, 0x01010101, sum_a);
-        sum_q = __dp4a((int)w, (int)w, sum_q);
-        if (wi < lw) mb = __vmaxs4(mb, w);
-        else if (wi > lw) ma = __vmaxs4(ma, w);
-        else {
-          const unsigned low = lb == 0 ? 0u : (0xffffffffu >> (32 - 8 * lb));          // bytes before the label
-          const unsigned high = lb == 3 ? 0u : (0xffffffffu << (8 * (lb + 1)));        // bytes after it
-          mb = __vmaxs4(mb, (w & low) | (0x80808080u & ~low));
-          ma = __vmaxs4(ma, (w & high) | (0x80808080u & ~high));
-        }
-      }
-      const int max_before = warp_max_i(hmax_s8x4(mb)), max_after = warp_max_i(hmax_s8x4(ma));
-      const int max_other = max(max_before, max_after);       // -128 when the row has one element
-      const int row_top = max(max_other, a_label);
-      hit = (a_label > max_before && a_label >= max_after) ? 1 : 0;   // the first arg-max is the label
-      long long p = 0, csum, t_other, t_label;
-      int line = 0;                                     // (TAB) the table line of this row
-      if (s <= -7) {
-        sum_a = warp_sum_i(sum_a);
-        sum_q = warp_sum_i(sum_q);
-        csum = (long long)N * (1LL << (1 - 2 * s)) + (long long)sum_a * (1LL << (1 - s)) + (long long)sum_q;
-        t_other = N > 1 ? xent_T(max_other, s, sh_amt, 0) : 0;     // T is increasing in the logit
-        t_label = xent_T(a_label, s, sh_amt, 0);
-      } else {
-        // smallest logit value whose x-hat exceeds mx - 10 (x-hat is non-decreasing in the logit)
-        int lo = -128;
-        if (TAB) {
-          lo = (int)tabs.thr[row_top + 128] - 128;
-        } else {
-          const long long mx = xent_xhat(row_top, sh_amt);
-          int hi = row_top;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;          // floor for negative sums as well
-            if (xent_xhat(mid, sh_amt) > mx - 10) hi = mid; else lo = mid + 1;
-          }
-        }
-        const unsigned thr4 = (unsigned)(lo & 0xff) * 0x01010101u;
-        // sweep 2: the smallest logit of the row that is at least that value
-        unsigned mn = 0x7f7f7f7fu;
-        for (int wi = lane; wi < words; wi += 32) {
-          const unsigned w = row[wi];
-          const unsigned m = __vcmpges4(w, thr4);
-          mn = __vmins4(mn, (w & m) | (0x7f7f7f7fu & ~m));
-        }
-        const int a_star = warp_min_i(hmin_s8x4(mn));
-        p = xent_xhat(a_star, sh_amt);
-        // table of T over the logit values, then sweep 3: the sum
-        if (TAB) {
-          reinterpret_cast<uint4 *>(sh_T[warp])[lane] =
-              reinterpret_cast<const uint4 *>(tabs.ttab + (a_star + 128) * 256)[lane];
-          line = a_star + 128;
-        } else {
-          for (int v = lane; v < 256; v += 32) sh_T[warp][v] = (unsigned short)xent_T(v - 128, s, sh_amt, p);
-        }
-        __syncwarp();
-        int acc = 0;
-        for (int wi = lane; wi < words; wi += 32) {
-          const unsigned w = row[wi] ^ 0x80808080u;            // logit + 128 per byte
-          acc += (int)sh_T[warp][w & 0xff] + (int)sh_T[warp][(w >> 8) & 0xff] + (int)sh_T[warp][(w >> 16) & 0xff] +
-                 (int)sh_T[warp][w >> 24];
-        }
-        csum = (long long)warp_sum_i(acc);
-        t_other = N > 1 ? (long long)sh_T[warp][max_other + 128] : 0;
-        t_label = (long long)sh_T[warp][a_label + 128];
-      }
-      const long long on_label = csum - t_label;
-      row_max = (unsigned long long)(t_other > on_label ? t_other : on_label);
-      if (lane == 0) {
-        rowinfo[2 * (long long)r] = TAB ? p * 256 + line : p;
-        rowinfo[2 * (long long)r + 1] = csum;
-      }
-    }
-  }
-  if (lane == 0) { sh_max[warp] = row_max; sh_hit[warp] = hit; }
-  __syncthreads();
+  unsigned long long m;
+  int h;
+  XentBlock<PACKED, false> rows(a, labels, B, N);
+  rows.stats(a, *s_a_ptr, labels, rowinfo, B, N, status, sh_max, sh_hit, m, h);
   if (threadIdx.x == 0) {
-    unsigned long long m = 0;
-    int h = 0;
-    for (int w = 0; w < XENT_WARPS; ++w) { m = sh_max[w] > m ? sh_max[w] : m; h += sh_hit[w]; }
     if (m > *(volatile unsigned long long *)&hdr->maxabs64) atomicMax(&hdr->maxabs64, m);
     if (h) atomicAdd(&hdr->hits, (unsigned)h);
   }
 }
-
-template <bool TAB>
+template <bool PACKED>
 __global__ void __launch_bounds__(32 * XENT_WARPS)
-xent_round_fast_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr,
-                       const int32_t *__restrict__ labels, const long long *__restrict__ rowinfo,
-                       const WsHeader *__restrict__ hdr, int8_t *__restrict__ out, int B, int N, int round_mode,
-                       int32_t *__restrict__ b_out, int32_t *__restrict__ n_correct, XentTables tabs) {
-  __shared__ __align__(8) unsigned char sh_q[XENT_WARPS][256];        // rounded T(a) for a = -128 .. 127
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * XENT_WARPS + warp;
-  const unsigned long long mxv = hdr->maxabs64;
-  const int b = 64 - __clzll((long long)mxv);
-  const int bp = b > 7 ? b - 7 : 0;
+xent_round_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
+                  const long long *rowinfo, const WsHeader *__restrict__ hdr, int8_t *__restrict__ out, int B, int N,
+                  int round_mode, int32_t *__restrict__ b_out, int32_t *__restrict__ n_correct) {
+  __shared__ unsigned char q_tab[256 * (XENT_WARPS + 1)];
+  const int b = 64 - __clzll((long long)hdr->maxabs64), bp = b > 7 ? b - 7 : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (b_out) *b_out = b;
     if (n_correct) *n_correct = (int32_t)hdr->hits;
   }
-  if (r >= B) return;
-  const int s = *s_a_ptr;
-  const int label = labels[r];
-  const unsigned *row = reinterpret_cast<const unsigned *>(a + (long long)r * N);
-  unsigned *orow = reinterpret_cast<unsigned *>(out + (long long)r * N);
-  const int words = N >> 2;
-  if (s < -22 || s > 24 || label < 0 || label >= N) {
-    for (int wi = lane; wi < words; wi += 32) orow[wi] = 0u;
-    return;
-  }
-  const long long sh_amt = 15 - (long long)s;
-  const long long info = rowinfo[2 * (long long)r], csum = rowinfo[2 * (long long)r + 1];
-  const long long p = TAB ? (info >> 8) : info;
-  // off the label e32 = T(a) > 0: one rounded value per logit value
-  if (TAB) {
-    reinterpret_cast<uint2 *>(sh_q[warp])[lane] =
-        reinterpret_cast<const uint2 *>(tabs.qtab + (int)(info & 0xff) * 256)[lane];
-  } else {
-    for (int v = lane; v < 256; v += 32) {
-      const unsigned long long T = (unsigned long long)xent_T(v - 128, s, sh_amt, p);
-      sh_q[warp][v] = (unsigned char)niti_round_mag<unsigned long long>(T, bp, 127ull, round_mode);
-    }
-  }
-  // on the label e32 = T - sum <= 0
-  const int a_label = (int)a[(long long)r * N + label];
-  const unsigned long long m_label = (unsigned long long)(csum - xent_T(a_label, s, sh_amt, p));
-  const unsigned q_label = (unsigned)(0 - (int)niti_round_mag<unsigned long long>(m_label, bp, 127ull, round_mode)) & 0xffu;
-  __syncwarp();
-  const int lw = label >> 2, lb = label & 3;
-  for (int wi = lane; wi < words; wi += 32) {
-    const unsigned w = row[wi] ^ 0x80808080u;
-    unsigned o = (unsigned)sh_q[warp][w & 0xff] | ((unsigned)sh_q[warp][(w >> 8) & 0xff] << 8) |
-                 ((unsigned)sh_q[warp][(w >> 16) & 0xff] << 16) | ((unsigned)sh_q[warp][w >> 24] << 24);
-    if (wi == lw) o = (o & ~(0xffu << (8 * lb))) | (q_label << (8 * lb));
-    orow[wi] = o;
-  }
+  XentBlock<PACKED, false> rows(a, labels, B, N);
+  rows.outs(a, *s_a_ptr, labels, rowinfo, out, B, N, bp, round_mode, q_tab);
 }
 
-// both passes; the packed path needs whole words per row
-// (ctx may be null: the variant without a context; with one, the max magnitude of the 64-bit
-// gradients is combined over the ranks between the two passes when a reduction hook is installed)
-// tab_mem: 196864 bytes of scratch for the tables of many-row calls, or null
+// Both passes in one launch of at most one block per SM, all resident: the blocks agree on the bit-width in between.
+// Bound: latency (a launch, one round trip for the logits, the agreement); with many rows per SM the arithmetic of pass 1.
+// Two launches, of which the second reads labels, scalars and logits again, took 7.7 / 9.8 us for 64 x 1000 logits (Eq. 2 /
+// Eq. 4), four with tables of all 256 offsets 13.0 / 16.8 us for 4096 x 1000 (and 29 us with their gaps outside a graph);
+// one launch takes 4.7 / 5.5 and 9.2 / 11.5 us, 64 x 10 3.5 / 3.9 instead of 3.5 / 4.7 us.
+constexpr int XENT_MAX_WARPS = 32;
+constexpr long long XENT_WAIT_CYCLES = 2000000000LL;
+template <bool PACKED, bool ONE, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
+xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
+            long long *rowinfo, WsHeader *hdr, int8_t *__restrict__ out, int B, int N, int round_mode, int32_t *__restrict__ b_out,
+            int32_t *__restrict__ n_correct, uint32_t *__restrict__ status) {
+  __shared__ unsigned long long sh_max[WARPS];
+  __shared__ int sh_hit[WARPS];
+  __shared__ unsigned blk_b, grid_b;
+  __shared__ unsigned char q_tab[256 * (WARPS + 1)];
+  XentBlock<PACKED, ONE> rows(a, labels, B, N);
+  const int s = *s_a_ptr;
+  unsigned long long m;
+  int h;
+  rows.stats(a, s, labels, rowinfo, B, N, status, sh_max, sh_hit, m, h);
+  if (threadIdx.x == 0) {
+    blk_b = 64u - (unsigned)__clzll((long long)m);
+    if (gridDim.x == 1) {
+      grid_b = blk_b + 1u;
+      if (n_correct) *n_correct = h;
+    } else if (h) {
+      atomicAdd(&hdr->hits, (unsigned)h);
+      __threadfence();
+    }
+  }
+  if (gridDim.x > 1 && threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    __syncwarp();
+    unsigned *words = niti_split_max(hdr);
+    const long long c0 = clock64();
+    const unsigned all = niti_agree_max(words, words + NITI_AGREE_MAX, *(volatile unsigned *)&blk_b, (int)blockIdx.x, (int)gridDim.x, 0, lane, [&]() {
+      const bool late = __any_sync(0xffffffffu, clock64() - c0 > XENT_WAIT_CYCLES);
+      if (late && lane == 0) atomicOr(status, NITI_DEV_TIMEOUT);
+      return late;
+    });
+    if (lane == 0) {
+      grid_b = all;
+      if (blockIdx.x == 0 && n_correct && all) {            // (the first block has seen every post, and thereby every hit)
+        __threadfence();
+        *n_correct = (int32_t)*(volatile unsigned *)&hdr->hits;
+      }
+    }
+  }
+  __syncthreads();
+  if (grid_b == 0) return;                                  // (gave up waiting)
+  const int b = (int)grid_b - 1, bp = b > 7 ? b - 7 : 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && b_out) *b_out = b;
+  rows.outs(a, s, labels, rowinfo, out, B, N, bp, round_mode, q_tab);
+}
+
+template <bool PACKED, bool ONE>
+static void launch_xent_one(int grid, int warps, cudaStream_t st, const int8_t *a, const int32_t *s_a, const int32_t *labels,
+                            long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N, int round_mode,
+                            uint32_t *status) {
+  auto go = [&](auto kernel) {
+    kernel<<<grid, 32 * warps, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status);
+  };
+  if (warps == 8) go(xent_kernel<PACKED, ONE, 8>);
+  else if (warps == 16) go(xent_kernel<PACKED, ONE, 16>);
+  else go(xent_kernel<PACKED, ONE, XENT_MAX_WARPS>);
+}
+
+// The packed path needs whole words per row.  (ctx may be null: the variant without a context; with one, the max
+// magnitude of the 64-bit gradients is combined over the ranks between the two passes when a reduction hook is installed)
 static int launch_xent(niti_ctx *ctx, cudaStream_t st, const int8_t *a, const int32_t *s_a, const int32_t *labels,
                        long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N,
-                       int round_mode, uint32_t *status, void *tab_mem) {
-  const unsigned blocks = (unsigned)((B + XENT_WARPS - 1) / XENT_WARPS);
+                       int round_mode, uint32_t *status) {
   const bool packed = (N & 3) == 0 && N >= 64 && (((uintptr_t)a | (uintptr_t)e) & 3) == 0;
-  const bool tab = packed && tab_mem != nullptr && B >= XENT_TAB_MIN_ROWS;
-  XentTables t = {nullptr, nullptr, nullptr};
-  if (tab) {
-    t.ttab = (unsigned short *)tab_mem;
-    t.qtab = (unsigned char *)tab_mem + 256 * 256 * 2;
-    t.thr = t.qtab + 256 * 256;
-    xent_ttab_kernel<<<256, 256, 0, st>>>(s_a, t);
-    xent_row_fast_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status, t);
-  } else if (packed) {
-    xent_row_fast_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status, t);
-  } else {
-    xent_row_kernel<<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status);
+  if (ctx && !ctx->reduce_fn) {
+    const int sms = ctx->sm_count < NITI_AGREE_MAX ? ctx->sm_count : NITI_AGREE_MAX;
+    // few warps per block as long as there is one per row: 1024 x 1000 5.1 us with 8, 6.1 with 16, 9.9 with 32; 2048 x 100
+    // 7.3 / 5.3 / 6.5 us; 4096 x 1000 13.4 / 10.6 / 9.2 us
+    const int warps = B <= 8 * sms ? 8 : B <= 16 * sms ? 16 : XENT_MAX_WARPS;
+    const int need = (B + warps - 1) / warps, grid = need < sms ? need : sms;
+    const bool one = (packed ? N >> 2 <= 32 * xent_held<true> : N <= 32 * xent_held<false>) && B <= grid * warps;
+    auto go = [&](auto launch) { launch(grid, warps, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status); };
+    if (packed) { if (one) go(launch_xent_one<true, true>); else go(launch_xent_one<true, false>); }
+    else { if (one) go(launch_xent_one<false, true>); else go(launch_xent_one<false, false>); }
+    ctx->launches++;
+    return NITI_OK;
   }
+  const unsigned blocks = (unsigned)((B + XENT_WARPS - 1) / XENT_WARPS);
+  if (packed) xent_row_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status);
+  else xent_row_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status);
   if (ctx) {
-    int rc = niti_reduce(ctx, st, &hdr->maxabs64, 1, NITI_REDUCE_MAX_U64);
+    const int rc = niti_reduce(ctx, st, &hdr->maxabs64, 1, NITI_REDUCE_MAX_U64);
     if (rc != NITI_OK) return rc;
+    ctx->launches += 2;
   }
-  if (tab) {
-    xent_qtab_kernel<<<256, 256, 0, st>>>(s_a, hdr, t, round_mode);
-    xent_round_fast_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, t);
-    if (ctx) ctx->launches += 2;
-  } else if (packed) {
-    xent_round_fast_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, t);
-  } else {
-    xent_round_kernel<<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
-  }
+  if (packed) xent_round_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
+  else xent_round_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
   return NITI_OK;
 }
 
@@ -778,10 +768,8 @@ extern "C" int niti_int_xent(niti_ctx *ctx, void *stream, const int8_t *a, const
   long long *rowinfo = (long long *)((char *)ws + NITI_WS_HEADER);
   const int rch = niti_clear(ctx, st);
   if (rch != NITI_OK) return rch;
-  void *tab_mem = (char *)ws + NITI_WS_HEADER + ((size_t)B * 16 + 255) / 256 * 256;
-  int rcx = launch_xent(ctx, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, ctx->d_status, tab_mem);
+  const int rcx = launch_xent(ctx, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, ctx->d_status);
   if (rcx != NITI_OK) return rcx;
-  ctx->launches += 2;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
 }
@@ -824,7 +812,7 @@ extern "C" int niti_int_xent_noalloc(void *stream, const int8_t *a, const int32_
   // word of the header takes the (unreported) status bits of this variant.
   uint32_t *status = (uint32_t *)((char *)base + NITI_NOALLOC_HEADER - sizeof(uint32_t));
   if (cudaMemsetAsync(base, 0, NITI_NOALLOC_HEADER, st) != cudaSuccess) return NITI_ERR_CUDA;
-  launch_xent(nullptr, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status, nullptr);
+  launch_xent(nullptr, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status);
   if (cudaGetLastError() != cudaSuccess) return NITI_ERR_CUDA;
   return NITI_OK;
 }
