@@ -175,8 +175,8 @@ extern "C" int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_
   }
   if (((uintptr_t)ws & 255) || ws_bytes < NITI_WS_HEADER)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "niti_begin_step: workspace misaligned or too small");
-  NITI_CUDA_TRY(ctx, cudaMemsetAsync(ws, 0, NITI_WS_HEADER, (cudaStream_t)stream));
-  ctx->launches++;
+  const int rc = niti_memset0(ctx, (cudaStream_t)stream, ws, NITI_WS_HEADER);
+  if (rc != NITI_OK) return rc;
   ctx->step_ws = ws;
   ctx->step_slot = 0;
   return NITI_OK;

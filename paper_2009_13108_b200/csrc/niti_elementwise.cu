@@ -18,6 +18,7 @@ round_i32_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict__ h
                  const int8_t *__restrict__ mask, const int32_t *__restrict__ s_a,
                  const int32_t *__restrict__ s_w, int32_t *__restrict__ s_out,
                  int32_t *__restrict__ b_out, uint32_t *__restrict__ status, int8_t *__restrict__ upd_w) {
+  niti_enter(acc, hdr, mask, s_a, s_w, upd_w);
   const int b = niti_bitlen32(hdr->maxabs32);
   const int bp = b > mbits ? b - mbits : 0;
   const unsigned qmax = (1u << mbits) - 1u;
@@ -90,7 +91,7 @@ int niti_launch_round(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const 
   long long cap = (long long)ctx->sm_count * 16;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  round_i32_kernel<<<(unsigned)blocks, 256, 0, st>>>(acc, hdr, out, n, mbits, round_mode, relu, mask,
+  niti_launch(st, (unsigned)blocks, 256, 0, round_i32_kernel, acc, hdr, out, n, mbits, round_mode, relu, mask,
                                                      s_a, s_w, s_out, b_out, ctx->d_status, upd_w);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
@@ -105,6 +106,7 @@ int niti_launch_round(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const 
 __global__ void __launch_bounds__(256)
 im2col32_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xcol, int B, int H, int W, int Ci, int R,
                 int S, int pad, int stride, int Ho, int Wo) {
+  niti_enter(x);
   const long long M = (long long)B * Ho * Wo;
   for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < M;
        m += (long long)gridDim.x * blockDim.x) {
@@ -142,6 +144,7 @@ __device__ __forceinline__ unsigned win_byte(const unsigned (&w)[5], int idx) {
 }
 __global__ void __launch_bounds__(128)
 im2col32_rgb3x3_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xcol, int B, int H, int W) {
+  niti_enter(x);
   extern __shared__ unsigned rgb_rows[];          // 3 rows x pitch words
   const int row_words = W * 3 / 4;                // data words per image row
   const int pitch = row_words + 2;                // one halo word on each side (3 of its 4 bytes are used)
@@ -186,11 +189,35 @@ im2col32_rgb3x3_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xcol, 
   }
 }
 
+__global__ void __launch_bounds__(256)
+clear_kernel(int8_t *p, unsigned vecs, unsigned bytes) {
+  niti_enter(p);
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += gridDim.x * blockDim.x)
+    reinterpret_cast<int4 *>(p)[i] = make_int4(0, 0, 0, 0);
+  const unsigned tail = vecs * 16u + 4u * threadIdx.x;
+  if (blockIdx.x == 0 && tail < bytes) *reinterpret_cast<int *>(p + tail) = 0;
+}
+
+int niti_memset0(niti_ctx *ctx, cudaStream_t st, void *p, size_t bytes) {
+  ctx->launches++;
+  if (bytes >= ((size_t)1 << 31) || (bytes & 3) || ((uintptr_t)p & 15)) {
+    NITI_CUDA_TRY(ctx, cudaMemsetAsync(p, 0, bytes, st));
+    return NITI_OK;
+  }
+  const unsigned vecs = (unsigned)(bytes >> 4);
+  unsigned blocks = (vecs + 255u) / 256u;
+  const unsigned most = 8u * (unsigned)ctx->sm_count;
+  blocks = blocks < 1u ? 1u : (blocks > most ? most : blocks);
+  NITI_CUDA_TRY(ctx, niti_launch(st, blocks, 256, 0, clear_kernel, (int8_t *)p, vecs, (unsigned)bytes));
+  return NITI_OK;
+}
+
 // Rows of n bytes -> rows of `pitch` bytes (a multiple of 4, pitch >= n), zero padded.  One output word per thread
 // from the two aligned source words around it (bound: memory; the byte-per-thread form with its 64-bit
 // divisions took 12.9 us for 4096 rows of 1000 bytes).
 __global__ void __launch_bounds__(256)
 pad_pitch_kernel(const int8_t *__restrict__ src, int8_t *__restrict__ dst, long long rows, int n, int pitch) {
+  niti_enter(src);
   const int words = pitch >> 2;
   const long long total = rows * n;                       // source bytes
   const int wpb = (int)(blockDim.x);
@@ -221,7 +248,7 @@ int niti_launch_pad_pitch(niti_ctx *ctx, cudaStream_t st, const int8_t *src, int
   const int words = pitch >> 2, rows_pb = words >= 256 ? 1 : 256 / words;
   long long blocks = (rows + rows_pb - 1) / rows_pb;
   if (blocks > (long long)ctx->sm_count * 32) blocks = (long long)ctx->sm_count * 32;
-  pad_pitch_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dst, rows, n, pitch);
+  niti_launch(st, (unsigned)blocks, 256, 0, pad_pitch_kernel, src, dst, rows, n, pitch);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -233,6 +260,7 @@ __global__ void __launch_bounds__(256)
 round_compact_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict__ hdr, int8_t *__restrict__ out,
                      int rows, int k, int pitch, int rowk, int rpitch, int Ci, int Cp, int mbits, int round_mode,
                      int32_t *__restrict__ b_out, int8_t *__restrict__ upd_w) {
+  niti_enter(acc, hdr, upd_w);
   const int b = niti_bitlen32(hdr->maxabs32);
   const int bp = b > mbits ? b - mbits : 0;
   const unsigned qmax = (1u << mbits) - 1u;
@@ -259,6 +287,7 @@ round_compact_kernel(const int32_t *__restrict__ acc, const WsHeader *__restrict
 __global__ void __launch_bounds__(256)
 widen_pixels_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xw, unsigned rows, int W, int Ci, int cp_shift, int pad,
                     unsigned row_parts) {
+  niti_enter(x);
   const unsigned total = rows * row_parts, stride = gridDim.x * blockDim.x;
   for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride) {
     const unsigned r = idx / row_parts, part = idx - r * row_parts;
@@ -275,6 +304,7 @@ widen_pixels_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ xw, unsig
 // weights [Cout][R][S][Ci] -> [Cout][R][pitch], tap column s in bytes s * Cp .. s * Cp + Ci - 1, zero elsewhere
 __global__ void __launch_bounds__(256)
 widen_weights_kernel(const int8_t *__restrict__ w, int8_t *__restrict__ ww, int rows, int S, int Ci, int Cp, int pitch) {
+  niti_enter(w);
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < (long long)rows * pitch) {
     const int r = (int)(idx / pitch), b = (int)(idx - (long long)r * pitch);
@@ -289,10 +319,10 @@ int niti_launch_widen(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *x
   long long blocks = (parts + 255) / 256;
   if (blocks > (long long)ctx->sm_count * 64) blocks = (long long)ctx->sm_count * 64;
   const int cp_shift = Cp == 4 ? 2 : (Cp == 8 ? 3 : 4);
-  widen_pixels_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, xw, (unsigned)rows, W, Ci, cp_shift, pad, (unsigned)(row_bytes / 16));
+  niti_launch(st, (unsigned)blocks, 256, 0, widen_pixels_kernel, x, xw, (unsigned)rows, W, Ci, cp_shift, pad, (unsigned)(row_bytes / 16));
   ctx->launches++;
   if (w) {
-    widen_weights_kernel<<<(unsigned)(((long long)wrows * pitch + 255) / 256), 256, 0, st>>>(w, ww, wrows, S, Ci, Cp, pitch);
+    niti_launch(st, (unsigned)(((long long)wrows * pitch + 255) / 256), 256, 0, widen_weights_kernel, w, ww, wrows, S, Ci, Cp, pitch);
     ctx->launches++;
   }
   NITI_CUDA_TRY(ctx, cudaGetLastError());
@@ -306,7 +336,7 @@ int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t
     const int threads = W / 4 >= 128 ? 128 : (W / 4 > 32 ? 64 : 32);
     const size_t smem = (size_t)3 * (W * 3 / 4 + 2) * sizeof(unsigned);
     if (smem <= 48 * 1024) {
-      im2col32_rgb3x3_kernel<<<(unsigned)(B * H), threads, smem, st>>>(x, xcol, B, H, W);
+      niti_launch(st, (unsigned)(B * H), threads, smem, im2col32_rgb3x3_kernel, x, xcol, B, H, W);
       ctx->launches++;
       NITI_CUDA_TRY(ctx, cudaGetLastError());
       return NITI_OK;
@@ -315,7 +345,7 @@ int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t
   long long M = (long long)B * Ho * Wo;
   long long blocks = (M + 255) / 256;
   if (blocks > (long long)ctx->sm_count * 16) blocks = (long long)ctx->sm_count * 16;
-  im2col32_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, xcol, B, H, W, Ci, R, S, pad, stride, Ho, Wo);
+  niti_launch(st, (unsigned)blocks, 256, 0, im2col32_kernel, x, xcol, B, H, W, Ci, R, S, pad, stride, Ho, Wo);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -324,7 +354,7 @@ int niti_launch_im2col32(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t
 int niti_launch_round_compact(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, const WsHeader *hdr, int8_t *out,
                               int rows, int k, int pitch, int rowk, int rpitch, int Ci, int Cp, int mbits, int round_mode,
                               int32_t *b_out, int8_t *upd_w) {
-  round_compact_kernel<<<(rows * k + 255) / 256, 256, 0, st>>>(acc, hdr, out, rows, k, pitch, rowk, rpitch, Ci, Cp, mbits,
+  niti_launch(st, (rows * k + 255) / 256, 256, 0, round_compact_kernel, acc, hdr, out, rows, k, pitch, rowk, rpitch, Ci, Cp, mbits,
                                                                round_mode, b_out, upd_w);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
@@ -628,6 +658,7 @@ template <bool PACKED>
 __global__ void __launch_bounds__(32 * XENT_WARPS)
 xent_row_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
                 long long *rowinfo, WsHeader *hdr, int B, int N, uint32_t *__restrict__ status) {
+  niti_enter(a, s_a_ptr, labels);
   __shared__ unsigned long long sh_max[XENT_WARPS];
   __shared__ int sh_hit[XENT_WARPS];
   unsigned long long m;
@@ -644,6 +675,7 @@ __global__ void __launch_bounds__(32 * XENT_WARPS)
 xent_round_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
                   const long long *rowinfo, const WsHeader *__restrict__ hdr, int8_t *__restrict__ out, int B, int N,
                   int round_mode, int32_t *__restrict__ b_out, int32_t *__restrict__ n_correct) {
+  niti_enter(a, s_a_ptr, labels, rowinfo, hdr);
   __shared__ unsigned char q_tab[256 * (XENT_WARPS + 1)];
   const int b = 64 - __clzll((long long)hdr->maxabs64), bp = b > 7 ? b - 7 : 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -666,6 +698,7 @@ __global__ void __launch_bounds__(32 * WARPS)
 xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
             long long *rowinfo, WsHeader *hdr, int8_t *__restrict__ out, int B, int N, int round_mode, int32_t *__restrict__ b_out,
             int32_t *__restrict__ n_correct, uint32_t *__restrict__ status) {
+  niti_enter(a, s_a_ptr, labels);
   __shared__ unsigned long long sh_max[WARPS];
   __shared__ int sh_hit[WARPS];
   __shared__ unsigned blk_b, grid_b;
@@ -715,7 +748,7 @@ static void launch_xent_one(int grid, int warps, cudaStream_t st, const int8_t *
                             long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N, int round_mode,
                             uint32_t *status) {
   auto go = [&](auto kernel) {
-    kernel<<<grid, 32 * warps, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status);
+    niti_launch(st, grid, 32 * warps, 0, kernel, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status);
   };
   if (warps == 8) go(xent_kernel<PACKED, ONE, 8>);
   else if (warps == 16) go(xent_kernel<PACKED, ONE, 16>);
@@ -742,15 +775,15 @@ static int launch_xent(niti_ctx *ctx, cudaStream_t st, const int8_t *a, const in
     return NITI_OK;
   }
   const unsigned blocks = (unsigned)((B + XENT_WARPS - 1) / XENT_WARPS);
-  if (packed) xent_row_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status);
-  else xent_row_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, B, N, status);
+  if (packed) niti_launch(st, blocks, 32 * XENT_WARPS, 0, xent_row_kernel<true>, a, s_a, labels, rowinfo, hdr, B, N, status);
+  else niti_launch(st, blocks, 32 * XENT_WARPS, 0, xent_row_kernel<false>, a, s_a, labels, rowinfo, hdr, B, N, status);
   if (ctx) {
     const int rc = niti_reduce(ctx, st, &hdr->maxabs64, 1, NITI_REDUCE_MAX_U64);
     if (rc != NITI_OK) return rc;
     ctx->launches += 2;
   }
-  if (packed) xent_round_kernel<true><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
-  else xent_round_kernel<false><<<blocks, 32 * XENT_WARPS, 0, st>>>(a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
+  if (packed) niti_launch(st, blocks, 32 * XENT_WARPS, 0, xent_round_kernel<true>, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
+  else niti_launch(st, blocks, 32 * XENT_WARPS, 0, xent_round_kernel<false>, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct);
   return NITI_OK;
 }
 
@@ -823,6 +856,7 @@ extern "C" int niti_int_xent_noalloc(void *stream, const int8_t *a, const int32_
 
 __global__ void __launch_bounds__(256)
 sgd_update_kernel(int8_t *__restrict__ w, const int8_t *__restrict__ g, long long n) {
+  niti_enter(w, g);
   const long long nvec = n >> 4;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -843,6 +877,7 @@ sgd_update_kernel(int8_t *__restrict__ w, const int8_t *__restrict__ g, long lon
 
 __global__ void __launch_bounds__(256)
 relu_fwd_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ y, long long n) {
+  niti_enter(x);
   const long long nvec = n >> 4;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -858,6 +893,7 @@ relu_fwd_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ y, long long 
 __global__ void __launch_bounds__(256)
 relu_bwd_kernel(const int8_t *__restrict__ y, const int8_t *__restrict__ eo, int8_t *__restrict__ ei,
                 long long n) {
+  niti_enter(y, eo);
   const long long nvec = n >> 4;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -876,6 +912,7 @@ relu_bwd_kernel(const int8_t *__restrict__ y, const int8_t *__restrict__ eo, int
 template <int VEC>
 __global__ void __launch_bounds__(256)
 maxpool2_fwd_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ y, int B, int H, int W, int C) {
+  niti_enter(x);
   const int Ho = H >> 1, Wo = W >> 1, Cv = C / VEC;
   const long long total = (long long)B * Ho * Wo * Cv;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -928,6 +965,7 @@ template <int VEC>
 __global__ void __launch_bounds__(256)
 maxpool2_bwd_kernel(const int8_t *__restrict__ x, const int8_t *__restrict__ eo,
                     int8_t *__restrict__ ei, int B, int H, int W, int C, int relu) {
+  niti_enter(x, eo);
   const int Ho = H >> 1, Wo = W >> 1, Cv = C / VEC;
   const long long total = (long long)B * Ho * Wo * Cv;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -996,6 +1034,7 @@ __device__ __forceinline__ unsigned pool_unpack_nibbles(unsigned p16) {
 __global__ void __launch_bounds__(256)
 maxpool2_fwd_idx_kernel(const int8_t *__restrict__ x, int8_t *__restrict__ y, uint8_t *__restrict__ idx, int B, int H,
                         int W, int C) {
+  niti_enter(x);
   const int Ho = H >> 1, Wo = W >> 1, Cv = C / 16;
   const long long total = (long long)B * Ho * Wo * Cv;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -1038,6 +1077,7 @@ __device__ __forceinline__ void pool_route_word(unsigned codes, unsigned e, int 
 __global__ void __launch_bounds__(256)
 maxpool2_bwd_idx_kernel(const int8_t *__restrict__ eo, const uint8_t *__restrict__ idx, int8_t *__restrict__ ei, int B,
                         int H, int W, int C, int relu) {
+  niti_enter(eo, idx);
   const int Ho = H >> 1, Wo = W >> 1, Cv = C / 16;
   const long long total = (long long)B * Ho * Wo * Cv;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -1073,7 +1113,7 @@ static inline unsigned ew_blocks(niti_ctx *ctx, long long work_items) {
 }
 
 int niti_launch_sgd_update(niti_ctx *ctx, cudaStream_t st, int8_t *w, const int8_t *g, long long n) {
-  sgd_update_kernel<<<ew_blocks(ctx, (n >> 4) + 16), 256, 0, st>>>(w, g, n);
+  niti_launch(st, ew_blocks(ctx, (n >> 4) + 16), 256, 0, sgd_update_kernel, w, g, n);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1084,7 +1124,7 @@ extern "C" int niti_int_sgd_update(niti_ctx *ctx, void *stream, int8_t *w, const
   if (!w || !g || n <= 0) return niti_fail(ctx, NITI_ERR_ARG, "niti_int_sgd_update: bad argument");
   if (((uintptr_t)w | (uintptr_t)g) & 15)
     return niti_fail(ctx, NITI_ERR_ARG, "niti_int_sgd_update: pointers must be 16-byte aligned");
-  sgd_update_kernel<<<ew_blocks(ctx, (n >> 4) + 16), 256, 0, (cudaStream_t)stream>>>(w, g, n);
+  niti_launch((cudaStream_t)stream, ew_blocks(ctx, (n >> 4) + 16), 256, 0, sgd_update_kernel, w, g, n);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1104,6 +1144,7 @@ struct CopyList {
 };
 __global__ void __launch_bounds__(256)
 copy_many_kernel(const __grid_constant__ CopyList l) {
+  niti_enter();
   int t = 0;
   while (t + 1 < l.n && (int)blockIdx.x >= l.first[t + 1]) ++t;
   const long long off = (long long)((int)blockIdx.x - l.first[t]) * COPY_BLOCK_BYTES;
@@ -1144,7 +1185,7 @@ extern "C" int niti_copy_tensors(niti_ctx *ctx, void *stream, int n, void *const
     l.first[l.n] = (int)blocks;
     if (blocks >= (1LL << 31)) return niti_fail(ctx, NITI_ERR_SHAPE, "niti_copy_tensors: too many bytes");
     if (!blocks) continue;
-    copy_many_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(l);
+    niti_launch((cudaStream_t)stream, (unsigned)blocks, 256, 0, copy_many_kernel, l);
     ctx->launches++;
     NITI_CUDA_TRY(ctx, cudaGetLastError());
   }
@@ -1155,7 +1196,7 @@ extern "C" int niti_relu_fwd(niti_ctx *ctx, void *stream, const int8_t *x, int8_
   if (!ctx) return NITI_ERR_ARG;
   if (!x || !y || n <= 0 || (((uintptr_t)x | (uintptr_t)y) & 15))
     return niti_fail(ctx, NITI_ERR_ARG, "niti_relu_fwd: bad argument");
-  relu_fwd_kernel<<<ew_blocks(ctx, (n >> 4) + 16), 256, 0, (cudaStream_t)stream>>>(x, y, n);
+  niti_launch((cudaStream_t)stream, ew_blocks(ctx, (n >> 4) + 16), 256, 0, relu_fwd_kernel, x, y, n);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1166,7 +1207,7 @@ extern "C" int niti_relu_bwd(niti_ctx *ctx, void *stream, const int8_t *y, const
   if (!ctx) return NITI_ERR_ARG;
   if (!y || !e_out || !e_in || n <= 0 || (((uintptr_t)y | (uintptr_t)e_out | (uintptr_t)e_in) & 15))
     return niti_fail(ctx, NITI_ERR_ARG, "niti_relu_bwd: bad argument");
-  relu_bwd_kernel<<<ew_blocks(ctx, (n >> 4) + 16), 256, 0, (cudaStream_t)stream>>>(y, e_out, e_in, n);
+  niti_launch((cudaStream_t)stream, ew_blocks(ctx, (n >> 4) + 16), 256, 0, relu_bwd_kernel, y, e_out, e_in, n);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1176,9 +1217,9 @@ int niti_launch_maxpool2_fwd(niti_ctx *ctx, cudaStream_t st, const int8_t *x, in
   bool vec = (C % 16 == 0) && !(((uintptr_t)x | (uintptr_t)y) & 15);
   long long items = (long long)B * (H / 2) * (W / 2) * (vec ? C / 16 : C);
   if (vec)
-    maxpool2_fwd_kernel<16><<<ew_blocks(ctx, items), 256, 0, st>>>(x, y, B, H, W, C);
+    niti_launch(st, ew_blocks(ctx, items), 256, 0, maxpool2_fwd_kernel<16>, x, y, B, H, W, C);
   else
-    maxpool2_fwd_kernel<1><<<ew_blocks(ctx, items), 256, 0, st>>>(x, y, B, H, W, C);
+    niti_launch(st, ew_blocks(ctx, items), 256, 0, maxpool2_fwd_kernel<1>, x, y, B, H, W, C);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1200,7 +1241,7 @@ extern "C" int niti_maxpool2_fwd_idx(niti_ctx *ctx, void *stream, const int8_t *
   if ((C % 16) != 0 || (((uintptr_t)x | (uintptr_t)y) & 15) || ((uintptr_t)idx & 7))
     return niti_fail(ctx, NITI_ERR_SHAPE, "niti_maxpool2_fwd_idx: C must be a multiple of 16 and the tensors aligned");
   const long long items = (long long)B * (H / 2) * (W / 2) * (C / 16);
-  maxpool2_fwd_idx_kernel<<<ew_blocks(ctx, items), 256, 0, (cudaStream_t)stream>>>(x, y, idx, B, H, W, C);
+  niti_launch((cudaStream_t)stream, ew_blocks(ctx, items), 256, 0, maxpool2_fwd_idx_kernel, x, y, idx, B, H, W, C);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1214,7 +1255,7 @@ extern "C" int niti_maxpool2_bwd_idx(niti_ctx *ctx, void *stream, const int8_t *
   if ((C % 16) != 0 || (((uintptr_t)e_out | (uintptr_t)e_in) & 15) || ((uintptr_t)idx & 7))
     return niti_fail(ctx, NITI_ERR_SHAPE, "niti_maxpool2_bwd_idx: C must be a multiple of 16 and the tensors aligned");
   const long long items = (long long)B * (H / 2) * (W / 2) * (C / 16);
-  maxpool2_bwd_idx_kernel<<<ew_blocks(ctx, items), 256, 0, (cudaStream_t)stream>>>(e_out, idx, e_in, B, H, W, C, relu);
+  niti_launch((cudaStream_t)stream, ew_blocks(ctx, items), 256, 0, maxpool2_bwd_idx_kernel, e_out, idx, e_in, B, H, W, C, relu);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -1228,9 +1269,9 @@ extern "C" int niti_maxpool2_bwd(niti_ctx *ctx, void *stream, const int8_t *x, c
   bool vec = (C % 16 == 0) && !(((uintptr_t)x | (uintptr_t)e_out | (uintptr_t)e_in) & 15);
   long long items = (long long)B * (H / 2) * (W / 2) * (vec ? C / 16 : C);
   if (vec)
-    maxpool2_bwd_kernel<16><<<ew_blocks(ctx, items), 256, 0, (cudaStream_t)stream>>>(x, e_out, e_in, B, H, W, C, relu);
+    niti_launch((cudaStream_t)stream, ew_blocks(ctx, items), 256, 0, maxpool2_bwd_kernel<16>, x, e_out, e_in, B, H, W, C, relu);
   else
-    maxpool2_bwd_kernel<1><<<ew_blocks(ctx, items), 256, 0, (cudaStream_t)stream>>>(x, e_out, e_in, B, H, W, C, relu);
+    niti_launch((cudaStream_t)stream, ew_blocks(ctx, items), 256, 0, maxpool2_bwd_kernel<1>, x, e_out, e_in, B, H, W, C, relu);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;

@@ -94,6 +94,7 @@ __device__ __forceinline__ int8_t load_b(const Addr &q, long long n, long long k
 template <bool SPLIT>
 __global__ void __launch_bounds__(256)
 simt_gemm_kernel(Addr q, int32_t *__restrict__ acc, WsHeader *hdr, long long k_per_split) {
+  niti_enter();
   __shared__ int As[TM][TK / 4 + 1];
   __shared__ int Bs[TN][TK / 4 + 1];
   __shared__ unsigned smax[8];
@@ -183,6 +184,7 @@ simt_gemm_kernel(Addr q, int32_t *__restrict__ acc, WsHeader *hdr, long long k_p
 // 2^31 the int32 contract cannot be vouched for.
 __global__ void __launch_bounds__(256)
 maxabs_i32_kernel(const int32_t *__restrict__ acc, long long n, WsHeader *hdr, int splits, uint32_t *status) {
+  niti_enter(acc);
   if (splits > 1 && blockIdx.x == 0 && threadIdx.x < 32) {
     unsigned long long bound = 0;
     const unsigned *sm = niti_split_max(hdr);
@@ -224,7 +226,7 @@ int niti_launch_maxabs(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, long 
   long long blocks = ((n >> 2) + 255) / 256;
   if (blocks > ctx->sm_count * 8) blocks = ctx->sm_count * 8;
   if (blocks < 1) blocks = 1;
-  maxabs_i32_kernel<<<(unsigned)blocks, 256, 0, st>>>(acc, n, hdr, splits, ctx->d_status);
+  niti_launch(st, (unsigned)blocks, 256, 0, maxabs_i32_kernel, acc, n, hdr, splits, ctx->d_status);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;
@@ -260,14 +262,14 @@ int niti_simt_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, int32_t
   if (splits > 1) {
     const int rc = niti_clear(ctx, st, acc, sizeof(int32_t) * (size_t)(p.gm * p.gn));
     if (rc != NITI_OK) return rc;
-    simt_gemm_kernel<true><<<grid, 256, 0, st>>>(q, acc, hdr, kps);
+    niti_launch(st, grid, 256, 0, simt_gemm_kernel<true>, q, acc, hdr, kps);
     ctx->launches++;
     NITI_CUDA_TRY(ctx, cudaGetLastError());
     return niti_launch_maxabs(ctx, st, acc, p.gm * p.gn, hdr, (int)splits);
   }
   const int rc = niti_clear(ctx, st);
   if (rc != NITI_OK) return rc;
-  simt_gemm_kernel<false><<<grid, 256, 0, st>>>(q, acc, hdr, kps);
+  niti_launch(st, grid, 256, 0, simt_gemm_kernel<false>, q, acc, hdr, kps);
   ctx->launches++;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
   return NITI_OK;

@@ -163,6 +163,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   int *acc = reinterpret_cast<int *>(smem);                 // [rm][rn + 4]
   int8_t *As = smem + (size_t)o.rm * acc_pitch * 4, *Bs = As + o.rm * (o.kc + 16);
   if (tid == 0) cta_max = 0;
+  niti_enter();
   unsigned mx = 0;
   {
     const int tiles_n = o.rn >> 5, tiles = (o.rm >> 5) * tiles_n;
@@ -381,17 +382,11 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
     const size_t s2 = region_smem(p.op[1].rm, p.op[1].rn, p.op[1].kc);
     if (s2 > smem) smem = s2;
   }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
   WsHeader *hdr = niti_take_header(ctx, ws);
   const int rc = niti_clear(ctx, st);
   if (rc != NITI_OK) return rc;
   p.words = niti_split_max(hdr);
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(SMALL_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, small_gemm_kernel, p));
+  NITI_CUDA_TRY(ctx, niti_launch(st, (unsigned)grid, SMALL_THREADS, smem, small_gemm_kernel, p));
   ctx->launches++;
   ctx->tc_launches += g2 ? 2 : 1;
   return NITI_OK;

@@ -900,11 +900,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                int8_t *__restrict__ out8, const int8_t *__restrict__ mask8, const int32_t *s_a,
                const int32_t *s_w, int32_t *s_out, int32_t *b_out, int32_t *spec_slot, int8_t *__restrict__ pool8) {
   constexpr bool I2C = MODE >= 1, STRIDED = MODE == 2, GENERAL = MODE >= 1;
-  if ((p.epi_mode == EPI_SPECULATE && !p.single_wave) || p.epi_mode == EPI_ATOMIC) {
-    // the follow-up launch may be scheduled now (it is launched as a programmatic dependent): its CTAs
-    // take the SMs as this grid's CTAs retire and wait there for the whole grid to finish
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
   if (p.epi_mode == EPI_KNOWN_B) {
     // follow-up of a speculative pass: publish the scalars, then leave unless the guess was wrong
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the first pass has completed and is visible
@@ -1010,6 +1005,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (CTAS == 2) cluster_sync_all();   // the peer's barriers exist before anyone signals them
   tc_fence_after();
   const unsigned tmem_base = tmem_base_slot;
+  // (the set-up above overlaps the kernel before this one; a follow-up launch that is scheduled from here on takes the SMs
+  // as this grid's CTAs retire)
+  niti_enter(mask8);
 
   if (warp < PROD_WARPS) {
     // ================= TMA producers (every CTA loads its own rows of A and its share of B) ========
@@ -2013,7 +2011,7 @@ finish_split_kernel(const int32_t *__restrict__ acc, int nvec, WsHeader *hdr, in
   __shared__ unsigned blk_max, grid_max;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, T = (int)gridDim.x * FIN_THREADS;
   if (tid == 0) blk_max = 0;
-  asm volatile("griddepcontrol.wait;" ::: "memory");          // the multiply has completed and is visible
+  niti_enter(acc, mask);                                      // the multiply has completed and is visible
   const int t0 = (int)blockIdx.x * FIN_THREADS + tid;
   int4 v[NV];
   unsigned mx = 0;
@@ -2860,13 +2858,9 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (p.epi_mode == EPI_KNOWN_B) {
-    // programmatic dependent launch: the launch latency of the follow-up overlaps the first pass
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
-  }
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (see niti_enter)
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = 2;
   const int units = tc_units<CTAS>(ctx);
   long long grid = (p.items < units ? p.items : units) * CTAS;
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
@@ -2983,18 +2977,8 @@ static int launch_finish(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, lon
   long long blocks = (nvec + FIN_THREADS - 1) / FIN_THREADS;
   if (blocks > most) blocks = most;
   const long long per = (nvec + blocks * FIN_THREADS - 1) / (blocks * FIN_THREADS);
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
-  cfg.blockDim = dim3(FIN_THREADS, 1, 1);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // (its launch overlaps the multiply)
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   auto go = [&](auto kernel) {
-    return cudaLaunchKernelEx(&cfg, kernel, acc, (int)nvec, hdr, splits, ctx->d_status, r.out, r.update_w, r.mask, r.relu, r.mbits,
+    return niti_launch(st, (unsigned)blocks, FIN_THREADS, 0, kernel, acc, (int)nvec, hdr, splits, ctx->d_status, r.out, r.update_w, r.mask, r.relu, r.mbits,
                               r.round_mode, r.s_a, r.s_w, r.s_out, r.b_out);
   };
   NITI_CUDA_TRY(ctx, per <= 1 ? go(finish_split_kernel<1>) : per <= 2 ? go(finish_split_kernel<2>)
