@@ -2276,6 +2276,15 @@ static int pick_bn(long long gn) {
 // Contractions up to this length run on single CTAs, deeper ones on CTA pairs (see niti_tc_gemm's choice of a plan).
 constexpr long long PAIR_MIN_K = 1152;
 
+// The same for an operand that is staged with its columns contiguous (errors and weight gradients): chunks of at least 64
+// columns, because 96 are staged as 32-byte rows.  Wide swizzles pay in deep contractions, where the operand copies and the
+// shared-memory reads are the bound (error of a 5 x 5 layer with 96 input channels 81.8 -> 71.8 us, weight gradient with
+// 160 channels at 28 x 28 33.4 -> 29.7 us); in short ones the wider accumulator only costs the epilogue (16.6 -> 17.7 us).
+static int pick_bn_mn(long long gn, long long gk) {
+  const int w = pick_bn(gn);
+  return w > 64 && gk > PAIR_MIN_K ? (w + 63) / 64 * 64 : w;
+}
+
 // Builds params and maps; returns false if the shape is not eligible for this engine.
 // `aligned`: output (and mask) pointers and rows are 32-byte aligned.
 // force_bn: column tile of an unsplit one-wave plan (see pick_one_wave), 0 for the planner's own choice, -1 for that
@@ -2319,7 +2328,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
     case GK_FC_DGRAD: {   // out [M][K'], contraction over N
       p.kdepth = pick_swizzle(g.gk);
       b_mn = 1;
-      p.bn = force_bn > 0 ? force_bn : pick_bn(g.gn);
+      p.bn = force_bn > 0 ? force_bn : pick_bn_mn(g.gn, g.gk);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       a_sw = p.kdepth;
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gk), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
@@ -2334,7 +2343,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       a_mn = b_mn = 1;
       a_sw = pick_swizzle(g.gm);
       p.kdepth = pick_swizzle(g.gk);
-      p.bn = force_bn > 0 ? force_bn : pick_bn(g.gn);
+      p.bn = force_bn > 0 ? force_bn : pick_bn_mn(g.gn, g.gk);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       const cuuint64_t ld0 = (cuuint64_t)(g.ld0 ? g.ld0 : g.gm), ld1 = (cuuint64_t)(g.ld1 ? g.ld1 : g.gn);
       sa = {2, {(cuuint64_t)g.gm, (cuuint64_t)g.gk}, {ld0}, {(cuuint32_t)a_sw, (cuuint32_t)p.kdepth}, a_sw, q0};
@@ -2411,7 +2420,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.b_tiles = (g.B + p.Bt - 1) / p.Bt;
       m_tiles = (long long)p.w_tiles * p.h_tiles * p.b_tiles;
       if (p.i2c) m_tiles = (m_tiles + BM - 1) / BM;
-      p.bn = force_bn > 0 ? force_bn : pick_bn(Cn);
+      p.bn = force_bn > 0 ? force_bn : fwd ? pick_bn(Cn) : pick_bn_mn(Cn, g.gk);
       if (fwd && ctas == 2 && Cn > 256 && force_bn <= 0) {
         // Whole waves: with 256-wide tiles the 14 x 14 layers are 98 tile pairs on 74 pairs of SMs, two
         // waves of which the second is a third full; 192-wide tiles make 147 items, two full waves.
@@ -2556,7 +2565,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.PW = g.Wo; p.PH = g.Ho; p.PB = g.B;
       p.R = g.R; p.S = g.S; p.pad = g.pad;
       p.Cn = g.Ci;
-      p.bn = force_bn > 0 ? force_bn : pick_bn(g.Ci);
+      p.bn = force_bn > 0 ? force_bn : pick_bn_mn(g.Ci, g.gk);
       b_sw = pick_swizzle_mn(p.bn / ctas);
       p.n_chunks = (g.Ci + p.bn - 1) / p.bn;
       p.tg = 1;
