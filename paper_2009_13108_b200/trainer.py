@@ -80,6 +80,7 @@ class NitiTrainer:
         # backward buffers: two ping-pong error buffers and one gradient buffer
         self.e_buf = [torch.empty(max_act, **i8), torch.empty(max_act, **i8)]
         self.g_buf = torch.empty(max_w, **i8)
+        self._e_views = {}                 # views of the error buffers by (buffer, shape)
         self.b_e = [niti.scalar(-1) for _ in net.layers]
         self.b_g = [niti.scalar(-1) for _ in net.layers]
         self.b_loss = niti.scalar()
@@ -160,6 +161,14 @@ class NitiTrainer:
             n *= d
         return buf[:n].view(shape)
 
+    def _e_view(self, k, shape):
+        """Error buffer k as `shape`.  (A fresh view costs the host 2 - 3 us, 16 of them 30 us of an eager step of a
+        four-layer network that the GPU computes in 190 us.)"""
+        v = self._e_views.get((k, shape))
+        if v is None:
+            v = self._e_views[k, shape] = self._view(self.e_buf[k], shape)
+        return v
+
     def forward(self):
         n, net = self.n, self.net
         a, s = self.x, self.s_in
@@ -180,7 +189,7 @@ class NitiTrainer:
                 s = self.s_act[li]
                 wi += 1
             elif L["op"] == "fc":
-                n.linear_fwd(a.reshape(a.shape[0], -1), s, self.weights[wi], self.s_w[li], out=out,
+                n.linear_fwd(a if a.dim() == 2 else a.reshape(a.shape[0], -1), s, self.weights[wi], self.s_w[li], out=out,
                              s_out=self.s_act[li], b_out=self.b_fwd[li], relu=L["relu"],
                              round_mode=self.round_mode)
                 s = self.s_act[li]
@@ -198,10 +207,10 @@ class NitiTrainer:
     def step(self):
         """Forward, integer loss gradient, backward with in-place weight update."""
         n, net = self.n, self.net
-        n.begin_step()                     # one memset instead of one per multiply (the workspace is sized by then)
+        n.begin_step()                     # one clear instead of one per multiply (the workspace is sized by then)
         logits, s_out = self.forward()
         cur = 0
-        e = self._view(self.e_buf[cur], logits.shape)
+        e = self._e_view(cur, logits.shape)
         n.int_xent(logits, s_out, self.labels, e=e, b_e=self.b_loss, n_correct=self.n_correct,
                    round_mode=self.round_mode)
         wi = len(self.weights)
@@ -209,13 +218,13 @@ class NitiTrainer:
             L = net.layers[li]
             a_in = self.x if li == 0 else self.acts[li - 1]
             if L["op"] == "pool":
-                nxt = self._view(self.e_buf[cur ^ 1], a_in.shape)
+                nxt = self._e_view(cur ^ 1, a_in.shape)
                 relu = bool(li > 0 and net.layers[li - 1].get("relu"))
                 if self.pool_idx[li] is not None:
-                    n.maxpool2_bwd_idx(e.view(self.acts[li].shape), self.pool_idx[li], a_in.shape, e_in=nxt,
+                    n.maxpool2_bwd_idx(self._e_view(cur, self.acts[li].shape), self.pool_idx[li], a_in.shape, e_in=nxt,
                                        relu=relu)
                 else:
-                    n.maxpool2_bwd(a_in, e.view(self.acts[li].shape), e_in=nxt, relu=relu)
+                    n.maxpool2_bwd(a_in, self._e_view(cur, self.acts[li].shape), e_in=nxt, relu=relu)
                 e, cur = nxt, cur ^ 1
                 continue
             wi -= 1
@@ -224,10 +233,10 @@ class NitiTrainer:
             mask = None
             if need_e and net.layers[li - 1]["op"] != "pool" and net.layers[li - 1].get("relu"):
                 mask = a_in
-            g = self._view(self.g_buf, w.shape)
-            nxt = self._view(self.e_buf[cur ^ 1], a_in.shape) if need_e else None
+            g = None if self.fused_update else self._view(self.g_buf, w.shape)
+            nxt = self._e_view(cur ^ 1, a_in.shape) if need_e else None
             if L["op"] == "conv":
-                ev = e.view(self.acts[li].shape)
+                ev = self._e_view(cur, self.acts[li].shape)
                 if self.fused_update:
                     if need_e:                     # from the weights as they are before the update
                         n.conv_dgrad(ev, w, a_in.shape[1:3], e_prev=nxt, relu_mask_src=mask,
@@ -242,15 +251,16 @@ class NitiTrainer:
                                      b_e=self.b_e[li], pad=1, round_mode=self.round_mode)
                     n.int_sgd_update(w, g)
             else:
-                a2 = a_in.reshape(a_in.shape[0], -1)
+                a2 = a_in if a_in.dim() == 2 else a_in.reshape(a_in.shape[0], -1)
+                ev = self._e_view(cur, self.acts[li].shape)
                 kw = dict(need_e_prev=need_e,
-                          relu_mask_src=None if mask is None else mask.reshape(a2.shape),
-                          e_prev=None if nxt is None else nxt.view(a2.shape),
+                          relu_mask_src=None if mask is None else a2,
+                          e_prev=None if nxt is None else self._e_view(cur ^ 1, a2.shape),
                           b_e=self.b_e[li], b_g=self.b_g[li], m_u=net.m_u, round_mode=self.round_mode)
                 if self.fused_update:
-                    n.linear_bwd_update(a2, e.view(a2.shape[0], -1), w, **kw)
+                    n.linear_bwd_update(a2, ev, w, **kw)
                 else:
-                    n.linear_bwd(a2, e.view(a2.shape[0], -1), w, g=g, **kw)
+                    n.linear_bwd(a2, ev, w, g=g, **kw)
                     n.int_sgd_update(w, g)
             if need_e:
                 e, cur = nxt, cur ^ 1
