@@ -116,7 +116,7 @@ size_t niti_workspace_bytes(int op, const int64_t *dims, int ndims);
  * value. */
 int niti_set_engine(niti_ctx *ctx, int engine);
 
-/* Number of kernels / memsets this context has enqueued so far. */
+/* Number of kernels and memsets this context has enqueued so far. */
 uint64_t niti_launch_count(niti_ctx *ctx);
 /* Of those, launches of the tensor-core matrix-multiply kernels: tcgen05 (without the instance that computes the
  * error of strided convolutions, which only niti_launch_count() counts) and the mma.sync kernel of small fully
@@ -287,9 +287,9 @@ int niti_linear_bwd_update(niti_ctx *ctx, void *stream, const int8_t *a, const i
 typedef int (*niti_reduce_fn)(void *user, void *stream, void *dev_ptr, int64_t count, int kind);
 int niti_set_reduce_hook(niti_ctx *ctx, niti_reduce_fn fn, void *user);
 /* Optional, once per training step (or per group of at most 64 calls): clears every header of the
- * workspace `ws` with one memset on `stream`.  The calls that follow on that workspace (in stream
+ * workspace `ws` with one launch on `stream`.  The calls that follow on that workspace (in stream
  * order, from this context) then take one zeroed header each instead of clearing their own, which
- * removes a memset node from in front of every multiply of the step.  After 64 calls, or for any other
+ * removes a clear from in front of every multiply of the step.  After 64 calls, or for any other
  * workspace, calls clear their header themselves as they do without this call.  The caller must not
  * use that workspace from two streams at once (as for any workspace) and must call niti_begin_step
  * again before the pattern repeats (each training step; a captured CUDA graph holds it as its first

@@ -197,7 +197,7 @@ class Niti:
             self._ws = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
 
     def begin_step(self):
-        """niti_begin_step on this object's workspace: one memset clears the headers that the next 64
+        """niti_begin_step on this object's workspace: one launch clears the headers that the next 64
         calls would otherwise clear one by one."""
         self._ck(self.lib.niti_begin_step(self.h, self._stream(), self._ws.data_ptr(), self._ws.numel()))
 

@@ -135,7 +135,7 @@ static inline cudaError_t niti_launch(cudaStream_t st, dim3 grid, dim3 block, si
 
 // A header for the call that is being enqueued: the next unused one of a workspace prepared by niti_begin_step()
 // (zeroed already), else the last one, which niti_clear() has to clear before the call's first kernel.  The last one
-// ends where the accumulators begin, so that a split contraction clears both with one memset.
+// ends where the accumulators begin, so that a split contraction clears both with one launch.
 static inline WsHeader *niti_take_header(niti_ctx *ctx, void *ws) {
   char *base = reinterpret_cast<char *>(ws);
   if (ws == ctx->step_ws && ctx->step_slot < NITI_HDR_SLOTS) {
