@@ -18,10 +18,18 @@ static inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 // runs as a plain K = 32 matrix multiply.
 static inline bool few_channel_conv(int Ci, int R, int S) { return R * S * Ci <= 32 && (Ci % 16) != 0; }
 
+// A forward pass or weight gradient with a stride above 8 has no operand copies on the tensor-core engine (the traversal
+// stride of a copy ends there): the CUDA-core engine reads the caller's tensors, nothing is widened or padded for it.
+static inline bool copies_refused(const GemmProblem &p) {
+  return (p.kind == GK_CONV_FWD || p.kind == GK_CONV_WGRAD) && p.stride > 8;
+}
+
 // With more taps nothing is gathered: a tap row of a window is S * Ci contiguous bytes of an image row.  Pixels are
 // widened to Cp bytes (4, 8 or 16: stride * Cp has to be a multiple of the 16 bytes that TMA strides are made of)
 // and image rows get their zero padding, and then the layer is a convolution with R x 1 taps over Wo "pixels" per
 // row that lie stride * Cp bytes apart and have S * Cp channels: windows that overlap in memory.
+//
+// The workspace query and the calls decide by the same rules here: what a call copies is what the query has room for.
 struct WindowGeometry {
   int Cp;                  // bytes per widened pixel, 0: the layer is not run this way
   int row_bytes;           // of a widened image row
@@ -31,12 +39,16 @@ struct WindowGeometry {
 static WindowGeometry window_geometry(const GemmProblem &p) {
   WindowGeometry g;
   memset(&g, 0, sizeof(g));
-  if (p.Ci >= 16 || few_channel_conv(p.Ci, p.R, p.S) || p.kind == GK_CONV_DGRAD) return g;
+  if (p.Ci >= 16 || few_channel_conv(p.Ci, p.R, p.S) || p.kind == GK_CONV_DGRAD || copies_refused(p)) return g;
+  // (the box of base pixels that an im2col copy walks starts and ends within 128 rows of the image's)
+  if (p.pad > 127 || p.R - 1 - p.pad > 128) return g;
   int cp = 4;
   while (cp < p.Ci || (p.stride * cp) % 16 != 0) cp *= 2;
   if (cp > 16) return g;
+  const long long row_bytes = (((p.Wo - 1LL) * p.stride + p.S) * cp + 15) / 16 * 16;
+  if ((long long)p.B * p.H * (row_bytes / 16) >= (1LL << 31)) return g;       // (the widening kernel counts in 32 bits)
   g.Cp = cp;
-  g.row_bytes = (((p.Wo - 1) * p.stride + p.S) * cp + 15) / 16 * 16;
+  g.row_bytes = (int)row_bytes;
   g.chans = p.S * cp;
   g.pitch = (g.chans + 15) / 16 * 16;
   g.x_bytes = round_up((size_t)p.B * p.H * g.row_bytes, 256);
@@ -78,13 +90,14 @@ static size_t pad_bytes(const GemmProblem &p, int which) {
   return o.width % 16 == 0 ? 0 : round_up((size_t)o.rows * pitch16(o.width), 256);
 }
 static size_t pad_bytes(const GemmProblem &p) { return pad_bytes(p, 0) + pad_bytes(p, 1); }
-// Copies what needs padding (and is not padded yet) into `mem` (pad_bytes(p) bytes).
-static int pad_operands(niti_ctx *ctx, cudaStream_t st, GemmProblem &p, char *mem) {
+// Copies what needs padding (and is not padded yet) into `mem` (pad_bytes(p) bytes); `end`: end of the workspace.
+static int pad_operands(niti_ctx *ctx, cudaStream_t st, GemmProblem &p, char *mem, const char *end) {
   for (int which = 0; which < 2; ++which) {
     const size_t bytes = pad_bytes(p, which);
     const int8_t *&q = which == 0 ? p.q0 : p.q1;
     if (bytes && !q) {
       const OperandRows o = operand_rows(p, which);
+      if (mem + bytes > end) return niti_fail(ctx, NITI_ERR_WORKSPACE, "the workspace has no room for padded operands");
       const int rc = niti_launch_pad_pitch(ctx, st, which == 0 ? p.p0 : p.p1, (int8_t *)mem, o.rows, o.width, pitch16(o.width));
       if (rc != NITI_OK) return rc;
       q = (int8_t *)mem;
@@ -358,7 +371,7 @@ extern "C" size_t niti_workspace_bytes(int op, const int64_t *d, int nd) {
         const size_t M = (size_t)d[0] * p.Ho * p.Wo;
         extra = round_up(M * 32, 256) + round_up((size_t)d[4] * 32, 256) + round_up((size_t)d[4] * 32 * 4, 256);
         if (op == NITI_OP_CONV_WGRAD) extra += pad_bytes(p, 0);           // e with padded pixels
-      } else {
+      } else if (!copies_refused(p)) {
         extra = pad_bytes(p);
       }
       if (upd) extra = round_up(extra, 256) + round_up((size_t)(p.gm * p.gn), 256);             // scratch gradient
@@ -417,26 +430,28 @@ int niti_reduce_after_gemm(niti_ctx *ctx, cudaStream_t st, int kind, int32_t *ac
 int niti_launch_maxpool2_fwd(niti_ctx *ctx, cudaStream_t st, const int8_t *x, int8_t *y, int B, int H, int W, int C);
 
 // tc_form: the problem in the form the tensor-core engine takes (operands prepared), where that is another one.
-// pad_mem: scratch for operands whose rows have to be padded (pad_bytes(p)).
+// pad_mem: scratch for operands whose rows have to be padded (pad_bytes(p)).  tc_refused: the tensor-core engine has
+// refused the problem already (nothing is padded for it).
 static int run_gemm_round(niti_ctx *ctx, cudaStream_t st, GemmProblem p, void *ws, size_t ws_bytes,
                           size_t need, char *pad_mem, int8_t *out, int mbits, int round_mode, int relu,
                           const int8_t *mask, const int32_t *s_a, const int32_t *s_w, int32_t *s_out,
                           int32_t *b_out, int8_t *update_w = nullptr, int8_t *pool_out = nullptr,
-                          const GemmProblem *tc_form = nullptr) {
+                          const GemmProblem *tc_form = nullptr, bool tc_refused = false) {
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
   WsHeader *hdr = niti_take_header(ctx, ws);
   int32_t *acc = (int32_t *)((char *)ws + NITI_WS_HEADER);
   int rc = NITI_OK;
   const bool narrow = p.kind <= GK_FC_WGRAD && p.N < 32 && p.kind != GK_FC_FWD;       // (the CUDA-core engine's)
-  if (rc == NITI_OK && ctx->engine != 1 && !narrow && !tc_form) rc = pad_operands(ctx, st, p, pad_mem);
+  const bool tc = ctx->engine != 1 && !tc_refused && !copies_refused(p);
+  if (tc && !narrow && !tc_form) rc = pad_operands(ctx, st, p, pad_mem, (const char *)ws + need);
   if (rc != NITI_OK) return rc;
   rc = NITI_ERR_SHAPE;
   bool fused = false;
   bool pooled = false;
   bool updated = false;
   RoundSpec rs = {out, mask, mbits, round_mode, relu, s_a, s_w, s_out, b_out, pool_out, update_w};
-  if (ctx->engine != 1) rc = niti_tc_gemm(ctx, st, tc_form ? *tc_form : p, rs, acc, hdr, &fused, &pooled, true, &updated);
+  if (tc) rc = niti_tc_gemm(ctx, st, tc_form ? *tc_form : p, rs, acc, hdr, &fused, &pooled, true, &updated);
   if (rc == NITI_ERR_SHAPE) {
     rc = niti_simt_gemm(ctx, st, p, acc, hdr);
     if (rc == NITI_OK) rc = niti_reduce_after_gemm(ctx, st, p.kind, acc, p.gm * p.gn, hdr, true);
@@ -703,7 +718,8 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
   if (update_w) g = (int8_t *)((char *)ws + need_base);       // scratch, used only where the rounding stores int8
   const WindowGeometry wg = window_geometry(p);
-  if ((wg.Cp || few_channel_conv(Cin, R, S)) && ctx->engine != 1) {
+  const bool own_form = (wg.Cp || few_channel_conv(Cin, R, S)) && ctx->engine != 1;
+  if (own_form) {
     // the multiply leaves int32 sums over widened windows (columns r, s * Cp + c) or over gathered 32-byte rows; the
     // columns that are taps are then rounded into g, or subtracted from the weights
     cudaStream_t st = (cudaStream_t)stream;
@@ -728,7 +744,7 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
       q.p0 = e; q.p1 = xcol;
     }
     if (rc != NITI_OK) return rc;
-    rc = pad_operands(ctx, st, q, pad_mem);
+    rc = pad_operands(ctx, st, q, pad_mem, (const char *)ws + need_base);
     if (rc != NITI_OK) return rc;
     bool fused = false;
     RoundSpec none = {nullptr, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -743,7 +759,7 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
     if (rc != NITI_ERR_SHAPE) return rc;
   }
   return run_gemm_round(ctx, (cudaStream_t)stream, p, ws, ws_bytes, need, conv_pad_mem(p, ws), g, m_u, round_mode, 0, nullptr,
-                        nullptr, nullptr, nullptr, b_g, update_w);
+                        nullptr, nullptr, nullptr, b_g, update_w, nullptr, nullptr, own_form);
 }
 
 extern "C" int niti_conv_wgrad_strided(niti_ctx *ctx, void *stream, const int8_t *x, const int8_t *e, int8_t *g,
