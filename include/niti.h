@@ -111,8 +111,10 @@ size_t niti_workspace_bytes(int op, const int64_t *dims, int ndims);
  * (falls back to CUDA cores where that kernel does not apply), 4 = tensor
  * cores with the two-pass epilogue (int32 accumulators spilled to the
  * workspace, rounded by a second kernel) instead of the fused one, 5 = tensor
- * cores without the weights-resident mode of small-channel 3x3 convolutions.
- * 1-5 exist so that tests can cross-check the engines.  Returns the previous
+ * cores without the weights-resident mode of small-channel 3x3 convolutions,
+ * 6 = automatic, but blocks that would wait for other blocks of their launch
+ * leave their share to a later one at once.
+ * 1-6 exist so that tests can cross-check the engines.  Returns the previous
  * value. */
 int niti_set_engine(niti_ctx *ctx, int engine);
 

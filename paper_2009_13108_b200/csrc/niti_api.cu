@@ -129,6 +129,7 @@ extern "C" int niti_create(niti_ctx **out, int device) {
     return NITI_ERR_SHAPE;
   }
   ctx->smem_optin = (size_t)smem_optin;
+  ctx->patience = NITI_PATIENCE;
   // one allocation: the status words, then the table of speculative-estimate errors
   const size_t dev_bytes = 256 + sizeof(int32_t) * 2 * NITI_SPEC_SLOTS;
   e = cudaMalloc(&ctx->d_status, dev_bytes);
@@ -167,8 +168,9 @@ extern "C" const char *niti_last_error(niti_ctx *ctx) { return ctx ? ctx->err : 
 
 extern "C" int niti_set_engine(niti_ctx *ctx, int engine) {
   if (!ctx) return -1;
-  int old = ctx->engine;
-  ctx->engine = engine;
+  const int old = ctx->patience ? ctx->engine : 6;
+  ctx->engine = engine == 6 ? 0 : engine;
+  ctx->patience = engine == 6 ? 0u : NITI_PATIENCE;
   return old;
 }
 
@@ -310,9 +312,10 @@ static bool fill_conv(GemmProblem &p, int kind, int B, int H, int W, int Ci, int
 }
 
 // int32 elements of the accumulator scratch of a fully connected backward call: the larger of the weight
-// gradient [N][K] and the error [M][K]
+// gradient [N][K] and the error [M][K], both where one launch may run both multiplies
 static size_t linear_bwd_acc_elems(long long M, long long N, long long K) {
   const size_t a = (size_t)(M * K), b = (size_t)(N * K);
+  if ((double)M * N * K <= NITI_SMALL_MACS * NITI_SMALL_NARROW) return a + b;
   return a > b ? a : b;
 }
 

@@ -47,12 +47,13 @@ struct niti_ctx {
   // per-device facts of the tensor-core kernel, indexed by CTAs per tile (1 or 2): co-resident CTAs /
   // CTA pairs (0 = not asked yet) and the dynamic shared-memory limit already set on the kernel
   int tc_units[3];
-  size_t tc_attr_smem[7];   // CTAs + 2 * mode of the instance
+  size_t tc_attr_smem[13];  // CTAs + 2 * mode + 6 * one of the instance
   // the device's opt-in limit of dynamic shared memory per CTA.  The limit set on a kernel belongs to the
   // device, not to a context: every context therefore sets this same value (a context that set only what it
   // needed would lower the limit under another context of the process)
   size_t smem_optin;
   int small_ready;          // attributes of the small-multiply kernel are set
+  unsigned patience;        // cycles that the blocks of a launch wait for each other (NITI_PATIENCE; 0: test switch)
 };
 
 
@@ -79,7 +80,7 @@ struct niti_ctx {
 // Scalars at the start of a workspace.
 struct WsHeader {
   unsigned int maxabs32;            // a value with the bit length of max |acc| (a max, or an OR of magnitudes)
-  unsigned int unused;
+  unsigned int arrived;             // agreement of a launch's blocks: low half blocks that have come, high half that left
   unsigned long long maxabs64;      // same for the 64-bit loss accumulators
   // the three words of the speculative agreement share one 16-byte line so that one load polls them all
   unsigned int est_max;             // max |acc| over the first tile of the CTAs that have reported
@@ -211,19 +212,32 @@ __device__ __forceinline__ unsigned niti_load_bytes4(const int8_t *p, int n) {
   return n >= 4 ? v : v & (0xffffffffu >> (32 - 8 * n));
 }
 
-// Maximum over n CTAs (at most NITI_AGREE_MAX), plus one, for one converged warp of every CTA; 0: gave up (`late()` said
-// so).  Words [0, n) of the area take what the CTAs post.  Up to NITI_AGREE_DIRECT CTAs all poll all words; with more, the
-// first CTA alone does and answers into a mailbox of 16 bytes per CTA that only that CTA polls, because the reads of a few
-// L2 lines by everybody delay the posts (3100 cycles for 64 CTAs, 6000 - 8000 for 128; one call with 98 CTAs 12.0 -> 10.5
-// us, with 64 14.1 -> 13.0 us, with 144 16.0 -> 13.7 us; with 16 6.9 us directly, 7.5 us through mailboxes).  `extra` more
-// words in front of the area have to be posted first.
+// Agreement of the blocks of one launch on the bit-width of a tensor of which every block holds a share: the largest bit
+// length over n blocks (at most NITI_AGREE_MAX), plus one, for one converged warp of every block; 0: the block ran out of
+// patience and has to leave.  Words [0, n) of the area take what the blocks post.  Up to NITI_AGREE_DIRECT CTAs all poll all
+// words; with more, the first CTA alone does and answers into a mailbox of 16 bytes per CTA that only that CTA polls, because
+// the reads of a few L2 lines by everybody delay the posts (3100 cycles for 64 CTAs, 6000 - 8000 for 128; one call with 98
+// CTAs 12.0 -> 10.5 us, with 64 14.1 -> 13.0 us, with 144 16.0 -> 13.7 us; with 16 6.9 us directly, 7.5 us through
+// mailboxes).  `extra` more words in front of the area have to be posted first.
+//
+// Nothing promises that all blocks of a launch are on the GPU at the same time: launches of two streams can each hold a part
+// of the SMs.  So no block waits until all have come.  Out of patience, it leaves its sums in memory, marks its post, counts
+// itself as left and exits, which frees its SM for the blocks that are still to come (niti_finish_left).  Arrivals and
+// departures are counted in one word, whose order decides who finishes the share of a block that left: the block itself
+// when all had arrived by then, else the block that arrived last.  (A cooperative launch would promise residency; it cost
+// every launch of a call-by-call program 1.3 us of host time: head of 4096 x 1000 x 512 66.1 -> 72.9 us, eager CNN step of
+// 37 launches 169 -> 187 us, one 256^3 multiply 7.8 -> 8.5 us, a captured MLP step 43.2 -> 45.0 us.)
 #define NITI_AGREE_MAX 160
 #define NITI_AGREE_DIRECT 48
 #define NITI_AGREE_WORDS (5 * NITI_AGREE_MAX)      // posts, then mailboxes
-template <typename Late>
-__device__ __forceinline__ unsigned niti_agree_max(unsigned *posts, unsigned *mail, unsigned mine, int cta, int n, int extra,
-                                                   int lane, Late late) {
-  if (lane == 0) *(volatile unsigned *)(posts + cta) = mine + 1u;
+#define NITI_LEFT 0x10000u                         // mark in a post: its block left its share in memory
+#define NITI_PATIENCE (1u << 19)                   // about 0.3 ms; the blocks of an undisturbed launch post within a few us
+__device__ __forceinline__ unsigned niti_agree_bits(unsigned *posts, unsigned *mail, int bits, int cta, int n, int extra, int lane,
+                                                    unsigned patience) {
+  if (lane == 0) *(volatile unsigned *)(posts + cta) = (unsigned)bits + 1u;
+  if (patience == 0u && (cta & 1)) return 0u;      // (test switch: every other block leaves, whoever has come)
+  const long long t0 = clock64();
+  auto late = [&]() { return __any_sync(0xffffffffu, clock64() - t0 > (long long)patience) != 0; };
   if (cta == 0 || n <= NITI_AGREE_DIRECT) {
     unsigned m;
     while (true) {
@@ -239,7 +253,7 @@ __device__ __forceinline__ unsigned niti_agree_max(unsigned *posts, unsigned *ma
       for (int u = 0; u < 5; ++u) {
         const int i = 32 * u + lane - extra;
         seen = seen && w[u] != 0;
-        if (i >= 0 && i < n) m = max(m, w[u]);
+        if (i >= 0 && i < n) m = max(m, w[u] & (NITI_LEFT - 1u));
       }
       if (__all_sync(0xffffffffu, seen)) break;
       if (late()) return 0u;
@@ -255,6 +269,55 @@ __device__ __forceinline__ unsigned niti_agree_max(unsigned *posts, unsigned *ma
     m = __shfl_sync(0xffffffffu, m, 0);
     if (m) return m;
     if (late()) return 0u;
+  }
+}
+// The same maximum when all n blocks have arrived: each of them posts without waiting for another.
+__device__ __forceinline__ unsigned niti_posted_bits(unsigned *posts, int n, uint32_t *status) {
+  unsigned m = 0;
+  const long long t0 = clock64();
+  for (int i = (int)(threadIdx.x & 31); i < n; i += 32) {
+    unsigned w;
+    while (!(w = *(volatile unsigned *)(posts + i)))
+      if (clock64() - t0 > 2000000000LL) {
+        atomicOr(status, NITI_DEV_TIMEOUT);
+        break;
+      }
+    m = max(m, w & (NITI_LEFT - 1u));
+  }
+  __syncwarp();
+  return __reduce_max_sync(0xffffffffu, m);
+}
+// At the start of every block of such a launch, by one thread, for niti_finish_left.
+__device__ __forceinline__ unsigned niti_arrive(WsHeader *hdr) { return atomicAdd(&hdr->arrived, 1u); }
+// The end of every block of such a launch, by all its threads: after its own output is stored, or (`left`) after its share
+// is in memory.  `ticket`: from niti_arrive, `posts`: of the whole grid.  finish(j) completes the share of block j, which
+// left, and is called for every such block by exactly one block.
+template <typename Finish>
+__device__ __forceinline__ void niti_finish_left(WsHeader *hdr, unsigned *posts, bool left, unsigned ticket, Finish finish) {
+  const unsigned n = gridDim.x;
+  __shared__ unsigned claimed;
+  bool look = (ticket & 0xffffu) == n - 1u && (ticket >> 16) != 0;              // the last to arrive, and some had left
+  if (left) {
+    __threadfence();                               // (each thread's part of the share)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      atomicOr(posts + blockIdx.x, NITI_LEFT);
+      __threadfence();
+      claimed = (atomicAdd(&hdr->arrived, 0x10000u) & 0xffffu) == n ? 1u : 0u;  // (nobody else looks at this block then)
+    }
+    __syncthreads();
+    look = look || claimed != 0;
+  }
+  if (!look) return;
+  __threadfence();
+  for (unsigned j = 0; j < n; ++j) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      claimed = (*(volatile unsigned *)(posts + j) & NITI_LEFT) && (atomicAnd(posts + j, ~NITI_LEFT) & NITI_LEFT) ? 1u : 0u;
+      __threadfence();
+    }
+    __syncthreads();
+    if (claimed) finish((int)j);
   }
 }
 
@@ -336,6 +399,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &p, const Rou
 // Small fully connected multiplies, one launch for one (g2 == null) or both multiplies of a backward call;
 // NITI_ERR_SHAPE when the problem is not small (nothing was enqueued).
 #define NITI_SMALL_MACS 200.0e6
+#define NITI_SMALL_NARROW 4                        // times that for layers of fewer than 32 outputs, backward
 int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem &g, const RoundSpec &r,
                     const GemmProblem *g2, const RoundSpec *r2);
 

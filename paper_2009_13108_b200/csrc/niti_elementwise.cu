@@ -581,12 +581,13 @@ template <bool PACKED, bool ONE>
 struct XentBlock {
   XentSweep<PACKED, ONE> held;
   XentRow mine;
-  int label;
-  __device__ __forceinline__ static long long first_row() {
-    return (long long)blockIdx.x * ((int)blockDim.x >> 5) + (threadIdx.x >> 5);
+  int label, blk;
+  __device__ __forceinline__ static long long first_row_of(int block) {
+    return (long long)block * ((int)blockDim.x >> 5) + (threadIdx.x >> 5);
   }
-  __device__ __forceinline__ XentBlock(const int8_t *__restrict__ a, const int32_t *__restrict__ labels, int B, int N)
-      : held(a + first_row() * N, ONE && first_row() < B ? (PACKED ? N >> 2 : N) : 0, (int)threadIdx.x & 31) {
+  __device__ __forceinline__ long long first_row() const { return first_row_of(blk); }
+  __device__ __forceinline__ XentBlock(const int8_t *__restrict__ a, const int32_t *__restrict__ labels, int B, int N, int block)
+      : held(a + first_row_of(block) * N, ONE && first_row_of(block) < B ? (PACKED ? N >> 2 : N) : 0, (int)threadIdx.x & 31), blk(block) {
     label = ONE && first_row() < B ? labels[first_row()] : 0;
   }
   // pass 1: the 64-bit maximum and the hits of the block, in m / h of thread 0
@@ -660,7 +661,7 @@ xent_row_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_pt
   __shared__ int sh_hit[XENT_WARPS];
   unsigned long long m;
   int h;
-  XentBlock<PACKED, false> rows(a, labels, B, N);
+  XentBlock<PACKED, false> rows(a, labels, B, N, (int)blockIdx.x);
   rows.stats(a, *s_a_ptr, labels, rowinfo, B, N, status, sh_max, sh_hit, m, h);
   if (threadIdx.x == 0) {
     if (m > *(volatile unsigned long long *)&hdr->maxabs64) atomicMax(&hdr->maxabs64, m);
@@ -679,28 +680,29 @@ xent_round_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_
     if (b_out) *b_out = b;
     if (n_correct) *n_correct = (int32_t)hdr->hits;
   }
-  XentBlock<PACKED, false> rows(a, labels, B, N);
+  XentBlock<PACKED, false> rows(a, labels, B, N, (int)blockIdx.x);
   rows.outs(a, *s_a_ptr, labels, rowinfo, out, B, N, bp, round_mode, q_tab);
 }
 
-// Both passes in one launch of at most one block per SM, all resident: the blocks agree on the bit-width in between.
+// Both passes in one launch of at most one block per SM: the blocks agree on the bit-width in between.
 // Bound: latency (a launch, one round trip for the logits, the agreement); with many rows per SM the arithmetic of pass 1.
 // Two launches, of which the second reads labels, scalars and logits again, took 7.7 / 9.8 us for 64 x 1000 logits (Eq. 2 /
 // Eq. 4), four with tables of all 256 offsets 13.0 / 16.8 us for 4096 x 1000 (and 29 us with their gaps outside a graph);
 // one launch takes 4.7 / 5.5 and 9.2 / 11.5 us, 64 x 10 3.5 / 3.9 instead of 3.5 / 4.7 us.
 constexpr int XENT_MAX_WARPS = 32;
-constexpr long long XENT_WAIT_CYCLES = 2000000000LL;
 template <bool PACKED, bool ONE, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS)
 xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
             long long *rowinfo, WsHeader *hdr, int8_t *__restrict__ out, int B, int N, int round_mode, int32_t *__restrict__ b_out,
-            int32_t *__restrict__ n_correct, uint32_t *__restrict__ status) {
+            int32_t *__restrict__ n_correct, uint32_t *__restrict__ status, unsigned patience) {
   niti_enter(a, s_a_ptr, labels);
   __shared__ unsigned long long sh_max[WARPS];
   __shared__ int sh_hit[WARPS];
-  __shared__ unsigned blk_b, grid_b;
+  __shared__ unsigned blk_b, grid_b, ticket;
   __shared__ unsigned char q_tab[256 * (WARPS + 1)];
-  XentBlock<PACKED, ONE> rows(a, labels, B, N);
+  unsigned came = 0;
+  if (threadIdx.x == 32 && gridDim.x > 1) came = niti_arrive(hdr);
+  XentBlock<PACKED, ONE> rows(a, labels, B, N, (int)blockIdx.x);
   const int s = *s_a_ptr;
   unsigned long long m;
   int h;
@@ -715,37 +717,48 @@ xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, c
       __threadfence();
     }
   }
+  unsigned *words = niti_split_max(hdr);
   if (gridDim.x > 1 && threadIdx.x < 32) {
-    const int lane = threadIdx.x;
     __syncwarp();
-    unsigned *words = niti_split_max(hdr);
-    const long long c0 = clock64();
-    const unsigned all = niti_agree_max(words, words + NITI_AGREE_MAX, *(volatile unsigned *)&blk_b, (int)blockIdx.x, (int)gridDim.x, 0, lane, [&]() {
-      const bool late = __any_sync(0xffffffffu, clock64() - c0 > XENT_WAIT_CYCLES);
-      if (late && lane == 0) atomicOr(status, NITI_DEV_TIMEOUT);
-      return late;
-    });
-    if (lane == 0) {
-      grid_b = all;
-      if (blockIdx.x == 0 && n_correct && all) {            // (the first block has seen every post, and thereby every hit)
-        __threadfence();
-        *n_correct = (int32_t)*(volatile unsigned *)&hdr->hits;
-      }
-    }
+    const unsigned all = niti_agree_bits(words, words + NITI_AGREE_MAX, (int)*(volatile unsigned *)&blk_b, (int)blockIdx.x,
+                                         (int)gridDim.x, 0, (int)threadIdx.x, patience);
+    if (threadIdx.x == 0) grid_b = all;
   }
+  if (threadIdx.x == 32) ticket = came;
   __syncthreads();
-  if (grid_b == 0) return;                                  // (gave up waiting)
-  const int b = (int)grid_b - 1, bp = b > 7 ? b - 7 : 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && b_out) *b_out = b;
-  rows.outs(a, s, labels, rowinfo, out, B, N, bp, round_mode, q_tab);
+  // the scalars, by whoever rounds the first block's rows
+  auto publish = [&](int b) {
+    if (threadIdx.x != 0) return;
+    if (b_out) *b_out = b;
+    if (gridDim.x > 1 && n_correct) {                       // (every post has been seen, and thereby every hit)
+      __threadfence();
+      *n_correct = (int32_t)*(volatile unsigned *)&hdr->hits;
+    }
+  };
+  const unsigned agreed = grid_b, came_as = ticket;
+  if (agreed) {
+    const int b = (int)agreed - 1;
+    if (blockIdx.x == 0) publish(b);
+    rows.outs(a, s, labels, rowinfo, out, B, N, b > 7 ? b - 7 : 0, round_mode, q_tab);
+  }
+  if (gridDim.x == 1 || (agreed && !(came_as >> 16))) return;
+  niti_finish_left(hdr, words, agreed == 0, came_as, [&](int j) {
+    const unsigned bits = niti_posted_bits(words, (int)gridDim.x, status);
+    if (bits == 0) return;
+    const int b = (int)bits - 1;
+    if (j == 0) publish(b);
+    XentBlock<PACKED, ONE> left(a, labels, B, N, j);
+    if (ONE) left.stats(a, s, labels, rowinfo, B, N, status, sh_max, sh_hit, m, h);      // (the others' are in memory)
+    left.outs(a, s, labels, rowinfo, out, B, N, b > 7 ? b - 7 : 0, round_mode, q_tab);
+  });
 }
 
 template <bool PACKED, bool ONE>
 static void launch_xent_one(int grid, int warps, cudaStream_t st, const int8_t *a, const int32_t *s_a, const int32_t *labels,
                             long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N, int round_mode,
-                            uint32_t *status) {
+                            uint32_t *status, unsigned patience) {
   auto go = [&](auto kernel) {
-    niti_launch(st, grid, 32 * warps, 0, kernel, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status);
+    niti_launch(st, grid, 32 * warps, 0, kernel, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status, patience);
   };
   if (warps == 8) go(xent_kernel<PACKED, ONE, 8>);
   else if (warps == 16) go(xent_kernel<PACKED, ONE, 16>);
@@ -765,7 +778,7 @@ static int launch_xent(niti_ctx *ctx, cudaStream_t st, const int8_t *a, const in
     const int warps = B <= 8 * sms ? 8 : B <= 16 * sms ? 16 : XENT_MAX_WARPS;
     const int need = (B + warps - 1) / warps, grid = need < sms ? need : sms;
     const bool one = (packed ? N >> 2 <= 32 * xent_held<true> : N <= 32 * xent_held<false>) && B <= grid * warps;
-    auto go = [&](auto launch) { launch(grid, warps, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status); };
+    auto go = [&](auto launch) { launch(grid, warps, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status, ctx->patience); };
     if (packed) { if (one) go(launch_xent_one<true, true>); else go(launch_xent_one<true, false>); }
     else { if (one) go(launch_xent_one<false, true>); else go(launch_xent_one<false, false>); }
     ctx->launches++;

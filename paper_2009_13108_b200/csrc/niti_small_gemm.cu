@@ -24,29 +24,30 @@ namespace {
 
 constexpr int SMALL_THREADS = 512;
 constexpr int SMALL_WARPS = SMALL_THREADS / 32;
-constexpr long long SMALL_WAIT_CYCLES = 2000000000LL;
 constexpr size_t SMALL_SMEM = 200 * 1024;
 
 // One multiply out[m][n] = sum_k A(m, k) B(n, k).  An operand is K-major (row r, element k at p[r * ld + k]) or
 // MN-major (p[k * ld + r]).
 struct SmallOp {
   const int8_t *a, *b;
-  int lda, ldb, a_mn, b_mn;
+  int lda, ldb;
   int gm, gn, gk;
   int rm, rn, cn;             // region of a CTA (multiples of 32), CTAs per row of regions
   int ctas;                   // CTAs of this multiply (0: this launch has no such multiply)
   int kc;                     // contraction elements staged at a time (multiple of 64)
+  uint8_t a_mn, b_mn, mbits, relu;
   int8_t *out;
   const int8_t *mask;         // output is zero where mask <= 0
   int8_t *upd;                // weights from which the rounded result is subtracted (out is then not written)
-  int mbits, relu;
   const int32_t *s_a, *s_w;
   int32_t *s_out, *b_out;
 };
 struct SmallParams {
   SmallOp op[2];              // op[0]: forward or error; op[1]: the weight gradient beside an error
   int round_mode;
-  unsigned *words;            // one cleared word per CTA
+  unsigned patience;
+  WsHeader *hdr;              // cleared
+  int32_t *left;              // in the workspace: sums of regions whose CTAs left, [gm][gn] of op[0], then of op[1]
   uint32_t *status;
 };
 
@@ -146,10 +147,85 @@ __device__ __forceinline__ void stage_operand(const int8_t *p, int ld, int mn, i
   }
 }
 
+// Rounds and stores the region at (m0, n0), of CTA c of its multiply, whose sums are in shared memory.
+__device__ __forceinline__ void round_region(const SmallParams &p, const SmallOp &o, const int *acc, int c, int m0, int n0,
+                                             unsigned agreed_bits) {
+  const int tid = threadIdx.x, acc_pitch = o.rn + 4;
+  const int b = (int)agreed_bits - 1, bp = b > o.mbits ? b - o.mbits : 0;
+  const unsigned qmax = (1u << o.mbits) - 1u;
+  if (c == 0 && tid == 0) {
+    if (o.b_out) *o.b_out = b;
+    if (o.s_out) {
+      const int s = bp + (o.s_a ? *o.s_a : 0) + (o.s_w ? *o.s_w : 0);
+      *o.s_out = s;
+      if (s < -128 || s > 127) atomicOr(p.status, NITI_DEV_EXP_RANGE);
+    }
+  }
+  const int q = o.rn >> 2;
+  int8_t *dst = o.upd ? o.upd : o.out;
+  const bool words_ok = (o.gn & 3) == 0 && (((uintptr_t)dst | (uintptr_t)o.mask) & 3) == 0;
+  for (int idx = tid; idx < o.rm * q; idx += SMALL_THREADS) {
+    const int r = idx / q, cc = (idx - r * q) * 4;
+    const int nv = o.gn - n0 - cc;
+    if (m0 + r >= o.gm || nv <= 0) continue;
+    const long long off = (long long)(m0 + r) * o.gn + n0 + cc;
+    const int4 v = *reinterpret_cast<const int4 *>(acc + r * acc_pitch + cc);
+    const int xs[4] = {v.x, v.y, v.z, v.w};
+    unsigned w = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      int x = niti_round_i32(xs[j], bp, qmax, p.round_mode);
+      if (o.relu && x < 0) x = 0;
+      w |= (unsigned)(x & 0xff) << (8 * j);
+    }
+    if (words_ok) {
+      if (o.mask) w &= __vcmpgts4(*reinterpret_cast<const unsigned *>(o.mask + off), 0u);
+      if (o.upd) w = __vmaxs4(__vsubss4(*reinterpret_cast<const unsigned *>(dst + off), w), 0x81818181u);
+      *reinterpret_cast<unsigned *>(dst + off) = w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (j >= nv) break;
+        int x = (int)(int8_t)(w >> (8 * j));
+        if (o.mask && o.mask[off + j] <= 0) x = 0;
+        if (o.upd) {
+          x = (int)dst[off + j] - x;
+          x = x > 127 ? 127 : (x < -127 ? -127 : x);
+        }
+        dst[off + j] = (int8_t)x;
+      }
+    }
+  }
+}
+__device__ __forceinline__ int32_t *left_sums(const SmallParams &p, int which) {
+  return p.left + (which ? (long long)p.op[0].gm * p.op[0].gn : 0);
+}
+// The regions of CTAs that left (see niti_agree_bits).
+__device__ __forceinline__ void finish_left_regions(const SmallParams &p, int *acc, bool left, unsigned ticket) {
+  unsigned *words = niti_split_max(p.hdr);
+  const int ctas0 = p.op[0].ctas;
+  niti_finish_left(p.hdr, words, left, ticket, [&](int j) {
+    const int which = (j < ctas0 || p.op[1].ctas == 0) ? 0 : 1;
+    const SmallOp &o = p.op[which];
+    const int c = which ? j - ctas0 : j, m0 = c / o.cn * o.rm, n0 = c % o.cn * o.rn;
+    const unsigned bits = niti_posted_bits(words + (which ? ctas0 : 0), o.ctas, p.status);
+    if (bits == 0 || (which && o.upd && niti_posted_bits(words, ctas0, p.status) == 0)) return;      // (op[0] reads the weights)
+    __threadfence();
+    __syncthreads();
+    const int32_t *sums = left_sums(p, which);
+    for (int idx = threadIdx.x; idx < o.rm * o.rn; idx += SMALL_THREADS) {
+      const int r = idx / o.rn, cc = idx - r * o.rn;
+      if (m0 + r < o.gm && n0 + cc < o.gn) acc[r * (o.rn + 4) + cc] = __ldcg(sums + (long long)(m0 + r) * o.gn + n0 + cc);
+    }
+    __syncthreads();
+    round_region(p, o, acc, c, m0, n0, bits);
+  });
+}
+
 __global__ void __launch_bounds__(SMALL_THREADS, 1)
 small_gemm_kernel(const __grid_constant__ SmallParams p) {
   extern __shared__ __align__(16) int8_t smem[];
-  __shared__ unsigned cta_max, group_max;
+  __shared__ unsigned cta_max, agreed, ticket;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // which multiply, which region
   const int ctas0 = p.op[0].ctas;
@@ -164,6 +240,8 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   int8_t *As = smem + (size_t)o.rm * acc_pitch * 4, *Bs = As + o.rm * (o.kc + 16);
   if (tid == 0) cta_max = 0;
   niti_enter();
+  unsigned came = 0;
+  if (tid == 32) came = niti_arrive(p.hdr);
   unsigned mx = 0;
   {
     const int tiles_n = o.rn >> 5, tiles = (o.rm >> 5) * tiles_n;
@@ -249,67 +327,27 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   mx = __reduce_max_sync(0xffffffffu, mx);
   if (lane == 0 && mx) atomicMax(&cta_max, mx);
   __syncthreads();
-  // agreement: maximum over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after
-  // op[0]'s reads of the same weights.
+  // agreement over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after op[0]'s reads of
+  // the same weights: an update waits for op[0]'s CTAs as well.
   if (warp == 0) {
-    const long long t0 = clock64();
-    // (an update waits for op[0] as well)
-    const unsigned m = niti_agree_max(p.words + first, p.words + NITI_AGREE_MAX + 4 * first, cta_max, cta, o.ctas,
-                                      o.upd ? first : 0, lane, [&]() {
-                                        const bool out = __any_sync(0xffffffffu, clock64() - t0 > SMALL_WAIT_CYCLES);
-                                        if (out && lane == 0) atomicOr(p.status, NITI_DEV_TIMEOUT);
-                                        return out;
-                                      });
-    if (lane == 0) group_max = m;
+    unsigned *words = niti_split_max(p.hdr);
+    const unsigned m = niti_agree_bits(words + first, words + NITI_AGREE_MAX + 4 * first, niti_bitlen32(cta_max), cta, o.ctas,
+                                       o.upd ? first : 0, lane, p.patience);
+    if (lane == 0) agreed = m;
   }
+  if (tid == 32) ticket = came;
   __syncthreads();
-  if (group_max == 0) return;                             // (gave up waiting)
-  mx = group_max - 1u;
-  const int b = niti_bitlen32(mx), bp = b > o.mbits ? b - o.mbits : 0;
-  const unsigned qmax = (1u << o.mbits) - 1u;
-  if (cta == 0 && tid == 0) {
-    if (o.b_out) *o.b_out = b;
-    if (o.s_out) {
-      const int s = bp + (o.s_a ? *o.s_a : 0) + (o.s_w ? *o.s_w : 0);
-      *o.s_out = s;
-      if (s < -128 || s > 127) atomicOr(p.status, NITI_DEV_EXP_RANGE);
+  const unsigned bits = agreed, came_as = ticket;
+  if (bits) {
+    round_region(p, o, acc, cta, m0, n0, bits);
+  } else {
+    int32_t *sums = left_sums(p, which);
+    for (int idx = tid; idx < o.rm * o.rn; idx += SMALL_THREADS) {
+      const int r = idx / o.rn, c = idx - r * o.rn;
+      if (m0 + r < o.gm && n0 + c < o.gn) sums[(long long)(m0 + r) * o.gn + n0 + c] = acc[r * acc_pitch + c];
     }
   }
-  const int q = o.rn >> 2;
-  int8_t *dst = o.upd ? o.upd : o.out;
-  const bool words_ok = (o.gn & 3) == 0 && (((uintptr_t)dst | (uintptr_t)o.mask) & 3) == 0;
-  for (int idx = tid; idx < o.rm * q; idx += SMALL_THREADS) {
-    const int r = idx / q, cc = (idx - r * q) * 4;
-    const int nv = o.gn - n0 - cc;
-    if (m0 + r >= o.gm || nv <= 0) continue;
-    const long long off = (long long)(m0 + r) * o.gn + n0 + cc;
-    const int4 v = *reinterpret_cast<const int4 *>(acc + r * acc_pitch + cc);
-    const int xs[4] = {v.x, v.y, v.z, v.w};
-    unsigned w = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int x = niti_round_i32(xs[j], bp, qmax, p.round_mode);
-      if (o.relu && x < 0) x = 0;
-      w |= (unsigned)(x & 0xff) << (8 * j);
-    }
-    if (words_ok) {
-      if (o.mask) w &= __vcmpgts4(*reinterpret_cast<const unsigned *>(o.mask + off), 0u);
-      if (o.upd) w = __vmaxs4(__vsubss4(*reinterpret_cast<const unsigned *>(dst + off), w), 0x81818181u);
-      *reinterpret_cast<unsigned *>(dst + off) = w;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= nv) break;
-        int x = (int)(int8_t)(w >> (8 * j));
-        if (o.mask && o.mask[off + j] <= 0) x = 0;
-        if (o.upd) {
-          x = (int)dst[off + j] - x;
-          x = x > 127 ? 127 : (x < -127 ? -127 : x);
-        }
-        dst[off + j] = (int8_t)x;
-      }
-    }
-  }
+  if (bits == 0 || came_as >> 16) finish_left_regions(p, acc, bits == 0, came_as);
 }
 
 inline int up32(long long v) { return (int)((v + 31) / 32 * 32); }
@@ -350,7 +388,7 @@ static void fill_op(SmallOp &o, const GemmProblem &g, const RoundSpec &r) {
   o.a_mn = g.kind == GK_FC_WGRAD;
   o.b_mn = g.kind != GK_FC_FWD;
   o.out = r.out; o.mask = r.mask; o.upd = r.update_w;
-  o.mbits = r.mbits; o.relu = r.relu;
+  o.mbits = (uint8_t)r.mbits; o.relu = r.relu ? 1 : 0;
   o.s_a = r.s_a; o.s_w = r.s_w; o.s_out = r.s_out; o.b_out = r.b_out;
 }
 
@@ -360,7 +398,7 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
                     const GemmProblem *g2, const RoundSpec *r2) {
   const double macs = (double)g.M * g.N * g.K;
   const bool narrow = g.N < 32 && g.kind != GK_FC_FWD;             // (the alternative is the CUDA-core engine)
-  if (ctx->engine != 0 || ctx->reduce_fn || g.kind > GK_FC_WGRAD || macs > NITI_SMALL_MACS * (narrow ? 4 : 1) || g.gk > NITI_SPLIT_MAX_K ||
+  if (ctx->engine != 0 || ctx->reduce_fn || g.kind > GK_FC_WGRAD || macs > NITI_SMALL_MACS * (narrow ? NITI_SMALL_NARROW : 1) || g.gk > NITI_SPLIT_MAX_K ||
       (g2 && g2->gk > NITI_SPLIT_MAX_K))
     return NITI_ERR_SHAPE;
   SmallParams p;
@@ -385,7 +423,9 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
   WsHeader *hdr = niti_take_header(ctx, ws);
   const int rc = niti_clear(ctx, st);
   if (rc != NITI_OK) return rc;
-  p.words = niti_split_max(hdr);
+  p.hdr = hdr;
+  p.patience = ctx->patience;
+  p.left = (int32_t *)((char *)ws + NITI_WS_HEADER);
   NITI_CUDA_TRY(ctx, niti_launch(st, (unsigned)grid, SMALL_THREADS, smem, small_gemm_kernel, p));
   ctx->launches++;
   ctx->tc_launches += g2 ? 2 : 1;

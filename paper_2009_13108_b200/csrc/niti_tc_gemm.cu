@@ -47,6 +47,7 @@ struct TcParams {
                                 // n * d < 2^32 (0: divide)
   int quorum;                   // CTAs whose first tile must have reported before the speculative bit-width
                                 // is fixed (launches that are not single-wave)
+  unsigned patience;            // cycles that CTAs wait for each other
   int nissue;                   // resident-weights mode: warps that issue MMAs (2: the warp that loaded the
                                 // weights takes every other tile)
   int one_commit;               // resident-weights mode with as many patch stages as accumulator buffers:
@@ -126,7 +127,7 @@ struct TcParams {
   int pool;                     // 1: the epilogue also stores the 2 x 2 max-pool of the (ReLU'd) output tile
   int pool_xh;                  // lane distance of the pixel one image row below (the pixel to the right is lane ^ 1)
   int single_wave;              // every CTA has at most one tile: the sample is the whole tensor, the shift
-                                // is exact, and the first CTA publishes b and the exponent
+                                // is exact, and whoever rounds the first CTA's tile publishes b and the exponent
 };
 
 // Epilogue modes.  The shift of Algorithm 2 needs the bit-width of the WHOLE accumulator tensor:
@@ -863,14 +864,88 @@ __device__ __forceinline__ void halo_mma_loop(const TcParams &p, int issuer, int
 // convolution (items run over the phases of the input grid).  With one kernel for all of them the index
 // arithmetic and the registers of the general forms cost the aligned layers 1 - 4 % (13 spilled registers more;
 // 14 x 14 weight gradients 28.8 -> 30.4 us, 56 x 56 ones 86.2 -> 89.7 us).
-template <int CTAS, int MODE>
+// ONE: single-wave launches, in which every CTA has at most one tile, the shift is exact and a CTA may leave (see
+// niti_agree_bits).  They have no use for the loops over tiles, and the others none for what leaving takes (with both in one
+// kernel a VGG-11 step took 514 us, with neither loop nor leaving apart 498 us, with these instances 485 us).
+
+// The tile of CTA `cta` of a single-wave launch, which left its sums in `acc`: rounded and stored element by element, by all
+// threads of another CTA.
+template <int CTAS, bool STRIDED>
+__device__ __forceinline__ void round_left_tile(const TcParams &p, int cta, int b, const int32_t *acc, int8_t *out8,
+                                                const int8_t *mask8, int8_t *pool8) {
+  const int item = cta / CTAS, rank = cta - item * CTAS;              // (one item per CTA pair, in the order of the CTAs)
+  const int lane = threadIdx.x & 31, bp = b > p.mbits ? b - p.mbits : 0;
+  const unsigned qmax = (1u << p.mbits) - 1u;
+  int tile = item, mu = 0, nt = 0, split = 0;
+  Phase phq = {0, 0, 1, 1};
+  if (STRIDED) phq = split_phase(p, item, tile);
+  if (!p.halo) decode_item(p, tile, mu, nt, split);
+  const int mt = mu * CTAS + rank;
+  long long col0 = (long long)nt * p.bn;
+  int cols = p.mrep > 1 ? (int)p.gn : (int)min((long long)p.bn, p.gn - col0);
+  if (p.kind == GK_CONV_WGRAD) {
+    const int tap = nt / p.n_chunks, ci0 = (nt - tap * p.n_chunks) * p.bn;
+    col0 = (long long)tap * p.Cn + ci0;
+    cols = min(p.bn, p.Cn - ci0);
+  }
+  const bool boxes = p.halo || ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !p.i2c);
+  auto rounded = [&](long long at) {
+    const int q = niti_round_i32(__ldcg(acc + at), bp, qmax, p.round_mode);
+    return p.relu && q < 0 ? 0 : q;
+  };
+  for (int r = (int)(threadIdx.x >> 5); r < BM * p.mrep; r += NUM_THREADS / 32) {
+    long long row;
+    bool ok;
+    int w = 0, h = 0, bb = 0;
+    if (STRIDED) {
+      row = phase_row(p, mt * BM + r, phq, ok);
+    } else if (boxes) {
+      if (p.halo) {
+        tile_coords(p, item, w, h, bb);
+        w = w * 8 + (r & 7);
+        h = h * 16 + (r >> 3);
+      } else {
+        pixel_box(p, mt, w, h, bb);
+        const int t = r / p.Wt;
+        w += r - t * p.Wt;
+        h += t % p.Ht;
+        bb += t / p.Ht;
+      }
+      ok = w < p.PW && h < p.PH && bb < p.PB;
+      row = ((long long)bb * p.PH + h) * p.PW + w;
+    } else {
+      row = (long long)mt * (BM * p.mrep) + r;
+      ok = row < p.gm;
+    }
+    if (!ok) continue;
+    const bool pools = p.pool && ((w | h) & 1) == 0;                  // (extents are even, windows lie inside the tile)
+    for (int c = lane; c < cols; c += 32) {
+      const long long at = row * p.gn + col0 + c;
+      int q = rounded(at);
+      if (pools) {
+        const int m = max(max(q, rounded(at + p.gn)), max(rounded(at + p.PW * p.gn), rounded(at + (p.PW + 1) * p.gn)));
+        pool8[(((long long)bb * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1)) * p.gn + col0 + c] = (int8_t)m;
+      }
+      if (p.update) {
+        const int d = (int)out8[at] - q;
+        q = d > 127 ? 127 : (d < -127 ? -127 : d);
+      } else if (mask8 && mask8[at] <= 0) {
+        q = 0;
+      }
+      out8[at] = (int8_t)q;
+    }
+  }
+}
+
+template <int CTAS, int MODE, bool ONE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_c, const TcParams p, int32_t *__restrict__ acc, WsHeader *hdr, uint32_t *status,
                int8_t *__restrict__ out8, const int8_t *__restrict__ mask8, const int32_t *s_a,
                const int32_t *s_w, int32_t *s_out, int32_t *b_out, int32_t *spec_slot, int8_t *__restrict__ pool8) {
   constexpr bool I2C = MODE >= 1, STRIDED = MODE == 2, GENERAL = MODE >= 1;
-  if (p.epi_mode == EPI_KNOWN_B) {
+  const int epi_mode = ONE ? (int)EPI_SPECULATE : p.epi_mode;
+  if (epi_mode == EPI_KNOWN_B) {
     // follow-up of a speculative pass: publish the scalars, then leave unless the guess was wrong
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the first pass has completed and is visible
     const int b_true = niti_bitlen32(hdr->maxabs32), b_est = (int)hdr->spec_b - 1;   // (stored + 1)
@@ -899,7 +974,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 2 * MAX_TBUF + 1];
   __shared__ unsigned tmem_base_slot;
   __shared__ volatile int abort_flag;
-  __shared__ volatile int spec_bp_ready;      // 0: not yet; else the speculative binary point + 1
+  __shared__ volatile int spec_bp_ready;      // 0: not yet; the speculative binary point + 1; -1: this CTA leaves
+  __shared__ unsigned ticket;                 // of the agreement of a single-wave launch
   __shared__ unsigned first_max, first_arrived;   // this CTA's first tile: max magnitude, warps that reported
   __shared__ unsigned cta_max;                    // max magnitude of everything this CTA rounded
 
@@ -929,7 +1005,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // The 16 epilogue warps are split into `egroups` groups that drain different tiles at the same
   // time (narrow tiles have too few 32-column chunks to keep every warp busy on one tile).  Inside a
   // group each TMEM lane quarter has wpq warps that interleave the tile's chunks.
-  const int egroups = p.halo == 2 ? 1 : p.egroups;
+  const int egroups = ONE || p.halo == 2 ? 1 : p.egroups;
   const int wpq = p.k_wpq;                                   // warps per quarter per tile
   const int wpq_active = p.k_wpq_active;
   const int epi_active = p.k_epi_active;                     // warps that drain one tile
@@ -977,7 +1053,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   const unsigned tmem_base = tmem_base_slot;
   // (the set-up above overlaps the kernel before this one; a follow-up launch that is scheduled from here on takes the SMs
   // as this grid's CTAs retire)
+  const int8_t *const mask_at_exit = mask8;          // (the parameter itself: costs the main loops no register)
   niti_enter(mask8);
+  if (ONE && threadIdx.x == NUM_THREADS - 1) ticket = niti_arrive(hdr);      // (a thread that has to wait anyway)
+
+  // the scalars of a single-wave launch: the shift is exact, and no second launch publishes them
+  auto publish_exact = [&](int b) {
+    const int bpf = b > p.mbits ? b - p.mbits : 0;
+    if (b_out) *b_out = b;
+    if (s_out) {
+      const int sv = bpf + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
+      *s_out = sv;
+      if (sv < -128 || sv > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
+    }
+  };
 
   if (warp < PROD_WARPS) {
     // ================= TMA producers (every CTA loads its own rows of A and its share of B) ========
@@ -1339,13 +1428,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     unsigned mx = 0;
     int bp = 0;
     int h_wt = 0, h_ht = 0, h_bt = 0;
-    if (p.epi_mode == EPI_KNOWN_B) {
+    if (epi_mode == EPI_KNOWN_B) {
       const int b = niti_bitlen32(hdr->maxabs32);
       bp = b > p.mbits ? b - p.mbits : 0;
     }
     bool ok = true;
     const unsigned red_buf = smem_base + (unsigned)p.red_off + (unsigned)(warp - EPI_WARP0) * 4096u;
-    if (p.halo == 2) {
+    if (!ONE && p.halo == 2) {
       // lane = (tap of the pair, input channel), column = output channel; partial sums of this
       // CTA's pixel range are added to g32[co][tap][ci]
       const int which = row_in_tile >> 6, ci = row_in_tile & 63;
@@ -1390,7 +1479,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             (mask8 == nullptr || ((uintptr_t)mask8 & 31) == 0);
     // the lean loop takes over after a warp's first item (which may be the CTA's speculative first
     // tile) when every chunk of every tile is whole and aligned
-    const bool lean_ok = (p.epi_mode == EPI_KNOWN_B || p.epi_mode == EPI_SPECULATE) && p.splits == 1 &&
+    const bool lean_ok = !ONE && (epi_mode == EPI_KNOWN_B || epi_mode == EPI_SPECULATE) && p.splits == 1 &&
                          (p.bn & 31) == 0 && p.halo != 2 && p.kind != GK_CONV_WGRAD &&
                          (p.mrep == 1 || (io_aligned && p.gn == p.bn_mma && mask8 == nullptr));
     // (otherwise: the largest store unit of the output rows, and this warp's staging buffer)
@@ -1476,7 +1565,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
       tc_fence_after();
       const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)p.bn;
-      if (p.epi_mode == EPI_ATOMIC && p.red) {
+      if (epi_mode == EPI_ATOMIC && p.red) {
         // partial sums of a split contraction: every chunk is staged and added by one copy
         unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
         int x0, x1, x2 = 0, x3 = 0;                            // tensor coordinates of the chunk at column 0
@@ -1520,7 +1609,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
         pmx = __reduce_max_sync(0xffffffffu, pmx);
         if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
-      } else if (p.epi_mode <= EPI_ATOMIC) {
+      } else if (epi_mode <= EPI_ATOMIC) {
         int32_t *dst = acc + out_row * p.gn + col0;
         const bool vec_ok = ((p.gn & 3) == 0) && ((col0 & 3) == 0);
         unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
@@ -1528,7 +1617,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           int v[32];
           tc_ld32(tm_row + (unsigned)c, v);
           if (row_ok && c < ncols_valid) {
-            if (p.epi_mode == EPI_ATOMIC) {
+            if (epi_mode == EPI_ATOMIC) {
 #pragma unroll
               for (int j = 0; j < 32; ++j)
                 if (c + j < ncols_valid && v[j] != 0) {
@@ -1558,12 +1647,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
           }
         }
-        if (p.epi_mode == EPI_ATOMIC) {
+        if (epi_mode == EPI_ATOMIC) {
           pmx = __reduce_max_sync(0xffffffffu, pmx);
           if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
         }
       } else {
-        if (p.epi_mode == EPI_SPECULATE && use == (unsigned)egroup && egroup != 0) {
+        bool leaves = false;                                   // (see niti_agree_bits)
+        if (!ONE && epi_mode == EPI_SPECULATE && use == (unsigned)egroup && egroup != 0) {
           // the group that drains this CTA's first tile publishes the shift through shared memory
           long long t0 = clock64();
           while (spec_bp_ready == 0) {
@@ -1578,7 +1668,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           bp = spec_bp_ready - 1;
           rk = make_round_const(bp, p.mbits, p.round_mode);
         }
-        if (p.epi_mode == EPI_SPECULATE && use == 0) {
+        if (epi_mode == EPI_SPECULATE && use == 0) {
           // first tile of this CTA: max only, then agree on the estimate with the whole grid
           // (columns of a partly filled chunk beyond the matrix accumulate zeros; whole chunks beyond it are left out)
           const int cend0 = p.mrep > 1 ? p.bn : (ncols_valid < p.bn ? ncols_valid : p.bn);
@@ -1608,30 +1698,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             __threadfence_block();
             last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
           }
-          if (p.single_wave) {
+          if (ONE) {
             // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
             if (__shfl_sync(0xffffffffu, last, 0)) {
               unsigned *words = niti_split_max(hdr);
-              const long long t0 = clock64();
-              const unsigned all_max = niti_agree_max(
-                  words, words + NITI_AGREE_MAX, *(volatile unsigned *)&first_max, (int)blockIdx.x, (int)gridDim.x, 0, lane, [&]() {
-                    const bool out = __any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES);
-                    if (out && lane == 0) {
-                      abort_flag = 1;
-                      atomicOr(status, NITI_DEV_TIMEOUT);
-                    }
-                    return out || __any_sync(0xffffffffu, abort_flag != 0);
-                  });
-              if (lane == 0 && all_max) {
-                const int b = niti_bitlen32(all_max - 1u), bpf = b > p.mbits ? b - p.mbits : 0;
-                spec_bp_ready = bpf + 1;
-                if (blockIdx.x == 0) {                       // (no second launch publishes the scalars)
-                  if (b_out) *b_out = b;
-                  if (s_out) {
-                    const int sv = bpf + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
-                    *s_out = sv;
-                    if (sv < -128 || sv > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
-                  }
+              const unsigned agreed = niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(*(volatile unsigned *)&first_max),
+                                                      (int)blockIdx.x, (int)gridDim.x, 0, lane, p.patience);
+              if (lane == 0) {
+                if (agreed) {
+                  const int b = (int)agreed - 1, bpf = b > p.mbits ? b - p.mbits : 0;
+                  spec_bp_ready = bpf + 1;
+                  if (blockIdx.x == 0) publish_exact(b);
+                } else {
+                  spec_bp_ready = -1;
                 }
               }
             }
@@ -1644,7 +1723,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               // The bit-width is fixed as soon as a quorum of CTAs has reported, by whichever CTA sees
               // that first (compare-and-swap on the published word); CTAs that start late find it
               // published and never wait.  Waiting for every CTA meant waiting out the launch ramp of
-              // the whole grid (~10 k cycles) in every launch.
+              // the whole grid (~10 k cycles) in every launch.  Where not even a quorum comes (launches of several
+              // streams share the SMs), a CTA out of patience fixes it from what has been reported: the bit-width
+              // is a guess in any case, and the follow-up launch corrects a wrong one.
               const unsigned quorum = (unsigned)p.quorum;
               unsigned pub = 0;
               long long t0 = clock64();
@@ -1656,7 +1737,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                              : "l"(&hdr->est_max)
                              : "memory");
                 if (v_pub) { pub = v_pub; break; }
-                if (v_cnt >= quorum) {
+                if (v_cnt >= quorum || clock64() - t0 > (long long)p.patience) {
                   // (the 16-byte load is not promised to be one atomic snapshot: once the count is seen,
                   // the maximum is read again, after a fence, so that it is at least as new as the count)
                   __threadfence();
@@ -1679,11 +1760,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                   break;
                 }
                 if (abort_flag) break;
-                if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
-                  abort_flag = 1;
-                  atomicOr(status, NITI_DEV_TIMEOUT);
-                  break;
-                }
               }
               const int b = (int)pub - 1;
               spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
@@ -1702,7 +1778,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
           __syncwarp();
           if (abort_flag) { ok = false; break; }
-          bp = spec_bp_ready - 1;
+          leaves = ONE && spec_bp_ready < 0;
+          bp = leaves ? 0 : spec_bp_ready - 1;
           rk = make_round_const(bp, p.mbits, p.round_mode);
         }
         // Whole 32-column chunks with 32-byte aligned rows (every layer of the networks): the chunk
@@ -1711,7 +1788,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // input channels: every instruction here is paid for 16 times per tile.)
         const bool whole_chunks = io_aligned && ((col0 & 31) == 0) &&
                                   (p.mrep > 1 ? ncols_valid >= p.bn_mma : (ncols_valid & 31) == 0);
-        if (whole_chunks) {
+        if (ONE && leaves) {
+          for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
+            int v[32];
+            tc_ld32(tm_row + (unsigned)c, v);
+            const int jt = p.mrep > 1 ? c / p.bn_mma : 0, cc = c - jt * p.bn_mma;
+            const long long orow = out_row + (long long)jt * BM;
+            if (!row_ok || (p.mrep > 1 && orow >= p.gm)) continue;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (cc + j < ncols_valid) acc[orow * p.gn + col0 + cc + j] = v[j];
+          }
+        } else if (whole_chunks) {
           const bool relu = p.relu != 0;
           // (the last column tile of a row may be narrower than the tile: its chunks beyond the
           // matrix are not read at all)
@@ -1811,7 +1899,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // input channels that pipe is the bound of the whole kernel: per tile and per chunk this loop
     // executes only what changes (measured on the first layer: the general loop above spends a third
     // of its integer instructions on tests whose outcome is the same for every tile).
-    if (ok && lean_item >= 0) {
+    if (!ONE && ok && lean_item >= 0) {
       auto lean = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c, auto narrow_c) {
         constexpr bool NARROW = decltype(narrow_c)::value;   // output rows that are not 32-byte aligned, short last chunks
         constexpr bool RELU = decltype(relu_c)::value, MASK = decltype(mask_c)::value, BATCHED = decltype(batched_c)::value;
@@ -1937,7 +2025,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       else { if (masked) lean(F{}, T{}, F{}, F{}, F{}, F{}); else lean(F{}, F{}, F{}, F{}, F{}, F{}); }
       mx |= ex_all.magnitude_bits();
     }
-    if (p.epi_mode == EPI_SPILL || p.epi_mode == EPI_SPECULATE) {
+    if (epi_mode == EPI_SPILL || epi_mode == EPI_SPECULATE) {
       for (int o = 16; o > 0; o >>= 1) {
         unsigned u = __shfl_xor_sync(0xffffffffu, mx, o);
         mx = u > mx ? u : mx;
@@ -1950,13 +2038,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // ================= common exit =================
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && cta_max && !(p.single_wave && p.epi_mode == EPI_SPECULATE)) atomicMax(&hdr->maxabs32, cta_max);
+  if (!ONE && threadIdx.x == 0 && cta_max) atomicMax(&hdr->maxabs32, cta_max);
   if (abort_flag) {
     // give copies and MMAs still in flight time to land before shared and tensor memory go away
     long long t0 = clock64();
     while (clock64() - t0 < 20000000LL) {
     }
     __syncthreads();
+  } else if (ONE) {
+    niti_finish_left(hdr, niti_split_max(hdr), spec_bp_ready < 0, ticket, [&](int j) {
+      const unsigned bits = niti_posted_bits(niti_split_max(hdr), (int)gridDim.x, status);
+      if (bits == 0) return;
+      if (j == 0 && threadIdx.x == 0) publish_exact((int)bits - 1);
+      round_left_tile<CTAS, STRIDED>(p, j, (int)bits - 1, acc, out8, mask_at_exit, pool8);
+    });
   }
   if (CTAS == 2) cluster_sync_all();   // nobody leaves while the peer may still touch this CTA
   if (warp == MMA_WARP) {
@@ -1977,19 +2072,24 @@ template <int NV>
 __global__ void __launch_bounds__(FIN_THREADS, 1)
 finish_split_kernel(const int32_t *__restrict__ acc, int nvec, WsHeader *hdr, int splits, uint32_t *status, int8_t *out,
                     int8_t *upd, const int8_t *__restrict__ mask, int relu, int mbits, int round_mode, const int32_t *s_a,
-                    const int32_t *s_w, int32_t *s_out, int32_t *b_out) {
-  __shared__ unsigned blk_max, grid_max;
+                    const int32_t *s_w, int32_t *s_out, int32_t *b_out, unsigned patience) {
+  __shared__ unsigned blk_max, agreed, ticket;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, T = (int)gridDim.x * FIN_THREADS;
   if (tid == 0) blk_max = 0;
   niti_enter(acc, mask);                                      // the multiply has completed and is visible
-  const int t0 = (int)blockIdx.x * FIN_THREADS + tid;
+  unsigned came = 0;
+  if (tid == 64) came = niti_arrive(hdr);
   int4 v[NV];
-  unsigned mx = 0;
+  auto load = [&](int blk) {
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    v[i] = make_int4(0, 0, 0, 0);
-    if (t0 + i * T < nvec) v[i] = __ldcg(reinterpret_cast<const int4 *>(acc) + t0 + i * T);
-  }
+    for (int i = 0; i < NV; ++i) {
+      const int idx = blk * FIN_THREADS + tid + i * T;
+      v[i] = make_int4(0, 0, 0, 0);
+      if (idx < nvec) v[i] = __ldcg(reinterpret_cast<const int4 *>(acc) + idx);
+    }
+  };
+  load((int)blockIdx.x);
+  unsigned mx = 0;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     mx = max(mx, max((unsigned)abs(v[i].x), (unsigned)abs(v[i].y)));
@@ -2006,41 +2106,49 @@ finish_split_kernel(const int32_t *__restrict__ acc, int nvec, WsHeader *hdr, in
     if (lane == 0 && bound >= 0x80000000ull) atomicOr(status, NITI_DEV_ACC_RANGE);
   }
   __syncthreads();
+  // (behind the split maxima: the caller leaves room)
+  unsigned *words = niti_split_max(hdr) + NITI_MAX_SPLITS - NITI_AGREE_WORDS;
   if (warp == 0) {
-    // (behind the split maxima: the caller leaves room)
-    unsigned *words = niti_split_max(hdr) + NITI_MAX_SPLITS - NITI_AGREE_WORDS;
-    const long long c0 = clock64();
-    const unsigned m = niti_agree_max(words, words + NITI_AGREE_MAX, blk_max, (int)blockIdx.x, (int)gridDim.x, 0, lane, [&]() {
-      const bool late = __any_sync(0xffffffffu, clock64() - c0 > WAIT_LIMIT_CYCLES);
-      if (late && lane == 0) atomicOr(status, NITI_DEV_TIMEOUT);
-      return late;
-    });
-    if (lane == 0) grid_max = m;
+    const unsigned m = niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(blk_max), (int)blockIdx.x, (int)gridDim.x, 0, lane,
+                                       patience);
+    if (lane == 0) agreed = m;
   }
+  if (tid == 64) ticket = came;
   __syncthreads();
-  if (grid_max == 0) return;                                  // (gave up waiting)
-  const int b = niti_bitlen32(grid_max - 1u), bp = b > mbits ? b - mbits : 0;
-  if (t0 == 0) {
-    if (b_out) *b_out = b;
-    if (s_out) {
-      const int s = bp + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
-      *s_out = s;
-      if (s < -128 || s > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
+  auto round_block = [&](int blk, unsigned bits) {
+    const int b = (int)bits - 1, bp = b > mbits ? b - mbits : 0;
+    if (blk == 0 && tid == 0) {
+      if (b_out) *b_out = b;
+      if (s_out) {
+        const int s = bp + (s_a ? *s_a : 0) + (s_w ? *s_w : 0);
+        *s_out = s;
+        if (s < -128 || s > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
+      }
     }
-  }
-  const RoundConst rk = make_round_const(bp, mbits, round_mode);
-  Extremes ex = {0, 0, 0u};
+    const RoundConst rk = make_round_const(bp, mbits, round_mode);
+    Extremes ex = {0, 0, 0u};
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const int idx = t0 + i * T;
-    if (idx >= nvec) break;
-    unsigned w = rk.aligned ? round_pack4_aligned<false>(v[i].x, v[i].y, v[i].z, v[i].w, rk, ex)
-                            : round_pack4<false, true>(v[i].x, v[i].y, v[i].z, v[i].w, rk, ex);
-    if (relu) w &= bytes_gt0(w);
-    if (mask) w &= bytes_gt0(reinterpret_cast<const unsigned *>(mask)[idx]);
-    if (upd) reinterpret_cast<unsigned *>(upd)[idx] = bytes_sub_clamp127(reinterpret_cast<unsigned *>(upd)[idx], w);
-    else reinterpret_cast<unsigned *>(out)[idx] = w;
-  }
+    for (int i = 0; i < NV; ++i) {
+      const int idx = blk * FIN_THREADS + tid + i * T;
+      if (idx >= nvec) break;
+      unsigned w = rk.aligned ? round_pack4_aligned<false>(v[i].x, v[i].y, v[i].z, v[i].w, rk, ex)
+                              : round_pack4<false, true>(v[i].x, v[i].y, v[i].z, v[i].w, rk, ex);
+      if (relu) w &= bytes_gt0(w);
+      if (mask) w &= bytes_gt0(reinterpret_cast<const unsigned *>(mask)[idx]);
+      if (upd) reinterpret_cast<unsigned *>(upd)[idx] = bytes_sub_clamp127(reinterpret_cast<unsigned *>(upd)[idx], w);
+      else reinterpret_cast<unsigned *>(out)[idx] = w;
+    }
+  };
+  const unsigned got = agreed, came_as = ticket;
+  if (got) round_block((int)blockIdx.x, got);
+  if (got && !(came_as >> 16)) return;
+  // (the sums of a block that left are in memory already)
+  niti_finish_left(hdr, words, got == 0, came_as, [&](int j) {
+    const unsigned bits = niti_posted_bits(words, (int)gridDim.x, status);
+    if (bits == 0) return;
+    load(j);
+    round_block(j, bits);
+  });
 }
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever completes, gives up
@@ -2777,13 +2885,13 @@ int niti_tc_timeout_probe(niti_ctx *ctx, cudaStream_t st) {
 // a second, short wave.
 // Dynamic shared-memory limit of the kernel: once per context, and always the most the device allows
 // beside the kernel's static shared memory (see niti_ctx::smem_optin for why not "what this launch needs").
-template <int CTAS, int MODE>
+template <int CTAS, int MODE, bool ONE>
 static int tc_set_smem_limit(niti_ctx *ctx) {
   cudaFuncAttributes fa;
-  NITI_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, tc_gemm_kernel<CTAS, MODE>));
+  NITI_CUDA_TRY(ctx, cudaFuncGetAttributes(&fa, tc_gemm_kernel<CTAS, MODE, ONE>));
   const size_t limit = ctx->smem_optin > fa.sharedSizeBytes ? ctx->smem_optin - fa.sharedSizeBytes : 0;
-  NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(tc_gemm_kernel<CTAS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
-  ctx->tc_attr_smem[CTAS + 2 * MODE] = limit;
+  NITI_CUDA_TRY(ctx, cudaFuncSetAttribute(tc_gemm_kernel<CTAS, MODE, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  ctx->tc_attr_smem[CTAS + 2 * MODE + 6 * ONE] = limit;
   return NITI_OK;
 }
 
@@ -2805,23 +2913,23 @@ static int tc_units(niti_ctx *ctx) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    (void)tc_set_smem_limit<2, 0>(ctx);
+    (void)tc_set_smem_limit<2, 0, false>(ctx);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2, 0>, &cfg) == cudaSuccess && n > 0 && n < cached) cached = n;
+    if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_kernel<2, 0, false>, &cfg) == cudaSuccess && n > 0 && n < cached) cached = n;
     else (void)cudaGetLastError();
   }
   return cached;
 }
 
-template <int CTAS, int MODE>
+template <int CTAS, int MODE, bool ONE>
 static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                      int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
   size_t smem = (size_t)p.stages * (p.a_bytes + p.b_bytes) + (size_t)p.b_res_bytes + 1024;
   if (p.red) smem = (size_t)p.red_off + RED_BYTES + 1024;
   if (p.nstg_off > 0) smem = (size_t)p.nstg_off + (size_t)EPI_WARPS * 32 * 36 + 1024;
-  size_t &attr_smem = ctx->tc_attr_smem[CTAS + 2 * MODE];
+  size_t &attr_smem = ctx->tc_attr_smem[CTAS + 2 * MODE + 6 * ONE];
   if (!attr_smem) {
-    const int rcs = tc_set_smem_limit<CTAS, MODE>(ctx);
+    const int rcs = tc_set_smem_limit<CTAS, MODE, ONE>(ctx);
     if (rcs != NITI_OK) return rcs;
   }
   if (smem > attr_smem) return niti_fail(ctx, NITI_ERR_SHAPE, "tensor-core kernel: stage buffers exceed the shared memory of an SM");
@@ -2871,7 +2979,7 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
     slot = ctx->d_spec_tab + 2 * (size_t)((key ^ (key >> 13)) % NITI_SPEC_SLOTS);
     q.spec_tag = (int)(unsigned)(key | 1u);
   }
-  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE>, ma, mb, mc, q, acc, hdr, ctx->d_status, r.out, r.mask,
+  NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE, ONE>, ma, mb, mc, q, acc, hdr, ctx->d_status, r.out, r.mask,
                                         r.s_a, r.s_w, r.s_out, r.b_out, slot, r.pool_out));
   ctx->launches++;
   if (MODE != 2) {                   // (the counters of the header cover the kernel without its strided form)
@@ -2883,11 +2991,18 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
 
 static int launch_tc(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mc,
                      int32_t *acc, WsHeader *hdr, const RoundSpec &r) {
-  if (p.mode == 2)
-    return p.ctas == 2 ? launch_tc_as<2, 2>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 2>(ctx, st, p, ma, mb, mc, acc, hdr, r);
-  if (p.mode == 1)
-    return p.ctas == 2 ? launch_tc_as<2, 1>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 1>(ctx, st, p, ma, mb, mc, acc, hdr, r);
-  return p.ctas == 2 ? launch_tc_as<2, 0>(ctx, st, p, ma, mb, mc, acc, hdr, r) : launch_tc_as<1, 0>(ctx, st, p, ma, mb, mc, acc, hdr, r);
+  auto go = [&](auto mode, auto one) {
+    constexpr int MODE = decltype(mode)::value;
+    constexpr bool ONE = decltype(one)::value;
+    return p.ctas == 2 ? launch_tc_as<2, MODE, ONE>(ctx, st, p, ma, mb, mc, acc, hdr, r)
+                       : launch_tc_as<1, MODE, ONE>(ctx, st, p, ma, mb, mc, acc, hdr, r);
+  };
+  auto pick = [&](auto mode) {
+    return p.single_wave && p.epi_mode == EPI_SPECULATE ? go(mode, std::true_type{}) : go(mode, std::false_type{});
+  };
+  if (p.mode == 2) return pick(std::integral_constant<int, 2>{});
+  if (p.mode == 1) return pick(std::integral_constant<int, 1>{});
+  return pick(std::integral_constant<int, 0>{});
 }
 
 // Profiling event of a launch.  On a stream that is being captured the record becomes an event-record
@@ -2958,7 +3073,7 @@ static int launch_finish(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, lon
   const long long per = (nvec + blocks * FIN_THREADS - 1) / (blocks * FIN_THREADS);
   auto go = [&](auto kernel) {
     return niti_launch(st, (unsigned)blocks, FIN_THREADS, 0, kernel, acc, (int)nvec, hdr, splits, ctx->d_status, r.out, r.update_w, r.mask, r.relu, r.mbits,
-                              r.round_mode, r.s_a, r.s_w, r.s_out, r.b_out);
+                              r.round_mode, r.s_a, r.s_w, r.s_out, r.b_out, ctx->patience);
   };
   NITI_CUDA_TRY(ctx, per <= 1 ? go(finish_split_kernel<1>) : per <= 2 ? go(finish_split_kernel<2>)
                      : per <= 4 ? go(finish_split_kernel<4>) : go(finish_split_kernel<8>));
@@ -3035,6 +3150,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     const long long units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
     const long long grid = (p.items < units ? p.items : units) * p.ctas;
     p.quorum = (int)((grid + 1) / 2);
+    p.patience = ctx->patience;
   }
   p.mbits = r.mbits;
   p.round_mode = r.round_mode;
@@ -3080,7 +3196,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
   if (rc != NITI_OK) return rc;
   if (p.epi_mode == EPI_SPECULATE && p.single_wave) {
-    *fused = true;                     // exact shift, scalars published by the last CTA: no second launch
+    *fused = true;                     // exact shift, scalars published by this launch: no second one
   } else if (p.epi_mode == EPI_SPECULATE) {
     // publishes b and the exponent; recomputes with the true bit-width only if the guess was low
     if (dp) {
