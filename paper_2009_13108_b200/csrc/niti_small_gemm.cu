@@ -35,7 +35,7 @@ struct SmallOp {
   int rm, rn, cn;             // region of a CTA (multiples of 32), CTAs per row of regions
   int ctas;                   // CTAs of this multiply (0: this launch has no such multiply)
   int kc;                     // contraction elements staged at a time (multiple of 64)
-  uint8_t a_mn, b_mn, mbits, relu;
+  int a_mn, b_mn, mbits, relu;
   int8_t *out;
   const int8_t *mask;         // output is zero where mask <= 0
   int8_t *upd;                // weights from which the rounded result is subtracted (out is then not written)
@@ -388,7 +388,7 @@ static void fill_op(SmallOp &o, const GemmProblem &g, const RoundSpec &r) {
   o.a_mn = g.kind == GK_FC_WGRAD;
   o.b_mn = g.kind != GK_FC_FWD;
   o.out = r.out; o.mask = r.mask; o.upd = r.update_w;
-  o.mbits = (uint8_t)r.mbits; o.relu = r.relu ? 1 : 0;
+  o.mbits = r.mbits; o.relu = r.relu ? 1 : 0;
   o.s_a = r.s_a; o.s_w = r.s_w; o.s_out = r.s_out; o.b_out = r.b_out;
 }
 
