@@ -2486,6 +2486,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
           p.u0_r = fr > 0 ? (fr + st - 1) / st : 0; p.u0_s = fs > 0 ? (fs + st - 1) / st : 0;
           const int u1_r = (g.H - 1 + g.pad) / st, u1_s = (g.W - 1 + g.pad) / st;
           p.PH = u1_r - p.u0_r + 1; p.PW = u1_s - p.u0_s + 1;
+          if (p.PH <= 0 || p.PW <= 0) return false;      // (every window row or column lies in the padding: all errors are 0)
           p.i2c_h0 = p.u0_r - (p.T_r - 1); p.i2c_w0 = p.u0_s - (p.T_s - 1);
           sa.hi[0] = p.i2c_w0 + p.PW - 1 - (OW - 1); sa.hi[1] = p.i2c_h0 + p.PH - 1 - (OH - 1);
           p.OH = g.H; p.OW = g.W;

@@ -30,6 +30,7 @@ CASES = [
     (1, 40, 33, 16, 48, 3, 0, 4),
     (2, 30, 30, 32, 32, 4, 1, 2),       # even filter, no phase is shorter
     (2, 31, 31, 64, 64, 7, 5, 2),       # padding larger than (R - 1) / 2
+    (2, 3, 9, 32, 32, 1, 1, 4), (2, 1, 7, 32, 32, 1, 1, 2),     # strided error without a single position: zeros
     (3, 29, 31, 3, 40, 11, 2, 4),       # gathered rows of 384 bytes
     (2, 33, 20, 3, 24, 7, 3, 2),
     (2, 21, 300, 1, 17, 5, 2, 1),       # two row segments
