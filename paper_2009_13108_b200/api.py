@@ -416,11 +416,28 @@ class Niti:
         return w
 
     def copy_tensors(self, dsts, srcs):
-        """Copies every source tensor to its destination (same sizes, contiguous) with one launch per 32."""
-        n = len(dsts)
-        sizes = [d.numel() * d.element_size() for d in dsts]
-        self._ck(self.lib.niti_copy_tensors(self.h, self._stream(), n, (C.c_void_p * n)(*[d.data_ptr() for d in dsts]),
-                                            (C.c_void_p * n)(*[s.data_ptr() for s in srcs]), (C.c_int64 * n)(*sizes)))
+        """Copies every source tensor to its destination (same shapes) with one launch per 32.  Tensors that are not
+        contiguous, differ in type or are not on this object's GPU are copied by torch, one by one."""
+        if len(dsts) != len(srcs):
+            raise NitiError(ERR_ARG, "copy_tensors: %d destinations, %d sources" % (len(dsts), len(srcs)))
+        to, frm, sizes, others, gpu = [], [], [], [], self.device.index
+        for d, s in zip(dsts, srcs):
+            if d.shape != s.shape:
+                raise NitiError(ERR_ARG, "copy_tensors: %s from %s" % (tuple(d.shape), tuple(s.shape)))
+            a, b = d.data_ptr(), s.data_ptr()
+            if (gpu is not None and d.get_device() == gpu and s.get_device() == gpu and d.dtype == s.dtype and
+                    d.is_contiguous() and s.is_contiguous() and not (a | b) & 15 and a and b):
+                to.append(a)
+                frm.append(b)
+                sizes.append(d.nbytes)
+            else:
+                others.append((d, s))
+        n = len(to)
+        if n:
+            self._ck(self.lib.niti_copy_tensors(self.h, self._stream(), n, (C.c_void_p * n)(*to), (C.c_void_p * n)(*frm),
+                                                (C.c_int64 * n)(*sizes)))
+        for d, s in others:
+            d.copy_(s, non_blocking=True)
 
     def relu_fwd(self, x, y=None):
         y = y if y is not None else torch.empty_like(x)
