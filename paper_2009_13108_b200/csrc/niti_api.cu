@@ -540,8 +540,12 @@ static int linear_bwd_impl(niti_ctx *ctx, void *stream, const int8_t *a, const i
   {
     const RoundSpec rd = {e_prev, relu_mask_src, 7, round_mode, 0, nullptr, nullptr, nullptr, b_e, nullptr, nullptr};
     const RoundSpec rw = {g, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, b_g, nullptr, update_w};
-    const int rc = e_prev ? niti_small_gemm(ctx, (cudaStream_t)stream, ws, pd, rd, &pw, &rw)
-                          : niti_small_gemm(ctx, (cudaStream_t)stream, ws, pw, rw, nullptr, nullptr);
+    // One launch runs both multiplies at once: an error that replaces the layer's input in place is left to the launches
+    // below, which read the input for the weight gradient before they write the error.
+    const uintptr_t e0 = (uintptr_t)e_prev, a0 = (uintptr_t)a, span = (uintptr_t)M * (uintptr_t)K;
+    int rc = NITI_ERR_SHAPE;
+    if (!e_prev) rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, pw, rw, nullptr, nullptr);
+    else if (e0 >= a0 + span || a0 >= e0 + span) rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, pd, rd, &pw, &rw);
     if (rc != NITI_ERR_SHAPE) return rc;
   }
   char *pad_a = pad_mem + pad_bytes(pd) - pad_bytes(pw, 0);      // (the weight gradient finds e padded already)

@@ -39,3 +39,18 @@ def test_small_multiplies(niti, oref, M, N, K):
     assert np.array_equal(eu.cpu().numpy(), we) and np.array_equal(wt.cpu().numpy(), oref.sgd_update(w, wg))
     niti.linear_bwd_update(T(a), T(e), wt, need_e_prev=False)
     assert np.array_equal(wt.cpu().numpy(), oref.sgd_update(oref.sgd_update(w, wg), wg))
+
+
+@pytest.mark.parametrize("M,N,K", [(64, 256, 784), (256, 10, 512), (300, 100, 90)])
+def test_error_in_place_of_the_input(niti, oref, M, N, K):
+    """niti_linear_bwd with e_prev in the storage of a: the weight gradient still sees the input."""
+    rng = np.random.default_rng(M + N + K)
+    i8 = lambda *s: rng.integers(-127, 128, size=s, dtype=np.int8)  # noqa: E731
+    T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(niti.device)  # noqa: E731
+    a, w, e = i8(M, K), i8(N, K), i8(M, N)
+    we, wg, be, bg = oref.linear_bwd(a, e, w, True, None, 5)
+    for _ in range(5):
+        at = T(a)
+        ep, g, b_e, b_g = niti.linear_bwd(at, T(e), T(w), True, e_prev=at)
+        assert np.array_equal(ep.cpu().numpy(), we) and np.array_equal(g.cpu().numpy(), wg)
+        assert (int(b_e), int(b_g)) == (be, bg)
