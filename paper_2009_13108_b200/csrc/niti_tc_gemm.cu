@@ -2038,6 +2038,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // ================= common exit =================
   tc_fence_before();
   __syncthreads();
+  // (a CTA that rounded with the agreed bit-width has met nothing wider: anything else means that the agreement was broken
+  // and its stored values are not exact)
+  if (ONE && threadIdx.x == 0 && spec_bp_ready > 0 && niti_bitlen32(cta_max) > p.mbits + spec_bp_ready - 1)
+    atomicOr(status, NITI_DEV_INTERNAL);
   if (!ONE && threadIdx.x == 0 && cta_max) atomicMax(&hdr->maxabs32, cta_max);
   if (abort_flag) {
     // give copies and MMAs still in flight time to land before shared and tensor memory go away
