@@ -120,9 +120,9 @@ int niti_set_engine(niti_ctx *ctx, int engine);
 
 /* Number of kernels and memsets this context has enqueued so far. */
 uint64_t niti_launch_count(niti_ctx *ctx);
-/* Of those, launches of the tensor-core matrix-multiply kernels: tcgen05 (without the instance that computes the
- * error of strided convolutions, which only niti_launch_count() counts) and the mma.sync kernel of small fully
- * connected multiplies, whose backward launch runs two multiplies and counts as two. */
+/* Launches of the tensor-core matrix-multiply kernels among them: tcgen05, and the mma.sync kernel of small fully
+ * connected multiplies.  A launch of the latter that runs both multiplies of a backward call counts as two here (and
+ * as one in niti_launch_count()). */
 uint64_t niti_tc_launch_count(niti_ctx *ctx);
 /* Of those, launches of the paired-CTA (cta_group::2) variant. */
 uint64_t niti_tc_pair_launch_count(niti_ctx *ctx);

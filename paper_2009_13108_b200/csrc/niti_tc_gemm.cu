@@ -2987,10 +2987,8 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
   NITI_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, tc_gemm_kernel<CTAS, MODE, ONE>, ma, mb, mc, q, acc, hdr, ctx->d_status, r.out, r.mask,
                                         r.s_a, r.s_w, r.s_out, r.b_out, slot, r.pool_out));
   ctx->launches++;
-  if (MODE != 2) {                   // (the counters of the header cover the kernel without its strided form)
-    ctx->tc_launches++;
-    if (CTAS == 2) ctx->tc2_launches++;
-  }
+  ctx->tc_launches++;
+  if (CTAS == 2) ctx->tc2_launches++;
   return NITI_OK;
 }
 
