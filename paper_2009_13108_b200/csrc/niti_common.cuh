@@ -218,8 +218,7 @@ __device__ __forceinline__ unsigned niti_load_bytes4(const int8_t *p, int n) {
 // words; with more, the first CTA alone does and answers into a mailbox of 16 bytes per CTA that only that CTA polls, because
 // the reads of a few L2 lines by everybody delay the posts (3100 cycles for 64 CTAs, 6000 - 8000 for 128; one call with 98
 // CTAs 12.0 -> 10.5 us, with 64 14.1 -> 13.0 us, with 144 16.0 -> 13.7 us; with 16 6.9 us directly, 7.5 us through
-// mailboxes).  `extra` more words in front of the area have to be posted first; `ordered`: what this block writes afterwards
-// comes after what the other blocks read before they posted (release at the post, acquire at the result).
+// mailboxes).  `extra` more words in front of the area have to be posted first.
 //
 // Nothing promises that all blocks of a launch are on the GPU at the same time: launches of two streams can each hold a part
 // of the SMs.  So no block waits until all have come.  Out of patience, it leaves its sums in memory, marks its post, counts
@@ -234,11 +233,8 @@ __device__ __forceinline__ unsigned niti_load_bytes4(const int8_t *p, int n) {
 #define NITI_LEFT 0x10000u                         // mark in a post: its block left its share in memory
 #define NITI_PATIENCE (1u << 19)                   // about 0.3 ms; the blocks of an undisturbed launch post within a few us
 __device__ __forceinline__ unsigned niti_agree_bits(unsigned *posts, unsigned *mail, int bits, int cta, int n, int extra, int lane,
-                                                    unsigned patience, bool ordered = false) {
-  if (lane == 0) {
-    if (ordered) __threadfence();
-    *(volatile unsigned *)(posts + cta) = (unsigned)bits + 1u;
-  }
+                                                    unsigned patience) {
+  if (lane == 0) *(volatile unsigned *)(posts + cta) = (unsigned)bits + 1u;
   if (patience == 0u && (cta & 1)) return 0u;      // (test switch: every other block leaves, whoever has come)
   const long long t0 = clock64();
   auto late = [&]() { return __any_sync(0xffffffffu, clock64() - t0 > (long long)patience) != 0; };
@@ -263,7 +259,6 @@ __device__ __forceinline__ unsigned niti_agree_bits(unsigned *posts, unsigned *m
       if (late()) return 0u;
     }
     m = __reduce_max_sync(0xffffffffu, m);
-    if (ordered) __threadfence();
     if (n > NITI_AGREE_DIRECT)
       for (int i = lane; i < n; i += 32) *(volatile unsigned *)(mail + 4 * i) = m;
     return m;
@@ -272,10 +267,7 @@ __device__ __forceinline__ unsigned niti_agree_bits(unsigned *posts, unsigned *m
   while (true) {
     if (lane == 0) m = *(volatile unsigned *)(mail + 4 * cta);
     m = __shfl_sync(0xffffffffu, m, 0);
-    if (m) {
-      if (ordered) __threadfence();
-      return m;
-    }
+    if (m) return m;
     if (late()) return 0u;
   }
 }

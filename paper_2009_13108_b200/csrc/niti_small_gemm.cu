@@ -328,11 +328,11 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   if (lane == 0 && mx) atomicMax(&cta_max, mx);
   __syncthreads();
   // agreement over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after op[0]'s reads of
-  // the same weights: an update waits for op[0]'s CTAs as well, and the fences of the exchange stand between the two.
+  // the same weights: an update waits for op[0]'s CTAs as well.
   if (warp == 0) {
     unsigned *words = niti_split_max(p.hdr);
     const unsigned m = niti_agree_bits(words + first, words + NITI_AGREE_MAX + 4 * first, niti_bitlen32(cta_max), cta, o.ctas,
-                                       o.upd ? first : 0, lane, p.patience, p.op[1].upd != nullptr);
+                                       o.upd ? first : 0, lane, p.patience);
     if (lane == 0) agreed = m;
   }
   if (tid == 32) ticket = came;
