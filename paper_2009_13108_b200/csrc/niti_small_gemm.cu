@@ -328,7 +328,9 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   if (lane == 0 && mx) atomicMax(&cta_max, mx);
   __syncthreads();
   // agreement over the CTAs of this multiply.  The exchange also orders the weight update of op[1] after op[0]'s reads of
-  // the same weights: an update waits for op[0]'s CTAs as well.
+  // the same weights: an update waits for op[0]'s CTAs as well.  (Those reads have returned, into shared memory and behind a
+  // barrier, before op[0] posts, and a write issued after the post was seen cannot reach a read that has returned.  Fences or
+  // acquiring loads on top of that cost a captured MLP step 43.4 -> 45.1 - 46.0 us.)
   if (warp == 0) {
     unsigned *words = niti_split_max(p.hdr);
     const unsigned m = niti_agree_bits(words + first, words + NITI_AGREE_MAX + 4 * first, niti_bitlen32(cta_max), cta, o.ctas,
