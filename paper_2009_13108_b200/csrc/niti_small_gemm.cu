@@ -8,11 +8,11 @@
 // (m16n8k32, int8) from shared memory, and the CTAs (at most one per SM) exchange their maxima through words of the
 // workspace header.  (One cluster of up to 16 CTAs that exchanges them through distributed shared memory measured the
 // same at 4 M multiply-accumulates, 5.4 against 5.2 us, and slower above, 8.2 against 5.8 us at 256^3.)
-// Measured (graph replay, forward / backward call, tcgen05 kernel -> this): 64 x 256 x 784 12.0 / 21.1 -> 7.0 / 8.4 us,
-// 256 x 256 x 256 9.8 / 20.7 -> 5.4 / 7.9 us, 512 x 512 x 512 10.8 / 22.7 -> 8.6 / 13.7 us, 1000 x 500 x 250 (rows that
-// TMA needs padded) 15.9 / 60.1 -> 15.2 / 17.4 us, 256 x 10 x 512 (CUDA-core backward before) 9.5 / 35.3 -> 5.8 / 7.5 us.
-// The line at NITI_SMALL_MACS: at 134 M 8.6 - 8.8 against 10.7 - 10.8 us forward and 13.7 - 15.4 against 22.7 - 27.0 us
-// backward; at 268 M 9.4 - 11.2 against 10.5 - 13.3 us and 19.2 - 27.6 against 27.4 - 29.3 us, about even.
+// Measured (graph replay, forward / backward call, other kernels -> this): 256 x 10 x 512 9.0 / 36.0 -> 6.6 / 8.0 us, 512 x 512
+// x 256 8.6 / 18.3 -> 7.0 / 12.0, 512 x 512 x 512 9.4 / 18.5 -> 8.7 / 14.2, 512 x 512 x 700 13.0 / 24.0 -> 11.9 / 15.2, 64 x
+// 1024 x 2048 12.3 / 20.0 -> 10.1 / 20.2.
+// The line at NITI_SMALL_MACS: at 134 - 185 M multiply-accumulates as above; at 268 M 10.4 - 10.6 -> 10.1 - 10.3 us forward and
+// 19.1 - 24.1 -> 16.8 - 24.0 us backward, about even; at 537 M 10.8 / 21.0 - 23.4 -> 11.9 - 12.1 / 23.4 - 27.9 us.
 //
 // Contraction order.  mma.sync wants k = 4t .. 4t+3 and 16 + 4t .. from thread t of a group; any permutation of k that
 // both operands share gives the same sums, so a thread takes the 16 contiguous bytes at 16 t of a 64-byte step: one
@@ -379,6 +379,22 @@ bool pick_regions(SmallOp &o, int max_ctas) {
   return best < 1e30;
 }
 
+// Staging that the tcgen05 kernel beats, whatever the number of multiply-accumulates.  (1) A contraction that does not fit
+// shared memory in one piece: the pieces are loaded one after the other, and the regions are few (forward 64 x 128 x 9216 25.6
+// against 9.7 us, 256 x 100 x 4096 15.6 / 10.5, 96 x 512 x 4000 15.5 / 11.4; backward 20000 x 64 x 64 128 / 24, 8192 x 128 x
+// 128 59 / 21, 4096 x 128 x 256 33 / 23; in one piece 64 x 1024 x 2600 13.0 / 17.2, 3000 x 300 x 200 23.6 / 30.7).  (2) Rows
+// that begin at any byte, which go through registers at about 0.125 us per KB: 1000 x 500 x 370 (47 KB per CTA) 15.6 / 12.8
+// us, 500 x 300 x 999 (96 KB) 21.3 / 14.9, with 368 and 992 elements 9.4 / 10.7 and 9.9 / 11.2.
+constexpr long long SMALL_ANY_BYTE = 24 * 1024;
+bool slow_staging(const SmallOp &o) {
+  const long long rows = (!o.a_mn && (o.lda & 3) ? o.rm : 0) + (!o.b_mn && (o.ldb & 3) ? o.rn : 0);
+  return o.kc < o.gk || rows * o.gk > SMALL_ANY_BYTE;
+}
+// Beside the CUDA-core engine (backward, fewer than 32 outputs) pieces still pay up to this contraction: gradient of 8192 x 10 x
+// 9216 90 against 503 us, 2048 x 31 x 4096 20 / 225, 4096 x 10 x 1024 28 / 101, 16384 x 10 x 1024 96 / 105, 32768 x 10 x 1024
+// 186 / 200, but 65536 x 10 x 784 360 / 276.
+constexpr long long SMALL_NARROW_K = 32768;
+
 }  // namespace
 
 static void fill_op(SmallOp &o, const GemmProblem &g, const RoundSpec &r) {
@@ -416,6 +432,8 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
   const int n = ctx->sm_count < NITI_AGREE_MAX ? ctx->sm_count : NITI_AGREE_MAX;
   if (!pick_regions(p.op[0], g2 ? n / 2 : n)) return NITI_ERR_SHAPE;
   if (g2 && !pick_regions(p.op[1], n - p.op[0].ctas)) return NITI_ERR_SHAPE;
+  if (narrow ? g.gk > SMALL_NARROW_K || (g2 && g2->gk > SMALL_NARROW_K) : slow_staging(p.op[0]) || (g2 && slow_staging(p.op[1])))
+    return NITI_ERR_SHAPE;
   const int grid = p.op[0].ctas + p.op[1].ctas;
   size_t smem = region_smem(p.op[0].rm, p.op[0].rn, p.op[0].kc);
   if (g2) {

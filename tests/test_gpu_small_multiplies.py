@@ -19,7 +19,8 @@ def niti():
 @pytest.mark.parametrize("M,N,K", [
     (1, 1, 1), (31, 33, 65), (33, 10, 257), (64, 31, 64), (65, 97, 130),       # remainders of tiles and steps
     (7, 129, 36), (40, 50, 72), (96, 64, 1023),                                # row pitches of 4, 8 and odd bytes
-    (16, 48, 20000), (128, 10, 6000),                                          # contractions staged in chunks
+    (16, 48, 20000), (128, 10, 6000), (4096, 10, 70), (5000, 31, 33),          # contractions staged in chunks
+    (33, 20, 511), (500, 300, 99), (64, 33, 3137), (96, 512, 4000),            # rows at any byte, on both sides of the line
     (3000, 300, 200), (300, 3000, 200), (64, 1400, 2200)])                     # near the size limit
 def test_small_multiplies(niti, oref, M, N, K):
     rng = np.random.default_rng(M + 3 * N + 7 * K)
