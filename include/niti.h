@@ -76,7 +76,8 @@ extern "C" {
 #define NITI_OP_CONV_WGRAD_UPDATE 7 /* dims as NITI_OP_CONV_FWD    */
 
 /* device status bits returned by niti_check() */
-#define NITI_DEV_TIMEOUT 1u      /* a bounded wait inside a kernel gave up     */
+#define NITI_DEV_TIMEOUT 1u      /* a bounded wait inside a kernel gave up (blocks that wait for other blocks of
+                                  * their launch do not: they leave their share to a later one) */
 #define NITI_DEV_EXP_RANGE 2u    /* an exponent left the int8 range            */
 #define NITI_DEV_XENT_RANGE 4u   /* s_a outside [-22, 24] in niti_int_xent     */
 #define NITI_DEV_BAD_LABEL 8u    /* a label outside [0, N)                     */
@@ -222,9 +223,10 @@ int niti_conv_wgrad(niti_ctx *ctx, void *stream, const int8_t *x, const int8_t *
  * respect to x and w.  H, W are always the INPUT sizes of the forward
  * convolution; y / e have the [B][Ho][Wo][Cout] shape.  Workspace: the same op
  * ids with the stride as a ninth entry of dims.  stride = 1 is the call
- * without the suffix.  Strides up to 8 run on the tensor cores: the stride
- * becomes the traversal stride of the operand copies, and the error is
- * computed phase by phase of the input grid. */
+ * without the suffix.  On the tensor cores the stride of a forward pass or
+ * weight gradient becomes the traversal stride of the operand copies, which
+ * ends at 8 (larger strides run on the CUDA cores); the error is computed
+ * phase by phase of the input grid, with any stride. */
 int niti_conv_fwd_strided(niti_ctx *ctx, void *stream, const int8_t *x, const int32_t *s_x,
                           const int8_t *w, const int32_t *s_w, int8_t *y, int32_t *s_y, int32_t *b_y, int B,
                           int H, int W, int Cin, int Cout, int R, int S, int pad, int stride, int relu,

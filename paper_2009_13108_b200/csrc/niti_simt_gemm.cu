@@ -1,8 +1,8 @@
 // Plain CUDA-core matrix-multiply engine (dp4a) with implicit operand addressing.
 //
-// It serves the shapes the tensor-core engine does not take (tiny or oddly strided operands:
-// 10-class heads, 1- and 3-channel inputs, general R x S / pad) and lets the tests cross-check the
-// two engines against each other.  D[m][n] = sum_k A(m,k) * B(n,k), int8 x int8 -> int32
+// It serves what the tensor-core engines do not take (backward calls of large layers with fewer than 32 outputs, forward
+// passes and gradients with strides above 8, copies that no tensor map describes) and lets the tests cross-check the
+// engines against each other.  D[m][n] = sum_k A(m,k) * B(n,k), int8 x int8 -> int32
 // (Int8MatrixMultiply of Algorithm 1), for the six operand mappings in NitiGemmKind.
 #include "niti_common.cuh"
 

@@ -2441,7 +2441,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       // error: the H x W input-shaped tensor); the shifted operand is the other activation tensor and
       // may have another size (padding other than (R-1)/2, strides): its copies start at any
       // coordinate and read zeros outside it.  A forward stride becomes the element stride of those
-      // copies.  The error of a strided convolution is left to the CUDA-core engine.
+      // copies; the error of a strided convolution runs over the phases of its input grid (see dstride).
       const bool fwd = g.kind == GK_CONV_FWD;
       const int st = g.stride > 1 ? g.stride : 1;
       const int RW = fwd ? g.Wo : g.W, RH = fwd ? g.Ho : g.H;      // pixel grid of the rows
@@ -2580,8 +2580,10 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
       p.stride = st;
       // (64 x 64)-channel blocks re-read the activations once per block of the other operand and their N = 64 MMAs run
       // at two thirds of the rate: this mode is kept where the tap groups below would leave half of the MMA's rows
-      // empty (64 output channels: 119 against 203 us at 224 x 224) or spend as much on copies (128 -> 128 channels at
-      // 112 x 112: 115 against 124 us); 64 -> 128 at 56 x 56 30.5 against 26.3 us, 128 -> 256 84 against 62 us
+      // empty (64 output channels, batch 64: this / groups 121 / 211 us at 224 x 224, 40 / 66 at 112 x 112, 21 / 23 at 56 x
+      // 56, 14.4 / 14.8 at 28 x 28; 128 input channels 65 / 113 and 29 / 38, 192 91 / 156, 256 47 / 62) or spend as much on
+      // copies (128 -> 128: 115 / 125 at 112 x 112, 43 / 43 at 56 x 56, 22 / 21 at 28 x 28).  Elsewhere the groups are as
+      // good or better: 64 -> 128 65 / 65, 28 / 24 and 17 / 16 us, 64 -> 192 35 / 38, 64 -> 256 41 / 39, 128 -> 256 75 / 59
       if (want == PLAN_HALO && same && ctas == 1 && g.R == 3 && g.S == 3 && g.pad == 1 && g.Ci % 64 == 0 && g.Co % 64 == 0 &&
           g.W >= 10 && g.H >= 18 && (long long)g.Ci * g.Co <= 16384 && (g.Co == 64 || g.Ci >= 128) && !g.q0 && !g.q1) {
         p.halo = 2;
@@ -2783,7 +2785,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   // split the contraction when the tiles alone cannot fill the SMs
   if (tiles < units && p.kb_total >= 8 && p.dstride <= 1 && force_bn <= 0) {
     // pick the split count with the least modelled time: waves of items, each item running its
-    // share of the k-blocks plus a fixed cost (pipeline fill and the atomic epilogue) of about
+    // share of the k-blocks plus a fixed cost (pipeline fill and the epilogue's reduce copies) of about
     // four k-blocks
     double best = 1e30;
     int best_s = 1;
@@ -3031,13 +3033,16 @@ static double kblock_cycles(const TcParams &p, int ctas, int bn, long long ctas_
 }
 // A multiply of at most one tile per SM: an unsplit plan whose every CTA (pair) has one tile rounds in its own epilogue
 // with an exact shift, in one launch.  Splitting the contraction shortens the main loop but costs a zeroed scratch, the
-// reduce copies and two passes over the int32 sums (measured 3.5 us + 5 us per million outputs); pairs of CTAs cost
-// 0.8 us more set-up than single ones.  Measured (graph replay, the former plan -> this one): 256 images of 4 x 4, 512
-// -> 512 channels, forward 33.3 -> 20.7, error 29.7 -> 21.7, weight gradient 30.3 -> 21.2 us; 100 images of 9 x 9, 96 ->
-// 160 channels, forward 21.5 -> 13.2, error 20.0 -> 14.2 us, but its weight gradient (64 k-blocks over 18 tiles) 16.4 us
-// split against 28.3 us unsplit: the model below draws that line.  (Splits that form a cluster and add their partial
-// tiles through distributed shared memory were built and measured: 24.3 - 25.0 us against 20.7 us unsplit on the first
-// of these; the agreement over twice as many CTAs and the exchange cost what the shorter main loop saves.)
+// reduce copies and a finishing launch over the int32 sums; pairs of CTAs cost 0.8 us more set-up than single ones.  (The
+// model's 3.5 us + 5 us per million outputs of a split were measured when two kernels finished it.)  Where the line lies
+// now, as kernels stand (graph replay, without one-wave plans -> with them): 256 images of 4 x 4, 512 -> 512 channels,
+// forward 30.6 -> 19.9, error 27.4 -> 21.1, weight gradient 27.2 -> 19.6 us; 100 images of 9 x 9, 96 -> 160, 19.3 -> 11.7,
+// 18.8 -> 13.7, 13.3 -> 14.6; 64 of 7 x 7, 256 -> 512, 26.3 -> 14.6, 19.8 -> 19.1, 21.9 -> 16.6; 128 of 8 x 8, 128 -> 256,
+// 20.8 -> 11.9, 20.6 -> 14.4, 16.8 -> 17.5; 256 of 2 x 2, 512 -> 512, 17.6 -> 18.3, 18.2 -> 18.9, 22.1 -> 12.7; fully
+// connected 1024^3 forward 16.1 -> 11.5, backward 32.7 -> 22.6 us, 4096 x 1000 x 512 14.0 -> 14.0 and 43.3 -> 33.2: a few
+// gradients are up to 10 % slower, nothing else is.  (Splits that form a cluster and add their partial tiles through
+// distributed shared memory were built and measured: 24.3 - 25.0 us against 20.7 us unsplit on the first of these; the
+// agreement over twice as many CTAs and the exchange cost what the shorter main loop saves.)
 static bool pick_one_wave(niti_ctx *ctx, const GemmProblem &g, const TcParams &p, int &ctas, int &bn) {
   const int units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
   if (p.halo || p.mrep > 1 || p.dstride > 1 || p.items > 4LL * units) return false;
