@@ -1068,6 +1068,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   };
 
+  const bool epi_warp = warp >= EPI_WARP0 && ((warp - EPI_WARP0) >> 2) % wpq < wpq_active;
   if (warp < PROD_WARPS) {
     // ================= TMA producers (every CTA loads its own rows of A and its share of B) ========
     // Each producer warp runs its loop in lock step and one elected lane issues the copies (warp-uniform
@@ -1417,17 +1418,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       }
     }
-  } else if (((warp - EPI_WARP0) >> 2) % wpq < wpq_active) {
+  } else if (epi_warp) {
     // ================= epilogue: TMEM -> int32 accumulators + max magnitude =================
     const int quarter = warp & 3;               // TMEM lanes [32 * quarter, +32)
     const int wq = (warp - EPI_WARP0) >> 2;     // index among the four warps of this quarter
     const int egroup = wq / wpq;                // tiles use % egroups == egroup are this warp's
     const int chunk_phase = wq % wpq;           // it takes 32-column chunks phase, phase + wpq, ...
     const int row_in_tile = quarter * 32 + lane;
-    unsigned use = 0;
     unsigned mx = 0;
     int bp = 0;
-    int h_wt = 0, h_ht = 0, h_bt = 0;
     if (epi_mode == EPI_KNOWN_B) {
       const int b = niti_bitlen32(hdr->maxabs32);
       bp = b > p.mbits ? b - p.mbits : 0;
@@ -1435,6 +1434,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     bool ok = true;
     const unsigned red_buf = smem_base + (unsigned)p.red_off + (unsigned)(warp - EPI_WARP0) * 4096u;
     if (!ONE && p.halo == 2) {
+      unsigned use = 0;
       // lane = (tap of the pair, input channel), column = output channel; partial sums of this
       // CTA's pixel range are added to g32[co][tap][ci]
       const int which = row_in_tile >> 6, ci = row_in_tile & 63;
@@ -1470,508 +1470,300 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       item_end = first_item;
     }
-    use = (unsigned)egroup;
-    unsigned ebuf = (unsigned)egroup, epar = 0;       // use % nbuf, (use / nbuf) & 1 (nbuf is a multiple of egroups)
-    // what the fused rounding needs and no tile changes: the rounding constants (replaced once, when the
-    // speculative binary point is agreed) and the alignment of the output and mask rows
-    RoundConst rk = make_round_const(bp, p.mbits, p.round_mode);
+    // alignment of the output and mask rows
     const bool io_aligned = ((p.gn & 31) == 0) && (((uintptr_t)out8 & 31) == 0) &&
-                            (mask8 == nullptr || ((uintptr_t)mask8 & 31) == 0);
-    // the lean loop takes over after a warp's first item (which may be the CTA's speculative first
-    // tile) when every chunk of every tile is whole and aligned
-    const bool lean_ok = !ONE && (epi_mode == EPI_KNOWN_B || epi_mode == EPI_SPECULATE) && p.splits == 1 &&
-                         (p.bn & 31) == 0 && p.halo != 2 && p.kind != GK_CONV_WGRAD &&
-                         (p.mrep == 1 || (io_aligned && p.gn == p.bn_mma && mask8 == nullptr));
-    // (otherwise: the largest store unit of the output rows, and this warp's staging buffer)
-    const unsigned io_bits = (unsigned)p.gn | (unsigned)(uintptr_t)out8 | 16u | (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
-    const int io_unit = (int)(io_bits & (0u - io_bits));
-    unsigned *nstg = reinterpret_cast<unsigned *>(smem_raw + (smem_base - smem_u32(smem_raw)) + p.nstg_off) +
-                     (warp - EPI_WARP0) * (32 * 9);
-    int lean_item = -1;
-    Extremes ex_all = {0, 0, 0u};
+                            (mask8 == nullptr || ((uintptr_t)mask8 & 31) == 0) &&
+                            (p.kind != GK_CONV_WGRAD || (p.Cn & 31) == 0);
+    const bool fused = epi_mode == EPI_KNOWN_B || epi_mode == EPI_SPECULATE;
+    bool unaligned_bp = false;                   // binary point above 24: the lean loop leaves the items to the general one
+    // (rows that are not 32-byte aligned: the largest store unit of the output rows, and this warp's staging buffer)
+    auto io_unit = [&]() {
+      const unsigned io_bits = (unsigned)p.gn | (unsigned)(uintptr_t)out8 | 16u | (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
+      return (int)(io_bits & (0u - io_bits));
+    };
+    auto nstg = [&]() {
+      return reinterpret_cast<unsigned *>(smem_raw + (smem_base - smem_u32(smem_raw)) + p.nstg_off) + (warp - EPI_WARP0) * (32 * 9);
+    };
     // this thread's pixel inside a pixel box (generic convolutions): the box sides are powers of two
-    const int wt_d = p.Wt > 0 ? p.Wt : 1, ht_d = p.Ht > 0 ? p.Ht : 1;     // (unset for plain matrix multiplies)
-    const int r_ww = row_in_tile % wt_d, r_t = row_in_tile / wt_d;
-    const int r_hh = r_t % ht_d, r_bb = r_t / ht_d;
-    for (int item = first_item + egroup * item_step; ok && item < item_end;
-         item += item_step * egroups, use += (unsigned)egroups) {
-      int mu = 0, nt = 0, split = 0;
+    struct BoxPixel { int w, h, b; };
+    auto box_pixel = [&]() {
+      const int wt_d = p.Wt > 0 ? p.Wt : 1, ht_d = p.Ht > 0 ? p.Ht : 1;   // (unset for plain matrix multiplies)
+      const int t = row_in_tile / wt_d;
+      return BoxPixel{row_in_tile - t * wt_d, t % ht_d, t / ht_d};
+    };
+    // an item's tile: this thread's output row (row-batched mode: in the first of the item's mrep tiles), first column,
+    // columns inside the matrix
+    struct Tile {
+      int mt, nt, split, ncols_valid;
+      long long out_row, col0;
+      bool row_ok;
+    };
+    auto tile_of = [&](int item) {
+      Tile t = {0, 0, 0, 0, 0, 0, false};
       Phase phq = {0, 0, 1, 1};
+      int mu = 0;
       if (!p.halo) {
         int tile = item;
         if (STRIDED) phq = split_phase(p, item, tile);
-        decode_item(p, tile, mu, nt, split);
+        decode_item(p, tile, mu, t.nt, t.split);
       }
-      const int mt = mu * CTAS + (int)rank;
-      const unsigned buf = ebuf;
-      const unsigned tpar = epar;
-      ebuf += (unsigned)egroups;
-      if (ebuf >= (unsigned)p.nbuf) { ebuf -= (unsigned)p.nbuf; epar ^= 1u; }
-      // output row / column base of this thread
-      long long out_row;
-      bool row_ok;
-      long long col0;
-      int ncols_valid;
+      t.mt = mu * CTAS + (int)rank;
+      t.col0 = (long long)t.nt * p.bn;
+      const long long rem = p.gn - t.col0;
+      t.ncols_valid = rem < p.bn ? (int)rem : p.bn;
       if (p.halo) {
-        // 8 x 16 pixel tiles of one image, visited in order: coordinates are stepped, not divided
-        if (use == (unsigned)egroup) {
-          tile_coords(p, item, h_wt, h_ht, h_bt);
-        }
-        const int w = h_wt * 8 + (row_in_tile & 7), h = h_ht * 16 + (row_in_tile >> 3);
-        row_ok = w < p.PW && h < p.PH;
-        out_row = ((long long)h_bt * p.PH + h) * p.PW + w;
-        col0 = 0;
-        ncols_valid = (int)p.gn;
-        for (int st = 0; st < egroups; ++st)
-          if (++h_wt == p.w_tiles) { h_wt = 0; if (++h_ht == p.h_tiles) { h_ht = 0; ++h_bt; } }
+        int wt, ht, bt;
+        tile_coords(p, item, wt, ht, bt);
+        const int w = wt * 8 + (row_in_tile & 7), h = ht * 16 + (row_in_tile >> 3);
+        t.row_ok = w < p.PW && h < p.PH;
+        t.out_row = ((long long)bt * p.PH + h) * p.PW + w;
       } else if (STRIDED) {
-        out_row = phase_row(p, mt * BM + row_in_tile, phq, row_ok);
-        col0 = (long long)nt * p.bn;
-        long long rem = p.gn - col0;
-        ncols_valid = rem < p.bn ? (int)rem : p.bn;
+        t.out_row = phase_row(p, t.mt * BM + row_in_tile, phq, t.row_ok);
       } else if ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) {
         int w0, h0, b0;
-        pixel_box(p, mt, w0, h0, b0);
-        const int ww = r_ww, hh = r_hh, bb = r_bb;
-        int w = w0 + ww, h = h0 + hh, b = b0 + bb;
-        row_ok = w < p.PW && h < p.PH && b < p.PB;
-        out_row = ((long long)b * p.PH + h) * p.PW + w;
-        col0 = (long long)nt * p.bn;
-        long long rem = p.gn - col0;
-        ncols_valid = rem < p.bn ? (int)rem : p.bn;
-      } else if (p.kind == GK_CONV_WGRAD) {
-        out_row = (long long)mt * BM + row_in_tile;
-        row_ok = out_row < p.gm;
-        int tap = nt / p.n_chunks, ci0 = (nt % p.n_chunks) * p.bn;
-        col0 = (long long)tap * p.Cn + ci0;
-        int rem = p.Cn - ci0;
-        ncols_valid = rem < p.bn && p.tg <= 1 ? rem : p.bn;
+        pixel_box(p, t.mt, w0, h0, b0);
+        const BoxPixel px = box_pixel();
+        const int w = w0 + px.w, h = h0 + px.h, b = b0 + px.b;
+        t.row_ok = w < p.PW && h < p.PH && b < p.PB;
+        t.out_row = ((long long)b * p.PH + h) * p.PW + w;
       } else {
-        // (row-batched mode: the row of the first of the item's mrep tiles; column chunk c of the
-        // accumulator then belongs to tile c / bn_mma)
-        out_row = (long long)mt * (BM * p.mrep) + row_in_tile;
-        row_ok = out_row < p.gm;
-        col0 = (long long)nt * p.bn;
-        long long rem = p.gn - col0;
-        ncols_valid = rem < p.bn ? (int)rem : p.bn;
-      }
-      // fused 2 x 2 max-pool (convolutions only): this lane's pixel and the row of its window in the pooled tensor
-      long long pool_row = 0;
-      if (p.pool) {
-        const long long pw = out_row % p.PW, t2 = out_row / p.PW;
-        const long long ph = t2 % p.PH, pb = t2 / p.PH;
-        pool_row = (pb * (p.PH >> 1) + (ph >> 1)) * (p.PW >> 1) + (pw >> 1);
-      }
-      if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
-      tc_fence_after();
-      const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)p.bn;
-      if (epi_mode == EPI_ATOMIC && p.red) {
-        // partial sums of a split contraction: every chunk is staged and added by one copy
-        unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
-        int x0, x1, x2 = 0, x3 = 0;                            // tensor coordinates of the chunk at column 0
+        t.out_row = (long long)t.mt * (BM * p.mrep) + row_in_tile;
+        t.row_ok = t.out_row < p.gm;
         if (p.kind == GK_CONV_WGRAD) {
-          const int tap = nt / p.n_chunks;
-          x0 = (nt - tap * p.n_chunks) * p.bn;
-          x1 = tap;
-          x2 = mt * BM + quarter * 32;
-        } else if (p.red == 2) {                               // pixel boxes
-          x0 = (int)col0;
-          int w0, h0, b0;
-          pixel_box(p, mt, w0, h0, b0);
-          x1 = __shfl_sync(0xffffffffu, w0 + r_ww, 0);
-          x2 = __shfl_sync(0xffffffffu, h0 + r_hh, 0);
-          x3 = __shfl_sync(0xffffffffu, b0 + r_bb, 0);
-        } else {
-          x0 = (int)col0;
-          x1 = mt * BM + quarter * 32;
+          const int tap = t.nt / p.n_chunks, ci0 = (t.nt - tap * p.n_chunks) * p.bn;
+          t.col0 = (long long)tap * p.Cn + ci0;
+          t.ncols_valid = p.Cn - ci0 < p.bn && p.tg <= 1 ? p.Cn - ci0 : p.bn;
         }
-        const bool any_row = __any_sync(0xffffffffu, row_ok);
-        for (int c = 32 * chunk_phase; c < p.bn && c < ncols_valid && any_row; c += 32 * wpq) {
-          int xc = x0 + c, xt = x1;
-          if (p.kind == GK_CONV_WGRAD && p.tg > 1) {           // tap group: tg_cols (a power of two) columns per tap
-            xt = nt * p.tg + c / p.tg_cols;
-            xc = c & (p.tg_cols - 1);
-            if (xt >= p.R * p.S || xc >= p.Cn) continue;
-          }
-          int v[32];
-          tc_ld32(tm_row + (unsigned)c, v);
-          // (rows and columns outside the matrix are clipped by the copy; they may hold anything)
-          if (row_ok) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) pmx = max(pmx, (unsigned)abs(v[j]));
-          }
-          if (lane == 0) tma_reduce_wait_read();
-          __syncwarp();
-          stage_tile32<false>(red_buf, lane, v);
-          fence_async_shared();
-          __syncwarp();
-          if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, xc, xt, x2, x3);
-        }
-        pmx = __reduce_max_sync(0xffffffffu, pmx);
-        if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
-      } else if (epi_mode <= EPI_ATOMIC) {
-        int32_t *dst = acc + out_row * p.gn + col0;
-        const bool vec_ok = ((p.gn & 3) == 0) && ((col0 & 3) == 0);
-        unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
-        for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
-          int v[32];
-          tc_ld32(tm_row + (unsigned)c, v);
-          if (row_ok && c < ncols_valid) {
-            if (epi_mode == EPI_ATOMIC) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (c + j < ncols_valid && v[j] != 0) {
-                  pmx = max(pmx, (unsigned)abs(v[j]));
-                  atomicAdd(dst + c + j, v[j]);
-                }
+      }
+      return t;
+    };
+    // The first tile of this CTA has largest magnitude m0 in this warp's share.  True in the warp that has spoken for the CTA.
+    auto report = [&](unsigned m0) {
+      m0 = __reduce_max_sync(0xffffffffu, m0);
+      // The warps of this CTA combine their maxima in shared memory; the last one to report speaks
+      // for the CTA in the grid-wide agreement (one atomic and one poller per CTA: with every warp
+      // of every CTA polling the same word the wait itself took microseconds) and publishes the
+      // shift to the others through shared memory.
+      unsigned last = 0;
+      if (lane == 0) {
+        if (m0) atomicMax(&first_max, m0);
+        __threadfence_block();
+        last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
+      }
+      if (ONE) {
+        // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
+        if (__shfl_sync(0xffffffffu, last, 0)) {
+          unsigned *words = niti_split_max(hdr);
+          const unsigned agreed = niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(*(volatile unsigned *)&first_max),
+                                                  (int)blockIdx.x, (int)gridDim.x, 0, lane, p.patience);
+          if (lane == 0) {
+            if (agreed) {
+              const int b = (int)agreed - 1, bpf = b > p.mbits ? b - p.mbits : 0;
+              spec_bp_ready = bpf + 1;
+              if (blockIdx.x == 0) publish_exact(b);
             } else {
-              if (vec_ok && c + 32 <= ncols_valid) {
-#pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                  *reinterpret_cast<int4 *>(dst + c + j) = make_int4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                }
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                  unsigned a = v[j] < 0 ? 0u - (unsigned)v[j] : (unsigned)v[j];
-                  mx = a > mx ? a : mx;
-                }
-              } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                  if (c + j < ncols_valid) {
-                    dst[c + j] = v[j];
-                    unsigned a = v[j] < 0 ? 0u - (unsigned)v[j] : (unsigned)v[j];
-                    mx = a > mx ? a : mx;
-                  }
-              }
+              spec_bp_ready = -1;
             }
           }
         }
-        if (epi_mode == EPI_ATOMIC) {
-          pmx = __reduce_max_sync(0xffffffffu, pmx);
-          if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
-        }
-      } else {
-        bool leaves = false;                                   // (see niti_agree_bits)
-        if (!ONE && epi_mode == EPI_SPECULATE && use == (unsigned)egroup && egroup != 0) {
-          // the group that drains this CTA's first tile publishes the shift through shared memory
+      } else if (lane == 0) {
+        if (last) {
+          const unsigned cm = *(volatile unsigned *)&first_max;
+          if (cm) atomicMax(&hdr->est_max, cm);
+          __threadfence();
+          atomicAdd(&hdr->tile_counter, 1u);
+          // The bit-width is fixed as soon as a quorum of CTAs has reported, by whichever CTA sees
+          // that first (compare-and-swap on the published word); CTAs that start late find it
+          // published and never wait.  Waiting for every CTA meant waiting out the launch ramp of
+          // the whole grid (~10 k cycles) in every launch.  Where not even a quorum comes (launches of several
+          // streams share the SMs), a CTA out of patience fixes it from what has been reported: the bit-width
+          // is a guess in any case, and the follow-up launch corrects a wrong one.
+          const unsigned quorum = (unsigned)p.quorum;
+          unsigned pub = 0;
           long long t0 = clock64();
-          while (spec_bp_ready == 0) {
-            if (abort_flag) break;
-            if (clock64() - t0 > WAIT_LIMIT_CYCLES) {
-              abort_flag = 1;
-              atomicOr(status, NITI_DEV_TIMEOUT);
+          while (true) {
+            // one 16-byte load: {est_max, tile_counter, spec_b, -}
+            unsigned v_max, v_cnt, v_pub, v_pad;
+            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v_max), "=r"(v_cnt), "=r"(v_pub), "=r"(v_pad)
+                         : "l"(&hdr->est_max)
+                         : "memory");
+            if (v_pub) { pub = v_pub; break; }
+            if (v_cnt >= quorum || clock64() - t0 > (long long)p.patience) {
+              // (the 16-byte load is not promised to be one atomic snapshot: once the count is seen,
+              // the maximum is read again, after a fence, so that it is at least as new as the count)
+              __threadfence();
+              v_max = *(volatile unsigned *)&hdr->est_max;
+              // the first tiles are a sample: scale their max by the growth expected from the sample
+              // to the whole tensor before taking the bit length (a wrong guess only costs the redo)
+              unsigned long long scaled = ((unsigned long long)v_max * p.spec_mul256) >> 8;
+              if (scaled > 0x7fffffffull) scaled = 0x7fffffffull;
+              // plus what the same estimate missed by at this call site last time (a systematic
+              // error of the sample, e.g. a tensor whose extremes sit outside the first tiles); never
+              // below the bit length of the sample's own maximum, which the tensor's cannot undercut
+              int guess = niti_bitlen32((unsigned)scaled);
+              if (spec_slot && p.spec_mul256 != 256 && *(volatile int *)&spec_slot[0] == p.spec_tag)
+                guess += spec_correction(*(volatile int *)&spec_slot[1]);
+              const int floor_b = niti_bitlen32(v_max);
+              guess = guess < floor_b ? floor_b : (guess > 31 ? 31 : guess);
+              const unsigned mine = (unsigned)guess + 1u;
+              const unsigned old = atomicCAS(&hdr->spec_b, 0u, mine);
+              pub = old ? old : mine;
               break;
             }
+            if (abort_flag) break;
           }
-          if (abort_flag) { ok = false; break; }
-          bp = spec_bp_ready - 1;
-          rk = make_round_const(bp, p.mbits, p.round_mode);
-        }
-        if (epi_mode == EPI_SPECULATE && use == 0) {
-          // first tile of this CTA: max only, then agree on the estimate with the whole grid
-          // (columns of a partly filled chunk beyond the matrix accumulate zeros; whole chunks beyond it are left out)
-          const int cend0 = p.mrep > 1 ? p.bn : (ncols_valid < p.bn ? ncols_valid : p.bn);
-          int hi0 = 0, lo0 = 0;
-          for (int c = 32 * chunk_phase; c < cend0; c += 32 * wpq) {
-            int v[32];
-            tc_ld32(tm_row + (unsigned)c, v);
-            bool rok = row_ok;
-            if (p.mrep > 1) rok = out_row + (long long)(c / p.bn_mma) * BM < p.gm;
-            if (rok) {
-#pragma unroll
-              for (int j = 0; j < 32; j += 2) {
-                hi0 = __vimax3_s32(hi0, v[j], v[j + 1]);
-                lo0 = __vimin3_s32(lo0, v[j], v[j + 1]);
-              }
-            }
-          }
-          unsigned m0 = max((unsigned)hi0, 0u - (unsigned)lo0);
-          m0 = __reduce_max_sync(0xffffffffu, m0);
-          // The warps of this CTA combine their maxima in shared memory; the last one to report speaks
-          // for the CTA in the grid-wide agreement (one atomic and one poller per CTA: with every warp
-          // of every CTA polling the same word the wait itself took microseconds) and publishes the
-          // shift to the others through shared memory.
-          unsigned last = 0;
-          if (lane == 0) {
-            if (m0) atomicMax(&first_max, m0);
-            __threadfence_block();
-            last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
-          }
-          if (ONE) {
-            // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
-            if (__shfl_sync(0xffffffffu, last, 0)) {
-              unsigned *words = niti_split_max(hdr);
-              const unsigned agreed = niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(*(volatile unsigned *)&first_max),
-                                                      (int)blockIdx.x, (int)gridDim.x, 0, lane, p.patience);
-              if (lane == 0) {
-                if (agreed) {
-                  const int b = (int)agreed - 1, bpf = b > p.mbits ? b - p.mbits : 0;
-                  spec_bp_ready = bpf + 1;
-                  if (blockIdx.x == 0) publish_exact(b);
-                } else {
-                  spec_bp_ready = -1;
-                }
-              }
-            }
-          } else if (lane == 0) {
-            if (last) {
-              const unsigned cm = *(volatile unsigned *)&first_max;
-              if (cm) atomicMax(&hdr->est_max, cm);
-              __threadfence();
-              atomicAdd(&hdr->tile_counter, 1u);
-              // The bit-width is fixed as soon as a quorum of CTAs has reported, by whichever CTA sees
-              // that first (compare-and-swap on the published word); CTAs that start late find it
-              // published and never wait.  Waiting for every CTA meant waiting out the launch ramp of
-              // the whole grid (~10 k cycles) in every launch.  Where not even a quorum comes (launches of several
-              // streams share the SMs), a CTA out of patience fixes it from what has been reported: the bit-width
-              // is a guess in any case, and the follow-up launch corrects a wrong one.
-              const unsigned quorum = (unsigned)p.quorum;
-              unsigned pub = 0;
-              long long t0 = clock64();
-              while (true) {
-                // one 16-byte load: {est_max, tile_counter, spec_b, -}
-                unsigned v_max, v_cnt, v_pub, v_pad;
-                asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                             : "=r"(v_max), "=r"(v_cnt), "=r"(v_pub), "=r"(v_pad)
-                             : "l"(&hdr->est_max)
-                             : "memory");
-                if (v_pub) { pub = v_pub; break; }
-                if (v_cnt >= quorum || clock64() - t0 > (long long)p.patience) {
-                  // (the 16-byte load is not promised to be one atomic snapshot: once the count is seen,
-                  // the maximum is read again, after a fence, so that it is at least as new as the count)
-                  __threadfence();
-                  v_max = *(volatile unsigned *)&hdr->est_max;
-                  // the first tiles are a sample: scale their max by the growth expected from the sample
-                  // to the whole tensor before taking the bit length (a wrong guess only costs the redo)
-                  unsigned long long scaled = ((unsigned long long)v_max * p.spec_mul256) >> 8;
-                  if (scaled > 0x7fffffffull) scaled = 0x7fffffffull;
-                  // plus what the same estimate missed by at this call site last time (a systematic
-                  // error of the sample, e.g. a tensor whose extremes sit outside the first tiles); never
-                  // below the bit length of the sample's own maximum, which the tensor's cannot undercut
-                  int guess = niti_bitlen32((unsigned)scaled);
-                  if (spec_slot && p.spec_mul256 != 256 && *(volatile int *)&spec_slot[0] == p.spec_tag)
-                    guess += spec_correction(*(volatile int *)&spec_slot[1]);
-                  const int floor_b = niti_bitlen32(v_max);
-                  guess = guess < floor_b ? floor_b : (guess > 31 ? 31 : guess);
-                  const unsigned mine = (unsigned)guess + 1u;
-                  const unsigned old = atomicCAS(&hdr->spec_b, 0u, mine);
-                  pub = old ? old : mine;
-                  break;
-                }
-                if (abort_flag) break;
-              }
-              const int b = (int)pub - 1;
-              spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
-            }
-          }
-          if (lane == 0) {
-            long long t1 = clock64();
-            while (spec_bp_ready == 0) {
-              if (abort_flag) break;
-              if (clock64() - t1 > WAIT_LIMIT_CYCLES) {
-                abort_flag = 1;
-                atomicOr(status, NITI_DEV_TIMEOUT);
-                break;
-              }
-            }
-          }
-          __syncwarp();
-          if (abort_flag) { ok = false; break; }
-          leaves = ONE && spec_bp_ready < 0;
-          bp = leaves ? 0 : spec_bp_ready - 1;
-          rk = make_round_const(bp, p.mbits, p.round_mode);
-        }
-        // Whole 32-column chunks with 32-byte aligned rows (every layer of the networks): the chunk
-        // loop below does nothing per chunk but load, round and store; pointers are stepped.  (The
-        // epilogue warps share their schedulers' integer pipe, which is the bound of layers with few
-        // input channels: every instruction here is paid for 16 times per tile.)
-        const bool whole_chunks = io_aligned && ((col0 & 31) == 0) &&
-                                  (p.mrep > 1 ? ncols_valid >= p.bn_mma : (ncols_valid & 31) == 0);
-        if (ONE && leaves) {
-          for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
-            int v[32];
-            tc_ld32(tm_row + (unsigned)c, v);
-            const int jt = p.mrep > 1 ? c / p.bn_mma : 0, cc = c - jt * p.bn_mma;
-            const long long orow = out_row + (long long)jt * BM;
-            if (!row_ok || (p.mrep > 1 && orow >= p.gm)) continue;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (cc + j < ncols_valid) acc[orow * p.gn + col0 + cc + j] = v[j];
-          }
-        } else if (whole_chunks) {
-          const bool relu = p.relu != 0;
-          // (the last column tile of a row may be narrower than the tile: its chunks beyond the
-          // matrix are not read at all)
-          const int cstep = 32 * wpq, bn = p.mrep > 1 ? p.bn : (ncols_valid < p.bn ? ncols_valid : p.bn);
-          const int bn_mma = p.mrep > 1 ? p.bn_mma : p.bn;
-          const long long row_off = out_row * p.gn + col0;
-          const long long sub_stride = (long long)BM * p.gn;      // next 128-row tile of a row-batched item
-          int8_t *drow = out8 + row_off;
-          const int8_t *mrow = mask8 ? mask8 + row_off : nullptr;
-          long long orow = out_row;
-          int cc = 32 * chunk_phase;
-          while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (mrow) mrow += sub_stride; }
-          for (int c = 32 * chunk_phase; c < bn; c += cstep) {
-            int v[32];
-            const bool rok = row_ok && orow < p.gm;
-            unsigned m[8];
-            unsigned pw8[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};     // pooling input of lanes outside the tensor
-            if ((mrow || p.update) && rok)        // the ReLU mask, or the weights this chunk updates
-              asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                           : "=r"(m[0]), "=r"(m[1]), "=r"(m[2]), "=r"(m[3]), "=r"(m[4]), "=r"(m[5]), "=r"(m[6]), "=r"(m[7])
-                           : "l"((p.update ? (const int8_t *)drow : mrow) + cc));
-            tc_ld32(tm_row + (unsigned)c, v);
-            if (rok) {
-              unsigned w8[8];
-              Extremes ex = {0, 0, 0u};
-              round_chunk32(v, w8, rk, relu, ex);
-              mx |= ex.magnitude_bits();
-              if (p.update) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) w8[j] = bytes_sub_clamp127(m[j], w8[j]);
-              } else if (mrow) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) w8[j] &= bytes_gt0(m[j]);
-              }
-              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                           ::"l"(drow + cc), "r"(w8[0]), "r"(w8[1]), "r"(w8[2]), "r"(w8[3]), "r"(w8[4]), "r"(w8[5]),
-                             "r"(w8[6]), "r"(w8[7])
-                           : "memory");
-              if (p.pool) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) pw8[j] = w8[j];
-              }
-            }
-            if (p.pool) {                          // (warp-uniform: every lane takes part in the exchange)
-              pool_chunk32(pw8, p.pool_xh);
-              if (rok && (lane & (1 | p.pool_xh)) == 0) store32(pool8 + pool_row * p.gn + col0 + cc, pw8);
-            }
-            cc += cstep;
-            while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (mrow) mrow += sub_stride; }
-          }
-        } else if (GENERAL)
-        for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
-          int v[32];
-          // chunk geometry: in row-batched mode chunk c holds columns cc of the item's tile c / bn_mma
-          int cc = c;
-          long long orow = out_row;
-          bool rok = row_ok;
-          if (p.mrep > 1) {
-            const int jt = c / p.bn_mma;
-            cc = c - jt * p.bn_mma;
-            orow = out_row + (long long)jt * BM;
-            rok = orow < p.gm;
-          }
-          const int nv = ncols_valid - cc;                       // (uniform across the warp)
-          if (nv <= 0) continue;
-          const long long off = orow * p.gn + col0 + cc;
-          // (the ReLU mask bytes are fetched first: their latency overlaps the TMEM load and the rounding)
-          unsigned m[8], w8[8];
-          if (mask8 && rok) load_row_narrow(mask8 + off, m, nv < 32 ? nv : 32);
-          tc_ld32(tm_row + (unsigned)c, v);
-          if (rok) {
-            Extremes ex = {0, 0, 0u};                            // (columns beyond the matrix accumulate zeros)
-            round_chunk32(v, w8, rk, p.relu != 0, ex);
-            mx |= ex.magnitude_bits();
-            if (mask8) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j) w8[j] &= bytes_gt0(m[j]);
-            }
-          }
-          store_rows_narrow(out8, off, rok, w8, nv, io_unit, nstg, lane);
+          const int b = (int)pub - 1;
+          spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
         }
       }
-      tc_fence_before();
-      __syncwarp();
+      return __shfl_sync(0xffffffffu, last, 0) != 0;
+    };
+    // The agreed binary point (in spec_bp_ready), once it is there; false: time to leave.
+    auto await_bp = [&]() {
       if (lane == 0) {
-        if (CTAS == 2 && rank != 0) mbar_arrive_cluster(lead_tempty0 + 8 * buf);
-        else mbar_arrive(tempty0 + 8 * buf);
+        const long long t1 = clock64();
+        while (spec_bp_ready == 0) {
+          if (abort_flag) break;
+          if (clock64() - t1 > WAIT_LIMIT_CYCLES) {
+            abort_flag = 1;
+            atomicOr(status, NITI_DEV_TIMEOUT);
+            break;
+          }
+        }
       }
-      if (lean_ok && rk.aligned) {                 // the rest of this warp's items: lean loop below
-        lean_item = item + item_step * egroups;
-        use += (unsigned)egroups;
-        break;
-      }
-    }
-    // ---- lean loop: fused rounding of whole, aligned chunks (every layer of the networks) ----
+      __syncwarp();
+      return abort_flag == 0;
+    };
+    // ---- lean loop: fused rounding (every layer of the networks) ----
     // The epilogue warps share their schedulers' integer pipe with everything else, and with few
     // input channels that pipe is the bound of the whole kernel: per tile and per chunk this loop
-    // executes only what changes (measured on the first layer: the general loop above spends a third
-    // of its integer instructions on tests whose outcome is the same for every tile).
-    if (!ONE && ok && lean_item >= 0) {
-      auto lean = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c, auto narrow_c) {
-        constexpr bool NARROW = decltype(narrow_c)::value;   // output rows that are not 32-byte aligned, short last chunks
-        constexpr bool RELU = decltype(relu_c)::value, MASK = decltype(mask_c)::value, BATCHED = decltype(batched_c)::value;
-        constexpr bool POOL = decltype(pool_c)::value;       // fused 2 x 2 max-pool of the ReLU'd tile
-        constexpr bool UPD = decltype(upd_c)::value;         // the output rows are weights: subtract the rounded gradient
-        const int pool_xh = p.pool_xh;
-        const bool pool_lane = (lane & (1 | pool_xh)) == 0;  // the window's top-left pixel stores the maximum
-        const int kind = STRIDED ? 3 : (p.halo ? 0 : (((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) ? 1 : 2));
-        const int istep = item_step * egroups, nbuf = p.nbuf, bn = p.bn, n_tiles_n = p.n_tiles_n;
-        const int cstep = 32 * wpq, c_first = 32 * chunk_phase;
-        const long long gn = p.gn, gm = p.gm;
-        const int bn_mma = BATCHED ? p.bn_mma : p.bn;
-        const long long sub_stride = (long long)BM * gn;
-        const bool counted = p.blocked && p.raster_g <= 0 && kind != 3;     // consecutive items: (mu, nt) are stepped
-        int mu = 0, nt = 0, split = 0;
-        Phase phq = {0, 0, 1, 1};
-        if (kind == 3) {
-          int tile;
-          phq = split_phase(p, lean_item, tile);
-          decode_item(p, tile, mu, nt, split);
-        } else if (kind != 0) decode_item(p, lean_item, mu, nt, split);
-        for (int item = lean_item; item < item_end; item += istep) {
-          const unsigned buf = ebuf, tpar = epar;
-          ebuf += (unsigned)egroups;
-          if (ebuf >= (unsigned)nbuf) { ebuf -= (unsigned)nbuf; epar ^= 1u; }
-          long long out_row;
-          bool row_ok;
-          long long pool_row = 0;
-          if (kind == 0) {
-            const int w = h_wt * 8 + (row_in_tile & 7), h = h_ht * 16 + (row_in_tile >> 3);
-            row_ok = w < p.PW && h < p.PH;
-            out_row = ((long long)h_bt * p.PH + h) * p.PW + w;
-            if (POOL) pool_row = ((long long)h_bt * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
-            h_wt += egroups;
-            while (h_wt >= p.w_tiles) { h_wt -= p.w_tiles; if (++h_ht == p.h_tiles) { h_ht = 0; ++h_bt; } }
-          } else if (kind == 1) {
-            int w0, h0, b0;
-            pixel_box(p, mu * CTAS + (int)rank, w0, h0, b0);
-            const int w = w0 + r_ww, h = h0 + r_hh, b = b0 + r_bb;
-            row_ok = w < p.PW && h < p.PH && b < p.PB;
-            out_row = ((long long)b * p.PH + h) * p.PW + w;
-            if (POOL) pool_row = ((long long)b * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
-          } else if (kind == 3) {
-            out_row = phase_row(p, (mu * CTAS + (int)rank) * BM + row_in_tile, phq, row_ok);
-          } else {
-            out_row = (long long)(mu * CTAS + (int)rank) * (BM * p.mrep) + row_in_tile;
-            row_ok = out_row < gm;
+    // executes only what changes (measured on the first layer: a loop that tests the launch's options per tile and
+    // chunk spends a third of its integer instructions on tests whose outcome is the same for every tile).
+    // Code that is not in the SM's instruction cache costs about 8 ns an instruction (lines of 128 bytes, 70 - 100 ns each), and
+    // in a program of different kernels that is every launch: rounding the first tile took 4.3 us instead of the 1.9 us of a
+    // launch that repeats.  While the bit-width is being agreed, the warps therefore take a chunk through the loop body without
+    // storing it (`live` false).
+    auto lean_as = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c, auto narrow_c) {
+      constexpr bool NARROW = decltype(narrow_c)::value;   // output rows that are not 32-byte aligned, short last chunks
+      constexpr bool RELU = decltype(relu_c)::value, MASK = decltype(mask_c)::value, BATCHED = decltype(batched_c)::value;
+      constexpr bool POOL = decltype(pool_c)::value;       // fused 2 x 2 max-pool of the ReLU'd tile
+      constexpr bool UPD = decltype(upd_c)::value;         // the output rows are weights: subtract the rounded gradient
+      const int pool_xh = p.pool_xh;
+      const bool pool_lane = (lane & (1 | pool_xh)) == 0;  // the window's top-left pixel stores the maximum
+      const int kind = STRIDED ? 3 : (p.halo ? 0 : (((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) ? 1
+                                                    : (p.kind == GK_CONV_WGRAD ? 4 : 2)));
+      const int istep = item_step * egroups, nbuf = p.nbuf, bn = p.bn, n_tiles_n = p.n_tiles_n;
+      const int cstep = 32 * wpq, c_first = 32 * chunk_phase;
+      const long long gn = p.gn, gm = p.gm;
+      const int bn_mma = BATCHED ? p.bn_mma : p.bn;
+      const long long sub_stride = (long long)BM * gn;      // next 128-row tile of a row-batched item
+      const bool counted = p.blocked && p.raster_g <= 0 && kind != 3;     // consecutive items: (mu, nt) are stepped
+      const int lean_item = first_item + egroup * item_step;
+      unsigned ebuf = (unsigned)egroup, epar = 0;           // use % nbuf, (use / nbuf) & 1 (nbuf is a multiple of egroups)
+      Extremes ex_all = {0, 0, 0u};
+      RoundConst rk = make_round_const(bp, p.mbits, p.round_mode);
+      const BoxPixel bpx = kind == 1 ? box_pixel() : BoxPixel{0, 0, 0};
+      int mu = 0, nt = 0, split = 0, h_wt = 0, h_ht = 0, h_bt = 0;
+      if (epi_mode == EPI_KNOWN_B && !rk.aligned) { unaligned_bp = true; return; }
+      Phase phq = {0, 0, 1, 1};
+      if (kind == 3) {
+        int tile;
+        phq = split_phase(p, lean_item, tile);
+        decode_item(p, tile, mu, nt, split);
+      } else if (kind != 0) decode_item(p, lean_item, mu, nt, split);
+      else tile_coords(p, lean_item, h_wt, h_ht, h_bt);
+      for (int item = lean_item; item < item_end; item += istep) {
+        const unsigned buf = ebuf, tpar = epar;
+        ebuf += (unsigned)egroups;
+        if (ebuf >= (unsigned)nbuf) { ebuf -= (unsigned)nbuf; epar ^= 1u; }
+        long long out_row;
+        bool row_ok;
+        long long pool_row = 0;
+        int col0 = nt * bn;
+        int cend = BATCHED ? bn : (int)(gn - col0);          // (whole chunks unless NARROW)
+        if (kind == 0) {
+          const int w = h_wt * 8 + (row_in_tile & 7), h = h_ht * 16 + (row_in_tile >> 3);
+          row_ok = w < p.PW && h < p.PH;
+          out_row = ((long long)h_bt * p.PH + h) * p.PW + w;
+          if (POOL) pool_row = ((long long)h_bt * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
+          h_wt += egroups;
+          while (h_wt >= p.w_tiles) { h_wt -= p.w_tiles; if (++h_ht == p.h_tiles) { h_ht = 0; ++h_bt; } }
+        } else if (kind == 1) {
+          int w0, h0, b0;
+          pixel_box(p, mu * CTAS + (int)rank, w0, h0, b0);
+          const int w = w0 + bpx.w, h = h0 + bpx.h, b = b0 + bpx.b;
+          row_ok = w < p.PW && h < p.PH && b < p.PB;
+          out_row = ((long long)b * p.PH + h) * p.PW + w;
+          if (POOL) pool_row = ((long long)b * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
+        } else if (kind == 3) {
+          out_row = phase_row(p, (mu * CTAS + (int)rank) * BM + row_in_tile, phq, row_ok);
+        } else {
+          out_row = (long long)(mu * CTAS + (int)rank) * (BM * p.mrep) + row_in_tile;
+          row_ok = out_row < gm;
+          if (kind == 4) {
+            const int tap = nt / p.n_chunks, ci0 = (nt - tap * p.n_chunks) * bn;
+            col0 = tap * p.Cn + ci0;
+            cend = p.Cn - ci0;
           }
-          const int col0 = nt * bn;
-          int cend = BATCHED ? bn : (int)(gn - col0);          // (whole chunks unless NARROW)
-          if (cend > bn) cend = bn;
-          if (kind != 0) {                                      // next item of this warp
-            if (counted) { nt += egroups; while (nt >= n_tiles_n) { nt -= n_tiles_n; ++mu; } }
-            else if (item + istep < item_end) {
-              int tile = item + istep;
-              if (kind == 3) phq = split_phase(p, item + istep, tile);
-              decode_item(p, tile, mu, nt, split);
+        }
+        if (cend > bn) cend = bn;
+        if (kind != 0) {                                      // next item of this warp
+          if (counted) { nt += egroups; while (nt >= n_tiles_n) { nt -= n_tiles_n; ++mu; } }
+          else if (item + istep < item_end) {
+            int tile = item + istep;
+            if (kind == 3) phq = split_phase(p, item + istep, tile);
+            decode_item(p, tile, mu, nt, split);
+          }
+        }
+        const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)bn;
+        int live = 1, warm_chunks = 1;
+        if (epi_mode == EPI_SPECULATE && item == lean_item) {
+          live = 0;
+          if (egroup == 0) {
+            // first tile of this CTA: max only, then agree on the estimate with the whole grid (columns of a partly filled
+            // chunk beyond the matrix accumulate zeros; whole chunks beyond it are left out)
+            int hi0 = 0, lo0 = 0, t = 0;
+            asm volatile("" : "+r"(t));                 // (one copy of the loop: the first, empty pass is for the instruction cache)
+#pragma unroll 1
+            for (; t < 2; ++t) {
+              if (t && !mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
+              tc_fence_after();
+              hi0 = lo0 = 0;
+              const int ce = t ? cend : c_first + 1;
+              for (int c = c_first; c < ce; c += cstep) {
+                int v[32];
+                tc_ld32(tm_row + (unsigned)c, v);
+                if (row_ok && (!BATCHED || out_row + (long long)(c / bn_mma) * BM < gm)) {
+#pragma unroll
+                  for (int j = 0; j < 32; j += 2) {
+                    hi0 = __vimax3_s32(hi0, v[j], v[j + 1]);
+                    lo0 = __vimin3_s32(lo0, v[j], v[j + 1]);
+                  }
+                }
+              }
             }
+            if (!ok) break;
+            if (report(max((unsigned)hi0, 0u - (unsigned)lo0))) warm_chunks = 0;
           }
-          if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
-          tc_fence_after();
-          const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)bn;
-          const long long row_off = out_row * gn + col0;
+        } else if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const long long row_off = out_row * gn + col0;
+#pragma unroll 1
+        while (true) {
           int8_t *drow = out8 + row_off;
           const int8_t *mrow = MASK ? mask8 + row_off : nullptr;
           int8_t *prow = POOL ? pool8 + pool_row * gn + col0 : nullptr;
           long long orow = out_row;
           int cc = c_first;
           if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (MASK) mrow += sub_stride; }
-          for (int c = c_first; c < cend; c += cstep) {
+          const int ce = live ? cend : c_first + warm_chunks;
+          for (int c = c_first; c < ce; c += cstep) {
             int v[32];
-            const bool rok = BATCHED ? (row_ok && orow < gm) : row_ok;
+            const bool rok = (BATCHED ? (row_ok && orow < gm) : row_ok) && live != 0;       // (rows that are read and written)
             unsigned m[8];
             if (NARROW) {
               if (MASK && rok) load_row_narrow(mrow + cc, m, cend - c < 32 ? cend - c : 32);
@@ -1982,19 +1774,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             tc_ld32(tm_row + (unsigned)c, v);
             unsigned w8[8];
             if (POOL) {
-#pragma unroll
+  #pragma unroll
               for (int j = 0; j < 8; ++j) w8[j] = 0u;          // lanes outside the tensor pool zeros
             }
-            if (rok) {
-#pragma unroll
+            if (rok || !live) {
+  #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 w8[j] = round_pack4_aligned<RELU>(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3], rk, ex_all);
                 if (MASK) w8[j] &= bytes_gt0(m[j]);
                 if (UPD) w8[j] = bytes_sub_clamp127(m[j], w8[j]);
               }
-              if (!NARROW) store32(drow + cc, w8);
+              if (!NARROW && rok) store32(drow + cc, w8);
             }
-            if (NARROW) store_rows_narrow(out8, row_off + cc, rok, w8, cend - c, io_unit, nstg, lane);
+            if (NARROW) store_rows_narrow(out8, drow - out8 + cc, rok, w8, BATCHED ? (int)gn - cc : cend - c, io_unit(), nstg(), lane);
             if (POOL) {                                        // (warp-uniform: all lanes exchange)
               pool_chunk32(w8, pool_xh);
               if (rok && pool_lane) store32(prow + cc, w8);
@@ -2002,29 +1794,202 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             cc += cstep;
             if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (MASK) mrow += sub_stride; }
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) {
-            if (CTAS == 2 && rank != 0) mbar_arrive_cluster(lead_tempty0 + 8 * buf);
-            else mbar_arrive(tempty0 + 8 * buf);
+          if (live) break;
+          if (!await_bp()) { ok = false; break; }
+          if (ONE && spec_bp_ready < 0) {                      // (this CTA leaves: see niti_agree_bits)
+            for (int c = c_first; c < cend; c += cstep) {
+              int v[32];
+              tc_ld32(tm_row + (unsigned)c, v);
+              if (!row_ok) continue;
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (c + j < cend) acc[row_off + c + j] = v[j];
+            }
+            ok = false;
+            break;
           }
+          bp = spec_bp_ready - 1;
+          rk = make_round_const(bp, p.mbits, p.round_mode);
+          ex_all = Extremes{0, 0, 0u};
+          if (!rk.aligned) { unaligned_bp = true; break; }
+          if (egroup != 0 && !mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
+          tc_fence_after();
+          live = 1;
+          asm volatile("" : "+r"(live));                       // (one copy of the loop)
         }
-      };
+        if (!ok || unaligned_bp) break;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (CTAS == 2 && rank != 0) mbar_arrive_cluster(lead_tempty0 + 8 * buf);
+          else mbar_arrive(tempty0 + 8 * buf);
+        }
+      }
+      mx |= ex_all.magnitude_bits();
+    };
+    auto lean = [&]() {
       using T = std::true_type;
       using F = std::false_type;
-      const bool relu = p.relu != 0, masked = mask8 != nullptr, batched = p.mrep > 1;
-      if (batched) { if (relu) lean(T{}, F{}, T{}, F{}, F{}, F{}); else lean(F{}, F{}, T{}, F{}, F{}, F{}); }   // (row-batched: forward only)
-      else if (GENERAL && !io_aligned) {
-        if (relu) lean(T{}, F{}, F{}, F{}, F{}, T{});                                                      // (ReLU: forward, no mask)
-        else if (masked) lean(F{}, T{}, F{}, F{}, F{}, T{});
-        else lean(F{}, F{}, F{}, F{}, F{}, T{});
+      const bool relu = p.relu != 0, masked = mask8 != nullptr;
+      if (!ONE && p.mrep > 1) {                                                                                 // (row-batched: forward only)
+        if (GENERAL && (!io_aligned || p.gn != p.bn_mma)) {
+          if (relu) lean_as(T{}, F{}, T{}, F{}, F{}, T{}); else lean_as(F{}, F{}, T{}, F{}, F{}, T{});
+        } else if (relu) lean_as(T{}, F{}, T{}, F{}, F{}, F{});
+        else lean_as(F{}, F{}, T{}, F{}, F{}, F{});
+      } else if (GENERAL && !io_aligned) {
+        if (relu) lean_as(T{}, F{}, F{}, F{}, F{}, T{});                                                  // (ReLU: forward, no mask)
+        else if (masked) lean_as(F{}, T{}, F{}, F{}, F{}, T{});
+        else lean_as(F{}, F{}, F{}, F{}, F{}, T{});
+      } else if (p.update) lean_as(F{}, F{}, F{}, F{}, T{}, F{});                                         // (weight gradients: signed, no mask)
+      else if (p.pool) lean_as(T{}, F{}, F{}, T{}, F{}, F{});                                             // (pooling: ReLU, no mask)
+      else if (relu) lean_as(T{}, F{}, F{}, F{}, F{}, F{});
+      else if (masked) lean_as(F{}, T{}, F{}, F{}, F{}, F{});
+      else lean_as(F{}, F{}, F{}, F{}, F{}, F{});
+    };
+    // ---- the loop for everything else: accumulators kept, partial sums, rounding that the lean loop does not do ----
+    auto general = [&]() {
+      unsigned use = (unsigned)egroup, ebuf = (unsigned)egroup, epar = 0;
+      const RoundConst rk = make_round_const(bp, p.mbits, p.round_mode);
+      for (int item = first_item + egroup * item_step; ok && item < item_end;
+           item += item_step * egroups, use += (unsigned)egroups) {
+        const Tile t = tile_of(item);
+        const int mt = t.mt, nt = t.nt, split = t.split, ncols_valid = t.ncols_valid;
+        const long long out_row = t.out_row, col0 = t.col0;
+        const bool row_ok = t.row_ok;
+        const unsigned buf = ebuf;
+        const unsigned tpar = epar;
+        ebuf += (unsigned)egroups;
+        if (ebuf >= (unsigned)p.nbuf) { ebuf -= (unsigned)p.nbuf; epar ^= 1u; }
+        if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
+        tc_fence_after();
+        const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)p.bn;
+        if (epi_mode == EPI_ATOMIC && p.red) {
+          // partial sums of a split contraction: every chunk is staged and added by one copy
+          unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
+          int x0, x1, x2 = 0, x3 = 0;                            // tensor coordinates of the chunk at column 0
+          if (p.kind == GK_CONV_WGRAD) {
+            const int tap = nt / p.n_chunks;
+            x0 = (nt - tap * p.n_chunks) * p.bn;
+            x1 = tap;
+            x2 = mt * BM + quarter * 32;
+          } else if (p.red == 2) {                               // pixel boxes
+            x0 = (int)col0;
+            int w0, h0, b0;
+            pixel_box(p, mt, w0, h0, b0);
+            const BoxPixel px = box_pixel();
+            x1 = __shfl_sync(0xffffffffu, w0 + px.w, 0);
+            x2 = __shfl_sync(0xffffffffu, h0 + px.h, 0);
+            x3 = __shfl_sync(0xffffffffu, b0 + px.b, 0);
+          } else {
+            x0 = (int)col0;
+            x1 = mt * BM + quarter * 32;
+          }
+          const bool any_row = __any_sync(0xffffffffu, row_ok);
+          for (int c = 32 * chunk_phase; c < p.bn && c < ncols_valid && any_row; c += 32 * wpq) {
+            int xc = x0 + c, xt = x1;
+            if (p.kind == GK_CONV_WGRAD && p.tg > 1) {           // tap group: tg_cols (a power of two) columns per tap
+              xt = nt * p.tg + c / p.tg_cols;
+              xc = c & (p.tg_cols - 1);
+              if (xt >= p.R * p.S || xc >= p.Cn) continue;
+            }
+            int v[32];
+            tc_ld32(tm_row + (unsigned)c, v);
+            // (rows and columns outside the matrix are clipped by the copy; they may hold anything)
+            if (row_ok) {
+  #pragma unroll
+              for (int j = 0; j < 32; ++j) pmx = max(pmx, (unsigned)abs(v[j]));
+            }
+            if (lane == 0) tma_reduce_wait_read();
+            __syncwarp();
+            stage_tile32<false>(red_buf, lane, v);
+            fence_async_shared();
+            __syncwarp();
+            if (lane == 0) tma_reduce_add_4d(&map_c, red_buf, xc, xt, x2, x3);
+          }
+          pmx = __reduce_max_sync(0xffffffffu, pmx);
+          if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
+        } else if (epi_mode <= EPI_ATOMIC) {
+          int32_t *dst = acc + out_row * p.gn + col0;
+          const bool vec_ok = ((p.gn & 3) == 0) && ((col0 & 3) == 0);
+          unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
+          for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
+            int v[32];
+            tc_ld32(tm_row + (unsigned)c, v);
+            if (row_ok && c < ncols_valid) {
+              if (epi_mode == EPI_ATOMIC) {
+  #pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  if (c + j < ncols_valid && v[j] != 0) {
+                    pmx = max(pmx, (unsigned)abs(v[j]));
+                    atomicAdd(dst + c + j, v[j]);
+                  }
+              } else {
+                if (vec_ok && c + 32 <= ncols_valid) {
+  #pragma unroll
+                  for (int j = 0; j < 32; j += 4) {
+                    *reinterpret_cast<int4 *>(dst + c + j) = make_int4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                  }
+  #pragma unroll
+                  for (int j = 0; j < 32; ++j) {
+                    unsigned a = v[j] < 0 ? 0u - (unsigned)v[j] : (unsigned)v[j];
+                    mx = a > mx ? a : mx;
+                  }
+                } else {
+  #pragma unroll
+                  for (int j = 0; j < 32; ++j)
+                    if (c + j < ncols_valid) {
+                      dst[c + j] = v[j];
+                      unsigned a = v[j] < 0 ? 0u - (unsigned)v[j] : (unsigned)v[j];
+                      mx = a > mx ? a : mx;
+                    }
+                }
+              }
+            }
+          }
+          if (epi_mode == EPI_ATOMIC) {
+            pmx = __reduce_max_sync(0xffffffffu, pmx);
+            if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
+          }
+        } else {
+          // Whole 32-column chunks with 32-byte aligned rows (binary points above 24), or any rows.
+          const bool whole_chunks = io_aligned && ((col0 & 31) == 0) &&
+                                    (p.mrep > 1 ? ncols_valid >= p.bn_mma : (ncols_valid & 31) == 0);
+          for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
+            // chunk geometry: in row-batched mode chunk c holds columns cc of the item's tile c / bn_mma
+            const int jt = p.mrep > 1 ? c / p.bn_mma : 0, cc = c - jt * p.bn_mma;
+            const long long orow = out_row + (long long)jt * BM, off = orow * p.gn + col0 + cc;
+            const bool rok = row_ok && (p.mrep == 1 || orow < p.gm);
+            const int nv = ncols_valid - cc;                     // (uniform across the warp)
+            if (nv <= 0) continue;
+            // (the bytes of the ReLU mask, or the weights this chunk updates, are fetched first)
+            int v[32];
+            unsigned m[8], w8[8];
+            const int8_t *const src = p.update ? (const int8_t *)out8 : mask8;
+            if (src && rok) load_row_narrow(src + off, m, nv < 32 ? nv : 32);
+            tc_ld32(tm_row + (unsigned)c, v);
+            if (rok) {
+              Extremes ex = {0, 0, 0u};                          // (columns beyond the matrix accumulate zeros)
+              round_chunk32(v, w8, rk, p.relu != 0, ex);
+              mx |= ex.magnitude_bits();
+              if (src) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) w8[j] = p.update ? bytes_sub_clamp127(m[j], w8[j]) : w8[j] & bytes_gt0(m[j]);
+              }
+            }
+            if (whole_chunks) { if (rok) store32(out8 + off, w8); }
+            else if (GENERAL) store_rows_narrow(out8, off, rok, w8, nv, io_unit(), nstg(), lane);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (CTAS == 2 && rank != 0) mbar_arrive_cluster(lead_tempty0 + 8 * buf);
+          else mbar_arrive(tempty0 + 8 * buf);
+        }
       }
-      else if (p.update) lean(F{}, F{}, F{}, F{}, T{}, F{});                                              // (weight gradients: signed, no mask)
-      else if (p.pool) lean(T{}, F{}, F{}, T{}, F{}, F{});                                                // (pooling: ReLU, no mask)
-      else if (relu) lean(T{}, F{}, F{}, F{}, F{}, F{});
-      else { if (masked) lean(F{}, T{}, F{}, F{}, F{}, F{}); else lean(F{}, F{}, F{}, F{}, F{}, F{}); }
-      mx |= ex_all.magnitude_bits();
-    }
+    };
+    if (fused) lean();
+    if (!fused || unaligned_bp) general();
     if (epi_mode == EPI_SPILL || epi_mode == EPI_SPECULATE) {
       for (int o = 16; o > 0; o >>= 1) {
         unsigned u = __shfl_xor_sync(0xffffffffu, mx, o);

@@ -1,0 +1,54 @@
+"""Forms of the fused rounding that the layers of the networks do not reach (bit-exact against the CPU oracle's rounding):
+binary points above 24, and row-batched first layers whose rows are not whole 32-byte chunks."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def niti():
+    from paper_2009_13108_b200 import Niti
+    n = Niti(0)
+    yield n
+    n.check()
+    n.close()
+
+
+@pytest.mark.parametrize("engine,N,K", [(2, 1280, 4096), (2, 1250, 4100), (0, 512, 1024)])   # many tiles, odd rows, one wave
+def test_binary_points_above_24(niti, oref, engine, N, K):
+    M = 4096
+    g = torch.Generator(device=niti.device)
+    g.manual_seed(N)
+    a = torch.full((M, K), 127, dtype=torch.int8, device=niti.device)
+    a[::3] = torch.randint(-127, 128, a[::3].shape, generator=g, dtype=torch.int8, device=niti.device)
+    e = torch.full((M, N), 127, dtype=torch.int8, device=niti.device)
+    e[:, 1::2] = torch.randint(-127, 128, e[:, 1::2].shape, generator=g, dtype=torch.int8, device=niti.device)
+    e[:, 2::4] = -127
+    w = torch.randint(-127, 128, (N, K), generator=g, dtype=torch.int8, device=niti.device)
+    acc = (e.double().T @ a.double()).cpu().numpy().astype(np.int32)       # (sums below 2^27: exact)
+    niti.set_engine(engine)
+    try:
+        for mode in (0, 1):
+            want, b, _ = oref.shift_round(acc, 1, mode)
+            assert b > 25
+            _, got, _, b_g = niti.linear_bwd(a, e, w, False, m_u=1, round_mode=mode)
+            assert int(b_g) == b and np.array_equal(got.cpu().numpy(), want)
+            wt = w.clone()
+            niti.linear_bwd_update(a, e, wt, need_e_prev=False, m_u=1, round_mode=mode)
+            assert np.array_equal(wt.cpu().numpy(), oref.sgd_update(w.cpu().numpy(), want))
+    finally:
+        niti.set_engine(0)
+
+
+@pytest.mark.parametrize("cout,cin", [(10, 3), (40, 1), (97, 3)])
+def test_row_batched_first_layers_with_odd_rows(niti, oref, cout, cin):
+    rng = np.random.default_rng(cout)
+    x = rng.integers(-127, 128, size=(48, 60, 64, cin), dtype=np.int8)
+    w = rng.integers(-127, 128, size=(cout, 3, 3, cin), dtype=np.int8)
+    for relu, mode in ((True, 0), (False, 1)):
+        want, s, b = oref.conv_fwd(x, -7, w, -9, 1, relu, mode)
+        y, s_y, b_y = niti.conv_fwd(torch.from_numpy(x).to(niti.device), niti.scalar(-7), torch.from_numpy(w).to(niti.device),
+                                    niti.scalar(-9), pad=1, relu=relu, round_mode=mode)
+        assert np.array_equal(y.cpu().numpy(), want) and (int(s_y), int(b_y)) == (s, b)
