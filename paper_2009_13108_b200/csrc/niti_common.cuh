@@ -82,13 +82,10 @@ struct WsHeader {
   unsigned int maxabs32;            // a value with the bit length of max |acc| (a max, or an OR of magnitudes)
   unsigned int arrived;             // agreement of a launch's blocks: low half blocks that have come, high half that left
   unsigned long long maxabs64;      // same for the 64-bit loss accumulators
-  // the three words of the speculative agreement share one 16-byte line so that one load polls them all
-  unsigned int est_max;             // max |acc| over the first tile of the CTAs that have reported
-  unsigned int tile_counter;        // CTAs that have reported
-  unsigned int spec_b;              // 0, or 1 + the bit-width the speculative epilogue rounds with
-  unsigned int hits;               // integer cross-entropy: rows whose first arg-max is the label
+  unsigned int spec_mask;           // bit b: a CTA of a speculative launch has rounded with bit-width b
+  unsigned int hits;                // integer cross-entropy: rows whose first arg-max is the label
 };
-static_assert(sizeof(WsHeader) == 32, "workspace header layout");
+static_assert(sizeof(WsHeader) == 24, "workspace header layout");
 static_assert(NITI_SPLIT_MAX_OFF + 4 * NITI_MAX_SPLITS <= NITI_HDR_SLOT_BYTES, "split maxima fit the header");
 __host__ __device__ __forceinline__ unsigned int *niti_split_max(WsHeader *hdr) {
   return reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(hdr) + NITI_SPLIT_MAX_OFF);

@@ -595,6 +595,60 @@ __device__ __forceinline__ int spec_correction(int packed) {
   return e1 == e2 ? e1 : 0;
 }
 
+// The guess at a tensor's bit-width from the first tiles of a launch's CTAs, for one converged warp of every CTA; m: largest
+// magnitude in its own first tile.  Posts and mailboxes as in niti_agree_bits: the first CTA decides as soon as a quorum has
+// posted (waiting for every CTA meant waiting out the launch ramp of the whole grid) and answers all of them.  (With a
+// maximum, a count and a published word that all CTAs poll, updated by atomics, the agreement took 3.7 - 4.4 us, a chain of
+// five trips to L2; this takes 2.0.)  A CTA out of patience (launches of several streams share the SMs) decides from what has
+// been posted by then.  Two CTAs may decide differently: every CTA reports what it rounded with (WsHeader::spec_mask), and
+// the follow-up launch recomputes unless all of them used the true bit-width.
+__device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, unsigned m, const TcParams &p,
+                                              const int32_t *spec_slot, int lane) {
+  const int cta = (int)blockIdx.x, n = (int)gridDim.x < NITI_AGREE_MAX ? (int)gridDim.x : NITI_AGREE_MAX;
+  m = min(m, 0x7ffffffeu) + 1u;
+  if (lane == 0 && cta < n) *(volatile unsigned *)(posts + cta) = m;
+  // what the same estimate missed by at this call site lately (a systematic error of the sample, e.g. a tensor whose
+  // extremes sit outside the first tiles); read while the posts are on their way
+  int correction = 0;
+  if (spec_slot && p.spec_mul256 != 256 && *(volatile const int *)&spec_slot[0] == p.spec_tag)
+    correction = spec_correction(*(volatile const int *)&spec_slot[1]);
+  const long long t0 = clock64();
+  auto late = [&]() { return __any_sync(0xffffffffu, clock64() - t0 > (long long)p.patience) != 0; };
+  if (cta != 0) {
+    unsigned answer = 0;
+    do {
+      if (lane == 0) answer = *(volatile unsigned *)(mail + 4 * (cta < n ? cta : 0));
+      answer = __shfl_sync(0xffffffffu, answer, 0);
+    } while (!answer && !late());
+    if (answer) return (int)answer - 1;
+  }
+  unsigned top;
+  while (true) {
+    unsigned seen = 0;
+    top = m;
+#pragma unroll
+    for (int u = 0; u < NITI_AGREE_MAX / 32; ++u) {
+      const int i = 32 * u + lane;
+      const unsigned w = i < n ? *(volatile unsigned *)(posts + i) : 0u;
+      seen += w ? 1u : 0u;
+      top = max(top, w);
+    }
+    if (cta != 0 || __reduce_add_sync(0xffffffffu, seen) >= (unsigned)p.quorum || late()) break;
+  }
+  top = __reduce_max_sync(0xffffffffu, top) - 1u;
+  // the first tiles are a sample: scale their max by the growth expected from the sample to the whole tensor before taking
+  // the bit length (a wrong guess only costs the second pass); never below the bit length of the sample's own maximum,
+  // which the tensor's cannot undercut
+  unsigned long long scaled = ((unsigned long long)top * p.spec_mul256) >> 8;
+  if (scaled > 0x7fffffffull) scaled = 0x7fffffffull;
+  int guess = niti_bitlen32((unsigned)scaled) + correction;
+  const int floor_b = niti_bitlen32(top);
+  guess = guess < floor_b ? floor_b : (guess > 31 ? 31 : guess);
+  if (cta == 0)
+    for (int i = lane; i < n; i += 32) *(volatile unsigned *)(mail + 4 * i) = (unsigned)guess + 1u;
+  return guess;
+}
+
 // n / d with the host's reciprocal (exact while n * d < 2^32, which the host checked), else a division
 __device__ __forceinline__ int div_tiles(int n, int d, unsigned magic) {
   return magic ? (int)__umulhi((unsigned)n, magic) : n / d;
@@ -948,7 +1002,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (epi_mode == EPI_KNOWN_B) {
     // follow-up of a speculative pass: publish the scalars, then leave unless the guess was wrong
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the first pass has completed and is visible
-    const int b_true = niti_bitlen32(hdr->maxabs32), b_est = (int)hdr->spec_b - 1;   // (stored + 1)
+    const unsigned used = hdr->spec_mask;                  // bit-widths that the CTAs rounded with
+    const int b_true = niti_bitlen32(hdr->maxabs32), b_est = used ? 31 - __clz(used) : b_true;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       if (spec_slot) {
         // remember, for the next calls from this call site, how far the sample-based estimate was off
@@ -967,7 +1022,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (s < -128 || s > 127) atomicOr(status, NITI_DEV_EXP_RANGE);
       }
     }
-    if (b_true == b_est) return;
+    if (used == 1u << (b_true & 31)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(status + 1, 1u);   // count of recomputations
   }
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -978,6 +1033,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __shared__ unsigned ticket;                 // of the agreement of a single-wave launch
   __shared__ unsigned first_max, first_arrived;   // this CTA's first tile: max magnitude, warps that reported
   __shared__ unsigned cta_max;                    // max magnitude of everything this CTA rounded
+  __shared__ int cta_b;                           // bit-width it rounded with (-1: nothing was agreed)
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const unsigned rank = CTAS == 2 ? cluster_ctarank() : 0u;
@@ -1026,6 +1082,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     first_max = 0;
     first_arrived = 0;
     cta_max = 0;
+    cta_b = -1;
   }
   if (threadIdx.x < 2 * MAX_STAGES + 2 * MAX_TBUF + 1) {
     const int bi = (int)threadIdx.x;
@@ -1541,83 +1598,32 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     auto report = [&](unsigned m0) {
       m0 = __reduce_max_sync(0xffffffffu, m0);
       // The warps of this CTA combine their maxima in shared memory; the last one to report speaks
-      // for the CTA in the grid-wide agreement (one atomic and one poller per CTA: with every warp
-      // of every CTA polling the same word the wait itself took microseconds) and publishes the
-      // shift to the others through shared memory.
+      // for the CTA in the grid-wide agreement (with every warp of every CTA polling the same word the wait
+      // itself took microseconds) and publishes the shift to the others through shared memory.
       unsigned last = 0;
       if (lane == 0) {
         if (m0) atomicMax(&first_max, m0);
         __threadfence_block();
         last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
       }
+      last = __shfl_sync(0xffffffffu, last, 0);
+      if (!last) return false;
+      unsigned *words = niti_split_max(hdr);
+      const unsigned cm = *(volatile unsigned *)&first_max;
+      int b;
       if (ONE) {
         // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
-        if (__shfl_sync(0xffffffffu, last, 0)) {
-          unsigned *words = niti_split_max(hdr);
-          const unsigned agreed = niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(*(volatile unsigned *)&first_max),
-                                                  (int)blockIdx.x, (int)gridDim.x, 0, lane, p.patience);
-          if (lane == 0) {
-            if (agreed) {
-              const int b = (int)agreed - 1, bpf = b > p.mbits ? b - p.mbits : 0;
-              spec_bp_ready = bpf + 1;
-              if (blockIdx.x == 0) publish_exact(b);
-            } else {
-              spec_bp_ready = -1;
-            }
-          }
-        }
-      } else if (lane == 0) {
-        if (last) {
-          const unsigned cm = *(volatile unsigned *)&first_max;
-          if (cm) atomicMax(&hdr->est_max, cm);
-          __threadfence();
-          atomicAdd(&hdr->tile_counter, 1u);
-          // The bit-width is fixed as soon as a quorum of CTAs has reported, by whichever CTA sees
-          // that first (compare-and-swap on the published word); CTAs that start late find it
-          // published and never wait.  Waiting for every CTA meant waiting out the launch ramp of
-          // the whole grid (~10 k cycles) in every launch.  Where not even a quorum comes (launches of several
-          // streams share the SMs), a CTA out of patience fixes it from what has been reported: the bit-width
-          // is a guess in any case, and the follow-up launch corrects a wrong one.
-          const unsigned quorum = (unsigned)p.quorum;
-          unsigned pub = 0;
-          long long t0 = clock64();
-          while (true) {
-            // one 16-byte load: {est_max, tile_counter, spec_b, -}
-            unsigned v_max, v_cnt, v_pub, v_pad;
-            asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(v_max), "=r"(v_cnt), "=r"(v_pub), "=r"(v_pad)
-                         : "l"(&hdr->est_max)
-                         : "memory");
-            if (v_pub) { pub = v_pub; break; }
-            if (v_cnt >= quorum || clock64() - t0 > (long long)p.patience) {
-              // (the 16-byte load is not promised to be one atomic snapshot: once the count is seen,
-              // the maximum is read again, after a fence, so that it is at least as new as the count)
-              __threadfence();
-              v_max = *(volatile unsigned *)&hdr->est_max;
-              // the first tiles are a sample: scale their max by the growth expected from the sample
-              // to the whole tensor before taking the bit length (a wrong guess only costs the redo)
-              unsigned long long scaled = ((unsigned long long)v_max * p.spec_mul256) >> 8;
-              if (scaled > 0x7fffffffull) scaled = 0x7fffffffull;
-              // plus what the same estimate missed by at this call site last time (a systematic
-              // error of the sample, e.g. a tensor whose extremes sit outside the first tiles); never
-              // below the bit length of the sample's own maximum, which the tensor's cannot undercut
-              int guess = niti_bitlen32((unsigned)scaled);
-              if (spec_slot && p.spec_mul256 != 256 && *(volatile int *)&spec_slot[0] == p.spec_tag)
-                guess += spec_correction(*(volatile int *)&spec_slot[1]);
-              const int floor_b = niti_bitlen32(v_max);
-              guess = guess < floor_b ? floor_b : (guess > 31 ? 31 : guess);
-              const unsigned mine = (unsigned)guess + 1u;
-              const unsigned old = atomicCAS(&hdr->spec_b, 0u, mine);
-              pub = old ? old : mine;
-              break;
-            }
-            if (abort_flag) break;
-          }
-          const int b = (int)pub - 1;
-          spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
-        }
+        b = (int)niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(cm), (int)blockIdx.x, (int)gridDim.x, 0, lane,
+                                 p.patience) - 1;
+      } else {
+        b = agree_on_guess(words, words + NITI_AGREE_MAX, cm, p, spec_slot, lane);
       }
-      return __shfl_sync(0xffffffffu, last, 0) != 0;
+      if (lane == 0) {
+        if (!ONE) cta_b = b;
+        spec_bp_ready = b < 0 ? -1 : (b > p.mbits ? b - p.mbits : 0) + 1;
+        if (ONE && b >= 0 && blockIdx.x == 0) publish_exact(b);
+      }
+      return true;
     };
     // The agreed binary point (in spec_bp_ready), once it is there; false: time to leave.
     auto await_bp = [&]() {
@@ -2007,7 +2013,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // and its stored values are not exact)
   if (ONE && threadIdx.x == 0 && spec_bp_ready > 0 && niti_bitlen32(cta_max) > p.mbits + spec_bp_ready - 1)
     atomicOr(status, NITI_DEV_INTERNAL);
-  if (!ONE && threadIdx.x == 0 && cta_max) atomicMax(&hdr->maxabs32, cta_max);
+  if (!ONE && threadIdx.x == 0) {
+    if (cta_max) atomicMax(&hdr->maxabs32, cta_max);
+    if (cta_b >= 0) atomicOr(&hdr->spec_mask, 1u << cta_b);
+  }
   if (abort_flag) {
     // give copies and MMAs still in flight time to land before shared and tensor memory go away
     long long t0 = clock64();
@@ -3122,7 +3131,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   {
     const long long units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
     const long long grid = (p.items < units ? p.items : units) * p.ctas;
-    p.quorum = (int)((grid + 1) / 2);
+    p.quorum = (int)(((grid < NITI_AGREE_MAX ? grid : NITI_AGREE_MAX) + 1) / 2);
     p.patience = ctx->patience;
   }
   p.mbits = r.mbits;
