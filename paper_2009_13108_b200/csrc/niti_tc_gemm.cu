@@ -33,8 +33,42 @@ constexpr int MAX_STAGES = 8;
 constexpr int MAX_TBUF = 8;
 constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;
 
+// n / d for 0 <= n < 2^31 as a multiplication: d > 1, s = ceil(log2 d), m = floor(2^(31 + s) / d) + 1 exceeds 2^(31 + s) / d by
+// at most 1 <= 2^s / d, so that n * m / 2^(31 + s) stays below the next integer.  (An integer division costs a lone warp 100 -
+// 200 cycles and 20 - 30 instructions, and the first copy of a launch used to wait for five of them.)
+struct Div {
+  unsigned m;               // 0: d = 1
+  int s;                    // s - 1 above
+};
+static Div make_div(long long d) {
+  if (d <= 1) return Div{0u, 0};
+  int s = 1;
+  while ((1LL << s) < d) ++s;
+  return Div{(unsigned)((1ull << (31 + s)) / (unsigned long long)d + 1), s - 1};
+}
+__device__ __forceinline__ int div_by(int n, Div d) { return d.m ? (int)(__umulhi((unsigned)n, d.m) >> d.s) : n; }
+
+// What the fused epilogue does with a launch's tiles; one instance of its loop each.
+enum LeanForm {
+  LEAN_PLAIN = 0, LEAN_RELU, LEAN_MASK, LEAN_POOL, LEAN_UPDATE,
+  LEAN_NARROW, LEAN_NARROW_RELU, LEAN_NARROW_MASK,                   // output rows that are not whole, aligned 32-byte chunks
+  LEAN_BATCHED, LEAN_BATCHED_RELU, LEAN_BATCHED_NARROW, LEAN_BATCHED_NARROW_RELU     // row-batched items
+};
+// How a tile's rows lie in the output
+enum RowKind { ROWS_HALO = 0, ROWS_BOXES, ROWS_PLAIN, ROWS_PHASES, ROWS_WGRAD };
+
 struct TcParams {
   int kind;
+  int form, row_kind;           // LeanForm, RowKind
+  int io_unit;                  // 32: output (and mask) rows are whole, aligned chunks; else the largest store unit, at most 16
+  Div d_w, d_h;                 // w_tiles, h_tiles
+  Div d_n, d_split;             // n_tiles_n, splits
+  Div d_group, d_units, d_last; // rasterisation: tiles of a group, its row units, those of the last group
+  int last_group;
+  Div d_chunks, d_S, d_cc;      // n_chunks, S, c_chunks
+  Div d_phases, d_phase_s;      // nph_r * nph_s, nph_s
+  int wt_shift, ht_shift;       // log2 of Wt, Ht (pixel boxes)
+  int k_wpq_shift;              // log2 of k_wpq
   int n_tiles_n;                // tiles along the output columns
   int kb_total;                 // k-blocks of the whole contraction
   int kb_per_split;
@@ -43,8 +77,6 @@ struct TcParams {
   // set-up arithmetic done on the host (integer divisions at kernel entry delay every launch)
   int blk_per, blk_extra;       // blocked assignment: items per CTA (pair) and how many take one more
   int k_wpq, k_wpq_active, k_epi_active, k_tmem_cols;
-  unsigned magic_w, magic_h;    // floor(2^32 / tiles) + 1 for w_tiles, h_tiles: n / d = umulhi(n, magic) while
-                                // n * d < 2^32 (0: divide)
   int quorum;                   // CTAs whose first tile must have reported before the speculative bit-width
                                 // is fixed (launches that are not single-wave)
   unsigned patience;            // cycles that CTAs wait for each other
@@ -57,7 +89,7 @@ struct TcParams {
   int nstg_off;                 // byte offset of the staging buffers for rows with a pitch that is no multiple of 8
   int mrep;                     // 128-row tiles per item (row-batched mode of short contractions), else 1
   int bn_mma;                   // N of one MMA; bn = mrep * bn_mma accumulator columns per item
-  long long gm, gn;             // output extent (rows, columns); row pitch of acc is gn
+  int gm, gn;                   // output extent (rows, columns; gm * gn < 2^31); row pitch of acc is gn
   int bn;                       // tile width (multiple of 32, <= 256)
   int kdepth;                   // contraction elements per k-block (32, 64 or 128)
   int ksteps;                   // kdepth / 32 MMAs per k-block
@@ -537,18 +569,18 @@ __device__ __forceinline__ void store32(int8_t *dst, const unsigned (&w8)[8]) {
 // costs 32 sector requests, so the chunk passes through shared memory (32 rows x 36 bytes per warp) and each
 // instruction writes whole rows.
 template <typename T>
-__device__ __forceinline__ void store_rows_staged(int8_t *out8, long long off, bool rok, int nv, const unsigned *stg, int lane) {
+__device__ __forceinline__ void store_rows_staged(int8_t *out8, unsigned off, bool rok, int nv, const unsigned *stg, int lane) {
   constexpr int LPR = 32 / (int)sizeof(T);                     // lanes per row
   const int part = lane % LPR;
   for (int r0 = 0; r0 < 32; r0 += (int)sizeof(T)) {
     const int r = r0 + lane / LPR;
-    const long long o = __shfl_sync(0xffffffffu, off, r);
+    const unsigned o = __shfl_sync(0xffffffffu, off, r);
     const int ok = __shfl_sync(0xffffffffu, rok ? 1 : 0, r);
     if (ok && part * (int)sizeof(T) < nv)
       reinterpret_cast<T *>(out8 + o)[part] = reinterpret_cast<const T *>(reinterpret_cast<const char *>(stg) + r * 36)[part];
   }
 }
-__device__ __forceinline__ void store_rows_narrow(int8_t *out8, long long off, bool rok, const unsigned (&w8)[8], int nv,
+__device__ __forceinline__ void store_rows_narrow(int8_t *out8, unsigned off, bool rok, const unsigned (&w8)[8], int nv,
                                                   int unit, unsigned *stg, int lane) {
   if (unit >= 8) {
     if (!rok) return;
@@ -649,15 +681,11 @@ __device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, u
   return guess;
 }
 
-// n / d with the host's reciprocal (exact while n * d < 2^32, which the host checked), else a division
-__device__ __forceinline__ int div_tiles(int n, int d, unsigned magic) {
-  return magic ? (int)__umulhi((unsigned)n, magic) : n / d;
-}
-// tile index -> (column tile, row tile, image) with two reciprocal multiplies
+// tile index -> (column tile, row tile, image)
 __device__ __forceinline__ void tile_coords(const TcParams &p, int idx, int &wt, int &ht, int &bt) {
-  const int t = div_tiles(idx, p.w_tiles, p.magic_w);
+  const int t = div_by(idx, p.d_w);
   wt = idx - t * p.w_tiles;
-  bt = div_tiles(t, p.h_tiles, p.magic_h);
+  bt = div_by(t, p.d_h);
   ht = t - bt * p.h_tiles;
 }
 // Coordinates of an output tile / k-block in the pixel grid of a convolution.
@@ -671,24 +699,24 @@ __device__ __forceinline__ void pixel_box(const TcParams &p, int idx, int &w0, i
 // range of items holds all phases, which have different numbers of taps, in equal shares.
 struct Phase { int r, s, n_r, n_s; };     // first tap row / column, taps of the phase
 __device__ __forceinline__ Phase split_phase(const TcParams &p, int item, int &tile) {
-  const int nph = p.nph_r * p.nph_s;
-  tile = item / nph;
-  const int ph = item - tile * nph;
+  tile = div_by(item, p.d_phases);
+  const int ph = item - tile * p.nph_r * p.nph_s;
   Phase q;
-  q.r = ph / p.nph_s;
+  q.r = div_by(ph, p.d_phase_s);
   q.s = ph - q.r * p.nph_s;
-  q.n_r = (p.R - q.r + p.dstride - 1) / p.dstride;
-  q.n_s = (p.S - q.s + p.dstride - 1) / p.dstride;
+  // (the phases before R mod stride have one tap more)
+  q.n_r = q.r + (p.T_r - 1) * p.dstride < p.R ? p.T_r : p.T_r - 1;
+  q.n_s = q.s + (p.T_s - 1) * p.dstride < p.S ? p.T_s : p.T_s - 1;
   return q;
 }
 
 // Output row of grid position `idx` of a phase of a strided error multiply; ok: it is inside the tensor.
-__device__ __forceinline__ long long phase_row(const TcParams &p, int idx, const Phase &q, bool &ok) {
+__device__ __forceinline__ int phase_row(const TcParams &p, int idx, const Phase &q, bool &ok) {
   int v, u, b;
   tile_coords(p, idx, v, u, b);
   const int jj = (v + p.u0_s) * p.dstride + q.s - p.pad, ii = (u + p.u0_r) * p.dstride + q.r - p.pad;
   ok = b < p.PB && ii >= 0 && ii < p.OH && jj >= 0 && jj < p.OW;
-  return ((long long)b * p.OH + ii) * p.OW + jj;
+  return (b * p.OH + ii) * p.OW + jj;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -829,22 +857,19 @@ __device__ __forceinline__ void decode_item(const TcParams &p, int item, int &mu
   int tile = item;
   split = 0;
   if (p.splits > 1) {
-    tile = item / p.splits;
+    tile = div_by(item, p.d_split);
     split = item - tile * p.splits;
   }
   if (p.raster_g <= 0) {
-    if (p.n_tiles_n == 1) { mu = tile; nt = 0; return; }
-    mu = tile / p.n_tiles_n;
+    mu = div_by(tile, p.d_n);
     nt = tile - mu * p.n_tiles_n;
     return;
   }
-  const int per_group = p.raster_g * p.n_tiles_n;
-  const int g = tile / per_group;
-  const int rem = tile - g * per_group;
-  int in_group = p.m_units - g * p.raster_g;
-  if (in_group > p.raster_g) in_group = p.raster_g;
-  mu = g * p.raster_g + rem % in_group;
-  nt = rem / in_group;
+  const int g = div_by(tile, p.d_group);
+  const int rem = tile - g * p.raster_g * p.n_tiles_n;
+  const bool last = g == p.last_group;
+  nt = div_by(rem, last ? p.d_last : p.d_units);
+  mu = g * p.raster_g + rem - nt * (last ? p.m_units - g * p.raster_g : p.raster_g);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -935,20 +960,20 @@ __device__ __forceinline__ void round_left_tile(const TcParams &p, int cta, int 
   if (STRIDED) phq = split_phase(p, item, tile);
   if (!p.halo) decode_item(p, tile, mu, nt, split);
   const int mt = mu * CTAS + rank;
-  long long col0 = (long long)nt * p.bn;
-  int cols = p.mrep > 1 ? (int)p.gn : (int)min((long long)p.bn, p.gn - col0);
+  int col0 = nt * p.bn;
+  int cols = min(p.bn, p.gn - col0);
   if (p.kind == GK_CONV_WGRAD) {
-    const int tap = nt / p.n_chunks, ci0 = (nt - tap * p.n_chunks) * p.bn;
-    col0 = (long long)tap * p.Cn + ci0;
+    const int tap = div_by(nt, p.d_chunks), ci0 = (nt - tap * p.n_chunks) * p.bn;
+    col0 = tap * p.Cn + ci0;
     cols = min(p.bn, p.Cn - ci0);
   }
   const bool boxes = p.halo || ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !p.i2c);
-  auto rounded = [&](long long at) {
+  auto rounded = [&](unsigned at) {
     const int q = niti_round_i32(__ldcg(acc + at), bp, qmax, p.round_mode);
     return p.relu && q < 0 ? 0 : q;
   };
-  for (int r = (int)(threadIdx.x >> 5); r < BM * p.mrep; r += NUM_THREADS / 32) {
-    long long row;
+  for (int r = (int)(threadIdx.x >> 5); r < BM; r += NUM_THREADS / 32) {
+    int row;
     bool ok;
     int w = 0, h = 0, bb = 0;
     if (STRIDED) {
@@ -960,25 +985,25 @@ __device__ __forceinline__ void round_left_tile(const TcParams &p, int cta, int 
         h = h * 16 + (r >> 3);
       } else {
         pixel_box(p, mt, w, h, bb);
-        const int t = r / p.Wt;
-        w += r - t * p.Wt;
-        h += t % p.Ht;
-        bb += t / p.Ht;
+        const int t = r >> p.wt_shift;
+        w += r & (p.Wt - 1);
+        h += t & (p.Ht - 1);
+        bb += t >> p.ht_shift;
       }
       ok = w < p.PW && h < p.PH && bb < p.PB;
-      row = ((long long)bb * p.PH + h) * p.PW + w;
+      row = (bb * p.PH + h) * p.PW + w;
     } else {
-      row = (long long)mt * (BM * p.mrep) + r;
+      row = mt * BM + r;
       ok = row < p.gm;
     }
     if (!ok) continue;
     const bool pools = p.pool && ((w | h) & 1) == 0;                  // (extents are even, windows lie inside the tile)
     for (int c = lane; c < cols; c += 32) {
-      const long long at = row * p.gn + col0 + c;
+      const unsigned at = (unsigned)row * (unsigned)p.gn + (unsigned)(col0 + c);
       int q = rounded(at);
       if (pools) {
         const int m = max(max(q, rounded(at + p.gn)), max(rounded(at + p.PW * p.gn), rounded(at + (p.PW + 1) * p.gn)));
-        pool8[(((long long)bb * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1)) * p.gn + col0 + c] = (int8_t)m;
+        pool8[(unsigned)((bb * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1)) * (unsigned)p.gn + (unsigned)(col0 + c)] = (int8_t)m;
       }
       if (p.update) {
         const int d = (int)out8[at] - q;
@@ -1125,7 +1150,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   };
 
-  const bool epi_warp = warp >= EPI_WARP0 && ((warp - EPI_WARP0) >> 2) % wpq < wpq_active;
+  const bool epi_warp = warp >= EPI_WARP0 && (((warp - EPI_WARP0) >> 2) & (wpq - 1)) < wpq_active;
   if (warp < PROD_WARPS) {
     // ================= TMA producers (every CTA loads its own rows of A and its share of B) ========
     // Each producer warp runs its loop in lock step and one elected lane issues the copies (warp-uniform
@@ -1142,13 +1167,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const int bn_cta = p.bn / CTAS;             // B rows (output columns) staged by this CTA
       if (p.halo == 2) {
         for (int item = first_item; ok && item < item_end; item += item_step) {
-          const int split = p.splits > 1 ? item % p.splits : 0;
-          const int blk = (int)(item / p.splits);
+          const int blk = div_by(item, p.d_split), split = item - blk * p.splits;
           const int ci0 = (blk % p.wg_nci) * 64, co0 = (blk / p.wg_nci) * 64;
           const int t0 = split * p.kb_per_split;
           int t1 = t0 + p.kb_per_split;
           if (t1 > p.kb_total) t1 = p.kb_total;
-          int wt = t0 % p.w_tiles, ht = (t0 / p.w_tiles) % p.h_tiles, bt = t0 / (p.w_tiles * p.h_tiles);
+          int wt, ht, bt;
+          tile_coords(p, t0, wt, ht, bt);
           for (int t = t0; t < t1; ++t) {
             if (owner == warp) {
               if (!mbar_wait_warp(empty0 + 8 * stage, phase ^ 1, &abort_flag, status)) { ok = false; break; }
@@ -1256,8 +1281,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (p.tg > 1) {
             tap_n = nt * p.tg + (int)rank * (p.tg / CTAS);
           } else {
-            tap_n = nt / p.n_chunks;
-            ci0 = (nt % p.n_chunks) * p.bn + (int)rank * bn_cta;
+            tap_n = div_by(nt, p.d_chunks);
+            ci0 = (nt - tap_n * p.n_chunks) * p.bn + (int)rank * bn_cta;
           }
         }
         // k-block counters, stepped instead of divided inside the loop (one thread issues all copies,
@@ -1267,8 +1292,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         int cc = 0, ts = 0, tr = 0, kwt = 0, kht = 0, kbt = 0;
         if (kb0 != 0) {
           if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) {
-            const int tap = kb0 / p.c_chunks;
-            cc = kb0 % p.c_chunks; tr = tap / p.S; ts = tap % p.S;
+            const int tap = div_by(kb0, p.d_cc);
+            cc = kb0 - tap * p.c_chunks; tr = div_by(tap, p.d_S); ts = tap - tr * p.S;
           } else if (p.kind == GK_CONV_WGRAD) {
             tile_coords(p, (I2C && p.i2c) ? kb0 * BM : kb0, kwt, kht, kbt);
           }
@@ -1276,7 +1301,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         int wg_r = 0, wg_s = 0;
         if (p.kind == GK_CONV_WGRAD) {
           if (tap_n >= p.R * p.S) tap_n = p.R * p.S - 1;          // (filler of a last, short tap group)
-          wg_r = tap_n / p.S; wg_s = tap_n % p.S;
+          wg_r = div_by(tap_n, p.d_S); wg_s = tap_n - wg_r * p.S;
         }
         const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + p.b_boxes * p.b_box_bytes));
         for (int kb = kb0; kb < kb1; ++kb) {
@@ -1387,7 +1412,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           a_pair[pi] = (unsigned)(ra * 4) | ((unsigned)(lbo_rows * 4) << 16);     // 64-byte rows, 16-byte units
         }
         for (int item = first_item; ok && item < item_end; item += item_step, ++use) {
-          const int split = p.splits > 1 ? item % p.splits : 0;
+          const int split = item - div_by(item, p.d_split) * p.splits;
           const int t0 = split * p.kb_per_split;
           int t1 = t0 + p.kb_per_split;
           if (t1 > p.kb_total) t1 = p.kb_total;
@@ -1427,7 +1452,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const unsigned g_bn_mma = (unsigned)p.bn_mma, g_slice16 = (unsigned)p.a_box_bytes >> 4;
       unsigned gbuf = 0, gpar = 0;            // use % nbuf, (use / nbuf) & 1, counted
       for (int item = first_item; ok && item < item_end; item += item_step, ++use) {
-        const int split = p.splits > 1 ? item % p.splits : 0;
+        const int split = p.splits > 1 ? item - div_by(item, p.d_split) * p.splits : 0;
         const int kb0 = split * p.kb_per_split;
         int kb1 = kb0 + p.kb_per_split;
         if (kb1 > p.kb_total) kb1 = p.kb_total;
@@ -1436,7 +1461,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           const Phase q = split_phase(p, item, tile);
           kb1 = q.n_r * q.n_s * p.c_chunks;
         }
-        int cc_left = g_tail ? p.c_chunks - kb0 % p.c_chunks : 0;     // chunks up to the short one (counted)
+        int cc_left = g_tail ? p.c_chunks - (kb0 - div_by(kb0, p.d_cc) * p.c_chunks) : 0;     // chunks up to the short one (counted)
         const unsigned buf = gbuf;
         // wait until the epilogue has drained this accumulator buffer (the first nbuf uses pass at once)
         if (!mbar_wait_warp(tempty0 + 8 * buf, gpar ^ 1u, &abort_flag, status)) { ok = false; break; }
@@ -1479,8 +1504,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // ================= epilogue: TMEM -> int32 accumulators + max magnitude =================
     const int quarter = warp & 3;               // TMEM lanes [32 * quarter, +32)
     const int wq = (warp - EPI_WARP0) >> 2;     // index among the four warps of this quarter
-    const int egroup = wq / wpq;                // tiles use % egroups == egroup are this warp's
-    const int chunk_phase = wq % wpq;           // it takes 32-column chunks phase, phase + wpq, ...
+    const int egroup = wq >> p.k_wpq_shift;                // tiles use % egroups == egroup are this warp's
+    const int chunk_phase = wq & (wpq - 1);           // it takes 32-column chunks phase, phase + wpq, ...
     const int row_in_tile = quarter * 32 + lane;
     unsigned mx = 0;
     int bp = 0;
@@ -1496,7 +1521,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       // CTA's pixel range are added to g32[co][tap][ci]
       const int which = row_in_tile >> 6, ci = row_in_tile & 63;
       for (int item = first_item; ok && item < item_end; item += item_step, ++use) {
-        const int blk = (int)(item / p.splits);
+        const int blk = div_by(item, p.d_split);
         const int ci0 = (blk % p.wg_nci) * 64, co0 = (blk / p.wg_nci) * 64;
         if (!mbar_wait(tfull0, use & 1u, &abort_flag, status)) { ok = false; break; }
         tc_fence_after();
@@ -1521,38 +1546,28 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (pmx) atomicMax(niti_split_max(hdr) + (p.splits > 1 ? item % p.splits : 0), pmx);
+          if (pmx) atomicMax(niti_split_max(hdr) + item - blk * p.splits, pmx);
           mbar_arrive(tempty0);
         }
       }
       item_end = first_item;
     }
-    // alignment of the output and mask rows
-    const bool io_aligned = ((p.gn & 31) == 0) && (((uintptr_t)out8 & 31) == 0) &&
-                            (mask8 == nullptr || ((uintptr_t)mask8 & 31) == 0) &&
-                            (p.kind != GK_CONV_WGRAD || (p.Cn & 31) == 0);
     const bool fused = epi_mode == EPI_KNOWN_B || epi_mode == EPI_SPECULATE;
     bool unaligned_bp = false;                   // binary point above 24: the lean loop leaves the items to the general one
-    // (rows that are not 32-byte aligned: the largest store unit of the output rows, and this warp's staging buffer)
-    auto io_unit = [&]() {
-      const unsigned io_bits = (unsigned)p.gn | (unsigned)(uintptr_t)out8 | 16u | (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
-      return (int)(io_bits & (0u - io_bits));
-    };
+    // (this warp's staging buffer for rows that are not 32-byte aligned)
     auto nstg = [&]() {
       return reinterpret_cast<unsigned *>(smem_raw + (smem_base - smem_u32(smem_raw)) + p.nstg_off) + (warp - EPI_WARP0) * (32 * 9);
     };
     // this thread's pixel inside a pixel box (generic convolutions): the box sides are powers of two
     struct BoxPixel { int w, h, b; };
     auto box_pixel = [&]() {
-      const int wt_d = p.Wt > 0 ? p.Wt : 1, ht_d = p.Ht > 0 ? p.Ht : 1;   // (unset for plain matrix multiplies)
-      const int t = row_in_tile / wt_d;
-      return BoxPixel{row_in_tile - t * wt_d, t % ht_d, t / ht_d};
+      const int t = row_in_tile >> p.wt_shift;
+      return BoxPixel{row_in_tile & ((1 << p.wt_shift) - 1), t & ((1 << p.ht_shift) - 1), t >> p.ht_shift};
     };
     // an item's tile: this thread's output row (row-batched mode: in the first of the item's mrep tiles), first column,
     // columns inside the matrix
     struct Tile {
-      int mt, nt, split, ncols_valid;
-      long long out_row, col0;
+      int mt, nt, split, ncols_valid, out_row, col0;
       bool row_ok;
     };
     auto tile_of = [&](int item) {
@@ -1565,15 +1580,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         decode_item(p, tile, mu, t.nt, t.split);
       }
       t.mt = mu * CTAS + (int)rank;
-      t.col0 = (long long)t.nt * p.bn;
-      const long long rem = p.gn - t.col0;
-      t.ncols_valid = rem < p.bn ? (int)rem : p.bn;
+      t.col0 = t.nt * p.bn;
+      t.ncols_valid = min(p.gn - t.col0, p.bn);
       if (p.halo) {
         int wt, ht, bt;
         tile_coords(p, item, wt, ht, bt);
         const int w = wt * 8 + (row_in_tile & 7), h = ht * 16 + (row_in_tile >> 3);
         t.row_ok = w < p.PW && h < p.PH;
-        t.out_row = ((long long)bt * p.PH + h) * p.PW + w;
+        t.out_row = (bt * p.PH + h) * p.PW + w;
       } else if (STRIDED) {
         t.out_row = phase_row(p, t.mt * BM + row_in_tile, phq, t.row_ok);
       } else if ((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) {
@@ -1582,13 +1596,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const BoxPixel px = box_pixel();
         const int w = w0 + px.w, h = h0 + px.h, b = b0 + px.b;
         t.row_ok = w < p.PW && h < p.PH && b < p.PB;
-        t.out_row = ((long long)b * p.PH + h) * p.PW + w;
+        t.out_row = (b * p.PH + h) * p.PW + w;
       } else {
-        t.out_row = (long long)t.mt * (BM * p.mrep) + row_in_tile;
+        t.out_row = t.mt * (BM * p.mrep) + row_in_tile;
         t.row_ok = t.out_row < p.gm;
         if (p.kind == GK_CONV_WGRAD) {
-          const int tap = t.nt / p.n_chunks, ci0 = (t.nt - tap * p.n_chunks) * p.bn;
-          t.col0 = (long long)tap * p.Cn + ci0;
+          const int tap = div_by(t.nt, p.d_chunks), ci0 = (t.nt - tap * p.n_chunks) * p.bn;
+          t.col0 = tap * p.Cn + ci0;
           t.ncols_valid = p.Cn - ci0 < p.bn && p.tg <= 1 ? p.Cn - ci0 : p.bn;
         }
       }
@@ -1657,68 +1671,68 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       constexpr bool UPD = decltype(upd_c)::value;         // the output rows are weights: subtract the rounded gradient
       const int pool_xh = p.pool_xh;
       const bool pool_lane = (lane & (1 | pool_xh)) == 0;  // the window's top-left pixel stores the maximum
-      const int kind = STRIDED ? 3 : (p.halo ? 0 : (((p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !(I2C && p.i2c)) ? 1
-                                                    : (p.kind == GK_CONV_WGRAD ? 4 : 2)));
+      const int kind = STRIDED ? (int)ROWS_PHASES : p.row_kind;
       const int istep = item_step * egroups, nbuf = p.nbuf, bn = p.bn, n_tiles_n = p.n_tiles_n;
       const int cstep = 32 * wpq, c_first = 32 * chunk_phase;
-      const long long gn = p.gn, gm = p.gm;
+      const int gn = p.gn, gm = p.gm;
       const int bn_mma = BATCHED ? p.bn_mma : p.bn;
-      const long long sub_stride = (long long)BM * gn;      // next 128-row tile of a row-batched item
-      const bool counted = p.blocked && p.raster_g <= 0 && kind != 3;     // consecutive items: (mu, nt) are stepped
+      const bool counted = p.blocked && p.raster_g <= 0 && kind != ROWS_PHASES;     // consecutive items: (mu, nt) are stepped
       const int lean_item = first_item + egroup * item_step;
       unsigned ebuf = (unsigned)egroup, epar = 0;           // use % nbuf, (use / nbuf) & 1 (nbuf is a multiple of egroups)
       Extremes ex_all = {0, 0, 0u};
-      RoundConst rk = make_round_const(bp, p.mbits, p.round_mode);
-      const BoxPixel bpx = kind == 1 ? box_pixel() : BoxPixel{0, 0, 0};
+      RoundConst rk = {0u, 0u, 0u, 0, 0, 0u, 0u, 0u, 0u, 0u, true};
+      const BoxPixel bpx = box_pixel();
       int mu = 0, nt = 0, split = 0, h_wt = 0, h_ht = 0, h_bt = 0;
-      if (epi_mode == EPI_KNOWN_B && !rk.aligned) { unaligned_bp = true; return; }
+      if (epi_mode == EPI_KNOWN_B) {
+        rk = make_round_const(bp, p.mbits, p.round_mode);
+        if (!rk.aligned) { unaligned_bp = true; return; }
+      }
       Phase phq = {0, 0, 1, 1};
-      if (kind == 3) {
+      if (kind == ROWS_PHASES) {
         int tile;
         phq = split_phase(p, lean_item, tile);
         decode_item(p, tile, mu, nt, split);
-      } else if (kind != 0) decode_item(p, lean_item, mu, nt, split);
+      } else if (kind != ROWS_HALO) decode_item(p, lean_item, mu, nt, split);
       else tile_coords(p, lean_item, h_wt, h_ht, h_bt);
       for (int item = lean_item; item < item_end; item += istep) {
         const unsigned buf = ebuf, tpar = epar;
         ebuf += (unsigned)egroups;
         if (ebuf >= (unsigned)nbuf) { ebuf -= (unsigned)nbuf; epar ^= 1u; }
-        long long out_row;
+        int out_row, pool_row = 0;
         bool row_ok;
-        long long pool_row = 0;
         int col0 = nt * bn;
-        int cend = BATCHED ? bn : (int)(gn - col0);          // (whole chunks unless NARROW)
-        if (kind == 0) {
+        int cend = BATCHED ? bn : gn - col0;          // (whole chunks unless NARROW)
+        if (kind == ROWS_HALO) {
           const int w = h_wt * 8 + (row_in_tile & 7), h = h_ht * 16 + (row_in_tile >> 3);
           row_ok = w < p.PW && h < p.PH;
-          out_row = ((long long)h_bt * p.PH + h) * p.PW + w;
-          if (POOL) pool_row = ((long long)h_bt * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
+          out_row = (h_bt * p.PH + h) * p.PW + w;
+          if (POOL) pool_row = (h_bt * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
           h_wt += egroups;
           while (h_wt >= p.w_tiles) { h_wt -= p.w_tiles; if (++h_ht == p.h_tiles) { h_ht = 0; ++h_bt; } }
-        } else if (kind == 1) {
+        } else if (kind == ROWS_BOXES) {
           int w0, h0, b0;
           pixel_box(p, mu * CTAS + (int)rank, w0, h0, b0);
           const int w = w0 + bpx.w, h = h0 + bpx.h, b = b0 + bpx.b;
           row_ok = w < p.PW && h < p.PH && b < p.PB;
-          out_row = ((long long)b * p.PH + h) * p.PW + w;
-          if (POOL) pool_row = ((long long)b * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
-        } else if (kind == 3) {
+          out_row = (b * p.PH + h) * p.PW + w;
+          if (POOL) pool_row = (b * (p.PH >> 1) + (h >> 1)) * (p.PW >> 1) + (w >> 1);
+        } else if (kind == ROWS_PHASES) {
           out_row = phase_row(p, (mu * CTAS + (int)rank) * BM + row_in_tile, phq, row_ok);
         } else {
-          out_row = (long long)(mu * CTAS + (int)rank) * (BM * p.mrep) + row_in_tile;
+          out_row = (mu * CTAS + (int)rank) * (BM * p.mrep) + row_in_tile;
           row_ok = out_row < gm;
-          if (kind == 4) {
-            const int tap = nt / p.n_chunks, ci0 = (nt - tap * p.n_chunks) * bn;
+          if (kind == ROWS_WGRAD) {
+            const int tap = div_by(nt, p.d_chunks), ci0 = (nt - tap * p.n_chunks) * bn;
             col0 = tap * p.Cn + ci0;
             cend = p.Cn - ci0;
           }
         }
         if (cend > bn) cend = bn;
-        if (kind != 0) {                                      // next item of this warp
+        if (kind != ROWS_HALO) {                                      // next item of this warp
           if (counted) { nt += egroups; while (nt >= n_tiles_n) { nt -= n_tiles_n; ++mu; } }
           else if (item + istep < item_end) {
             int tile = item + istep;
-            if (kind == 3) phq = split_phase(p, item + istep, tile);
+            if (kind == ROWS_PHASES) phq = split_phase(p, item + istep, tile);
             decode_item(p, tile, mu, nt, split);
           }
         }
@@ -1740,7 +1754,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               for (int c = c_first; c < ce; c += cstep) {
                 int v[32];
                 tc_ld32(tm_row + (unsigned)c, v);
-                if (row_ok && (!BATCHED || out_row + (long long)(c / bn_mma) * BM < gm)) {
+                if (row_ok && (!BATCHED || out_row + c / bn_mma * BM < gm)) {
 #pragma unroll
                   for (int j = 0; j < 32; j += 2) {
                     hi0 = __vimax3_s32(hi0, v[j], v[j + 1]);
@@ -1757,26 +1771,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           break;
         }
         tc_fence_after();
-        const long long row_off = out_row * gn + col0;
+        const unsigned row_off = (unsigned)out_row * (unsigned)gn + (unsigned)col0;       // (used where row_ok)
 #pragma unroll 1
         while (true) {
-          int8_t *drow = out8 + row_off;
-          const int8_t *mrow = MASK ? mask8 + row_off : nullptr;
-          int8_t *prow = POOL ? pool8 + pool_row * gn + col0 : nullptr;
-          long long orow = out_row;
+          unsigned off = row_off;                              // (row-batched mode: steps to the item's next 128-row tile)
+          int orow = out_row;
           int cc = c_first;
-          if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (MASK) mrow += sub_stride; }
+          if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; off += BM * (unsigned)gn; }
           const int ce = live ? cend : c_first + warm_chunks;
           for (int c = c_first; c < ce; c += cstep) {
             int v[32];
             const bool rok = (BATCHED ? (row_ok && orow < gm) : row_ok) && live != 0;       // (rows that are read and written)
             unsigned m[8];
             if (NARROW) {
-              if (MASK && rok) load_row_narrow(mrow + cc, m, cend - c < 32 ? cend - c : 32);
+              if (MASK && rok) load_row_narrow(mask8 + (off + cc), m, cend - c < 32 ? cend - c : 32);
             } else if ((MASK || UPD) && rok)
               asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                            : "=r"(m[0]), "=r"(m[1]), "=r"(m[2]), "=r"(m[3]), "=r"(m[4]), "=r"(m[5]), "=r"(m[6]), "=r"(m[7])
-                           : "l"((UPD ? (const int8_t *)drow : mrow) + cc));
+                           : "l"((UPD ? (const int8_t *)out8 : mask8) + (off + cc)));
             tc_ld32(tm_row + (unsigned)c, v);
             unsigned w8[8];
             if (POOL) {
@@ -1790,15 +1802,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (MASK) w8[j] &= bytes_gt0(m[j]);
                 if (UPD) w8[j] = bytes_sub_clamp127(m[j], w8[j]);
               }
-              if (!NARROW && rok) store32(drow + cc, w8);
+              if (!NARROW && rok) store32(out8 + (off + cc), w8);
             }
-            if (NARROW) store_rows_narrow(out8, drow - out8 + cc, rok, w8, BATCHED ? (int)gn - cc : cend - c, io_unit(), nstg(), lane);
+            if (NARROW) store_rows_narrow(out8, off + cc, rok, w8, BATCHED ? gn - cc : cend - c, p.io_unit, nstg(), lane);
             if (POOL) {                                        // (warp-uniform: all lanes exchange)
               pool_chunk32(w8, pool_xh);
-              if (rok && pool_lane) store32(prow + cc, w8);
+              if (rok && pool_lane) store32(pool8 + ((unsigned)pool_row * (unsigned)gn + (unsigned)(col0 + cc)), w8);
             }
             cc += cstep;
-            if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; drow += sub_stride; if (MASK) mrow += sub_stride; }
+            if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; off += BM * (unsigned)gn; }
           }
           if (live) break;
           if (!await_bp()) { ok = false; break; }
@@ -1836,21 +1848,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     auto lean = [&]() {
       using T = std::true_type;
       using F = std::false_type;
-      const bool relu = p.relu != 0, masked = mask8 != nullptr;
-      if (!ONE && p.mrep > 1) {                                                                                 // (row-batched: forward only)
-        if (GENERAL && (!io_aligned || p.gn != p.bn_mma)) {
-          if (relu) lean_as(T{}, F{}, T{}, F{}, F{}, T{}); else lean_as(F{}, F{}, T{}, F{}, F{}, T{});
-        } else if (relu) lean_as(T{}, F{}, T{}, F{}, F{}, F{});
-        else lean_as(F{}, F{}, T{}, F{}, F{}, F{});
-      } else if (GENERAL && !io_aligned) {
-        if (relu) lean_as(T{}, F{}, F{}, F{}, F{}, T{});                                                  // (ReLU: forward, no mask)
-        else if (masked) lean_as(F{}, T{}, F{}, F{}, F{}, T{});
-        else lean_as(F{}, F{}, F{}, F{}, F{}, T{});
-      } else if (p.update) lean_as(F{}, F{}, F{}, F{}, T{}, F{});                                         // (weight gradients: signed, no mask)
-      else if (p.pool) lean_as(T{}, F{}, F{}, T{}, F{}, F{});                                             // (pooling: ReLU, no mask)
-      else if (relu) lean_as(T{}, F{}, F{}, F{}, F{}, F{});
-      else if (masked) lean_as(F{}, T{}, F{}, F{}, F{}, F{});
-      else lean_as(F{}, F{}, F{}, F{}, F{}, F{});
+      const int form = p.form;
+      if (form == LEAN_RELU) lean_as(T{}, F{}, F{}, F{}, F{}, F{});
+      else if (form == LEAN_MASK) lean_as(F{}, T{}, F{}, F{}, F{}, F{});
+      else if (form == LEAN_POOL) lean_as(T{}, F{}, F{}, T{}, F{}, F{});
+      else if (form == LEAN_PLAIN) lean_as(F{}, F{}, F{}, F{}, F{}, F{});
+      else if (form == LEAN_UPDATE) lean_as(F{}, F{}, F{}, F{}, T{}, F{});
+      else if (GENERAL && form == LEAN_NARROW_RELU) lean_as(T{}, F{}, F{}, F{}, F{}, T{});
+      else if (GENERAL && form == LEAN_NARROW_MASK) lean_as(F{}, T{}, F{}, F{}, F{}, T{});
+      else if (GENERAL && form == LEAN_NARROW) lean_as(F{}, F{}, F{}, F{}, F{}, T{});
+      else if (!ONE && form == LEAN_BATCHED_RELU) lean_as(T{}, F{}, T{}, F{}, F{}, F{});
+      else if (!ONE && form == LEAN_BATCHED) lean_as(F{}, F{}, T{}, F{}, F{}, F{});
+      else if (!ONE && GENERAL && form == LEAN_BATCHED_NARROW_RELU) lean_as(T{}, F{}, T{}, F{}, F{}, T{});
+      else if (!ONE && GENERAL && form == LEAN_BATCHED_NARROW) lean_as(F{}, F{}, T{}, F{}, F{}, T{});
     };
     // ---- the loop for everything else: accumulators kept, partial sums, rounding that the lean loop does not do ----
     auto general = [&]() {
@@ -1860,7 +1870,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
            item += item_step * egroups, use += (unsigned)egroups) {
         const Tile t = tile_of(item);
         const int mt = t.mt, nt = t.nt, split = t.split, ncols_valid = t.ncols_valid;
-        const long long out_row = t.out_row, col0 = t.col0;
+        const int out_row = t.out_row, col0 = t.col0;
         const bool row_ok = t.row_ok;
         const unsigned buf = ebuf;
         const unsigned tpar = epar;
@@ -1874,7 +1884,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
           int x0, x1, x2 = 0, x3 = 0;                            // tensor coordinates of the chunk at column 0
           if (p.kind == GK_CONV_WGRAD) {
-            const int tap = nt / p.n_chunks;
+            const int tap = div_by(nt, p.d_chunks);
             x0 = (nt - tap * p.n_chunks) * p.bn;
             x1 = tap;
             x2 = mt * BM + quarter * 32;
@@ -1915,7 +1925,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           pmx = __reduce_max_sync(0xffffffffu, pmx);
           if (lane == 0 && pmx) atomicMax(niti_split_max(hdr) + split, pmx);
         } else if (epi_mode <= EPI_ATOMIC) {
-          int32_t *dst = acc + out_row * p.gn + col0;
+          int32_t *dst = acc + ((long long)out_row * p.gn + col0);
           const bool vec_ok = ((p.gn & 3) == 0) && ((col0 & 3) == 0);
           unsigned pmx = 0;                                      // largest partial-sum magnitude of this item
           for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
@@ -1958,12 +1968,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
         } else {
           // Whole 32-column chunks with 32-byte aligned rows (binary points above 24), or any rows.
-          const bool whole_chunks = io_aligned && ((col0 & 31) == 0) &&
-                                    (p.mrep > 1 ? ncols_valid >= p.bn_mma : (ncols_valid & 31) == 0);
+          const bool whole_chunks = p.io_unit == 32;
           for (int c = 32 * chunk_phase; c < p.bn; c += 32 * wpq) {
             // chunk geometry: in row-batched mode chunk c holds columns cc of the item's tile c / bn_mma
             const int jt = p.mrep > 1 ? c / p.bn_mma : 0, cc = c - jt * p.bn_mma;
-            const long long orow = out_row + (long long)jt * BM, off = orow * p.gn + col0 + cc;
+            const int orow = out_row + jt * BM;
+            const unsigned off = (unsigned)orow * (unsigned)p.gn + (unsigned)(col0 + cc);
             const bool rok = row_ok && (p.mrep == 1 || orow < p.gm);
             const int nv = ncols_valid - cc;                     // (uniform across the warp)
             if (nv <= 0) continue;
@@ -1983,7 +1993,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               }
             }
             if (whole_chunks) { if (rok) store32(out8 + off, w8); }
-            else if (GENERAL) store_rows_narrow(out8, off, rok, w8, nv, io_unit(), nstg(), lane);
+            else if (GENERAL) store_rows_narrow(out8, off, rok, w8, nv, p.io_unit, nstg(), lane);
           }
         }
         tc_fence_before();
@@ -1997,10 +2007,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (fused) lean();
     if (!fused || unaligned_bp) general();
     if (epi_mode == EPI_SPILL || epi_mode == EPI_SPECULATE) {
-      for (int o = 16; o > 0; o >>= 1) {
-        unsigned u = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = u > mx ? u : mx;
-      }
+      mx = __reduce_max_sync(0xffffffffu, mx);
       if (lane == 0 && mx) atomicMax(&cta_max, mx);     // (one global atomic per CTA, below)
     }
     if (p.red && lane == 0) tma_reduce_wait_all();      // (shared memory stays valid until the copies are done)
@@ -2363,7 +2370,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   int a_sw = 0, b_sw = 0;
   int tail = 0;                  // contraction elements of the last chunk of c_chunks when it is not a whole one
   long long m_tiles = 0;
-  if (g.gm * g.gn >= (1LL << 31)) return false;
+  if (g.gm * g.gn >= (1LL << 31) || g.gm >= (1LL << 31) - 1024) return false;      // (rows are counted in 32 bits)
   // operands as they are copied: padded where the caller's rows are no multiple of 16 bytes
   const int8_t *q0 = g.q0 ? g.q0 : g.p0, *q1 = g.q1 ? g.q1 : g.p1;
   if (g.kind == GK_FC_DGRAD && g.gk < 32) return false;            // (10-class heads: the CUDA-core engine is faster)
@@ -2947,11 +2954,40 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
     int cols = 32;
     while (cols < p.nbuf * p.bn) cols <<= 1;
     q.k_tmem_cols = cols;
-    // reciprocals for tile index -> coordinates; dividends stay below the tile count
-    const unsigned long long n_max = (unsigned long long)(p.w_tiles > 0 ? p.w_tiles : 1) * (p.h_tiles > 0 ? p.h_tiles : 1) *
-                                     (p.b_tiles > 0 ? p.b_tiles : 1) + 512;
-    q.magic_w = (p.w_tiles > 1 && n_max * p.w_tiles < (1ull << 32)) ? (unsigned)((1ull << 32) / p.w_tiles + 1) : 0u;
-    q.magic_h = (p.h_tiles > 1 && n_max * p.h_tiles < (1ull << 32)) ? (unsigned)((1ull << 32) / p.h_tiles + 1) : 0u;
+    // (dividends are items, tiles or grid positions, all below 2^31)
+    q.d_w = make_div(p.w_tiles);
+    q.d_h = make_div(p.h_tiles);
+    q.d_n = make_div(p.n_tiles_n);
+    q.d_split = make_div(p.splits);
+    if (p.raster_g > 0) {
+      q.last_group = (p.m_units - 1) / p.raster_g;
+      q.d_group = make_div((long long)p.raster_g * p.n_tiles_n);
+      q.d_units = make_div(p.raster_g);
+      q.d_last = make_div(p.m_units - q.last_group * p.raster_g);
+    }
+    q.d_chunks = make_div(p.n_chunks);
+    q.d_S = make_div(p.S);
+    q.d_cc = make_div(p.c_chunks);
+    q.d_phases = make_div((long long)p.nph_r * p.nph_s);
+    q.d_phase_s = make_div(p.nph_s);
+    for (int v = p.Wt; v > 1; v >>= 1) q.wt_shift++;
+    for (int v = p.Ht; v > 1; v >>= 1) q.ht_shift++;
+    for (int v = q.k_wpq; v > 1; v >>= 1) q.k_wpq_shift++;
+    // how the rows of the output lie and what is done to them
+    q.row_kind = p.dstride > 1 ? ROWS_PHASES : p.halo ? ROWS_HALO
+                 : p.kind == GK_CONV_WGRAD ? ROWS_WGRAD
+                 : (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) && !p.i2c ? ROWS_BOXES : ROWS_PLAIN;
+    const unsigned bits = (unsigned)p.gn | (unsigned)(uintptr_t)r.out | (r.mask ? (unsigned)(uintptr_t)r.mask : 0u) | 32u |
+                          (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
+    q.io_unit = (int)(bits & (0u - bits));
+    if (q.io_unit < 32) {
+      const unsigned out_bits = (unsigned)p.gn | (unsigned)(uintptr_t)r.out | 16u | (p.kind == GK_CONV_WGRAD ? (unsigned)p.Cn : 0u);
+      q.io_unit = (int)(out_bits & (0u - out_bits));          // (gate bytes are read at any alignment)
+    }
+    const bool narrow = q.io_unit < 32;
+    q.form = p.mrep > 1 ? (narrow ? (r.relu ? LEAN_BATCHED_NARROW_RELU : LEAN_BATCHED_NARROW) : r.relu ? LEAN_BATCHED_RELU : LEAN_BATCHED)
+             : narrow ? (r.relu ? LEAN_NARROW_RELU : r.mask ? LEAN_NARROW_MASK : LEAN_NARROW)
+             : p.update ? LEAN_UPDATE : p.pool ? LEAN_POOL : r.relu ? LEAN_RELU : r.mask ? LEAN_MASK : LEAN_PLAIN;
   }
   // per call site (keyed by the address of its bit-width scalar): the error of the last speculative estimate
   int32_t *slot = nullptr;
