@@ -77,8 +77,6 @@ struct TcParams {
   // set-up arithmetic done on the host (integer divisions at kernel entry delay every launch)
   int blk_per, blk_extra;       // blocked assignment: items per CTA (pair) and how many take one more
   int k_wpq, k_wpq_active, k_epi_active, k_tmem_cols;
-  int quorum;                   // CTAs whose first tile must have reported before the speculative bit-width
-                                // is fixed (launches that are not single-wave)
   unsigned patience;            // cycles that CTAs wait for each other
   int nissue;                   // resident-weights mode: warps that issue MMAs (2: the warp that loaded the
                                 // weights takes every other tile)
@@ -154,6 +152,7 @@ struct TcParams {
   int epi_mode;                 // EPI_SPILL / EPI_ATOMIC / EPI_SPECULATE / EPI_KNOWN_B
   int mbits, round_mode, relu;
   unsigned spec_mul256;         // the sampled max is scaled by this / 256 before taking its bit length
+  unsigned trial_mul256;        // the same for the maximum of a CTA's own first tile (see lean_as), 0: no trial
   int spec_tag;                 // identifies the call site (its b_out scalar) in the table of estimate errors
   int update;                   // 1: out8 holds weights: the epilogue stores clamp(w - rounded gradient, +-127)
   int pool;                     // 1: the epilogue also stores the 2 x 2 max-pool of the (ReLU'd) output tile
@@ -628,10 +627,10 @@ __device__ __forceinline__ int spec_correction(int packed) {
 }
 
 // The guess at a tensor's bit-width from the first tiles of a launch's CTAs, for one converged warp of every CTA; m: largest
-// magnitude in its own first tile.  Posts and mailboxes as in niti_agree_bits: the first CTA decides as soon as a quorum has
-// posted (waiting for every CTA meant waiting out the launch ramp of the whole grid) and answers all of them.  (With a
-// maximum, a count and a published word that all CTAs poll, updated by atomics, the agreement took 3.7 - 4.4 us, a chain of
-// five trips to L2; this takes 2.0.)  A CTA out of patience (launches of several streams share the SMs) decides from what has
+// magnitude in its own first tile.  Posts and mailboxes as in niti_agree_bits: the first CTA decides when all have posted
+// (deciding at half of them saved 0.2 us and made the guess depend on who came first: 50 of 100 launches of a 5 x 5 layer's
+// error were recomputed, now none) and answers all of them.  (With a maximum, a count and a published word that all CTAs
+// poll, updated by atomics, the agreement took 3.7 - 4.4 us, a chain of five trips to L2; this takes 2.2.)  A CTA out of patience (launches of several streams share the SMs) decides from what has
 // been posted by then.  Two CTAs may decide differently: every CTA reports what it rounded with (WsHeader::spec_mask), and
 // the follow-up launch recomputes unless all of them used the true bit-width.
 __device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, unsigned m, const TcParams &p,
@@ -665,7 +664,7 @@ __device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, u
       seen += w ? 1u : 0u;
       top = max(top, w);
     }
-    if (cta != 0 || __reduce_add_sync(0xffffffffu, seen) >= (unsigned)p.quorum || late()) break;
+    if (cta != 0 || __reduce_add_sync(0xffffffffu, seen) >= (unsigned)n || late()) break;
   }
   top = __reduce_max_sync(0xffffffffu, top) - 1u;
   // the first tiles are a sample: scale their max by the growth expected from the sample to the whole tensor before taking
@@ -1500,6 +1499,28 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       }
     }
+    if (ONE) {
+      // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.  This warp has nothing else to do and
+      // speaks for its CTA as soon as the epilogue's warps have reported.
+      const long long t0 = clock64();
+      while (__any_sync(0xffffffffu, *(volatile unsigned *)&first_arrived < (unsigned)epi_active)) {
+        if (__any_sync(0xffffffffu, abort_flag != 0)) break;
+        if (__any_sync(0xffffffffu, clock64() - t0 > WAIT_LIMIT_CYCLES)) {
+          abort_flag = 1;
+          atomicOr(status, NITI_DEV_TIMEOUT);
+          break;
+        }
+      }
+      if (__all_sync(0xffffffffu, abort_flag == 0)) {
+        unsigned *words = niti_split_max(hdr);
+        const int b = (int)niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(*(volatile unsigned *)&first_max),
+                                           (int)blockIdx.x, (int)gridDim.x, 0, lane, p.patience) - 1;
+        if (lane == 0) {
+          spec_bp_ready = b < 0 ? -1 : (b > p.mbits ? b - p.mbits : 0) + 1;
+          if (b >= 0 && blockIdx.x == 0) publish_exact(b);
+        }
+      }
+    }
   } else if (epi_warp) {
     // ================= epilogue: TMEM -> int32 accumulators + max magnitude =================
     const int quarter = warp & 3;               // TMEM lanes [32 * quarter, +32)
@@ -1608,36 +1629,38 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       return t;
     };
-    // The first tile of this CTA has largest magnitude m0 in this warp's share.  True in the warp that has spoken for the CTA.
+    // The first tile of this CTA has largest magnitude m0 in this warp's share.  The warps combine their maxima in shared
+    // memory; one warp speaks for the CTA in the grid-wide agreement (with every warp of every CTA polling the same word the
+    // wait itself took microseconds) and publishes the shift to the others through shared memory: the issuing warp, idle by
+    // then, in single-wave launches, else the last one to report, for which this is true.
     auto report = [&](unsigned m0) {
       m0 = __reduce_max_sync(0xffffffffu, m0);
-      // The warps of this CTA combine their maxima in shared memory; the last one to report speaks
-      // for the CTA in the grid-wide agreement (with every warp of every CTA polling the same word the wait
-      // itself took microseconds) and publishes the shift to the others through shared memory.
       unsigned last = 0;
       if (lane == 0) {
         if (m0) atomicMax(&first_max, m0);
         __threadfence_block();
         last = atomicAdd(&first_arrived, 1u) + 1u == (unsigned)epi_active ? 1u : 0u;
       }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (!last) return false;
+      if (ONE) return false;
+      if (!__shfl_sync(0xffffffffu, last, 0)) return false;
       unsigned *words = niti_split_max(hdr);
-      const unsigned cm = *(volatile unsigned *)&first_max;
-      int b;
-      if (ONE) {
-        // Every CTA has one tile: the sample is the whole tensor, and the shift is exact.
-        b = (int)niti_agree_bits(words, words + NITI_AGREE_MAX, niti_bitlen32(cm), (int)blockIdx.x, (int)gridDim.x, 0, lane,
-                                 p.patience) - 1;
-      } else {
-        b = agree_on_guess(words, words + NITI_AGREE_MAX, cm, p, spec_slot, lane);
-      }
+      const int b = agree_on_guess(words, words + NITI_AGREE_MAX, *(volatile unsigned *)&first_max, p, spec_slot, lane);
       if (lane == 0) {
-        if (!ONE) cta_b = b;
-        spec_bp_ready = b < 0 ? -1 : (b > p.mbits ? b - p.mbits : 0) + 1;
-        if (ONE && b >= 0 && blockIdx.x == 0) publish_exact(b);
+        cta_b = b;
+        spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
       }
       return true;
+    };
+    // What this CTA's first tile alone says about the tensor's binary point, once all its warps have reported.
+    auto own_guess = [&]() {
+      const long long t0 = clock64();
+      while (*(volatile unsigned *)&first_arrived < (unsigned)epi_active && !abort_flag && clock64() - t0 < WAIT_LIMIT_CYCLES) {
+      }
+      __syncwarp();
+      const unsigned own = *(volatile unsigned *)&first_max;
+      const unsigned long long scaled = ((unsigned long long)own * p.trial_mul256) >> 8;
+      const int b = niti_bitlen32(scaled > 0x7fffffffull ? 0x7fffffffu : (unsigned)scaled);
+      return __shfl_sync(0xffffffffu, b > p.mbits ? b - p.mbits : 0, 0);
     };
     // The agreed binary point (in spec_bp_ready), once it is there; false: time to leave.
     auto await_bp = [&]() {
@@ -1662,8 +1685,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // chunk spends a third of its integer instructions on tests whose outcome is the same for every tile).
     // Code that is not in the SM's instruction cache costs about 8 ns an instruction (lines of 128 bytes, 70 - 100 ns each), and
     // in a program of different kernels that is every launch: rounding the first tile took 4.3 us instead of the 1.9 us of a
-    // launch that repeats.  While the bit-width is being agreed, the warps therefore take a chunk through the loop body without
-    // storing it (`live` false).
+    // launch that repeats.  While the bit-width is being agreed (2 us), the warps therefore round and store the first tile
+    // with what the tile itself says of the bit-width (`trial`), and again only where the grid has agreed on another one; where
+    // a store could not be taken back (weight updates, outputs in the storage of an operand) a chunk passes without it.
     auto lean_as = [&](auto relu_c, auto mask_c, auto batched_c, auto pool_c, auto upd_c, auto narrow_c) {
       constexpr bool NARROW = decltype(narrow_c)::value;   // output rows that are not 32-byte aligned, short last chunks
       constexpr bool RELU = decltype(relu_c)::value, MASK = decltype(mask_c)::value, BATCHED = decltype(batched_c)::value;
@@ -1728,7 +1752,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
         }
         if (cend > bn) cend = bn;
-        if (kind != ROWS_HALO) {                                      // next item of this warp
+        if (!ONE && kind != ROWS_HALO) {                       // next item of this warp
           if (counted) { nt += egroups; while (nt >= n_tiles_n) { nt -= n_tiles_n; ++mu; } }
           else if (item + istep < item_end) {
             int tile = item + istep;
@@ -1737,9 +1761,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
         }
         const unsigned tm_row = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * (unsigned)bn;
-        int live = 1, warm_chunks = 1;
+        int live = 1, ce = cend, trial_bp = -1;                // columns of this pass; the binary point of a trial
         if (epi_mode == EPI_SPECULATE && item == lean_item) {
           live = 0;
+          ce = c_first + 1;
           if (egroup == 0) {
             // first tile of this CTA: max only, then agree on the estimate with the whole grid (columns of a partly filled
             // chunk beyond the matrix accumulate zeros; whole chunks beyond it are left out)
@@ -1750,8 +1775,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               if (t && !mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) { ok = false; break; }
               tc_fence_after();
               hi0 = lo0 = 0;
-              const int ce = t ? cend : c_first + 1;
-              for (int c = c_first; c < ce; c += cstep) {
+              for (int c = c_first; c < (t ? cend : c_first + 1); c += cstep) {
                 int v[32];
                 tc_ld32(tm_row + (unsigned)c, v);
                 if (row_ok && (!BATCHED || out_row + c / bn_mma * BM < gm)) {
@@ -1764,7 +1788,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               }
             }
             if (!ok) break;
-            if (report(max((unsigned)hi0, 0u - (unsigned)lo0))) warm_chunks = 0;
+            if (report(max((unsigned)hi0, 0u - (unsigned)lo0))) {
+              ce = c_first;                                    // (the agreement is there)
+            } else if (!UPD && p.trial_mul256) {
+              trial_bp = own_guess();
+              if (trial_bp <= 24) {
+                rk = make_round_const(trial_bp, p.mbits, p.round_mode);
+                ce = cend;
+              } else {
+                trial_bp = -1;
+              }
+            }
           }
         } else if (!mbar_wait(tfull0 + 8 * buf, tpar, &abort_flag, status)) {
           ok = false;
@@ -1778,10 +1812,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           int orow = out_row;
           int cc = c_first;
           if (BATCHED) while (cc >= bn_mma) { cc -= bn_mma; orow += BM; off += BM * (unsigned)gn; }
-          const int ce = live ? cend : c_first + warm_chunks;
           for (int c = c_first; c < ce; c += cstep) {
             int v[32];
-            const bool rok = (BATCHED ? (row_ok && orow < gm) : row_ok) && live != 0;       // (rows that are read and written)
+            const bool rok = (BATCHED ? (row_ok && orow < gm) : row_ok) && (live != 0 || trial_bp >= 0);   // (rows that are read and written)
             unsigned m[8];
             if (NARROW) {
               if (MASK && rok) load_row_narrow(mask8 + (off + cc), m, cend - c < 32 ? cend - c : 32);
@@ -1792,11 +1825,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             tc_ld32(tm_row + (unsigned)c, v);
             unsigned w8[8];
             if (POOL) {
-  #pragma unroll
+#pragma unroll
               for (int j = 0; j < 8; ++j) w8[j] = 0u;          // lanes outside the tensor pool zeros
             }
-            if (rok || !live) {
-  #pragma unroll
+            if (rok || (!live && trial_bp < 0)) {
+#pragma unroll
               for (int j = 0; j < 8; ++j) {
                 w8[j] = round_pack4_aligned<RELU>(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3], rk, ex_all);
                 if (MASK) w8[j] &= bytes_gt0(m[j]);
@@ -1827,6 +1860,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             break;
           }
           bp = spec_bp_ready - 1;
+          if (bp == trial_bp) break;                           // (stored already)
+          trial_bp = -1;
+          ce = cend;
           rk = make_round_const(bp, p.mbits, p.round_mode);
           ex_all = Extremes{0, 0, 0u};
           if (!rk.aligned) { unaligned_bp = true; break; }
@@ -1835,7 +1871,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           live = 1;
           asm volatile("" : "+r"(live));                       // (one copy of the loop)
         }
-        if (!ok || unaligned_bp) break;
+        if (ONE || !ok || unaligned_bp) break;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
@@ -2008,7 +2044,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (!fused || unaligned_bp) general();
     if (epi_mode == EPI_SPILL || epi_mode == EPI_SPECULATE) {
       mx = __reduce_max_sync(0xffffffffu, mx);
-      if (lane == 0 && mx) atomicMax(&cta_max, mx);     // (one global atomic per CTA, below)
+      if (ONE) {
+        // (a CTA that rounded with the agreed bit-width has met nothing wider: anything else means that the agreement was
+        // broken and its stored values are not exact)
+        if (lane == 0 && spec_bp_ready > 0 && niti_bitlen32(mx) > p.mbits + spec_bp_ready - 1) atomicOr(status, NITI_DEV_INTERNAL);
+      } else if (lane == 0 && mx) {
+        atomicMax(&cta_max, mx);                        // (one global atomic per CTA, below)
+      }
     }
     if (p.red && lane == 0) tma_reduce_wait_all();      // (shared memory stays valid until the copies are done)
   }
@@ -2016,10 +2058,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   // ================= common exit =================
   tc_fence_before();
   __syncthreads();
-  // (a CTA that rounded with the agreed bit-width has met nothing wider: anything else means that the agreement was broken
-  // and its stored values are not exact)
-  if (ONE && threadIdx.x == 0 && spec_bp_ready > 0 && niti_bitlen32(cta_max) > p.mbits + spec_bp_ready - 1)
-    atomicOr(status, NITI_DEV_INTERNAL);
   if (!ONE && threadIdx.x == 0) {
     if (cta_max) atomicMax(&hdr->maxabs32, cta_max);
     if (cta_b >= 0) atomicOr(&hdr->spec_mask, 1u << cta_b);
@@ -3099,6 +3137,30 @@ static int launch_finish(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, lon
   return NITI_OK;
 }
 
+// Is no operand (nor the gate) in the storage of an output?  Then the first tile's outputs may be stored before all operands
+// have been read, and stored again.
+static bool may_store_twice(const GemmProblem &g, const RoundSpec &r) {
+  const long long x = (long long)g.B * g.H * g.W * g.Ci, y = (long long)g.B * g.Ho * g.Wo * g.Co;
+  const long long out_bytes = g.gm * g.gn;
+  long long n0, n1;
+  switch (g.kind) {
+    case GK_FC_FWD: n0 = (long long)g.M * g.K; n1 = (long long)g.N * g.K; break;
+    case GK_FC_DGRAD: n0 = (long long)g.M * g.N; n1 = (long long)g.N * g.K; break;
+    case GK_FC_WGRAD: n0 = (long long)g.M * g.N; n1 = (long long)g.M * g.K; break;
+    case GK_CONV_FWD: n0 = x; n1 = (long long)g.Co * g.R * g.S * g.Ci; break;
+    case GK_CONV_DGRAD: n0 = y; n1 = (long long)g.Co * g.R * g.S * g.Ci; break;
+    default: n0 = y; n1 = x; break;
+  }
+  auto apart = [](const void *a, long long na, const void *b, long long nb) {
+    const uintptr_t u = (uintptr_t)a, v = (uintptr_t)b;
+    return !a || !b || u + (uintptr_t)na <= v || v + (uintptr_t)nb <= u;
+  };
+  auto output_apart = [&](const int8_t *out, long long n) {
+    return apart(out, n, g.p0, n0) && apart(out, n, g.p1, n1) && apart(out, n, r.mask, out_bytes);
+  };
+  return output_apart(r.out, out_bytes) && output_apart(r.pool_out, out_bytes / 4);
+}
+
 int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const RoundSpec &r_in, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled, bool shard_ok, bool *updated) {
   TcParams p;
@@ -3154,22 +3216,18 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     const int units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
     const double n_all = (double)g.gm * (double)g.gn;
     const double frac = p.items > units ? (double)units / (double)p.items : 1.0;
-    // (when the tensor has more tiles than the grid, the bit-width is fixed once half of the CTAs have
-    // reported; typically a few more have by then)
-    const double n_s = n_all * frac * (frac < 1.0 ? 0.6 : 1.0);
+    const double n_s = n_all * frac;
     double f = (n_s > 16.0 && frac < 1.0) ? sqrt(log(n_all) / log(n_s)) : 1.0;
     p.spec_mul256 = (unsigned)(f * 256.0 + 0.5);
+    const double n_own = n_all / ((double)p.items * p.ctas);
+    const double f_own = n_own > 16.0 ? sqrt(log(n_all) / log(n_own)) : 1.0;
+    p.trial_mul256 = may_store_twice(g, r) ? (unsigned)(f_own * 256.0 + 0.5) : 0u;
   }
   // data parallelism (niti_set_reduce_hook): the max magnitude is combined over the ranks between the
   // two launches, so there is always a second launch; weight gradients keep their int32 sums
   const bool dp = ctx->reduce_fn != nullptr, dp_sum = dp && niti_is_wgrad(g.kind);
   p.single_wave = (!dp && p.items * p.ctas <= NITI_AGREE_MAX && p.items <= (p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx)) && p.spec_mul256 == 256) ? 1 : 0;
-  {
-    const long long units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
-    const long long grid = (p.items < units ? p.items : units) * p.ctas;
-    p.quorum = (int)(((grid < NITI_AGREE_MAX ? grid : NITI_AGREE_MAX) + 1) / 2);
-    p.patience = ctx->patience;
-  }
+  p.patience = ctx->patience;
   p.mbits = r.mbits;
   p.round_mode = r.round_mode;
   p.relu = r.relu;
@@ -3206,6 +3264,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
       p.epi_mode == EPI_SPECULATE && p.single_wave && p.mrep == 1 && !p.halo && !r.mask && !r.relu && (g.gn % 32) == 0 &&
       ((uintptr_t)r.update_w & 31) == 0) {
     p.update = 1;
+    p.trial_mul256 = 0;
     r.out = r.update_w;
     *updated = true;
   }

@@ -52,3 +52,22 @@ def test_row_batched_first_layers_with_odd_rows(niti, oref, cout, cin):
         y, s_y, b_y = niti.conv_fwd(torch.from_numpy(x).to(niti.device), niti.scalar(-7), torch.from_numpy(w).to(niti.device),
                                     niti.scalar(-9), pad=1, relu=relu, round_mode=mode)
         assert np.array_equal(y.cpu().numpy(), want) and (int(s_y), int(b_y)) == (s, b)
+
+
+@pytest.mark.parametrize("M,N", [(1024, 1024), (500, 736)])
+def test_outputs_in_the_storage_of_an_operand(niti, oref, M, N):
+    """One-wave multiplies read all operands before they store: outputs may replace an operand or the gate."""
+    rng = np.random.default_rng(M)
+    i8 = lambda *s: rng.integers(-127, 128, size=s, dtype=np.int8)  # noqa: E731
+    T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(niti.device)  # noqa: E731
+    a, w, e = np.maximum(i8(M, N), 0), i8(N, N), i8(M, N)
+    want, s, b = oref.linear_fwd(a, -7, w, -9, True)
+    we, wg, be, bg = oref.linear_bwd(a, e, w, True, a, 5)
+    for _ in range(3):
+        at = T(a)
+        _, s_out, b_out = niti.linear_fwd(at, niti.scalar(-7), T(w), niti.scalar(-9), out=at, relu=True)
+        assert np.array_equal(at.cpu().numpy(), want) and (int(s_out), int(b_out)) == (s, b)
+        at = T(a)
+        _, g, b_e, b_g = niti.linear_bwd(at, T(e), T(w), True, at, e_prev=at)
+        assert np.array_equal(at.cpu().numpy(), we) and np.array_equal(g.cpu().numpy(), wg)
+        assert (int(b_e), int(b_g)) == (be, bg)
