@@ -1237,154 +1237,172 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       // next tile no copy is issued and the ring runs dry; measured: ~1500 cycles of integer divisions
       // per tile cost a third of a 256-channel convolution).  Consecutive items of the convolutions
       // are consecutive tiles, so tile and pixel-box coordinates are stepped, not divided.
-      const bool stepped = p.blocked && p.splits == 1 && p.raster_g <= 0 && !STRIDED;
-      int c_mu = 0, c_nt = 0, c_wt = 0, c_ht = 0, c_bt = 0;
-      for (int item = first_item; ok && item < item_end; item += item_step) {
-        int mu, nt, split;
-        int w0 = 0, h0 = 0, b0 = 0, tap_n = 0, ci0 = 0;
-        Phase phq = {0, 0, p.R, p.S};
-        if (stepped) {
-          if (item == first_item) {
-            decode_item(p, item, c_mu, c_nt, split);
-            const int mt0 = c_mu * CTAS + (int)rank;
-            tile_coords(p, (I2C && p.i2c) ? mt0 * BM : mt0, c_wt, c_ht, c_bt);
-          } else if (++c_nt == p.n_tiles_n) {
-            c_nt = 0;
-            ++c_mu;
-            if (I2C && p.i2c) {
-              tile_coords(p, (c_mu * CTAS + (int)rank) * BM, c_wt, c_ht, c_bt);
-            } else {
-              c_wt += CTAS;
-              while (c_wt >= p.w_tiles) { c_wt -= p.w_tiles; if (++c_ht == p.h_tiles) { c_ht = 0; ++c_bt; } }
-            }
-          }
-          mu = c_mu; nt = c_nt; split = 0;
-          w0 = c_wt * p.Wt; h0 = c_ht * p.Ht; b0 = c_bt * p.Bt;
-        } else {
-          int tile = item;
-          if (STRIDED) phq = split_phase(p, item, tile);
-          decode_item(p, tile, mu, nt, split);
-          if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD)
-            pixel_box(p, (mu * CTAS + (int)rank) * ((I2C && p.i2c) ? BM : 1), w0, h0, b0);
-        }
-        if (p.kind == GK_CONV_FWD) { w0 *= p.stride_w; h0 *= p.stride; }     // output pixel -> window origin in x
-        if (I2C && p.i2c) { w0 += p.i2c_w0; h0 += p.i2c_h0; }
-        const int n_ts = phq.n_s;
-        const int mt = mu * CTAS + (int)rank;     // this CTA's 128-row tile
-        const int nb = nt * p.bn + (int)rank * bn_cta;
-        const int kb0 = split * p.kb_per_split;
-        int kb1 = kb0 + p.kb_per_split;
-        if (kb1 > p.kb_total) kb1 = p.kb_total;
-        if (STRIDED) kb1 = phq.n_r * phq.n_s * p.c_chunks;
-        if (p.kind == GK_CONV_WGRAD) {
-          if (p.tg > 1) {
-            tap_n = nt * p.tg + (int)rank * (p.tg / CTAS);
-          } else {
-            tap_n = div_by(nt, p.d_chunks);
-            ci0 = (nt - tap_n * p.n_chunks) * p.bn + (int)rank * bn_cta;
-          }
-        }
-        // k-block counters, stepped instead of divided inside the loop (one thread issues all copies,
-        // so every scalar instruction here is on the critical path):
-        //   forward / dgrad: k-block = (tap row r, tap column s, channel chunk cc)
-        //   wgrad:           k-block = pixel box (kwt, kht, kbt)
-        int cc = 0, ts = 0, tr = 0, kwt = 0, kht = 0, kbt = 0;
-        if (kb0 != 0) {
-          if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) {
-            const int tap = div_by(kb0, p.d_cc);
-            cc = kb0 - tap * p.c_chunks; tr = div_by(tap, p.d_S); ts = tap - tr * p.S;
-          } else if (p.kind == GK_CONV_WGRAD) {
-            tile_coords(p, (I2C && p.i2c) ? kb0 * BM : kb0, kwt, kht, kbt);
-          }
-        }
-        int wg_r = 0, wg_s = 0;
-        if (p.kind == GK_CONV_WGRAD) {
-          if (tap_n >= p.R * p.S) tap_n = p.R * p.S - 1;          // (filler of a last, short tap group)
-          wg_r = div_by(tap_n, p.d_S); wg_s = tap_n - wg_r * p.S;
-        }
-        const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + p.b_boxes * p.b_box_bytes));
-        for (int kb = kb0; kb < kb1; ++kb) {
-         if (owner == warp) {
-          if (!mbar_wait_warp(empty0 + 8 * stage, phase ^ 1, &abort_flag, status)) { ok = false; break; }
-          const unsigned full = lead_full0 + 8 * stage;
-          const unsigned sa = smem_base + stage * stage_bytes;
-          const unsigned sb = sa + p.a_bytes;
-          if (leader) {
-          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, tx_bytes);
-          switch (p.kind) {
-            case GK_FC_FWD:       // A [M][K] K-major, B [N][K] K-major
-              for (int j = 0; j < p.mrep; ++j)     // rows past the end of A are zero-filled by the copy
-                load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, kb * p.kdepth, (mt * p.mrep + j) * BM);
-              load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
-              break;
-            case GK_FC_DGRAD:     // A = e [M][N] K-major; B(k', n) = w[n][k'] MN-major
-              load2<CTAS>(sa, &map_a, full, kb * p.kdepth, mt * BM);
-              for (int j = 0; j < p.b_boxes; ++j)
-                load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
-              break;
-            case GK_FC_WGRAD:     // A(n, m) = e[m][n] MN-major; B(k', m) = a[m][k'] MN-major
-              for (int j = 0; j < p.a_boxes; ++j)
-                load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * p.kdepth);
-              for (int j = 0; j < p.b_boxes; ++j)
-                load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
-              break;
-            case GK_CONV_FWD:     // k-block = (tap, channel chunk); B = w[co][tap][ci]
-              if (I2C && p.i2c) load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, ts, tr);
-              else load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 + ts - p.pad, h0 + tr - p.pad, b0);
-              if (GENERAL) load3<CTAS>(sb, &map_b, full, cc * p.kdepth, tr * p.S + ts, nb);
-              else load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
-              break;
-            case GK_CONV_DGRAD: { // A = e shifted the other way; B(ci, (tap, co)) = w[co][tap][ci]
-              int tap = tr * p.S + ts;
-              if (I2C && p.i2c) {
-                load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, p.T_s - 1 - ts, p.T_r - 1 - tr);
-                if (STRIDED) tap = (phq.r + p.dstride * tr) * p.S + phq.s + p.dstride * ts;
+      // One instance of the loop per kind of multiply: a producer that finds out what to copy for every k-block issues a third
+      // fewer copies.
+      auto produce = [&](auto kind_c, auto i2c_c) {
+        constexpr int KIND = decltype(kind_c)::value;
+        constexpr bool IC = decltype(i2c_c)::value;           // im2col copies
+        const bool stepped = p.blocked && p.splits == 1 && p.raster_g <= 0 && !STRIDED;
+        int c_mu = 0, c_nt = 0, c_wt = 0, c_ht = 0, c_bt = 0;
+        for (int item = first_item; ok && item < item_end; item += item_step) {
+          int mu, nt, split;
+          int w0 = 0, h0 = 0, b0 = 0, tap_n = 0, ci0 = 0;
+          Phase phq = {0, 0, p.R, p.S};
+          if (stepped) {
+            if (item == first_item) {
+              decode_item(p, item, c_mu, c_nt, split);
+              const int mt0 = c_mu * CTAS + (int)rank;
+              tile_coords(p, (IC) ? mt0 * BM : mt0, c_wt, c_ht, c_bt);
+            } else if (++c_nt == p.n_tiles_n) {
+              c_nt = 0;
+              ++c_mu;
+              if (IC) {
+                tile_coords(p, (c_mu * CTAS + (int)rank) * BM, c_wt, c_ht, c_bt);
               } else {
-                load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 - ts + p.pad, h0 - tr + p.pad, b0);
+                c_wt += CTAS;
+                while (c_wt >= p.w_tiles) { c_wt -= p.w_tiles; if (++c_ht == p.h_tiles) { c_ht = 0; ++c_bt; } }
               }
-              for (int j = 0; j < p.b_boxes; ++j)
-                if (GENERAL) load3<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, tap, cc * p.kdepth);
-                else load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, tap * p.Cn + nb + j * p.b_box_step, cc * p.kdepth);
-              break;
             }
-            default: {            // GK_CONV_WGRAD: k-block = pixel box; A = e, B = x shifted by the tap
-              const int kw0 = kwt * p.Wt, kh0 = kht * p.Ht, kbb0 = kbt * p.Bt;
-              if (I2C && p.i2c) {        // consecutive pixels: e as a plain matrix, x as im2col rows of the same pixels
+            mu = c_mu; nt = c_nt; split = 0;
+            w0 = c_wt * p.Wt; h0 = c_ht * p.Ht; b0 = c_bt * p.Bt;
+          } else {
+            int tile = item;
+            if (STRIDED) phq = split_phase(p, item, tile);
+            decode_item(p, tile, mu, nt, split);
+            if (KIND == GK_CONV_FWD || KIND == GK_CONV_DGRAD)
+              pixel_box(p, (mu * CTAS + (int)rank) * ((IC) ? BM : 1), w0, h0, b0);
+          }
+          if (KIND == GK_CONV_FWD) { w0 *= p.stride_w; h0 *= p.stride; }     // output pixel -> window origin in x
+          if (IC) { w0 += p.i2c_w0; h0 += p.i2c_h0; }
+          const int n_ts = phq.n_s;
+          const int mt = mu * CTAS + (int)rank;     // this CTA's 128-row tile
+          const int nb = nt * p.bn + (int)rank * bn_cta;
+          const int kb0 = split * p.kb_per_split;
+          int kb1 = kb0 + p.kb_per_split;
+          if (kb1 > p.kb_total) kb1 = p.kb_total;
+          if (STRIDED) kb1 = phq.n_r * phq.n_s * p.c_chunks;
+          if (KIND == GK_CONV_WGRAD) {
+            if (p.tg > 1) {
+              tap_n = nt * p.tg + (int)rank * (p.tg / CTAS);
+            } else {
+              tap_n = div_by(nt, p.d_chunks);
+              ci0 = (nt - tap_n * p.n_chunks) * p.bn + (int)rank * bn_cta;
+            }
+          }
+          // k-block counters, stepped instead of divided inside the loop (one thread issues all copies,
+          // so every scalar instruction here is on the critical path):
+          //   forward / dgrad: k-block = (tap row r, tap column s, channel chunk cc)
+          //   wgrad:           k-block = pixel box (kwt, kht, kbt)
+          int cc = 0, ts = 0, tr = 0, kwt = 0, kht = 0, kbt = 0;
+          if (kb0 != 0) {
+            if (KIND == GK_CONV_FWD || KIND == GK_CONV_DGRAD) {
+              const int tap = div_by(kb0, p.d_cc);
+              cc = kb0 - tap * p.c_chunks; tr = div_by(tap, p.d_S); ts = tap - tr * p.S;
+            } else if (KIND == GK_CONV_WGRAD) {
+              tile_coords(p, (IC) ? kb0 * BM : kb0, kwt, kht, kbt);
+            }
+          }
+          int wg_r = 0, wg_s = 0;
+          if (KIND == GK_CONV_WGRAD) {
+            if (tap_n >= p.R * p.S) tap_n = p.R * p.S - 1;          // (filler of a last, short tap group)
+            wg_r = div_by(tap_n, p.d_S); wg_s = tap_n - wg_r * p.S;
+          }
+          const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + p.b_boxes * p.b_box_bytes));
+          for (int kb = kb0; kb < kb1; ++kb) {
+           if (owner == warp) {
+            if (!mbar_wait_warp(empty0 + 8 * stage, phase ^ 1, &abort_flag, status)) { ok = false; break; }
+            const unsigned full = lead_full0 + 8 * stage;
+            const unsigned sa = smem_base + stage * stage_bytes;
+            const unsigned sb = sa + p.a_bytes;
+            if (leader) {
+            if (rank == 0) mbar_expect_tx(full0 + 8 * stage, tx_bytes);
+            switch (KIND) {                       // (one case per instance of the loop)
+              case GK_FC_FWD:       // A [M][K] K-major, B [N][K] K-major
+                for (int j = 0; j < p.mrep; ++j)     // rows past the end of A are zero-filled by the copy
+                  load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, kb * p.kdepth, (mt * p.mrep + j) * BM);
+                load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+                break;
+              case GK_FC_DGRAD:     // A = e [M][N] K-major; B(k', n) = w[n][k'] MN-major
+                load2<CTAS>(sa, &map_a, full, kb * p.kdepth, mt * BM);
+                for (int j = 0; j < p.b_boxes; ++j)
+                  load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
+                break;
+              case GK_FC_WGRAD:     // A(n, m) = e[m][n] MN-major; B(k', m) = a[m][k'] MN-major
                 for (int j = 0; j < p.a_boxes; ++j)
-                  load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * BM);
-                for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
-                  load_im2col<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step,
-                                    kwt * p.stride_w + p.i2c_w0, kht * p.stride + p.i2c_h0, kbt, ts2, tr2);
-                  if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
+                  load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * p.kdepth);
+                for (int j = 0; j < p.b_boxes; ++j)
+                  load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
+                break;
+              case GK_CONV_FWD:     // k-block = (tap, channel chunk); B = w[co][tap][ci]
+                if (IC) load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, ts, tr);
+                else load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 + ts - p.pad, h0 + tr - p.pad, b0);
+                if (GENERAL) load3<CTAS>(sb, &map_b, full, cc * p.kdepth, tr * p.S + ts, nb);
+                else load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+                break;
+              case GK_CONV_DGRAD: { // A = e shifted the other way; B(ci, (tap, co)) = w[co][tap][ci]
+                int tap = tr * p.S + ts;
+                if (IC) {
+                  load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, p.T_s - 1 - ts, p.T_r - 1 - tr);
+                  if (STRIDED) tap = (phq.r + p.dstride * tr) * p.S + phq.s + p.dstride * ts;
+                } else {
+                  load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 - ts + p.pad, h0 - tr + p.pad, b0);
+                }
+                for (int j = 0; j < p.b_boxes; ++j)
+                  if (GENERAL) load3<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, tap, cc * p.kdepth);
+                  else load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, tap * p.Cn + nb + j * p.b_box_step, cc * p.kdepth);
+                break;
+              }
+              default: {            // GK_CONV_WGRAD: k-block = pixel box; A = e, B = x shifted by the tap
+                const int kw0 = kwt * p.Wt, kh0 = kht * p.Ht, kbb0 = kbt * p.Bt;
+                if (IC) {        // consecutive pixels: e as a plain matrix, x as im2col rows of the same pixels
+                  for (int j = 0; j < p.a_boxes; ++j)
+                    load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kb * BM);
+                  for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
+                    load_im2col<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step,
+                                      kwt * p.stride_w + p.i2c_w0, kht * p.stride + p.i2c_h0, kbt, ts2, tr2);
+                    if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
+                  }
+                } else {
+                  for (int j = 0; j < p.a_boxes; ++j)
+                    load4<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kw0, kh0, kbb0);
+                  for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
+                    load4<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step, kw0 * p.stride + ts2 - p.pad,
+                                kh0 * p.stride + tr2 - p.pad, kbb0);
+                    if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
+                  }
                 }
                 break;
               }
-              for (int j = 0; j < p.a_boxes; ++j)
-                load4<CTAS>(sa + j * p.a_box_bytes, &map_a, full, mt * BM + j * p.a_box_step, kw0, kh0, kbb0);
-              for (int j = 0, jb = 0, tr2 = wg_r, ts2 = wg_s; j < p.b_boxes; ++j) {
-                load4<CTAS>(sb + j * p.b_box_bytes, &map_b, full, ci0 + jb * p.b_box_step, kw0 * p.stride + ts2 - p.pad,
-                            kh0 * p.stride + tr2 - p.pad, kbb0);
-                if (++jb == p.tg_boxes) next_tap(p, jb, tr2, ts2);
-              }
-              break;
             }
+            }
+           }
+            if (KIND == GK_CONV_FWD || KIND == GK_CONV_DGRAD) {
+              if (++cc == p.c_chunks) { cc = 0; if (++ts == n_ts) { ts = 0; ++tr; } }
+            } else if (KIND == GK_CONV_WGRAD) {
+              if (IC) {          // 128 pixels further in the grid
+                kwt += p.i2c_dj;
+                if (kwt >= p.w_tiles) { kwt -= p.w_tiles; ++kht; }
+                kht += p.i2c_di;
+                if (kht >= p.h_tiles) { kht -= p.h_tiles; ++kbt; }
+                kbt += p.i2c_db;
+              } else if (++kwt == p.w_tiles) { kwt = 0; if (++kht == p.h_tiles) { kht = 0; ++kbt; } }
+            }
+            if (++owner == nprod) owner = 0;
+            if (++stage == p.stages) { stage = 0; phase ^= 1; }
           }
-          }
-         }
-          if (p.kind == GK_CONV_FWD || p.kind == GK_CONV_DGRAD) {
-            if (++cc == p.c_chunks) { cc = 0; if (++ts == n_ts) { ts = 0; ++tr; } }
-          } else if (p.kind == GK_CONV_WGRAD) {
-            if (I2C && p.i2c) {          // 128 pixels further in the grid
-              kwt += p.i2c_dj;
-              if (kwt >= p.w_tiles) { kwt -= p.w_tiles; ++kht; }
-              kht += p.i2c_di;
-              if (kht >= p.h_tiles) { kht -= p.h_tiles; ++kbt; }
-              kbt += p.i2c_db;
-            } else if (++kwt == p.w_tiles) { kwt = 0; if (++kht == p.h_tiles) { kht = 0; ++kbt; } }
-          }
-          if (++owner == nprod) owner = 0;
-          if (++stage == p.stages) { stage = 0; phase ^= 1; }
         }
+      };
+      if (ok && first_item < item_end) {
+        auto run = [&](auto kind_c) {
+          if (I2C && p.i2c) produce(kind_c, std::integral_constant<bool, I2C>{});
+          else if (!STRIDED) produce(kind_c, std::false_type{});
+        };
+        if (STRIDED || p.kind == GK_CONV_DGRAD) run(std::integral_constant<int, GK_CONV_DGRAD>{});
+        else if (p.kind == GK_CONV_FWD) run(std::integral_constant<int, GK_CONV_FWD>{});
+        else if (p.kind == GK_CONV_WGRAD) run(std::integral_constant<int, GK_CONV_WGRAD>{});
+        else if (p.kind == GK_FC_FWD) produce(std::integral_constant<int, GK_FC_FWD>{}, std::false_type{});
+        else if (p.kind == GK_FC_DGRAD) produce(std::integral_constant<int, GK_FC_DGRAD>{}, std::false_type{});
+        else produce(std::integral_constant<int, GK_FC_WGRAD>{}, std::false_type{});
       }
     }
   } else if (warp == MMA_WARP) {
