@@ -300,6 +300,13 @@ int niti_set_reduce_hook(niti_ctx *ctx, niti_reduce_fn fn, void *user);
  * node).  ws = NULL ends the arrangement.  Results do not change. */
 int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_bytes);
 
+/* Declares `ws` this context's own: between the calls that use it nobody else writes to its first
+ * 256 KB (the headers), and the calls that use it through this context are ordered one after the
+ * other, on whatever streams.  Calls outside a niti_begin_step arrangement on it then leave a zeroed header for their
+ * successor instead of clearing one first.  (Calls that are being captured clear theirs themselves.)  A new buffer, also
+ * one at the same address, has to be declared again.  ws = NULL ends the arrangement.  Results do not change. */
+int niti_own_workspace(niti_ctx *ctx, void *ws, size_t ws_bytes);
+
 /* Convolutions with very few input channels (R * S * Cin <= 32: the first layer of an image network)
  * are run as a matrix multiply over rows of gathered taps, 32 bytes per output pixel.  Forward and
  * weight gradient of such a layer read the same rows.  With a tap cache installed (a caller-owned

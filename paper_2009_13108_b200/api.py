@@ -22,7 +22,7 @@ _REDUCE_FN = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64,
 
 EXPORTS = [
     "niti_create", "niti_destroy", "niti_last_error", "niti_check", "niti_workspace_bytes",
-    "niti_set_engine", "niti_set_reduce_hook", "niti_set_dp_shard", "niti_set_tap_cache", "niti_begin_step", "niti_launch_count", "niti_tc_launch_count", "niti_tc_pair_launch_count",
+    "niti_set_engine", "niti_set_reduce_hook", "niti_set_dp_shard", "niti_set_tap_cache", "niti_begin_step", "niti_own_workspace", "niti_launch_count", "niti_tc_launch_count", "niti_tc_pair_launch_count",
     "niti_redo_count", "niti_selftest_timeout", "niti_profile_enable", "niti_profile_read_launches",
     "niti_profile_read", "niti_linear_fwd", "niti_linear_bwd", "niti_conv_fwd",
     "niti_conv_dgrad", "niti_conv_wgrad", "niti_conv_fwd_pool", "niti_conv_fwd_strided", "niti_conv_dgrad_strided", "niti_conv_wgrad_strided",
@@ -67,6 +67,7 @@ def load_library():
     lib.niti_set_dp_shard.argtypes = [vp, i32, i32]
     lib.niti_set_tap_cache.argtypes = [vp, vp, sz]
     lib.niti_begin_step.argtypes = [vp, vp, vp, sz]
+    lib.niti_own_workspace.argtypes = [vp, vp, sz]
     lib.niti_launch_count.argtypes = [vp]
     lib.niti_launch_count.restype = C.c_uint64
     lib.niti_tc_launch_count.argtypes = [vp]
@@ -122,7 +123,7 @@ class Niti:
         if rc != OK:
             raise NitiError(rc, "niti_create failed (needs an sm_100 device)")
         self.h = h
-        self._ws = torch.empty(1 << 20, dtype=torch.uint8, device=self.device)
+        self._own_workspace(1 << 20)
         self._ws_need = {}                 # workspace bytes of (op, dims) already asked for
 
     def close(self):
@@ -194,7 +195,12 @@ class Niti:
     def reserve_workspace(self, nbytes: int):
         if self._ws.numel() < nbytes:
             self._ck(self.lib.niti_begin_step(self.h, None, None, 0))      # the old buffer's headers are gone
-            self._ws = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
+            self._own_workspace(nbytes)
+
+    def _own_workspace(self, nbytes: int):
+        """A new workspace, declared to the library as nobody else's (see niti_own_workspace)."""
+        self._ws = self._owned_ws = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
+        self._ck(self.lib.niti_own_workspace(self.h, self._ws.data_ptr(), nbytes))
 
     def begin_step(self):
         """niti_begin_step on this object's workspace: one launch clears the headers that the next 64
@@ -211,6 +217,9 @@ class Niti:
                 self._ws_need.clear()
             self._ws_need[op, dims] = need
         ws = self._ws
+        if ws is not self._owned_ws:                       # (somebody put another buffer in its place)
+            self._owned_ws = ws
+            self._ck(self.lib.niti_own_workspace(self.h, None, 0))
         if ws.numel() < need:
             self.reserve_workspace(need)
             ws = self._ws

@@ -194,6 +194,17 @@ extern "C" int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_
   if (rc != NITI_OK) return rc;
   ctx->step_ws = ws;
   ctx->step_slot = 0;
+  if (ws == ctx->own_ws) ctx->own_clean = 0;
+  return NITI_OK;
+}
+
+extern "C" int niti_own_workspace(niti_ctx *ctx, void *ws, size_t ws_bytes) {
+  if (!ctx) return NITI_ERR_ARG;
+  if (ws && (((uintptr_t)ws & 255) || ws_bytes < NITI_WS_HEADER))
+    return niti_fail(ctx, NITI_ERR_WORKSPACE, "niti_own_workspace: workspace misaligned or too small");
+  ctx->own_ws = ws;
+  ctx->own_next = 0;
+  ctx->own_clean = 0;
   return NITI_OK;
 }
 
@@ -442,7 +453,7 @@ static int run_gemm_round(niti_ctx *ctx, cudaStream_t st, GemmProblem p, void *w
                           const GemmProblem *tc_form = nullptr, bool tc_refused = false) {
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < need)
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "workspace missing, misaligned or too small");
-  WsHeader *hdr = niti_take_header(ctx, ws);
+  WsHeader *hdr = niti_take_header(ctx, st, ws);
   int32_t *acc = (int32_t *)((char *)ws + NITI_WS_HEADER);
   int rc = NITI_OK;
   const bool narrow = p.kind <= GK_FC_WGRAD && p.N < 32 && p.kind != GK_FC_FWD;       // (the CUDA-core engine's)
@@ -731,7 +742,7 @@ static int conv_wgrad_impl(niti_ctx *ctx, void *stream, const int8_t *x, const i
     // columns that are taps are then rounded into g, or subtracted from the weights
     cudaStream_t st = (cudaStream_t)stream;
     const size_t M = (size_t)B * p.Ho * p.Wo;
-    WsHeader *hdr = niti_take_header(ctx, ws);
+    WsHeader *hdr = niti_take_header(ctx, st, ws);
     int rc = NITI_OK;
     int8_t *xcol = (int8_t *)conv_pad_mem(p, ws);
     const size_t x_bytes = wg.Cp ? wg.x_bytes + wg.w_bytes : round_up(M * 32, 256) + round_up((size_t)Cout * 32, 256);

@@ -694,8 +694,9 @@ template <bool PACKED, bool ONE, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS)
 xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, const int32_t *__restrict__ labels,
             long long *rowinfo, WsHeader *hdr, int8_t *__restrict__ out, int B, int N, int round_mode, int32_t *__restrict__ b_out,
-            int32_t *__restrict__ n_correct, uint32_t *__restrict__ status, unsigned patience) {
+            int32_t *__restrict__ n_correct, uint32_t *__restrict__ status, unsigned patience, WsHeader *next) {
   niti_enter(a, s_a_ptr, labels);
+  if (next && blockIdx.x == 0 && threadIdx.x >= 32 * (WARPS - 1)) niti_zero_header(next, (int)threadIdx.x & 31);
   __shared__ unsigned long long sh_max[WARPS];
   __shared__ int sh_hit[WARPS];
   __shared__ unsigned blk_b, grid_b, ticket;
@@ -756,9 +757,9 @@ xent_kernel(const int8_t *__restrict__ a, const int32_t *__restrict__ s_a_ptr, c
 template <bool PACKED, bool ONE>
 static void launch_xent_one(int grid, int warps, cudaStream_t st, const int8_t *a, const int32_t *s_a, const int32_t *labels,
                             long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N, int round_mode,
-                            uint32_t *status, unsigned patience) {
+                            uint32_t *status, unsigned patience, WsHeader *next) {
   auto go = [&](auto kernel) {
-    niti_launch(st, grid, 32 * warps, 0, kernel, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status, patience);
+    niti_launch(st, grid, 32 * warps, 0, kernel, a, s_a, labels, rowinfo, hdr, e, B, N, round_mode, b_e, n_correct, status, patience, next);
   };
   if (warps == 8) go(xent_kernel<PACKED, ONE, 8>);
   else if (warps == 16) go(xent_kernel<PACKED, ONE, 16>);
@@ -769,7 +770,7 @@ static void launch_xent_one(int grid, int warps, cudaStream_t st, const int8_t *
 // magnitude of the 64-bit gradients is combined over the ranks between the two passes when a reduction hook is installed)
 static int launch_xent(niti_ctx *ctx, cudaStream_t st, const int8_t *a, const int32_t *s_a, const int32_t *labels,
                        long long *rowinfo, WsHeader *hdr, int8_t *e, int32_t *b_e, int32_t *n_correct, int B, int N,
-                       int round_mode, uint32_t *status) {
+                       int round_mode, uint32_t *status, WsHeader *next = nullptr) {
   const bool packed = (N & 3) == 0 && N >= 64 && (((uintptr_t)a | (uintptr_t)e) & 3) == 0;
   if (ctx && !ctx->reduce_fn) {
     const int sms = ctx->sm_count < NITI_AGREE_MAX ? ctx->sm_count : NITI_AGREE_MAX;
@@ -778,7 +779,7 @@ static int launch_xent(niti_ctx *ctx, cudaStream_t st, const int8_t *a, const in
     const int warps = B <= 8 * sms ? 8 : B <= 16 * sms ? 16 : XENT_MAX_WARPS;
     const int need = (B + warps - 1) / warps, grid = need < sms ? need : sms;
     const bool one = (packed ? N >> 2 <= 32 * xent_held<true> : N <= 32 * xent_held<false>) && B <= grid * warps;
-    auto go = [&](auto launch) { launch(grid, warps, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status, ctx->patience); };
+    auto go = [&](auto launch) { launch(grid, warps, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, status, ctx->patience, next); };
     if (packed) { if (one) go(launch_xent_one<true, true>); else go(launch_xent_one<true, false>); }
     else { if (one) go(launch_xent_one<false, true>); else go(launch_xent_one<false, false>); }
     ctx->launches++;
@@ -807,13 +808,14 @@ extern "C" int niti_int_xent(niti_ctx *ctx, void *stream, const int8_t *a, const
   if (!ws || ((uintptr_t)ws & 255) || ws_bytes < niti_workspace_bytes(NITI_OP_INT_XENT, dims, 2))
     return niti_fail(ctx, NITI_ERR_WORKSPACE, "niti_int_xent: workspace missing, misaligned or too small");
   cudaStream_t st = (cudaStream_t)stream;
-  WsHeader *hdr = niti_take_header(ctx, ws);
+  WsHeader *hdr = niti_take_header(ctx, st, ws), *next = nullptr;
   long long *rowinfo = (long long *)((char *)ws + NITI_WS_HEADER);
-  const int rch = niti_clear(ctx, st);
+  const int rch = niti_clear(ctx, st, nullptr, 0, ctx->reduce_fn ? nullptr : &next);
   if (rch != NITI_OK) return rch;
-  const int rcx = launch_xent(ctx, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, ctx->d_status);
+  const int rcx = launch_xent(ctx, st, a, s_a, labels, rowinfo, hdr, e, b_e, n_correct, B, N, round_mode, ctx->d_status, next);
   if (rcx != NITI_OK) return rcx;
   NITI_CUDA_TRY(ctx, cudaGetLastError());
+  niti_header_passed_on(ctx, next);
   return NITI_OK;
 }
 

@@ -47,6 +47,7 @@ struct SmallParams {
   int round_mode;
   unsigned patience;
   WsHeader *hdr;              // cleared
+  WsHeader *next;             // to be cleared for the next call, or null
   int32_t *left;              // in the workspace: sums of regions whose CTAs left, [gm][gn] of op[0], then of op[1]
   uint32_t *status;
 };
@@ -241,6 +242,7 @@ small_gemm_kernel(const __grid_constant__ SmallParams p) {
   if (tid == 0) cta_max = 0;
   niti_enter();
   unsigned came = 0;
+  if (blockIdx.x == 0 && warp == SMALL_WARPS - 1 && p.next) niti_zero_header(p.next, lane);
   if (tid == 32) came = niti_arrive(p.hdr);
   unsigned mx = 0;
   {
@@ -440,13 +442,14 @@ int niti_small_gemm(niti_ctx *ctx, cudaStream_t st, void *ws, const GemmProblem 
     const size_t s2 = region_smem(p.op[1].rm, p.op[1].rn, p.op[1].kc);
     if (s2 > smem) smem = s2;
   }
-  WsHeader *hdr = niti_take_header(ctx, ws);
-  const int rc = niti_clear(ctx, st);
+  WsHeader *hdr = niti_take_header(ctx, st, ws);
+  const int rc = niti_clear(ctx, st, nullptr, 0, &p.next);
   if (rc != NITI_OK) return rc;
   p.hdr = hdr;
   p.patience = ctx->patience;
   p.left = (int32_t *)((char *)ws + NITI_WS_HEADER);
   NITI_CUDA_TRY(ctx, niti_launch(st, (unsigned)grid, SMALL_THREADS, smem, small_gemm_kernel, p));
+  niti_header_passed_on(ctx, p.next);
   ctx->launches++;
   ctx->tc_launches += g2 ? 2 : 1;
   return NITI_OK;

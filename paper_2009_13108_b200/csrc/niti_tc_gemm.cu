@@ -157,6 +157,7 @@ struct TcParams {
   int update;                   // 1: out8 holds weights: the epilogue stores clamp(w - rounded gradient, +-127)
   int pool;                     // 1: the epilogue also stores the 2 x 2 max-pool of the (ReLU'd) output tile
   int pool_xh;                  // lane distance of the pixel one image row below (the pixel to the right is lane ^ 1)
+  WsHeader *next;               // header to be zeroed for the next call, or null
   int single_wave;              // every CTA has at most one tile: the sample is the whole tensor, the shift
                                 // is exact, and whoever rounds the first CTA's tile publishes b and the exponent
 };
@@ -1137,6 +1138,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   const int8_t *const mask_at_exit = mask8;          // (the parameter itself: costs the main loops no register)
   niti_enter(mask8);
   if (ONE && threadIdx.x == NUM_THREADS - 1) ticket = niti_arrive(hdr);      // (a thread that has to wait anyway)
+  if (p.next && blockIdx.x == 0 && warp == NUM_THREADS / 32 - 2) niti_zero_header(p.next, lane);
 
   // the scalars of a single-wave launch: the shift is exact, and no second launch publishes them
   auto publish_exact = [&](int b) {
@@ -3256,7 +3258,8 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     else NITI_CUDA_TRY(ctx, cudaMemsetAsync(r.out, 0, (size_t)(g.gm * g.gn), st));
     ctx->launches++;
   }
-  int rc = p.epi_mode == EPI_ATOMIC ? niti_clear(ctx, st, acc, sizeof(int32_t) * (size_t)(g.gm * g.gn)) : niti_clear(ctx, st);
+  const bool sums = p.epi_mode == EPI_ATOMIC;
+  int rc = niti_clear(ctx, st, sums ? acc : nullptr, sums ? sizeof(int32_t) * (size_t)(g.gm * g.gn) : 0, &p.next);
   if (rc != NITI_OK) return rc;
   // Fused 2 x 2 max-pool: the fused epilogue of a forward convolution with ReLU also stores the pooled
   // tile when every pooling window lies inside one warp's 32 pixels (8 x 16 pixel tiles of the
@@ -3290,6 +3293,8 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   if (prof) prof_record(ctx->prof_ev[2 * ctx->prof_used], st);
   rc = launch_tc(ctx, st, p, ma, mb, mc, acc, hdr, r);
   if (rc != NITI_OK) return rc;
+  niti_header_passed_on(ctx, p.next);
+  p.next = nullptr;
   if (p.epi_mode == EPI_SPECULATE && p.single_wave) {
     *fused = true;                     // exact shift, scalars published by this launch: no second one
   } else if (p.epi_mode == EPI_SPECULATE) {

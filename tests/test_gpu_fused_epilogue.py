@@ -71,3 +71,65 @@ def test_outputs_in_the_storage_of_an_operand(niti, oref, M, N):
         _, g, b_e, b_g = niti.linear_bwd(at, T(e), T(w), True, at, e_prev=at)
         assert np.array_equal(at.cpu().numpy(), we) and np.array_equal(g.cpu().numpy(), wg)
         assert (int(b_e), int(b_g)) == (be, bg)
+
+
+def test_headers_of_an_own_workspace(oref):
+    """Calls outside a step leave a clean header for the next one, whatever the path of either, a captured call (whose replays
+    repeat) and a step between them, and a buffer put in the workspace's place."""
+    from paper_2009_13108_b200 import Niti
+    n = Niti(0)
+    rng = np.random.default_rng(5)
+    i8 = lambda *s: rng.integers(-127, 128, size=s, dtype=np.int8)  # noqa: E731
+    T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(n.device)  # noqa: E731
+    x, w, e, lab = i8(4, 20, 20, 64), i8(64, 3, 3, 64), i8(4, 20, 20, 64), rng.integers(0, 64, 33).astype(np.int32)
+    a, wl = i8(33, 70), i8(64, 70)
+    xt, wt, et, at, wlt, labt = T(x), T(w), T(e), T(a), T(wl), T(lab)
+    sx, sw = n.scalar(-7), n.scalar(-9)
+    want = [oref.conv_fwd(x, -7, w, -9, 1, True)[0], oref.conv_dgrad(e, w, (20, 20), 1, None)[0], oref.conv_wgrad(x, e, (3, 3), 1, 5)[0],
+            oref.linear_fwd(a, -7, wl, -9, False)[0]]
+    want.append(oref.int_xent(want[3], -3, lab)[0])
+    logits, s3 = T(want[3]), n.scalar(-3)
+    calls = [lambda: n.conv_fwd(xt, sx, wt, sw, relu=True)[0], lambda: n.conv_dgrad(et, wt, (20, 20))[0],
+             lambda: n.conv_wgrad(xt, et, (3, 3))[0], lambda: n.linear_fwd(at, sx, wlt, sw)[0],
+             lambda: n.int_xent(logits, s3, labt)[0]]
+
+    def check(order):
+        for k in order:
+            assert np.array_equal(calls[k]().cpu().numpy(), want[k]), k
+
+    def all_pairs():
+        for engine in (0, 6, 2, 4, 1):                       # (one wave, leaving CTAs, single CTAs, two passes, CUDA cores)
+            n.set_engine(engine)
+            check([i for p in range(5) for q in range(5) for i in (p, q)])
+        n.set_engine(0)
+
+    all_pairs()
+    launches = []
+    for _ in range(3):
+        l0 = n.launch_count()
+        calls[3]()
+        launches.append(n.launch_count() - l0)
+    assert launches == [1, 1, 1]                             # no clear of its own
+    y = torch.empty((4, 20, 20, 64), dtype=torch.int8, device=n.device)
+    st = torch.cuda.Stream(device=n.device)
+    st.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    s_y, b_y = n.scalar(), n.scalar()
+    with torch.cuda.graph(graph, stream=st):
+        n.conv_fwd(xt, sx, wt, sw, y=y, s_y=s_y, b_y=b_y, relu=True)
+    for k in (3, 0, 4, 2):
+        y.zero_()
+        graph.replay()
+        graph.replay()
+        check([k])
+        assert np.array_equal(y.cpu().numpy(), want[0])
+    n.begin_step()
+    check(list(range(5)) * 14)                               # (70 calls: past the step's headers)
+    n._ck(n.lib.niti_begin_step(n.h, None, None, 0))
+    check(range(5))
+    n._ws = torch.full((n._ws.numel(),), 0x5A, dtype=torch.uint8, device=n.device)
+    check(list(range(5)) * 2)
+    n.reserve_workspace(2 * n._ws.numel())
+    all_pairs()
+    n.check()
+    n.close()
