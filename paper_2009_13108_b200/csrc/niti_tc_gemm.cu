@@ -148,6 +148,7 @@ struct TcParams {
   int wg_nci;                   // 64-channel blocks of the input channels
   int b_tile_bytes;             // bytes of one tap's weight tile
   int b_res_bytes;              // bytes of the resident weights (all taps), multiple of 1024
+  int b_resident;               // generic loops: the B tiles of all k-blocks (b_tile_bytes each) stay in shared memory as well
   // epilogue
   int epi_mode;                 // EPI_SPILL / EPI_ATOMIC / EPI_SPECULATE / EPI_KNOWN_B
   int mbits, round_mode, relu;
@@ -1244,6 +1245,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       auto produce = [&](auto kind_c, auto i2c_c) {
         constexpr int KIND = decltype(kind_c)::value;
         constexpr bool IC = decltype(i2c_c)::value;           // im2col copies
+        // the B tile of a k-block (forward and error multiplies)
+        auto load_b = [&](unsigned sb, unsigned full, int kb, int cc, int tap, int nb) {
+          if (KIND == GK_FC_FWD) {
+            load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+          } else if (KIND == GK_CONV_FWD) {
+            if (GENERAL) load3<CTAS>(sb, &map_b, full, cc * p.kdepth, tap, nb);
+            else load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+          } else {
+            for (int j = 0; j < p.b_boxes; ++j)
+              if (KIND == GK_FC_DGRAD) load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
+              else if (GENERAL) load3<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, tap, cc * p.kdepth);
+              else load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, tap * p.Cn + nb + j * p.b_box_step, cc * p.kdepth);
+          }
+        };
+        constexpr bool RES = CTAS == 1 && !ONE && !STRIDED && KIND != GK_FC_WGRAD && KIND != GK_CONV_WGRAD;
+        const bool resident = RES && p.b_resident != 0;
         const bool stepped = p.blocked && p.splits == 1 && p.raster_g <= 0 && !STRIDED;
         int c_mu = 0, c_nt = 0, c_wt = 0, c_ht = 0, c_bt = 0;
         for (int item = first_item; ok && item < item_end; item += item_step) {
@@ -1309,25 +1326,25 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             if (tap_n >= p.R * p.S) tap_n = p.R * p.S - 1;          // (filler of a last, short tap group)
             wg_r = div_by(tap_n, p.d_S); wg_s = tap_n - wg_r * p.S;
           }
-          const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + p.b_boxes * p.b_box_bytes));
+          const bool with_b = !resident || item == first_item;       // (resident: the first tile's copies bring them)
+          const unsigned tx_bytes = (unsigned)(CTAS * (p.a_boxes * p.a_box_bytes + (with_b ? p.b_boxes * p.b_box_bytes : 0)));
           for (int kb = kb0; kb < kb1; ++kb) {
            if (owner == warp) {
             if (!mbar_wait_warp(empty0 + 8 * stage, phase ^ 1, &abort_flag, status)) { ok = false; break; }
             const unsigned full = lead_full0 + 8 * stage;
-            const unsigned sa = smem_base + stage * stage_bytes;
-            const unsigned sb = sa + p.a_bytes;
+            const unsigned sa = smem_base + p.b_res_bytes + stage * stage_bytes;
+            const unsigned sb = resident ? smem_base + kb * p.b_tile_bytes : sa + p.a_bytes;
             if (leader) {
             if (rank == 0) mbar_expect_tx(full0 + 8 * stage, tx_bytes);
             switch (KIND) {                       // (one case per instance of the loop)
               case GK_FC_FWD:       // A [M][K] K-major, B [N][K] K-major
                 for (int j = 0; j < p.mrep; ++j)     // rows past the end of A are zero-filled by the copy
                   load2<CTAS>(sa + j * p.a_box_bytes, &map_a, full, kb * p.kdepth, (mt * p.mrep + j) * BM);
-                load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+                if (with_b) load_b(sb, full, kb, 0, 0, nb);
                 break;
               case GK_FC_DGRAD:     // A = e [M][N] K-major; B(k', n) = w[n][k'] MN-major
                 load2<CTAS>(sa, &map_a, full, kb * p.kdepth, mt * BM);
-                for (int j = 0; j < p.b_boxes; ++j)
-                  load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, kb * p.kdepth);
+                if (with_b) load_b(sb, full, kb, 0, 0, nb);
                 break;
               case GK_FC_WGRAD:     // A(n, m) = e[m][n] MN-major; B(k', m) = a[m][k'] MN-major
                 for (int j = 0; j < p.a_boxes; ++j)
@@ -1338,8 +1355,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               case GK_CONV_FWD:     // k-block = (tap, channel chunk); B = w[co][tap][ci]
                 if (IC) load_im2col<CTAS>(sa, &map_a, full, cc * p.kdepth, w0, h0, b0, ts, tr);
                 else load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 + ts - p.pad, h0 + tr - p.pad, b0);
-                if (GENERAL) load3<CTAS>(sb, &map_b, full, cc * p.kdepth, tr * p.S + ts, nb);
-                else load2<CTAS>(sb, &map_b, full, kb * p.kdepth, nb);
+                if (with_b) load_b(sb, full, kb, cc, tr * p.S + ts, nb);
                 break;
               case GK_CONV_DGRAD: { // A = e shifted the other way; B(ci, (tap, co)) = w[co][tap][ci]
                 int tap = tr * p.S + ts;
@@ -1349,9 +1365,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 } else {
                   load4<CTAS>(sa, &map_a, full, cc * p.kdepth, w0 - ts + p.pad, h0 - tr + p.pad, b0);
                 }
-                for (int j = 0; j < p.b_boxes; ++j)
-                  if (GENERAL) load3<CTAS>(sb + j * p.b_box_bytes, &map_b, full, nb + j * p.b_box_step, tap, cc * p.kdepth);
-                  else load2<CTAS>(sb + j * p.b_box_bytes, &map_b, full, tap * p.Cn + nb + j * p.b_box_step, cc * p.kdepth);
+                if (with_b) load_b(sb, full, kb, cc, tap, nb);
                 break;
               }
               default: {            // GK_CONV_WGRAD: k-block = pixel box; A = e, B = x shifted by the tap
@@ -1470,6 +1484,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const int g_ksteps = p.ksteps, g_mrep = p.mrep, g_tail = GENERAL ? p.tail_ks : 0;
       const unsigned g_bn_mma = (unsigned)p.bn_mma, g_slice16 = (unsigned)p.a_box_bytes >> 4;
       unsigned gbuf = 0, gpar = 0;            // use % nbuf, (use / nbuf) & 1, counted
+      const bool resident = CTAS == 1 && !ONE && !STRIDED && p.b_resident != 0;
+      const unsigned g_btile16 = (unsigned)p.b_tile_bytes >> 4;
       for (int item = first_item; ok && item < item_end; item += item_step, ++use) {
         const int split = p.splits > 1 ? item - div_by(item, p.d_split) * p.splits : 0;
         const int kb0 = split * p.kb_per_split;
@@ -1490,8 +1506,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait_warp(full0 + 8 * stage, phase, &abort_flag, status)) { ok = false; break; }
           tc_fence_after();
-          const unsigned sa = smem_base + stage * stage_bytes;
-          const unsigned a_lo = g_a_lo0 + ((sa >> 4) & 0x3fff), b_lo = g_b_lo0 + (((sa + g_a_bytes) >> 4) & 0x3fff);
+          const unsigned sa = smem_base + p.b_res_bytes + stage * stage_bytes;
+          const unsigned a_lo = g_a_lo0 + ((sa >> 4) & 0x3fff);
+          const unsigned b_lo = g_b_lo0 + (resident ? ((smem_base >> 4) & 0x3fff) + (unsigned)kb * g_btile16 : ((sa + g_a_bytes) >> 4) & 0x3fff);
           const unsigned first_acc = kb > kb0 ? 1u : 0u;
           int ks = g_ksteps;
           if (g_tail && --cc_left == 0) { ks = g_tail; cc_left = p.c_chunks; }
@@ -2862,14 +2879,30 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   }
   // (tap groups only where the sums leave through reduce copies, which place every tap's columns)
   if (p.tg > 1 && !(p.splits > 1 && p.red)) return plan(ctx, g, ctas, want, aligned, -1, acc, p, ma, mb, mc);
+  // All of B resident: with one column tile every tile reads the same B tiles again, and short contractions are bound by their
+  // copies (about 4 cycles a row).  Where they leave room for the A stages, the first tile of a CTA copies them and the others
+  // find them.  Before -> after: 11 x 11 stride 4 RGB 75.1 -> 50.5 us, 5 x 5 RGB at 64 x 64 56.6 -> 41.9, 1 x 1 64 -> 256 at 56 x 56
+  // 31.0 -> 27.4, error of 1 x 1 48 -> 384 at 45 x 45 17.8 -> 15.4, row-batched 3 x 3 RGB at 32 x 32 16.6 -> 15.3; not with 32-byte
+  // rows (5 x 5 32 -> 96 35.9 -> 37.6, 7 x 7 stride 2 RGB 33.4 -> 34.0) or few tiles per CTA (64 -> 128 stride 2, 2.6 of them, 15.5 ->
+  // 15.9).
+  if (ctas == 1 && !p.halo && p.splits == 1 && p.n_tiles_n == 1 && p.dstride <= 1 && g.kind != GK_FC_WGRAD && g.kind != GK_CONV_WGRAD &&
+      (p.mrep > 1 || (p.kdepth >= 64 && tiles >= 3LL * units)) && (long long)p.kb_total * p.b_bytes <= 112 * 1024 && p.kb_total * p.b_bytes + 4 * p.a_bytes <= 200 * 1024) {
+    p.b_resident = 1;
+    p.b_tile_bytes = p.b_bytes;
+    p.b_res_bytes = p.kb_total * p.b_bytes;
+    p.b_bytes = 0;
+    stage_bytes = p.a_bytes;
+    p.stages = (200 * 1024 - p.b_res_bytes) / stage_bytes;
+    if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
+  }
   // rows with a pitch that is no multiple of 8: staging buffers of the fused epilogue's stores
   p.nstg_off = 0;
   if (p.splits == 1 && !p.halo && ((g.gn & 7) != 0 || (g.kind == GK_CONV_WGRAD && (p.Cn & 7) != 0))) {
-    int st = (200 * 1024 - EPI_WARPS * 32 * 36) / stage_bytes;
+    int st = (200 * 1024 - p.b_res_bytes - EPI_WARPS * 32 * 36) / stage_bytes;
     if (st > MAX_STAGES) st = MAX_STAGES;
     if (st < 2) return false;
     p.stages = st;
-    p.nstg_off = st * stage_bytes;
+    p.nstg_off = p.b_res_bytes + st * stage_bytes;
   }
   if (p.halo) {
     p.splits = 1;

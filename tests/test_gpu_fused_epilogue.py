@@ -133,3 +133,30 @@ def test_headers_of_an_own_workspace(oref):
     all_pairs()
     n.check()
     n.close()
+
+
+@pytest.mark.parametrize("B,S,Ci,Co,R,pad,stride", [(60, 32, 72, 40, 1, 0, 1), (64, 61, 64, 100, 3, 1, 2), (20, 111, 3, 96, 11, 2, 2),
+                                                    (15, 64, 130, 64, 1, 0, 1)])
+def test_weights_resident_over_many_tiles(niti, oref, B, S, Ci, Co, R, pad, stride):
+    """One column tile and three row tiles per CTA or more: short chunks, odd rows, windows, errors."""
+    rng = np.random.default_rng(S + Ci)
+    i8 = lambda *s: rng.integers(-127, 128, size=s, dtype=np.int8)  # noqa: E731
+    T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(niti.device)  # noqa: E731
+    x, w = i8(B, S, S, Ci), i8(Co, R, R, Ci)
+    want, s, b = oref.conv_fwd(x, -7, w, -9, pad, True, stride=stride)
+    y, s_y, b_y = niti.conv_fwd(T(x), niti.scalar(-7), T(w), niti.scalar(-9), pad=pad, relu=True, stride=stride)
+    assert np.array_equal(y.cpu().numpy(), want) and (int(s_y), int(b_y)) == (s, b)
+    if stride == 1:
+        e = i8(*want.shape)
+        wd, bd = oref.conv_dgrad(e, w, (S, S), pad, x)
+        ep, b_e = niti.conv_dgrad(T(e), T(w), (S, S), relu_mask_src=T(x), pad=pad)
+        assert np.array_equal(ep.cpu().numpy(), wd) and int(b_e) == bd
+
+
+def test_fully_connected_weights_resident(niti, oref):
+    rng = np.random.default_rng(3)
+    a, w = rng.integers(-127, 128, size=(60000, 130), dtype=np.int8), rng.integers(-127, 128, size=(200, 130), dtype=np.int8)
+    want, s, b = oref.linear_fwd(a, -7, w, -9, False)
+    out, s_out, b_out = niti.linear_fwd(torch.from_numpy(a).to(niti.device), niti.scalar(-7), torch.from_numpy(w).to(niti.device),
+                                        niti.scalar(-9))
+    assert np.array_equal(out.cpu().numpy(), want) and (int(s_out), int(b_out)) == (s, b)
