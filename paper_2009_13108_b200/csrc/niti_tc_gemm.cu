@@ -632,30 +632,41 @@ __device__ __forceinline__ int spec_correction(int packed) {
 // magnitude in its own first tile.  Posts and mailboxes as in niti_agree_bits: the first CTA decides when all have posted
 // (deciding at half of them saved 0.2 us and made the guess depend on who came first: 50 of 100 launches of a 5 x 5 layer's
 // error were recomputed, now none) and answers all of them.  (With a maximum, a count and a published word that all CTAs
-// poll, updated by atomics, the agreement took 3.7 - 4.4 us, a chain of five trips to L2; this takes 2.2.)  A CTA out of patience (launches of several streams share the SMs) decides from what has
-// been posted by then.  Two CTAs may decide differently: every CTA reports what it rounded with (WsHeader::spec_mask), and
-// the follow-up launch recomputes unless all of them used the true bit-width.
-__device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, unsigned m, const TcParams &p,
+// poll, updated by atomics, the agreement took 3.7 - 4.4 us, a chain of five trips to L2; this takes 2.2.)
+//
+// Nothing promises that all CTAs are on the GPU at the same time: where a kernel of another stream holds a single SM, the
+// last CTA starts when one of this launch exits.  So the first CTA decides from half of the posts or more once no new one has
+// come for GUESS_QUIET cycles, and marks the launch (WsHeader::hurried: its error is not remembered).  Beside a kernel that
+// holds 1 - 60 SMs for longer, 8192 x 4096 x 512 took 322 us where it waited for all posts and takes 65 (38 undisturbed),
+// the error of the 5 x 5 layer 375 - 400 and 130 - 164 (91).  Of 500 passes over fifty layers alone on the GPU none was
+// marked, with 2048, 4096, 8192 or 16384 cycles.  Where more than half of the SMs are held it waits for its whole patience.
+// The other CTAs wait for its answer; out of patience twice as long as its own, one decides from what has been posted by then.
+// Two CTAs may decide differently that way: every CTA reports what it rounded with (WsHeader::spec_mask), and the follow-up
+// launch recomputes unless all of them used the true bit-width.
+constexpr long long GUESS_QUIET = 8192;                  // about 4 us; the posts of an undisturbed launch come within 2
+__device__ __forceinline__ int agree_on_guess(WsHeader *hdr, unsigned m, unsigned patience, unsigned mul256, int tag,
                                               const int32_t *spec_slot, int lane) {
+  unsigned *const posts = niti_split_max(hdr), *const mail = posts + NITI_AGREE_MAX;
   const int cta = (int)blockIdx.x, n = (int)gridDim.x < NITI_AGREE_MAX ? (int)gridDim.x : NITI_AGREE_MAX;
   m = min(m, 0x7ffffffeu) + 1u;
   if (lane == 0 && cta < n) *(volatile unsigned *)(posts + cta) = m;
   // what the same estimate missed by at this call site lately (a systematic error of the sample, e.g. a tensor whose
   // extremes sit outside the first tiles); read while the posts are on their way
   int correction = 0;
-  if (spec_slot && p.spec_mul256 != 256 && *(volatile const int *)&spec_slot[0] == p.spec_tag)
+  if (spec_slot && mul256 != 256 && *(volatile const int *)&spec_slot[0] == tag)
     correction = spec_correction(*(volatile const int *)&spec_slot[1]);
   const long long t0 = clock64();
-  auto late = [&]() { return __any_sync(0xffffffffu, clock64() - t0 > (long long)p.patience) != 0; };
+  auto past = [&](long long since, long long limit) { return __any_sync(0xffffffffu, clock64() - since > limit) != 0; };
   if (cta != 0) {
     unsigned answer = 0;
     do {
       if (lane == 0) answer = *(volatile unsigned *)(mail + 4 * (cta < n ? cta : 0));
       answer = __shfl_sync(0xffffffffu, answer, 0);
-    } while (!answer && !late());
+    } while (!answer && !past(t0, 2LL * patience));
     if (answer) return (int)answer - 1;
   }
-  unsigned top;
+  unsigned top, came = 0;
+  long long news = t0;                                   // when the last new post was seen
   while (true) {
     unsigned seen = 0;
     top = m;
@@ -666,13 +677,22 @@ __device__ __forceinline__ int agree_on_guess(unsigned *posts, unsigned *mail, u
       seen += w ? 1u : 0u;
       top = max(top, w);
     }
-    if (cta != 0 || __reduce_add_sync(0xffffffffu, seen) >= (unsigned)n || late()) break;
+    seen = __reduce_add_sync(0xffffffffu, seen);
+    if (cta != 0 || seen >= (unsigned)n) break;
+    if (seen != came) {
+      came = seen;
+      news = clock64();
+    }
+    if (past(t0, (long long)patience) || (2u * seen >= (unsigned)n && past(news, GUESS_QUIET))) {
+      if (lane == 0) hdr->hurried = 1u;
+      break;
+    }
   }
   top = __reduce_max_sync(0xffffffffu, top) - 1u;
   // the first tiles are a sample: scale their max by the growth expected from the sample to the whole tensor before taking
   // the bit length (a wrong guess only costs the second pass); never below the bit length of the sample's own maximum,
   // which the tensor's cannot undercut
-  unsigned long long scaled = ((unsigned long long)top * p.spec_mul256) >> 8;
+  unsigned long long scaled = ((unsigned long long)top * mul256) >> 8;
   if (scaled > 0x7fffffffull) scaled = 0x7fffffffull;
   int guess = niti_bitlen32((unsigned)scaled) + correction;
   const int floor_b = niti_bitlen32(top);
@@ -1031,7 +1051,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const unsigned used = hdr->spec_mask;                  // bit-widths that the CTAs rounded with
     const int b_true = niti_bitlen32(hdr->maxabs32), b_est = used ? 31 - __clz(used) : b_true;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      if (spec_slot) {
+      if (spec_slot && !hdr->hurried) {
         // remember, for the next calls from this call site, how far the sample-based estimate was off
         // (b_est = raw estimate + the correction this call applied): the last two errors are kept
         const int packed = spec_slot[0] == p.spec_tag ? spec_slot[1] : 0x22;
@@ -1680,8 +1700,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       if (ONE) return false;
       if (!__shfl_sync(0xffffffffu, last, 0)) return false;
-      unsigned *words = niti_split_max(hdr);
-      const int b = agree_on_guess(words, words + NITI_AGREE_MAX, *(volatile unsigned *)&first_max, p, spec_slot, lane);
+      const int b = agree_on_guess(hdr, *(volatile unsigned *)&first_max, p.patience, p.spec_mul256, p.spec_tag, spec_slot, lane);
       if (lane == 0) {
         cta_b = b;
         spec_bp_ready = (b > p.mbits ? b - p.mbits : 0) + 1;
@@ -1918,7 +1937,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       mx |= ex_all.magnitude_bits();
     };
-    auto lean = [&]() {
+    auto lean = [&]() __attribute__((always_inline)) {
       using T = std::true_type;
       using F = std::false_type;
       const int form = p.form;
