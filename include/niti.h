@@ -297,14 +297,17 @@ int niti_set_reduce_hook(niti_ctx *ctx, niti_reduce_fn fn, void *user);
  * workspace, calls clear their header themselves as they do without this call.  The caller must not
  * use that workspace from two streams at once (as for any workspace) and must call niti_begin_step
  * again before the pattern repeats (each training step; a captured CUDA graph holds it as its first
- * node).  ws = NULL ends the arrangement.  Results do not change. */
+ * node).  Calls that are captured while niti_begin_step was not, or the other way round, take no part: they clear
+ * their own header.  ws = NULL ends the arrangement, which a program does after the last call of a step if other
+ * calls, or replays of a captured step on the same workspace, come before the next one.  Results do not change. */
 int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_bytes);
 
 /* Declares `ws` this context's own: between the calls that use it nobody else writes to its first
  * 256 KB (the headers), and the calls that use it through this context are ordered one after the
  * other, on whatever streams.  Calls outside a niti_begin_step arrangement on it then leave a zeroed header for their
  * successor instead of clearing one first.  (Calls that are being captured clear theirs themselves.)  A new buffer, also
- * one at the same address, has to be declared again.  ws = NULL ends the arrangement.  Results do not change. */
+ * one at the same address, has to be declared again, and the same one after a niti_begin_step arrangement of 62 calls or
+ * more, which uses all headers.  ws = NULL ends the arrangement.  Results do not change. */
 int niti_own_workspace(niti_ctx *ctx, void *ws, size_t ws_bytes);
 
 /* Convolutions with very few input channels (R * S * Cin <= 32: the first layer of an image network)

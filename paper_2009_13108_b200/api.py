@@ -207,6 +207,10 @@ class Niti:
         calls would otherwise clear one by one."""
         self._ck(self.lib.niti_begin_step(self.h, self._stream(), self._ws.data_ptr(), self._ws.numel()))
 
+    def end_step(self):
+        """The end of begin_step's arrangement: what follows is not part of the step."""
+        self._ck(self.lib.niti_begin_step(self.h, None, None, 0))
+
     def _ws_for(self, op, *dims):
         need = self._ws_need.get((op, dims))
         if need is None:

@@ -194,6 +194,7 @@ extern "C" int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_
   if (rc != NITI_OK) return rc;
   ctx->step_ws = ws;
   ctx->step_slot = 0;
+  ctx->step_capture = niti_capture_id((cudaStream_t)stream);
   if (ws == ctx->own_ws) ctx->own_clean = 0;
   return NITI_OK;
 }

@@ -41,6 +41,7 @@ struct niti_ctx {
   // niti_begin_step: workspace whose headers were cleared in one go, and how many of them are used up
   void *step_ws;
   int step_slot;
+  unsigned long long step_capture;  // the capture that niti_begin_step was part of (0: none)
   struct WsHeader *dirty_hdr;   // header of the call being enqueued that has not been cleared yet, or null
   // niti_own_workspace: calls alternate between two headers of this workspace, each clearing the other one's
   void *own_ws;
@@ -144,25 +145,38 @@ int niti_memset0(niti_ctx *ctx, cudaStream_t st, void *p, size_t bytes);
 static inline WsHeader *niti_own_header(void *ws, int which) {
   return reinterpret_cast<WsHeader *>(reinterpret_cast<char *>(ws) + (size_t)NITI_HDR_SLOT_BYTES * (NITI_HDR_OWN + which));
 }
+// The capture that a stream is part of; 0: none, NITI_CAPTURE_UNKNOWN: the stream cannot say (another one is being captured).
+#define NITI_CAPTURE_UNKNOWN (~0ull)
+static inline unsigned long long niti_capture_id(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return NITI_CAPTURE_UNKNOWN;
+  }
+  return status == cudaStreamCaptureStatusNone ? 0ull : status == cudaStreamCaptureStatusActive ? id : NITI_CAPTURE_UNKNOWN;
+}
 // A header for the call that is being enqueued: the next unused one of a workspace prepared by niti_begin_step()
-// (zeroed already); in a workspace that is this context's own one of two that the calls use in turn, the kernel of each
-// clearing the other one for the next (a launch of its own for that took 1.2 us of each call: one 256^3 multiply 7.9 -> 6.3 us,
-// forward, error and gradient of a 56 x 56 layer 73.2 -> 71.0 us); else the last one, which niti_clear() has to clear before the
-// call's first kernel.  The last one ends where the accumulators begin, so that a split contraction clears both with one
-// launch.  A call that is being captured takes the last one too: its replays do not alternate.
+// (zeroed already, if the call and niti_begin_step are enqueued alike: a begin that is being captured has cleared nothing yet,
+// and one in front of a capture does not repeat with the replays); in a workspace that is this context's own one of two that
+// the calls use in turn, the kernel of each clearing the other one for the next (a launch of its own for that took 1.2 us of
+// each call: one 256^3 multiply 7.9 -> 6.3 us, forward, error and gradient of a 56 x 56 layer 73.2 -> 71.0 us); else the last
+// one, which niti_clear() has to clear before the call's first kernel.  The last one ends where the accumulators begin, so
+// that a split contraction clears both with one launch.  A call that is being captured takes the last one too: its replays
+// do not alternate.  (So do calls past the 64th of a step, and those without patience, whose test looks there.)
 static inline WsHeader *niti_take_header(niti_ctx *ctx, cudaStream_t st, void *ws) {
   char *base = reinterpret_cast<char *>(ws);
   ctx->own_taken = 0;
   ctx->dirty_hdr = nullptr;
-  if (ws == ctx->step_ws && ctx->step_slot < NITI_HDR_SLOTS) {
-    if (ws == ctx->own_ws && ctx->step_slot >= NITI_HDR_OWN) ctx->own_ws = nullptr;      // (a graph of this step uses them, too)
-    return reinterpret_cast<WsHeader *>(base + (size_t)NITI_HDR_SLOT_BYTES * ctx->step_slot++);
-  }
-  if (ws == ctx->own_ws && ws != ctx->step_ws && ctx->patience) {
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
-      (void)cudaGetLastError();
-    } else if (capture == cudaStreamCaptureStatusNone) {
+  const bool step = ws == ctx->step_ws;
+  if (step || ws == ctx->own_ws) {
+    const unsigned long long capture = niti_capture_id(st);
+    const bool in_step = step && capture == ctx->step_capture && capture != NITI_CAPTURE_UNKNOWN;
+    if (in_step && ctx->step_slot < NITI_HDR_SLOTS) {
+      if (ws == ctx->own_ws && ctx->step_slot >= NITI_HDR_OWN) ctx->own_ws = nullptr;      // (a graph of this step uses them, too)
+      return reinterpret_cast<WsHeader *>(base + (size_t)NITI_HDR_SLOT_BYTES * ctx->step_slot++);
+    }
+    if (ws == ctx->own_ws && !in_step && capture == 0 && ctx->patience) {
       if (!ctx->own_clean) ctx->own_clean = niti_memset0(ctx, st, niti_own_header(ws, 0), 2 * NITI_HDR_SLOT_BYTES) == NITI_OK;
       if (ctx->own_clean) {
         ctx->own_taken = 1;

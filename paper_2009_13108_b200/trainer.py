@@ -206,8 +206,14 @@ class NitiTrainer:
 
     def step(self):
         """Forward, integer loss gradient, backward with in-place weight update."""
+        self.n.begin_step()                # one clear instead of one per multiply (the workspace is sized by then)
+        try:
+            return self._step()
+        finally:
+            self.n.end_step()              # (calls of the program between two steps have headers of their own)
+
+    def _step(self):
         n, net = self.n, self.net
-        n.begin_step()                     # one clear instead of one per multiply (the workspace is sized by then)
         logits, s_out = self.forward()
         cur = 0
         e = self._e_view(cur, logits.shape)
