@@ -306,8 +306,8 @@ int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_bytes);
  * 256 KB (the headers), and the calls that use it through this context are ordered one after the
  * other, on whatever streams.  Calls outside a niti_begin_step arrangement on it then leave a zeroed header for their
  * successor instead of clearing one first.  (Calls that are being captured clear theirs themselves.)  A new buffer, also
- * one at the same address, has to be declared again, and the same one after a niti_begin_step arrangement of 62 calls or
- * more, which uses all headers.  ws = NULL ends the arrangement.  Results do not change. */
+ * one at the same address, has to be declared again, and the same one after a captured niti_begin_step arrangement of 62
+ * calls or more, whose replays use all headers.  ws = NULL ends the arrangement.  Results do not change. */
 int niti_own_workspace(niti_ctx *ctx, void *ws, size_t ws_bytes);
 
 /* Convolutions with very few input channels (R * S * Cin <= 32: the first layer of an image network)

@@ -195,7 +195,7 @@ extern "C" int niti_begin_step(niti_ctx *ctx, void *stream, void *ws, size_t ws_
   ctx->step_ws = ws;
   ctx->step_slot = 0;
   ctx->step_capture = niti_capture_id((cudaStream_t)stream);
-  if (ws == ctx->own_ws) ctx->own_clean = 0;
+  if (ws == ctx->own_ws && ctx->step_capture == 0) ctx->own_clean = 1;        // (its two headers are among the cleared ones)
   return NITI_OK;
 }
 

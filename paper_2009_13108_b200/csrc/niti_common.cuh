@@ -173,7 +173,10 @@ static inline WsHeader *niti_take_header(niti_ctx *ctx, cudaStream_t st, void *w
     const unsigned long long capture = niti_capture_id(st);
     const bool in_step = step && capture == ctx->step_capture && capture != NITI_CAPTURE_UNKNOWN;
     if (in_step && ctx->step_slot < NITI_HDR_SLOTS) {
-      if (ws == ctx->own_ws && ctx->step_slot >= NITI_HDR_OWN) ctx->own_ws = nullptr;      // (a graph of this step uses them, too)
+      if (ws == ctx->own_ws && ctx->step_slot >= NITI_HDR_OWN) {
+        ctx->own_clean = 0;
+        if (capture) ctx->own_ws = nullptr;                  // (the replays will use them, too)
+      }
       return reinterpret_cast<WsHeader *>(base + (size_t)NITI_HDR_SLOT_BYTES * ctx->step_slot++);
     }
     if (ws == ctx->own_ws && !in_step && capture == 0 && ctx->patience) {

@@ -108,6 +108,24 @@ def test_calls_between_the_steps_of_two_networks(niti):
     assert all(torch.equal(t, u) for t, u in zip(big.weights, want))
 
 
+@pytest.mark.parametrize("calls", [1, 64])
+def test_no_clears_after_a_step(niti, calls):
+    """After a step, whether it used all headers or not, at most the first call clears anything."""
+    a, w, sa = torch.ones((64, 64), dtype=torch.int8, device=niti.device), torch.ones((64, 64), dtype=torch.int8, device=niti.device), niti.scalar(-7)
+
+    def launches():
+        l0 = niti.launch_count()
+        out, _, b = niti.linear_fwd(a, sa, w, sa)
+        assert int(b) == 7 and bool((out == 64).all())
+        return niti.launch_count() - l0
+    niti.begin_step()
+    for _ in range(calls):
+        launches()
+    niti.end_step()
+    launches()
+    assert [launches() for _ in range(70)] == [1] * 70
+
+
 def test_no_clears_after_a_training_step(niti):
     tr = _trainer(niti, 0, 64)
     tr.step()
