@@ -111,7 +111,8 @@ def _ptr(t):
 
 
 class Niti:
-    """One library context on one CUDA device plus a growable workspace."""
+    """One library context on one CUDA device plus a growable workspace.  A program that captures calls into a graph keeps
+    ``buffers()`` for as long as it replays it (``NitiTrainer.capture`` does)."""
 
     def __init__(self, device: int = 0):
         if not torch.cuda.is_available():
@@ -196,6 +197,10 @@ class Niti:
         if self._ws.numel() < nbytes:
             self._ck(self.lib.niti_begin_step(self.h, None, None, 0))      # the old buffer's headers are gone
             self._own_workspace(nbytes)
+
+    def buffers(self):
+        """The device buffers that calls use now: a program that captures calls keeps them as long as it replays."""
+        return [self._ws, getattr(self, "_tap", None)]
 
     def _own_workspace(self, nbytes: int):
         """A new workspace, declared to the library as nobody else's (see niti_own_workspace)."""

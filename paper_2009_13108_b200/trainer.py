@@ -121,6 +121,8 @@ class NitiTrainer:
                     self.reset_weights()
                 self.step()
         torch.cuda.current_stream(self.n.device).wait_stream(stream)
+        # the graph reads and writes these buffers of the library object, which may replace them by larger ones later
+        graph.buffers_in_use = self.n.buffers()
         self._graph = graph
         return graph.replay
 
