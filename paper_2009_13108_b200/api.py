@@ -190,12 +190,15 @@ class Niti:
     def set_tap_cache(self, nbytes: int):
         """niti_set_tap_cache with a buffer of ``nbytes`` owned by this object (0 removes it): the gathered
         taps of a few-channel first layer are kept between its forward and its weight-gradient call."""
+        if getattr(self, "_tap", None) is not None:
+            self._tap.record_stream(torch.cuda.current_stream(self.device))    # (calls enqueued here still use it)
         self._tap = torch.empty(nbytes, dtype=torch.uint8, device=self.device) if nbytes else None
         self._ck(self.lib.niti_set_tap_cache(self.h, _ptr(self._tap), nbytes))
 
     def reserve_workspace(self, nbytes: int):
         if self._ws.numel() < nbytes:
             self._ck(self.lib.niti_begin_step(self.h, None, None, 0))      # the old buffer's headers are gone
+            self._ws.record_stream(torch.cuda.current_stream(self.device))     # (calls enqueued here still use it)
             self._own_workspace(nbytes)
 
     def buffers(self):

@@ -44,3 +44,23 @@ def test_a_captured_step_keeps_its_buffers():
     assert all(torch.equal(w, u) for w, u in zip(tr.weights, want))
     n.check()
     n.close()
+
+
+def test_a_workspace_replaced_behind_calls_of_another_stream():
+    from paper_2009_13108_b200 import Niti
+    n = Niti(0)
+    size = n._ws.numel()
+    ones, sa = torch.ones((64, 64), dtype=torch.int8, device=n.device), n.scalar(-7)
+    n.linear_fwd(ones, sa, ones, sa)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)             # about 10 ms
+        out, _, b = n.linear_fwd(ones, sa, ones, sa)
+        n.reserve_workspace(64 << 20)
+    held = _patterns([size])                      # written while the call still waits
+    torch.cuda.synchronize()
+    assert all(bool((t == 0x5A).all()) for t in held)
+    assert int(b) == 7 and bool((out == 64).all())
+    n.check()
+    n.close()
