@@ -411,6 +411,7 @@ struct GemmProblem {
   // of image rows in the widened input; W and S then count windows and tap rows' windows (Wo and 1), and only rows
   // have a stride and padding
   int win_chans, win_sw, win_sh;
+  int in_place;             // an output is in the storage of an operand or of the gate (set and read by niti_tc_gemm)
 };
 
 // shard_ok: the caller rounds only this rank's shard afterwards (niti_dp_shard) and all-gathers the result

@@ -2805,7 +2805,7 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   // stage holds their A boxes, one MMA per tile writes its own bn_mma columns of the accumulator,
   // and the barriers, commits and tile decoding are paid once per item.
   p.mrep = 1;
-  if (g.kind == GK_FC_FWD && ctas == 1 && ctx->engine != 4 && p.n_tiles_n == 1 && p.kb_total <= 2 && p.bn <= 128 &&
+  if (g.kind == GK_FC_FWD && ctas == 1 && ctx->engine != 4 && !g.in_place && p.n_tiles_n == 1 && p.kb_total <= 2 && p.bn <= 128 &&
       m_tiles >= 8LL * ctx->sm_count) {
     p.mrep = p.bn <= 64 ? 4 : 2;
     p.a_boxes = p.mrep;
@@ -3209,8 +3209,8 @@ static int launch_finish(niti_ctx *ctx, cudaStream_t st, const int32_t *acc, lon
   return NITI_OK;
 }
 
-// Is no operand (nor the gate) in the storage of an output?  Then the first tile's outputs may be stored before all operands
-// have been read, and stored again.
+// Is no operand (nor the gate) in the storage of an output?  Then outputs may be stored before all operands have been read,
+// and stored again: a CTA's first tile during the agreement, all of them where a guess was wrong.
 static bool may_store_twice(const GemmProblem &g, const RoundSpec &r) {
   const long long x = (long long)g.B * g.H * g.W * g.Ci, y = (long long)g.B * g.Ho * g.Wo * g.Co;
   const long long out_bytes = g.gm * g.gn;
@@ -3228,13 +3228,16 @@ static bool may_store_twice(const GemmProblem &g, const RoundSpec &r) {
     return !a || !b || u + (uintptr_t)na <= v || v + (uintptr_t)nb <= u;
   };
   auto output_apart = [&](const int8_t *out, long long n) {
-    return apart(out, n, g.p0, n0) && apart(out, n, g.p1, n1) && apart(out, n, r.mask, out_bytes);
+    // (a padded or widened copy is read in place of the operand, whose extents are then others)
+    return (g.q0 || apart(out, n, g.p0, n0)) && (g.q1 || apart(out, n, g.p1, n1)) && apart(out, n, r.mask, out_bytes);
   };
   return output_apart(r.out, out_bytes) && output_apart(r.pool_out, out_bytes / 4);
 }
 
-int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const RoundSpec &r_in, int32_t *acc,
+int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g_in, const RoundSpec &r_in, int32_t *acc,
                  WsHeader *hdr, bool *fused, bool *pooled, bool shard_ok, bool *updated) {
+  GemmProblem g = g_in;
+  g.in_place = !may_store_twice(g_in, r_in);
   TcParams p;
   CUtensorMap ma, mb, mc;
   memset(&mc, 0, sizeof(mc));
@@ -3293,7 +3296,7 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
     p.spec_mul256 = (unsigned)(f * 256.0 + 0.5);
     const double n_own = n_all / ((double)p.items * p.ctas);
     const double f_own = n_own > 16.0 ? sqrt(log(n_all) / log(n_own)) : 1.0;
-    p.trial_mul256 = may_store_twice(g, r) ? (unsigned)(f_own * 256.0 + 0.5) : 0u;
+    p.trial_mul256 = !g.in_place ? (unsigned)(f_own * 256.0 + 0.5) : 0u;
   }
   // data parallelism (niti_set_reduce_hook): the max magnitude is combined over the ranks between the
   // two launches, so there is always a second launch; weight gradients keep their int32 sums
@@ -3303,7 +3306,10 @@ int niti_tc_gemm(niti_ctx *ctx, cudaStream_t st, const GemmProblem &g, const Rou
   p.mbits = r.mbits;
   p.round_mode = r.round_mode;
   p.relu = r.relu;
-  p.epi_mode = (p.splits > 1 || p.halo == 2) ? EPI_ATOMIC : ((ctx->engine == 4 || dp_sum || !r.out) ? EPI_SPILL : EPI_SPECULATE);
+  // (an output in the storage of an operand or of the gate: rounded after the whole multiply, where not in one wave, whose
+  // CTAs store when all have read.  A strided error with phases that no window reaches clears its output beforehand.)
+  const bool sums_first = g.in_place && (!p.single_wave || p.dstride > 1);
+  p.epi_mode = (p.splits > 1 || p.halo == 2) ? EPI_ATOMIC : ((ctx->engine == 4 || dp_sum || !r.out || sums_first) ? EPI_SPILL : EPI_SPECULATE);
   if (p.dstride > 1 && (p.nph_r < p.dstride || p.nph_s < p.dstride)) {
     // filter smaller than the stride: no window reaches the input pixels of the other phases
     if (p.epi_mode == EPI_SPILL) NITI_CUDA_TRY(ctx, cudaMemsetAsync(acc, 0, sizeof(int32_t) * (size_t)(g.gm * g.gn), st));
