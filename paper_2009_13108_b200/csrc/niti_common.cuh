@@ -91,10 +91,8 @@ struct WsHeader {
   unsigned long long maxabs64;      // same for the 64-bit loss accumulators
   unsigned int spec_mask;           // bit b: a CTA of a speculative launch has rounded with bit-width b
   unsigned int hits;                // integer cross-entropy: rows whose first arg-max is the label
-  unsigned int hurried;             // a speculative launch guessed the bit-width without having heard from all of its CTAs
-  unsigned int unused;
 };
-static_assert(sizeof(WsHeader) == 32, "workspace header layout");
+static_assert(sizeof(WsHeader) == 24, "workspace header layout");
 static_assert(NITI_SPLIT_MAX_OFF + 4 * NITI_MAX_SPLITS <= NITI_HDR_SLOT_BYTES, "split maxima fit the header");
 __host__ __device__ __forceinline__ unsigned int *niti_split_max(WsHeader *hdr) {
   return reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(hdr) + NITI_SPLIT_MAX_OFF);

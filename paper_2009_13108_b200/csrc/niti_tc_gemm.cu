@@ -636,14 +636,15 @@ __device__ __forceinline__ int spec_correction(int packed) {
 //
 // Nothing promises that all CTAs are on the GPU at the same time: where a kernel of another stream holds a single SM, the
 // last CTA starts when one of this launch exits.  So the first CTA decides from half of the posts or more once no new one has
-// come for GUESS_QUIET cycles, and marks the launch (WsHeader::hurried: its error is not remembered).  Beside a kernel that
-// holds 1 - 60 SMs for longer, 8192 x 4096 x 512 took 322 us where it waited for all posts and takes 65 (38 undisturbed),
-// the error of the 5 x 5 layer 375 - 400 and 130 - 164 (91).  Of 500 passes over fifty layers alone on the GPU none was
-// marked, with 2048, 4096, 8192 or 16384 cycles.  Where more than half of the SMs are held it waits for its whole patience.
-// The other CTAs wait for its answer; out of patience twice as long as its own, one decides from what has been posted by then.
-// Two CTAs may decide differently that way: every CTA reports what it rounded with (WsHeader::spec_mask), and the follow-up
-// launch recomputes unless all of them used the true bit-width.
-constexpr long long GUESS_QUIET = 8192;                  // about 4 us; the posts of an undisturbed launch come within 2
+// come for GUESS_QUIET cycles, and from fewer after its whole patience.  Beside a kernel that holds 1 - 60 SMs for longer,
+// 8192 x 4096 x 512 took 322 us where it waited for all posts and takes 65 (38 undisturbed), the error of the 5 x 5 layer 375
+// - 400 and 130 - 164 (91).  In 500 passes over fifty layers alone on the GPU no launch went on early, with 2048, 4096, 8192
+// or 16384 cycles.  (Marking early ones in the header, so that the follow-up does not remember their error, cost every
+// follow-up 0.2 - 1.2 us; an error has to repeat before it is followed in any case.)  The other CTAs wait for the answer; out
+// of patience twice as long as the first one's, a CTA decides from what has been posted by then.  Two CTAs may decide
+// differently that way: every CTA reports what it rounded with (WsHeader::spec_mask), and the follow-up launch recomputes
+// unless all of them used the true bit-width.
+constexpr unsigned GUESS_QUIET = 8192;                  // about 4 us; the posts of an undisturbed launch come within 2
 __device__ __forceinline__ int agree_on_guess(WsHeader *hdr, unsigned m, unsigned patience, unsigned mul256, int tag,
                                               const int32_t *spec_slot, int lane) {
   unsigned *const posts = niti_split_max(hdr), *const mail = posts + NITI_AGREE_MAX;
@@ -655,18 +656,17 @@ __device__ __forceinline__ int agree_on_guess(WsHeader *hdr, unsigned m, unsigne
   int correction = 0;
   if (spec_slot && mul256 != 256 && *(volatile const int *)&spec_slot[0] == tag)
     correction = spec_correction(*(volatile const int *)&spec_slot[1]);
-  const long long t0 = clock64();
-  auto past = [&](long long since, long long limit) { return __any_sync(0xffffffffu, clock64() - since > limit) != 0; };
+  unsigned since = (unsigned)clock64();                   // the start, or when the first CTA saw the last new post
+  auto past = [&](unsigned limit) { return __any_sync(0xffffffffu, (unsigned)clock64() - since > limit) != 0; };
   if (cta != 0) {
     unsigned answer = 0;
     do {
       if (lane == 0) answer = *(volatile unsigned *)(mail + 4 * (cta < n ? cta : 0));
       answer = __shfl_sync(0xffffffffu, answer, 0);
-    } while (!answer && !past(t0, 2LL * patience));
+    } while (!answer && !past(2u * patience));
     if (answer) return (int)answer - 1;
   }
   unsigned top, came = 0;
-  long long news = t0;                                   // when the last new post was seen
   while (true) {
     unsigned seen = 0;
     top = m;
@@ -679,14 +679,9 @@ __device__ __forceinline__ int agree_on_guess(WsHeader *hdr, unsigned m, unsigne
     }
     seen = __reduce_add_sync(0xffffffffu, seen);
     if (cta != 0 || seen >= (unsigned)n) break;
-    if (seen != came) {
-      came = seen;
-      news = clock64();
-    }
-    if (past(t0, (long long)patience) || (2u * seen >= (unsigned)n && past(news, GUESS_QUIET))) {
-      if (lane == 0) hdr->hurried = 1u;
-      break;
-    }
+    if (seen != came) since = (unsigned)clock64();
+    came = seen;
+    if (past(2u * seen >= (unsigned)n ? GUESS_QUIET : patience)) break;
   }
   top = __reduce_max_sync(0xffffffffu, top) - 1u;
   // the first tiles are a sample: scale their max by the growth expected from the sample to the whole tensor before taking
@@ -1051,7 +1046,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const unsigned used = hdr->spec_mask;                  // bit-widths that the CTAs rounded with
     const int b_true = niti_bitlen32(hdr->maxabs32), b_est = used ? 31 - __clz(used) : b_true;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-      if (spec_slot && !hdr->hurried) {
+      if (spec_slot) {
         // remember, for the next calls from this call site, how far the sample-based estimate was off
         // (b_est = raw estimate + the correction this call applied): the last two errors are kept
         const int packed = spec_slot[0] == p.spec_tag ? spec_slot[1] : 0x22;
