@@ -98,7 +98,7 @@ def test_headers_of_an_own_workspace(oref):
             assert np.array_equal(calls[k]().cpu().numpy(), want[k]), k
 
     def all_pairs():
-        for engine in (0, 6, 2, 4, 1):                       # (one wave, leaving CTAs, single CTAs, two passes, CUDA cores)
+        for engine in (0, 6, 2, 4, 1):                       # (one wave, leaving CTAs on a header of their own, single CTAs, ...)
             n.set_engine(engine)
             check([i for p in range(5) for q in range(5) for i in (p, q)])
         n.set_engine(0)

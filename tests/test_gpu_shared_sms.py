@@ -85,3 +85,49 @@ def test_several_waves_beside_held_sms(hold, form):
         assert best < 2 * alone + 60, (sms, best, alone)
     n.check()
     n.close()
+
+
+def _one_wave(n):
+    sx, sw = n.scalar(-7), n.scalar(-9)
+    a, w = _i8(1, 1024, 1024).clamp_(min=0), _i8(2, 1024, 1024)
+    a2, w2 = _i8(4, 256, 300).clamp_(min=0), _i8(5, 250, 300)
+    a3, w3, e3 = _i8(6, 64, 2048).clamp_(min=0), _i8(7, 1024, 2048), _i8(8, 64, 1024)
+    x, ex = _i8(9, 16, 14, 14, 256).clamp_(min=0), _i8(10, 16, 14, 14, 256)
+    labels = (torch.arange(4096, dtype=torch.int32) % 1000).cuda()
+    logits = _i8(11, 4096, 1000)
+
+    def update():
+        wt = w3.clone()
+        return list(n.linear_bwd_update(a3, e3, wt, need_e_prev=False)[2:]) + [wt]
+    return {"small": lambda: n.linear_fwd(a2, sx, w2, sw), "fc": lambda: n.linear_fwd(a, sx, w, sw, relu=True),
+            "update": update, "split": lambda: n.conv_wgrad(x, ex), "loss": lambda: n.int_xent(logits, n.scalar(-6), labels)}
+
+
+def _left(n):
+    """Blocks that left in the last two calls: upper halves of the second words of the two headers used in turn."""
+    torch.cuda.synchronize()
+    return sum(int(w) >> 16 for w in n._ws[61 * 4096:63 * 4096].view(torch.int32).view(2, 1024)[:, 1])
+
+
+@pytest.mark.parametrize("form", ["small", "fc", "update", "split", "loss"])
+def test_blocks_leave_on_headers_used_in_turn(hold, form):
+    """Blocks that wait for others leave their share when these cannot start; the header that such a call leaves for the next
+    one is clean, whichever of the two it is."""
+    from paper_2009_13108_b200 import Niti
+    n = Niti(0)
+    n.reserve_workspace(256 << 20)
+    call = _one_wave(n)[form]
+    want = [t.clone() for t in call() if t is not None]
+    call()
+    assert _left(n) == 0
+    left = 0
+    for _ in range(3):
+        hold(140)
+        got = [t for t in call() if t is not None]
+        left += _left(n)
+        assert all(torch.equal(t, u) for t, u in zip(got, want))
+        for _ in range(2):
+            assert all(torch.equal(t, u) for t, u in zip([t for t in call() if t is not None], want))
+    assert left > 0
+    n.check()
+    n.close()
