@@ -14,6 +14,7 @@
 // NITI_DEV_TIMEOUT in the status word, and all roles drain and leave through the common exit
 // that frees the tensor memory.
 #include "niti_common.cuh"
+#include "niti_div.h"
 #include <math.h>
 #include <type_traits>
 
@@ -32,21 +33,6 @@ constexpr int NUM_THREADS = 32 * (PROD_WARPS + 1 + EPI_WARPS);
 constexpr int MAX_STAGES = 8;
 constexpr int MAX_TBUF = 8;
 constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;
-
-// n / d for 0 <= n < 2^31 as a multiplication: d > 1, s = ceil(log2 d), m = floor(2^(31 + s) / d) + 1 exceeds 2^(31 + s) / d by
-// at most 1 <= 2^s / d, so that n * m / 2^(31 + s) stays below the next integer.  (An integer division costs a lone warp 100 -
-// 200 cycles and 20 - 30 instructions, and the first copy of a launch used to wait for five of them.)
-struct Div {
-  unsigned m;               // 0: d = 1
-  int s;                    // s - 1 above
-};
-static Div make_div(long long d) {
-  if (d <= 1) return Div{0u, 0};
-  int s = 1;
-  while ((1LL << s) < d) ++s;
-  return Div{(unsigned)((1ull << (31 + s)) / (unsigned long long)d + 1), s - 1};
-}
-__device__ __forceinline__ int div_by(int n, Div d) { return d.m ? (int)(__umulhi((unsigned)n, d.m) >> d.s) : n; }
 
 // What the fused epilogue does with a launch's tiles; one instance of its loop each.
 enum LeanForm {
@@ -2459,7 +2445,8 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   int a_sw = 0, b_sw = 0;
   int tail = 0;                  // contraction elements of the last chunk of c_chunks when it is not a whole one
   long long m_tiles = 0;
-  if (g.gm * g.gn >= (1LL << 31) || g.gm >= (1LL << 31) - 1024) return false;      // (rows are counted in 32 bits)
+  // (rows, columns and contraction elements are counted in 32 bits, and divided by div_by)
+  if (g.gm * g.gn >= (1LL << 31) || g.gm >= (1LL << 31) - 1024 || g.gk >= (1LL << 31) - 1024) return false;
   // operands as they are copied: padded where the caller's rows are no multiple of 16 bytes
   const int8_t *q0 = g.q0 ? g.q0 : g.p0, *q1 = g.q1 ? g.q1 : g.p1;
   if (g.kind == GK_FC_DGRAD && g.gk < 32) return false;            // (10-class heads: the CUDA-core engine is faster)
@@ -3059,7 +3046,7 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
     int cols = 32;
     while (cols < p.nbuf * p.bn) cols <<= 1;
     q.k_tmem_cols = cols;
-    // (dividends are items, tiles or grid positions, all below 2^31)
+    // (dividends are items, tiles, grid positions or k-blocks, all below 2^31: plan() refuses others)
     q.d_w = make_div(p.w_tiles);
     q.d_h = make_div(p.h_tiles);
     q.d_n = make_div(p.n_tiles_n);
