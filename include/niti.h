@@ -127,6 +127,9 @@ uint64_t niti_launch_count(niti_ctx *ctx);
 uint64_t niti_tc_launch_count(niti_ctx *ctx);
 /* Of those, launches of the paired-CTA (cta_group::2) variant. */
 uint64_t niti_tc_pair_launch_count(niti_ctx *ctx);
+/* And launches that keep the weights of their only column tile in shared memory (beside the mode of small-channel 3x3
+ * convolutions, which is not counted here). */
+uint64_t niti_tc_resident_launch_count(niti_ctx *ctx);
 
 /* The fused epilogue of the tensor-core kernel rounds with a bit-width guessed from the first
  * tile of every CTA and recomputes the multiply when the whole tensor turns out to need a larger

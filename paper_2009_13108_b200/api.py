@@ -22,7 +22,7 @@ _REDUCE_FN = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64,
 
 EXPORTS = [
     "niti_create", "niti_destroy", "niti_last_error", "niti_check", "niti_workspace_bytes",
-    "niti_set_engine", "niti_set_reduce_hook", "niti_set_dp_shard", "niti_set_tap_cache", "niti_begin_step", "niti_own_workspace", "niti_launch_count", "niti_tc_launch_count", "niti_tc_pair_launch_count",
+    "niti_set_engine", "niti_set_reduce_hook", "niti_set_dp_shard", "niti_set_tap_cache", "niti_begin_step", "niti_own_workspace", "niti_launch_count", "niti_tc_launch_count", "niti_tc_pair_launch_count", "niti_tc_resident_launch_count",
     "niti_redo_count", "niti_selftest_timeout", "niti_profile_enable", "niti_profile_read_launches",
     "niti_profile_read", "niti_linear_fwd", "niti_linear_bwd", "niti_conv_fwd",
     "niti_conv_dgrad", "niti_conv_wgrad", "niti_conv_fwd_pool", "niti_conv_fwd_strided", "niti_conv_dgrad_strided", "niti_conv_wgrad_strided",
@@ -70,6 +70,8 @@ def load_library():
     lib.niti_own_workspace.argtypes = [vp, vp, sz]
     lib.niti_launch_count.argtypes = [vp]
     lib.niti_launch_count.restype = C.c_uint64
+    lib.niti_tc_resident_launch_count.argtypes = [vp]
+    lib.niti_tc_resident_launch_count.restype = C.c_uint64
     lib.niti_tc_launch_count.argtypes = [vp]
     lib.niti_tc_launch_count.restype = C.c_uint64
     lib.niti_tc_pair_launch_count.argtypes = [vp]
@@ -251,6 +253,9 @@ class Niti:
 
     def tc_pair_launch_count(self) -> int:
         return int(self.lib.niti_tc_pair_launch_count(self.h))
+
+    def tc_resident_launch_count(self) -> int:
+        return int(self.lib.niti_tc_resident_launch_count(self.h))
 
     def redo_count(self) -> int:
         return int(self.lib.niti_redo_count(self.h, self._stream()))

@@ -238,6 +238,7 @@ extern "C" int niti_set_dp_shard(niti_ctx *ctx, int rank, int world) {
 extern "C" uint64_t niti_launch_count(niti_ctx *ctx) { return ctx ? ctx->launches : 0; }
 extern "C" uint64_t niti_tc_launch_count(niti_ctx *ctx) { return ctx ? ctx->tc_launches : 0; }
 extern "C" uint64_t niti_tc_pair_launch_count(niti_ctx *ctx) { return ctx ? ctx->tc2_launches : 0; }
+extern "C" uint64_t niti_tc_resident_launch_count(niti_ctx *ctx) { return ctx ? ctx->res_launches : 0; }
 
 extern "C" int64_t niti_redo_count(niti_ctx *ctx, void *stream) {
   if (!ctx) return -1;

@@ -19,6 +19,7 @@ struct niti_ctx {
   uint64_t launches;
   uint64_t tc_launches;     // launches of the tensor-core matrix-multiply kernels (two multiplies in one count as two)
   uint64_t tc2_launches;    // of those, launches of the paired-CTA (cta_group::2) variant
+  uint64_t res_launches;    // and launches of the generic loops with all of B resident
   char err[256];
   // optional timing of the tensor-core kernel: event pairs recorded around each launch
   int profile_on;

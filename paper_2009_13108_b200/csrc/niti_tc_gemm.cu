@@ -3093,6 +3093,7 @@ static int launch_tc_as(niti_ctx *ctx, cudaStream_t st, const TcParams &p, const
   ctx->launches++;
   ctx->tc_launches++;
   if (CTAS == 2) ctx->tc2_launches++;
+  if (p.b_resident) ctx->res_launches++;
   return NITI_OK;
 }
 

@@ -135,21 +135,27 @@ def test_headers_of_an_own_workspace(oref):
     n.close()
 
 
-@pytest.mark.parametrize("B,S,Ci,Co,R,pad,stride", [(60, 32, 72, 40, 1, 0, 1), (64, 61, 64, 100, 3, 1, 2), (20, 111, 3, 96, 11, 2, 2),
-                                                    (15, 64, 130, 64, 1, 0, 1)])
-def test_weights_resident_over_many_tiles(niti, oref, B, S, Ci, Co, R, pad, stride):
+@pytest.mark.parametrize("B,S,Ci,Co,R,pad,stride,resident", [
+    (60, 32, 72, 40, 1, 0, 1, True), (64, 61, 64, 100, 3, 1, 2, True), (15, 64, 130, 64, 1, 0, 1, True),
+    # windows of few channels: 444 row tiles and more, and 439, which are copied tile by tile
+    (70, 119, 3, 96, 11, 2, 4, True), (16, 60, 3, 40, 5, 2, 1, True), (60, 66, 1, 33, 7, 2, 2, True), (20, 111, 3, 96, 11, 2, 2, False)])
+def test_weights_resident_over_many_tiles(niti, oref, B, S, Ci, Co, R, pad, stride, resident):
     """One column tile and three row tiles per CTA or more: short chunks, odd rows, windows, errors."""
     rng = np.random.default_rng(S + Ci)
     i8 = lambda *s: rng.integers(-127, 128, size=s, dtype=np.int8)  # noqa: E731
     T = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(niti.device)  # noqa: E731
     x, w = i8(B, S, S, Ci), i8(Co, R, R, Ci)
     want, s, b = oref.conv_fwd(x, -7, w, -9, pad, True, stride=stride)
+    before = niti.tc_resident_launch_count()
     y, s_y, b_y = niti.conv_fwd(T(x), niti.scalar(-7), T(w), niti.scalar(-9), pad=pad, relu=True, stride=stride)
+    assert (niti.tc_resident_launch_count() > before) == resident
     assert np.array_equal(y.cpu().numpy(), want) and (int(s_y), int(b_y)) == (s, b)
-    if stride == 1:
+    if stride == 1 and Ci >= 32:
         e = i8(*want.shape)
         wd, bd = oref.conv_dgrad(e, w, (S, S), pad, x)
+        before = niti.tc_resident_launch_count()
         ep, b_e = niti.conv_dgrad(T(e), T(w), (S, S), relu_mask_src=T(x), pad=pad)
+        assert niti.tc_resident_launch_count() > before
         assert np.array_equal(ep.cpu().numpy(), wd) and int(b_e) == bd
 
 
@@ -157,6 +163,8 @@ def test_fully_connected_weights_resident(niti, oref):
     rng = np.random.default_rng(3)
     a, w = rng.integers(-127, 128, size=(60000, 130), dtype=np.int8), rng.integers(-127, 128, size=(200, 130), dtype=np.int8)
     want, s, b = oref.linear_fwd(a, -7, w, -9, False)
+    before = niti.tc_resident_launch_count()
     out, s_out, b_out = niti.linear_fwd(torch.from_numpy(a).to(niti.device), niti.scalar(-7), torch.from_numpy(w).to(niti.device),
                                         niti.scalar(-9))
+    assert niti.tc_resident_launch_count() > before
     assert np.array_equal(out.cpu().numpy(), want) and (int(s_out), int(b_out)) == (s, b)
