@@ -438,11 +438,12 @@ def measured_traffic(kernel_file):
 
 def kernel_device_digest(kernel_file):
     """SHA-256 of the device part of the kernel's source file: everything above its 'Host side' banner
-    (the kernel, its helpers and its parameter block), so that host-only edits keep a capture valid."""
+    (the kernel, its helpers and its parameter block) and its divisions, so that host-only edits keep a capture valid."""
     import hashlib
     text = open(kernel_file, "rb").read()
     cut = text.find(b"// Host side: tensor maps")
-    return hashlib.sha256(text if cut < 0 else text[:cut]).hexdigest()
+    div = open(os.path.join(os.path.dirname(kernel_file), "niti_div.h"), "rb").read()
+    return hashlib.sha256((text if cut < 0 else text[:cut]) + div).hexdigest()
 
 
 def spawn_ranks(args):

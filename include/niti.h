@@ -132,8 +132,8 @@ uint64_t niti_tc_pair_launch_count(niti_ctx *ctx);
 uint64_t niti_tc_resident_launch_count(niti_ctx *ctx);
 
 /* The fused epilogue of the tensor-core kernel rounds with a bit-width guessed from the first
- * tile of every CTA and recomputes the multiply when the whole tensor turns out to need a larger
- * shift (results are exact either way).  A call that passes a bit-width scalar (b_out / b_e / b_g)
+ * tile of every CTA and recomputes the multiply when the whole tensor turns out to need another
+ * one (results are exact either way).  A call that passes a bit-width scalar (b_out / b_e / b_g)
  * is recognised by that scalar's address when it comes again (the same layer in the next training
  * step): an estimate that missed by the same amount twice in a row is corrected by that amount, which
  * removes the recomputations of tensors whose extremes the sample systematically misses.  Returns how many recomputations this

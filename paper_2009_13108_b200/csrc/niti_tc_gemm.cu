@@ -157,9 +157,9 @@ struct TcParams {
 //                 and 11 us for a 128 x 256 one; the reduce copies add at L2 in whole lines.)
 //  EPI_SPECULATE  every CTA computes its first tile, the grid agrees on the max over those tiles
 //                 (one bounded grid-wide wait), and all tiles are rounded and stored as int8 with the
-//                 shift that max implies, while the true max is tracked.  If the true bit-width turns
-//                 out larger, the EPI_KNOWN_B pass recomputes everything with it (exact in all cases;
-//                 the common case costs one multiply and no int32 traffic)
+//                 shift that max implies, while the true max is tracked.  Unless every CTA has used
+//                 exactly the true bit-width, the EPI_KNOWN_B pass recomputes everything with it (exact in
+//                 all cases; the common case costs one multiply and no int32 traffic)
 //  EPI_KNOWN_B    bit-width known (hdr->maxabs32): round and store directly.  The kernel returns at
 //                 once when the speculative pass was right.
 enum { EPI_SPILL = 0, EPI_ATOMIC = 1, EPI_SPECULATE = 2, EPI_KNOWN_B = 3 };
@@ -2882,10 +2882,13 @@ static bool plan(niti_ctx *ctx, const GemmProblem &g, int ctas, PlanWant want, b
   if (p.tg > 1 && !(p.splits > 1 && p.red)) return plan(ctx, g, ctas, want, aligned, -1, acc, p, ma, mb, mc);
   // All of B resident: with one column tile every tile reads the same B tiles again, and short contractions are bound by their
   // copies (about 4 cycles a row).  Where they leave room for the A stages, the first tile of a CTA copies them and the others
-  // find them.  Before -> after: 11 x 11 stride 4 RGB 75.1 -> 50.5 us, 5 x 5 RGB at 64 x 64 56.6 -> 41.9, 1 x 1 64 -> 256 at 56 x 56
-  // 31.0 -> 27.4, error of 1 x 1 48 -> 384 at 45 x 45 17.8 -> 15.4, row-batched 3 x 3 RGB at 32 x 32 16.6 -> 15.3; not with 32-byte
-  // rows (5 x 5 32 -> 96 35.9 -> 37.6, 7 x 7 stride 2 RGB 33.4 -> 34.0) or few tiles per CTA (64 -> 128 stride 2, 2.6 of them, 15.5 ->
-  // 15.9).
+  // find them.  Before -> after: 11 x 11 stride 4 RGB 61.7 -> 49.8 us, 5 x 5 RGB at 64 x 64 to 64 and 96 channels 45.0 -> 30.1
+  // and 51.2 -> 34.9, 1 x 1 64 -> 256 at 56 x 56 28.6 -> 27.3, error of 1 x 1 48 -> 384 at 45 x 45 27.8 -> 18.5, 72 -> 40 at 32 x
+  // 32 19.0 -> 17.3; row-batched, at any row width, 3 x 3 RGB at 112 x 112 47.4 -> 44.1, 200000 x 32 x 27 18.8 -> 17.8, x 64 x 64
+  // 16.0 -> 15.8.  Nothing at 96 KB of B tiles (1 x 1 512 -> 192 at 45 x 45 23.8 -> 23.7) or 2 - 5 tiles per CTA (64 -> 128 stride 2
+  // at 56 x 56, batch 48, 64, 128: 13.2, 15.3, 22.9 -> 22.8).  Outside the rule, forced: 128 KB 27.5 -> 27.0, three A stages of a
+  // row-batched multiply 18.5 -> 18.4; 32-byte rows were slower when the rule was made (5 x 5 32 -> 96 35.9 -> 37.6, 7 x 7
+  // stride 2 RGB 33.4 -> 34.0) and as kernels stand 5 x 5 32 -> 96 is the same, 16 -> 64 70.4 -> 61.9, 1 x 1 32 -> 256 24.4 -> 21.5.
   if (ctas == 1 && !p.halo && p.splits == 1 && p.n_tiles_n == 1 && p.dstride <= 1 && g.kind != GK_FC_WGRAD && g.kind != GK_CONV_WGRAD &&
       (p.mrep > 1 || (p.kdepth >= 64 && tiles >= 3LL * units)) && (long long)p.kb_total * p.b_bytes <= 112 * 1024 && p.kb_total * p.b_bytes + 4 * p.a_bytes <= 200 * 1024) {
     p.b_resident = 1;
@@ -3137,15 +3140,19 @@ static double kblock_cycles(const TcParams &p, int ctas, int bn, long long ctas_
 // A multiply of at most one tile per SM: an unsplit plan whose every CTA (pair) has one tile rounds in its own epilogue
 // with an exact shift, in one launch.  Splitting the contraction shortens the main loop but costs a zeroed scratch, the
 // reduce copies and a finishing launch over the int32 sums; pairs of CTAs cost 0.8 us more set-up than single ones.  (The
-// model's 3.5 us + 5 us per million outputs of a split were measured when two kernels finished it.)  Where the line lies
-// now, as kernels stand (graph replay, without one-wave plans -> with them): 256 images of 4 x 4, 512 -> 512 channels,
-// forward 30.6 -> 19.9, error 27.4 -> 21.1, weight gradient 27.2 -> 19.6 us; 100 images of 9 x 9, 96 -> 160, 19.3 -> 11.7,
-// 18.8 -> 13.7, 13.3 -> 14.6; 64 of 7 x 7, 256 -> 512, 26.3 -> 14.6, 19.8 -> 19.1, 21.9 -> 16.6; 128 of 8 x 8, 128 -> 256,
-// 20.8 -> 11.9, 20.6 -> 14.4, 16.8 -> 17.5; 256 of 2 x 2, 512 -> 512, 17.6 -> 18.3, 18.2 -> 18.9, 22.1 -> 12.7; fully
-// connected 1024^3 forward 16.1 -> 11.5, backward 32.7 -> 22.6 us, 4096 x 1000 x 512 14.0 -> 14.0 and 43.3 -> 33.2: a few
-// gradients are up to 10 % slower, nothing else is.  (Splits that form a cluster and add their partial tiles through
-// distributed shared memory were built and measured: 24.3 - 25.0 us against 20.7 us unsplit on the first of these; the
-// agreement over twice as many CTAs and the exchange cost what the shorter main loop saves.)
+// constants of the model were measured on earlier kernels: a split's 3.5 us + 5 us per million outputs when two kernels
+// finished it, several waves' when their agreement took twice as long.)  What it decides, as kernels stand (graph replay, without
+// one-wave plans -> with them, forward / error / gradient, where the plan changes): 256 images of 4 x 4, 512 -> 512 channels, 27.9
+// -> 18.8 / 24.9 -> 17.6 / 25.5 -> 16.7 us; 100 of 9 x 9, 96 -> 160, 17.7 -> 10.0 / 17.9 -> 12.2; 64 of 7 x 7, 256 -> 512, 26.1 ->
+// 12.4 / 19.3 -> 17.0 / 20.8 -> 14.5; 128 of 8 x 8, 128 -> 256, 20.1 -> 11.0 / 19.8 -> 13.6; 256 of 2 x 2, 512 -> 512, 16.5 ->
+// 16.2 / 17.1 -> 17.7 / 21.2 -> 11.7; 32 of 14 x 14, 256 -> 256, 20.6 -> 12.3 / 21.5 -> 13.7; 77 of 11 x 11, 64 -> 192, 19.0 ->
+// 9.1 / 16.5 -> 12.0; 30 of 13 x 13, 192 -> 384, 28.0 -> 11.8 / 21.0 -> 14.7; 5 x 5, 64 of 8 x 8, 256 -> 256, 21.1 -> 20.7 / 21.8 ->
+// 21.9 / 22.9 -> 16.2; fully connected, forward / backward, 1024^3 15.6 -> 10.6 / 31.6 -> 20.3, 4096 x 1000 x 512 11.2 / 42.4 ->
+// 29.9, 2048 x 2048 x 512 9.7 / 37.5 -> 25.0, 512 x 4096 x 1024 20.5 -> 11.3 / 28.8 -> 25.1, 1500 x 700 x 3000 25.4 -> 20.8 / 45.3 ->
+// 36.9, 256 x 4096 x 4096 19.5 -> 17.1 / 42.5 -> 38.0: of 53 multiplies one is 3.5 % slower, none of the others by more than
+// two measurements differ.  (Splits that form a cluster and add their partial tiles through distributed shared memory were built and measured: 24.3 -
+// 25.0 us against 20.7 us unsplit on the first of these; the agreement over twice as many CTAs and the exchange cost what the
+// shorter main loop saves.)
 static bool pick_one_wave(niti_ctx *ctx, const GemmProblem &g, const TcParams &p, int &ctas, int &bn) {
   const int units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
   if (p.halo || p.mrep > 1 || p.dstride > 1 || p.items > 4LL * units) return false;
