@@ -193,15 +193,20 @@ class Niti:
         """niti_set_tap_cache with a buffer of ``nbytes`` owned by this object (0 removes it): the gathered
         taps of a few-channel first layer are kept between its forward and its weight-gradient call."""
         if getattr(self, "_tap", None) is not None:
-            self._tap.record_stream(torch.cuda.current_stream(self.device))    # (calls enqueued here still use it)
-        self._tap = torch.empty(nbytes, dtype=torch.uint8, device=self.device) if nbytes else None
+            self._used_here(self._tap, self._tap_stream)
+        self._tap, self._tap_stream = torch.empty(nbytes, dtype=torch.uint8, device=self.device) if nbytes else None, self._stream()
         self._ck(self.lib.niti_set_tap_cache(self.h, _ptr(self._tap), nbytes))
 
     def reserve_workspace(self, nbytes: int):
         if self._ws.numel() < nbytes:
             self._ck(self.lib.niti_begin_step(self.h, None, None, 0))      # the old buffer's headers are gone
-            self._ws.record_stream(torch.cuda.current_stream(self.device))     # (calls enqueued here still use it)
+            self._used_here(self._ws, self._ws_stream)
             self._own_workspace(nbytes)
+
+    def _used_here(self, buf, stream):
+        """Before a buffer allocated on ``stream`` is let go: calls enqueued on the current stream still use it."""
+        if stream != self._stream():                       # (else the allocator's order is the calls')
+            buf.record_stream(torch.cuda.current_stream(self.device))
 
     def buffers(self):
         """The device buffers that calls use now: a program that captures calls keeps them as long as it replays."""
@@ -210,6 +215,7 @@ class Niti:
     def _own_workspace(self, nbytes: int):
         """A new workspace, declared to the library as nobody else's (see niti_own_workspace)."""
         self._ws = self._owned_ws = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
+        self._ws_stream = self._stream()
         self._ck(self.lib.niti_own_workspace(self.h, self._ws.data_ptr(), nbytes))
 
     def begin_step(self):

@@ -3150,9 +3150,9 @@ static double kblock_cycles(const TcParams &p, int ctas, int bn, long long ctas_
 // 21.9 / 22.9 -> 16.2; fully connected, forward / backward, 1024^3 15.6 -> 10.6 / 31.6 -> 20.3, 4096 x 1000 x 512 11.2 / 42.4 ->
 // 29.9, 2048 x 2048 x 512 9.7 / 37.5 -> 25.0, 512 x 4096 x 1024 20.5 -> 11.3 / 28.8 -> 25.1, 1500 x 700 x 3000 25.4 -> 20.8 / 45.3 ->
 // 36.9, 256 x 4096 x 4096 19.5 -> 17.1 / 42.5 -> 38.0: of 53 multiplies one is 3.5 % slower, none of the others by more than
-// two measurements differ.  (Splits that form a cluster and add their partial tiles through distributed shared memory were built and measured: 24.3 -
-// 25.0 us against 20.7 us unsplit on the first of these; the agreement over twice as many CTAs and the exchange cost what the
-// shorter main loop saves.)
+// two measurements differ.  (Splits that form a cluster and add their partial tiles through distributed shared memory were
+// built and measured: 24.3 - 25.0 us against 20.7 us unsplit on the first of these; the agreement over twice as many CTAs and
+// the exchange cost what the shorter main loop saves.)
 static bool pick_one_wave(niti_ctx *ctx, const GemmProblem &g, const TcParams &p, int &ctas, int &bn) {
   const int units = p.ctas == 2 ? tc_units<2>(ctx) : tc_units<1>(ctx);
   if (p.halo || p.mrep > 1 || p.dstride > 1 || p.items > 4LL * units) return false;
