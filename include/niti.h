@@ -173,7 +173,10 @@ int niti_linear_fwd(niti_ctx *ctx, void *stream, const int8_t *a, const int32_t 
  * Both use w as it is on entry (the update is a separate call).  e_prev may be
  * NULL (first layer).  relu_mask_src, if not NULL, is an int8 [M][K] tensor
  * (the ReLU output that fed this layer); e_prev is zeroed where it is <= 0.
- * b_e, b_g: device scalars, may be NULL. */
+ * b_e, b_g: device scalars, may be NULL.  e_prev may be the storage of a, of
+ * e or of relu_mask_src, here and in niti_linear_bwd_update; likewise an
+ * output of the other multiplies that of their operands or gate (large ones
+ * then round in a second pass over int32 sums). */
 int niti_linear_bwd(niti_ctx *ctx, void *stream, const int8_t *a, const int8_t *e, const int8_t *w,
                     int8_t *e_prev, const int8_t *relu_mask_src, int8_t *g, int32_t *b_e,
                     int32_t *b_g, int M, int N, int K, int m_u, int round_mode, void *ws,

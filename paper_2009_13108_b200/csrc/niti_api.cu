@@ -550,15 +550,19 @@ static int linear_bwd_impl(niti_ctx *ctx, void *stream, const int8_t *a, const i
   pd.p0 = e; pd.p1 = w;
   fill_fc(pw, GK_FC_WGRAD, M, N, K);
   pw.p0 = e; pw.p1 = a;
+  const auto replaces = [&](const int8_t *operand, int width) {
+    const uintptr_t out = (uintptr_t)e_prev, in = (uintptr_t)operand;
+    return out < in + (uintptr_t)M * (uintptr_t)width && in < out + (uintptr_t)M * (uintptr_t)K;
+  };
+  const bool in_place = e_prev && (replaces(a, K) || replaces(e, N));      // (an operand of the gradient, too)
   {
     const RoundSpec rd = {e_prev, relu_mask_src, 7, round_mode, 0, nullptr, nullptr, nullptr, b_e, nullptr, nullptr};
     const RoundSpec rw = {g, nullptr, m_u, round_mode, 0, nullptr, nullptr, nullptr, b_g, nullptr, update_w};
-    // One launch runs both multiplies at once: an error that replaces the layer's input in place is left to the launches
-    // below, which read the input for the weight gradient before they write the error.
-    const uintptr_t e0 = (uintptr_t)e_prev, a0 = (uintptr_t)a, span = (uintptr_t)M * (uintptr_t)K;
+    // One launch runs both multiplies at once: an error that replaces the layer's input or the error above it is left to the
+    // launches below, which read them for the weight gradient before they write the error.
     int rc = NITI_ERR_SHAPE;
     if (!e_prev) rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, pw, rw, nullptr, nullptr);
-    else if (e0 >= a0 + span || a0 >= e0 + span) rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, pd, rd, &pw, &rw);
+    else if (!in_place) rc = niti_small_gemm(ctx, (cudaStream_t)stream, ws, pd, rd, &pw, &rw);
     if (rc != NITI_ERR_SHAPE) return rc;
   }
   char *pad_a = pad_mem + pad_bytes(pd) - pad_bytes(pw, 0);      // (the weight gradient finds e padded already)
@@ -568,17 +572,20 @@ static int linear_bwd_impl(niti_ctx *ctx, void *stream, const int8_t *a, const i
     pd.q0 = pw.q0 = (int8_t *)pad_mem;
     pd.ld0 = pw.ld0 = pitch16(N);
   }
-  int rc;
-  if (e_prev && update_w) {                // the error below needs the weights as they were
-    rc = run_gemm_round(ctx, (cudaStream_t)stream, pd, ws, ws_bytes, need, pad_mem, e_prev, 7, round_mode, 0,
-                        relu_mask_src, nullptr, nullptr, nullptr, b_e);
-    if (rc != NITI_OK) return rc;
-  }
-  rc = run_gemm_round(ctx, (cudaStream_t)stream, pw, ws, ws_bytes, need, pad_a, g, m_u, round_mode, 0, nullptr,
-                      nullptr, nullptr, nullptr, b_g, update_w);
-  if (rc != NITI_OK || !e_prev || update_w) return rc;
-  return run_gemm_round(ctx, (cudaStream_t)stream, pd, ws, ws_bytes, need, pad_mem, e_prev, 7, round_mode, 0,
-                        relu_mask_src, nullptr, nullptr, nullptr, b_e);
+  const auto error_below = [&]() {
+    return run_gemm_round(ctx, (cudaStream_t)stream, pd, ws, ws_bytes, need, pad_mem, e_prev, 7, round_mode, 0, relu_mask_src,
+                          nullptr, nullptr, nullptr, b_e);
+  };
+  // The error below needs the weights as they were, the gradient its operands as they were: beside an error that replaces one
+  // of them the gradient is kept until the error is there.
+  const bool error_first = e_prev && update_w && !in_place;
+  int rc = error_first ? error_below() : NITI_OK;
+  if (rc == NITI_OK)
+    rc = run_gemm_round(ctx, (cudaStream_t)stream, pw, ws, ws_bytes, need, pad_a, g, m_u, round_mode, 0, nullptr, nullptr, nullptr,
+                        nullptr, b_g, in_place ? nullptr : update_w);
+  if (rc != NITI_OK || !e_prev || error_first) return rc;
+  rc = error_below();
+  return rc == NITI_OK && update_w ? niti_launch_sgd_update(ctx, (cudaStream_t)stream, update_w, g, (long long)N * K) : rc;
 }
 
 extern "C" int niti_linear_bwd(niti_ctx *ctx, void *stream, const int8_t *a, const int8_t *e,

@@ -58,3 +58,32 @@ def test_convolution_errors_in_place_of_the_gate(niti, B, S, Ci, Co, R, pad, str
         gt = gate.clone()
         got, b_e = n.conv_dgrad(e, w, (S, S), e_prev=gt, relu_mask_src=gt, pad=pad, stride=stride)
         assert torch.equal(got, want) and int(b_e) == int(b)
+
+
+@pytest.mark.parametrize("M,N,K", [(64, 100, 256), (96, 768, 1056), (8192, 256, 2048), (500, 1000, 3000)])
+def test_update_with_the_error_in_place_of_the_input(niti, M, N, K):
+    """The gradient is that of the input as it was, the error that of the weights as they were."""
+    n = niti
+    a, e, w = _i8(9, M, K).clamp_(min=0), _i8(10, M, N), _i8(11, N, K)
+    w_want = w.clone()
+    want, b, b_g = n.linear_bwd_update(a, e, w_want, relu_mask_src=a)
+    for _ in range(2):
+        at, wt = a.clone(), w.clone()
+        got, b_e, b_gt = n.linear_bwd_update(at, e, wt, relu_mask_src=at, e_prev=at)
+        assert torch.equal(got, want) and torch.equal(wt, w_want) and (int(b_e), int(b_gt)) == (int(b), int(b_g))
+
+
+@pytest.mark.parametrize("M,N", [(64, 96), (512, 1024), (8192, 1024)])
+def test_error_in_place_of_the_error_above(niti, M, N):
+    n = niti
+    a, e, w = _i8(12, M, N).clamp_(min=0), _i8(13, M, N), _i8(14, N, N)
+    w_want = w.clone()
+    want, g, b, b_g = n.linear_bwd(a, e, w, relu_mask_src=a)
+    n.linear_bwd_update(a, e, w_want, relu_mask_src=a)
+    for _ in range(2):
+        et = e.clone()
+        got, g_t, b_e, b_gt = n.linear_bwd(a, et, w, relu_mask_src=a, e_prev=et)
+        assert torch.equal(got, want) and torch.equal(g_t, g) and (int(b_e), int(b_gt)) == (int(b), int(b_g))
+        et, wt = e.clone(), w.clone()
+        got, _, _ = n.linear_bwd_update(a, et, wt, relu_mask_src=a, e_prev=et)
+        assert torch.equal(got, want) and torch.equal(wt, w_want)

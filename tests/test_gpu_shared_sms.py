@@ -98,7 +98,7 @@ def _one_wave(n):
 
     def update():
         wt = w3.clone()
-        return list(n.linear_bwd_update(a3, e3, wt, need_e_prev=False)[2:]) + [wt]
+        return [n.linear_bwd_update(a3, e3, wt, need_e_prev=False)[-1], wt]
     return {"small": lambda: n.linear_fwd(a2, sx, w2, sw), "fc": lambda: n.linear_fwd(a, sx, w, sw, relu=True),
             "update": update, "split": lambda: n.conv_wgrad(x, ex), "loss": lambda: n.int_xent(logits, n.scalar(-6), labels)}
 
