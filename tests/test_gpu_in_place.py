@@ -87,3 +87,18 @@ def test_error_in_place_of_the_error_above(niti, M, N):
         et, wt = e.clone(), w.clone()
         got, _, _ = n.linear_bwd_update(a, et, wt, relu_mask_src=a, e_prev=et)
         assert torch.equal(got, want) and torch.equal(wt, w_want)
+
+
+@pytest.mark.parametrize("engine", [0, 1, 2, 4, 5])
+@pytest.mark.parametrize("B,S,C,R", [(64, 56, 64, 3), (20, 45, 72, 5), (40, 64, 200, 1), (100, 9, 160, 3)])
+def test_convolution_in_place_of_its_input(niti, B, S, C, R, engine):
+    n = niti
+    x, w, sx = _i8(15, B, S, S, C), _i8(16, C, R, R, C), n.scalar(-7)
+    want, _, b = n.conv_fwd(x, sx, w, sx, pad=R // 2, relu=True)
+    n.set_engine(engine)
+    try:
+        xt = x.clone()
+        _, _, b_y = n.conv_fwd(xt, sx, w, sx, y=xt, pad=R // 2, relu=True)
+    finally:
+        n.set_engine(0)
+    assert torch.equal(xt, want) and int(b_y) == int(b)
